@@ -15,6 +15,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "update.h"
+#include "wheel.h"
 
 namespace mert {
 
@@ -265,6 +266,19 @@ struct mertens_plan_s {
     WideEntry *dwide = nullptr;
     std::vector<uint32_t> wide_grid;
     bool mg_built = false;
+    // whole runs over the integers coprime to 6 (wheel.h)
+    bool wheel = false;
+    bool wheel_long = false;     // 64-bit remainders for every gathered term
+    WheelSieve ws;
+    uint32_t *dJL = nullptr, *dJD = nullptr;
+    uint64_t *dA = nullptr, *dR6 = nullptr;
+    WheelGroup *dwgroups = nullptr;
+    WheelDenseItem *dwitems = nullptr;
+    WheelGatherTile *dwtiles = nullptr;
+    uint4 *dwgitems = nullptr;
+    uint16_t *dwl = nullptr;
+    uint32_t *dwl_cnt = nullptr;
+    uint64_t wchunks = 0;        // chunks of the dense list
     // run state
     cudaEvent_t done = nullptr;
     bool ran = false;
@@ -294,6 +308,13 @@ static void block_range(const mertens_plan_s *p, uint64_t b, uint64_t *y1, uint6
 {
     *y1 = p->y_first + b * p->block_len;
     *y2 = std::min(*y1 + p->block_len - 1, p->y_last);
+}
+
+// y of block b of a wheel plan: (b block_len, b block_len + this], whole segments.
+static uint64_t wheel_block_len(const mertens_plan_s *p, uint64_t b)
+{
+    const uint64_t left = p->y_last - b * p->block_len;
+    return std::min(p->block_len, (left + kWheelSegY - 1) / kWheelSegY * kWheelSegY);
 }
 
 // Tuning in force for new plans (mertens_set_tuning); MERTENS_* environment
@@ -399,7 +420,8 @@ size_t plan_device_bytes(mertens_plan_t p)
     size_t b = 0;
     for (auto &a : p->allocs)
         b += a.second;
-    b += (size_t)p->pt.np * 25 + 2 * kPatternWords * 4;
+    b += (size_t)p->pt.np * 25 + 2 * kPatternWords * 4 + (size_t)p->ws.np * 28 +
+         p->ws.max_len / 96 + (4u << 20);
     return b;
 }
 }  // namespace mert
@@ -511,6 +533,367 @@ int mertens_describe(mertens_u128 n, mertens_u128 u, mertens_query_info *info)
     return MERTENS_OK;
 }
 
+// The rest of plan_create for a plan over the integers coprime to 6: K, JLO and
+// the dense cut-offs YCE of every entry are given.  Blocks are whole segments
+// (6144 y) of about block_len y.
+static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::vector<uint64_t> &K,
+                             const std::vector<uint64_t> &JLO, std::vector<uint64_t> &YC,
+                             uint64_t block_len, const mertens_tuning &tn)
+{
+    const size_t count = p->nq, E = K.size();
+    // cut-offs common to 64 consecutive entries of a target, at most
+    // floor(k/jlo) (beyond it no term is left); jd, the last gathered j
+    std::vector<uint32_t> JL(E), JD(E);
+    std::vector<WheelGroup> groups;
+    p->ydense = p->dense_y = p->gather_j_exec = p->jmax = 0;
+    for (size_t i = 0; i < count; ++i) {
+        const size_t o = p->off[i], X = p->X[i], ng = (X + kWheelGroup - 1) / kWheelGroup;
+        const size_t gs = groups.size();
+        groups.resize(gs + ng);
+        std::mutex mu;
+        parallel_for(ng, 256, [&](size_t glo, size_t ghi) {
+            uint64_t y_max = 0, ydense = 0, jmax = 0, dense_y = 0, exec = 0;
+            for (size_t g = glo; g < ghi; ++g) {
+                const size_t e0 = o + g * kWheelGroup, e1 = std::min(e0 + kWheelGroup, o + X);
+                uint64_t yc = UINT64_MAX;
+                for (size_t e = e0; e < e1; ++e)
+                    yc = std::min(yc, std::min(YC[e], K[e] / JLO[e]));
+                yc -= yc % 6;  // so that yc + 1 is a wheel number (tile_uniform)
+                WheelGroup &G = groups[gs + g];
+                G.first = (uint32_t)e0;
+                G.count = (uint32_t)(e1 - e0);
+                G.yc = yc;
+                G.kmax = K[e0];
+                ydense = std::max(ydense, yc);
+                dense_y += yc * (e1 - e0);
+                for (size_t e = e0; e < e1; ++e) {
+                    const uint64_t jd = std::max(K[e] / (yc + 1), JLO[e] - 1);
+                    YC[e] = yc;
+                    JL[e] = (uint32_t)JLO[e];
+                    JD[e] = (uint32_t)jd;
+                    y_max = std::max(y_max, std::max(yc, K[e] / JLO[e]));
+                    jmax = std::max(jmax, jd);
+                    exec += phi6(jd) - phi6(JLO[e] - 1);
+                }
+            }
+            std::lock_guard<std::mutex> lk(mu);
+            p->y_max = std::max(p->y_max, y_max);
+            p->ydense = std::max(p->ydense, ydense);
+            p->jmax = std::max(p->jmax, jmax);
+            p->dense_y += dense_y;
+            p->gather_j_exec += exec;
+        });
+    }
+    p->y_first = 1;
+    p->y_last = p->y_max;
+    if (block_len == 0) {
+        // one block when it fits 2^28 y, else 2^28 (up to 2^36 y) or 2^30 y blocks
+        uint64_t cap = p->y_last > (1ull << 36) ? (1ull << 30) : (1ull << 28);
+        if (tn.block_cap >= kSieveTile && tn.block_cap <= (1ull << 31))
+            cap = tn.block_cap;
+        block_len = std::min(p->y_last, cap);
+    }
+    if (block_len > (1ull << 31)) {
+        set_last_error("mertens_plan: block_len must be <= 2^31");
+        delete p;
+        return MERTENS_EINVAL;
+    }
+    block_len = std::min(block_len, p->y_last);
+    p->block_len = (block_len + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
+    p->nblocks = (p->y_last + p->block_len - 1) / p->block_len;
+
+    // ---- dense work items ----
+    std::stable_sort(groups.begin(), groups.end(),
+                     [](const WheelGroup &a, const WheelGroup &b) { return a.yc > b.yc; });
+    std::vector<uint64_t> kmax(groups.size() + 1, 0);  // largest k of the groups from g on
+    for (size_t g = groups.size(); g-- > 0;)
+        kmax[g] = std::max(kmax[g + 1], groups[g].kmax);
+    p->wchunks = (p->ydense + kWheelSegY - 1) / kWheelSegY;
+    std::vector<WheelDenseItem> ditems;
+    {
+        const size_t gpi = kWheelDenseThreads / 32;
+        double pairs = 0;
+        for (const WheelGroup &G : groups)
+            pairs += (double)(G.yc / kWheelSegY + 1);
+        // parts of a chunk's list while the items would not fill the device
+        const uint32_t parts =
+            (uint32_t)std::min(8.0, std::max(1.0, std::ceil(2400.0 * gpi / std::max(pairs, 1.0))));
+        size_t pref = groups.size();
+        for (uint64_t c = 0; c < p->wchunks; ++c) {
+            const uint64_t ys = c * kWheelSegY + 1;
+            while (pref > 0 && groups[pref - 1].yc < ys)
+                --pref;
+            // groups [0, gw) wide, [gw, gf) high-word, [gf, pref) float
+            const auto first_below = [&](double lim, bool ok) {
+                if (!ok)
+                    return pref;
+                size_t lo = 0, hi = pref;
+                while (lo < hi) {
+                    const size_t mid = (lo + hi) / 2;
+                    if ((double)kmax[mid] < lim * 6.0 * (double)ys)
+                        hi = mid;
+                    else
+                        lo = mid + 1;
+                }
+                return lo;
+            };
+            const bool small_y = ys + kWheelSegY < 350000000ull;
+            const size_t gf = first_below(1.5e6, small_y);
+            const size_t gw = std::min(gf, first_below(6.0e7, small_y && c > 0));
+            const size_t cut[4] = {0, gw, gf, pref};
+            const int mode[3] = {kDenseWide, kDenseHigh, kDenseFloat};
+            for (int m = 0; m < 3; ++m)
+                for (size_t g0 = cut[m]; g0 < cut[m + 1]; g0 += gpi)
+                    for (uint32_t q = 0; q < parts; ++q) {
+                        WheelDenseItem it;
+                        it.c = (uint32_t)c;
+                        it.g0 = (uint32_t)g0;
+                        it.g1 = (uint32_t)std::min(g0 + gpi, cut[m + 1]);
+                        it.mode_parts = (uint32_t)mode[m] | (q << 8) | (parts << 16);
+                        ditems.push_back(it);
+                    }
+        }
+    }
+    p->nitems = (uint32_t)ditems.size();
+
+    // ---- shared-memory gather tiles ----
+    std::vector<uint64_t> ycmin(E);
+    std::vector<double> kpre(E + 1, 0.0);  // prefix sums of k over all entries
+    for (size_t e = 0; e < E; ++e)
+        kpre[e + 1] = kpre[e] + (double)K[e];
+    double acc = 0;
+    for (size_t i = 0; i < count; ++i) {
+        uint64_t run = UINT64_MAX;
+        for (uint64_t x = 0; x < p->X[i]; ++x) {
+            const size_t e = p->off[i] + x;
+            run = std::min(run, YC[e]);
+            ycmin[e] = run;
+        }
+        acc += (double)p->n[i] * std::log((double)std::max<uint64_t>(p->X[i], 2));
+    }
+    {
+        // Gathered terms per y near y are about (n / y^2) ln X / 3 summed over
+        // the targets, 32768 (sum n ln X) / y^2 per tile: tiles of all entries
+        // pay while that is at least two thirds per y and a quarter of the
+        // entries a tile must check.
+        const double gs = tn.gather_scale > 0 ? tn.gather_scale : 1.0;
+        uint64_t ys = (uint64_t)(gs * std::min(std::sqrt(acc / 2.0),
+                                               std::sqrt(4.0 * kGatherTile * acc / (double)E)));
+        if (const char *e = getenv("MERTENS_GATHER_END"))
+            ys = strtoull(e, nullptr, 10);
+        p->gather_smem_end = std::min(ys, p->y_max);
+    }
+    // Blocks above: tiles over the whole block for the entries with
+    // k >= kt_fac y0^2 / 32768 (about kt_fac terms or more per tile; a prefix of
+    // each target's entries) when they have at least kt_min terms per tile
+    // together; the global path takes the others.
+    double kt_fac = 1.0, kt_min = 700.0;
+    if (const char *e = getenv("MERTENS_TILE_KT"))
+        kt_fac = atof(e);
+    if (const char *e = getenv("MERTENS_TILE_MIN"))
+        kt_min = atof(e);
+    const double item_work =
+        std::min(2.0e5, std::max(4096.0, (double)p->gather_j_exec / 2000.0));
+    std::vector<WheelGatherTile> gtiles;
+    std::vector<uint4> gitems;
+    for (uint64_t b = 0; b < p->nblocks; ++b) {
+        const uint64_t y0 = b * p->block_len, blen = wheel_block_len(p, b);
+        p->gblk.push_back((uint32_t)gitems.size());
+        uint64_t end = y0;  // y in (y0, end] goes to tiles
+        if (p->gather_smem_end > y0)
+            end = std::min(y0 + blen,
+                           (p->gather_smem_end + kWheelSegY - 1) / kWheelSegY * kWheelSegY);
+        p->gend.push_back(end);
+        uint64_t kt = UINT64_MAX;  // entries with k >= kt take this block's tiles
+        if (y0 >= p->gather_smem_end && kt_fac > 0) {
+            const double y1 = (double)y0 + 1.0, k0 = kt_fac * y1 * y1 / kGatherTile;
+            double ksum = 0;
+            for (size_t i = 0; i < count; ++i) {
+                const double xt = std::min((double)p->X[i], std::floor((double)p->n[i] / k0));
+                ksum += kpre[p->off[i] + (uint64_t)xt] - kpre[p->off[i]];
+            }
+            if (ksum * kGatherTile / (y1 * y1) >= kt_min) {
+                kt = (uint64_t)std::ceil(k0);
+                end = y0 + blen;
+            }
+        }
+        p->ktile.push_back(kt);
+        const uint64_t ntile = (end - y0 + kWheelTileY - 1) / kWheelTileY;
+        std::vector<WheelGatherTile> btiles(ntile);
+        std::vector<std::vector<uint4>> bitems(ntile);
+        parallel_for(ntile, 64, [&](size_t qlo, size_t qhi) {
+            std::vector<std::pair<uint64_t, uint64_t>> ranges;
+            for (size_t q = qlo; q < qhi; ++q) {
+                const uint64_t t0 = y0 + q * kWheelTileY;
+                WheelGatherTile &T = btiles[q];
+                T.t0 = t0;
+                T.len = (uint32_t)std::min(kWheelTileY, end - t0);
+                T.m1 = magic_of(t0 + 1);
+                T.l1 = magic_shift(t0 + 1);
+                T.m2 = magic_of(t0 + T.len + 1);
+                T.l2 = magic_shift(t0 + T.len + 1);
+                T.pad = 0;
+                // entries that can have terms: per target the suffix whose
+                // cut-off lies below the tile's end (and k >= kt: a prefix);
+                // suffixes separated by short gaps are merged
+                ranges.clear();
+                for (size_t i = 0; i < count; ++i) {
+                    const uint64_t o = p->off[i], X = p->X[i];
+                    uint64_t lo = 0, hi = X;
+                    while (lo < hi) {
+                        const uint64_t mid = (lo + hi) / 2;
+                        if (ycmin[o + mid] < t0 + T.len)
+                            hi = mid;
+                        else
+                            lo = mid + 1;
+                    }
+                    uint64_t top = X;
+                    if (kt != UINT64_MAX) {
+                        uint64_t a = 0, z = X;  // first x index with k < kt
+                        while (a < z) {
+                            const uint64_t mid = (a + z) / 2;
+                            if (K[o + mid] >= kt)
+                                a = mid + 1;
+                            else
+                                z = mid;
+                        }
+                        top = a;
+                    }
+                    if (lo >= top)
+                        continue;
+                    if (!ranges.empty() && o + lo <= ranges.back().second + 4096 &&
+                        kt == UINT64_MAX)
+                        ranges.back().second = o + top;
+                    else
+                        ranges.push_back({o + lo, o + top});
+                }
+                const double per_k = (double)T.len / 3.0 / ((double)(t0 + 1) * (double)(t0 + 1));
+                for (const auto &rg : ranges) {
+                    for (uint64_t f = rg.first; f < rg.second;) {
+                        uint64_t g = std::min<uint64_t>(f + 1024, rg.second);
+                        while (g < rg.second &&
+                               (double)(g - f) + per_k * (kpre[g] - kpre[f]) < item_work)
+                            g = std::min<uint64_t>(g + 1024, rg.second);
+                        bitems[q].push_back(make_uint4(0u, (uint32_t)f, (uint32_t)g, 0u));
+                        f = g;
+                    }
+                }
+            }
+        });
+        for (size_t q = 0; q < ntile; ++q) {
+            if (bitems[q].empty())
+                continue;
+            for (uint4 it : bitems[q]) {
+                it.x = (uint32_t)gtiles.size();
+                gitems.push_back(it);
+            }
+            gtiles.push_back(btiles[q]);
+        }
+    }
+    p->gblk.push_back((uint32_t)gitems.size());
+
+    // ---- device buffers ----
+    {
+        // chunk records of a block's global gather: an entry with cnt > 16
+        // terms posts ceil(cnt / kSparseItem); cnt is at most
+        // k (1/ylo - 1/(yend + 1)) / 3 + 2
+        double most = 0;
+        for (uint64_t b = 0; b < p->nblocks; ++b) {
+            const uint64_t y0 = b * p->block_len, yend = y0 + wheel_block_len(p, b);
+            const uint64_t ylo = p->gend[b] + 1;
+            if (ylo > yend)
+                continue;
+            const double C =
+                kpre[E] * (1.0 / (double)ylo - 1.0 / ((double)yend + 1.0)) / 3.0 + 2.0 * (double)E;
+            most = std::max(most, C / kSparseItem + std::min((double)E, C / 16.0));
+        }
+        p->qcap = (uint32_t)std::min(most * 1.01 + 256.0, 4.0e9);
+    }
+    const uint64_t wlen = p->block_len / 3;
+    p->serial = true;
+    p->dK = p->alloc<uint64_t>(E);
+    p->dYCE = p->alloc<uint64_t>(E);
+    p->dJL = p->alloc<uint32_t>(E);
+    p->dJD = p->alloc<uint32_t>(E);
+    p->dS = p->alloc<uint64_t>(2 * E);  // S, then A
+    p->dA = p->dS ? p->dS + E : nullptr;
+    p->dR6 = p->alloc<uint64_t>(E);
+    p->dR = p->alloc<uint64_t>(E);
+    p->dqueue = p->alloc<uint4>(p->qcap);
+    p->dMloc[0] = p->alloc<int16_t>(wlen);
+    p->dsegsum[0] = p->alloc<int32_t>(wlen / kSegY);
+    p->dsegoff[0] = p->alloc<int64_t>(wlen / kSegY);
+    p->dcarry = p->alloc<int64_t>(p->nblocks + 1);
+    p->derr = p->alloc<uint32_t>(4);  // status, chunk count, two work counters
+    p->dqlen = p->derr ? p->derr + 1 : nullptr;
+    p->dcounter_dense = p->derr ? p->derr + 2 : nullptr;
+    p->dcounter_gather = p->derr ? p->derr + 3 : nullptr;
+    p->dwgroups = p->alloc<WheelGroup>(groups.size());
+    p->dwitems = p->alloc<WheelDenseItem>(ditems.size());
+    p->dwtiles = p->alloc<WheelGatherTile>(gtiles.size());
+    p->dwgitems = p->alloc<uint4>(gitems.size());
+    p->dwl = p->alloc<uint16_t>(p->wchunks * kSegY);
+    p->dwl_cnt = p->alloc<uint32_t>(p->wchunks);
+    p->dqs = p->alloc<QueryDev>(count);
+    int rc = MERTENS_OK;
+    if (!p->dK || !p->dYCE || !p->dJL || !p->dJD || !p->dS || !p->dR6 || !p->dR || !p->dqueue ||
+        !p->dMloc[0] || !p->dsegsum[0] || !p->dsegoff[0] || !p->dcarry || !p->derr ||
+        !p->dwgroups || !p->dwitems || !p->dwtiles || !p->dwgitems || !p->dwl || !p->dwl_cnt ||
+        !p->dqs)
+        rc = MERTENS_ENOMEM;
+    if (rc == MERTENS_OK) {
+        const int prc = wheel_sieve_create(&p->ws, p->al, p->y_last, wlen, nullptr);
+        if (prc != 0)
+            rc = prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA;
+    }
+    if (rc == MERTENS_OK) {
+        // sieve updates: sum of 1/p + 1/p^2 over the primes 5 <= p <= sqrt(block
+        // end), per wheel number
+        std::vector<double> pre(p->ws.np + 1, 0.0);
+        for (uint32_t i = 0; i < p->ws.np; ++i) {
+            const double q = (double)p->ws.host_p[i];
+            pre[i + 1] = pre[i] + 1.0 / q + 1.0 / (q * q);
+        }
+        for (uint64_t b = 0; b < p->nblocks; ++b) {
+            const uint64_t len = wheel_block_len(p, b);
+            p->sieve_updates += (double)len / 3.0 *
+                                pre[wheel_primes_upto(&p->ws, isqrt64(b * p->block_len + len))];
+        }
+        std::vector<QueryDev> qs(count);
+        for (size_t i = 0; i < count; ++i) {
+            qs[i].X = p->X[i];
+            qs[i].off = p->off[i];
+        }
+        const auto up = [&](void *d, const void *h, size_t bytes) {
+            if (bytes)
+                cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
+            p->h2d_bytes += bytes;
+        };
+        up(p->dK, K.data(), E * 8);
+        up(p->dYCE, YC.data(), E * 8);
+        up(p->dJL, JL.data(), E * 4);
+        up(p->dJD, JD.data(), E * 4);
+        up(p->dwgroups, groups.data(), groups.size() * sizeof(WheelGroup));
+        up(p->dwitems, ditems.data(), ditems.size() * sizeof(WheelDenseItem));
+        up(p->dwtiles, gtiles.data(), gtiles.size() * sizeof(WheelGatherTile));
+        up(p->dwgitems, gitems.data(), gitems.size() * sizeof(uint4));
+        up(p->dqs, qs.data(), count * sizeof(QueryDev));
+        if (cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) != cudaSuccess ||
+            cudaGetLastError() != cudaSuccess)
+            rc = MERTENS_ECUDA;
+    }
+    if (rc != MERTENS_OK) {
+        if (rc == MERTENS_ENOMEM)
+            set_last_error("mertens_plan: device allocation failed");
+        else
+            set_last_error("mertens_plan: CUDA error %s", cudaGetErrorString(cudaGetLastError()));
+        mertens_destroy(p);
+        return rc;
+    }
+    *out = p;
+    return MERTENS_OK;
+}
+
 static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count, mertens_u128 u,
                        uint64_t block_len, const mertens_tuning &tn, bool window = false,
                        uint64_t w_first = 1, uint64_t w_last = UINT64_MAX,
@@ -568,7 +951,22 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     std::vector<uint64_t> K, JLO, JC0, YCE;
     std::vector<Group> groups;
     const char *share_env = getenv("MERTENS_SHARE");
-    const bool share_dense = !window && !(share_env && share_env[0] == '0');
+    const bool share = !(share_env && share_env[0] == '0');
+    // whole runs of one-word targets take the sums over integers coprime to 6
+    // (window plans return sums over all y; MERTENS_SHARE=0 and
+    // MERTENS_GATHER_QUOT=0 keep the full sums, MERTENS_OVERLAP the three-stream
+    // schedule, which is the full path's)
+    {
+        const char *q = getenv("MERTENS_GATHER_QUOT");
+        p->wheel = !window && !table && share && !(q && q[0] == '0') && !getenv("MERTENS_OVERLAP");
+        p->wheel_long = q && q[0] == '2';
+        for (size_t i = 0; i < count && p->wheel; ++i) {
+            const uint64_t uu = u.lo ? u.lo : target_u(n128[i], ub);
+            p->wheel = n128[i] < wide_threshold() && n128[i] / uu < (1ull << 31) &&
+                       wheel_sieve_exact(uu + 2 * kWheelSegY);
+        }
+    }
+    const bool share_dense = !window && share && !p->wheel;
     for (size_t i = 0; i < count; ++i) {
         const u128 nn = to_u128(n[i]);
         const uint64_t uu = u.lo ? u.lo : (table ? on_table_u(nn, ub, table->y_max)
@@ -816,6 +1214,8 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         delete p;
         return MERTENS_ENOTSUP;
     }
+    if (p->wheel)
+        return plan_create_wheel(out, p, K, JLO, YCE, block_len, tn);
     // ---- gathered terms shared along chains x, 2x, 4x, 8x, 16x ----
     // floor(floor(n/x)/j) = floor(n/(x j)), so entry 2x's term at j' is entry
     // x's term at j = 2j'.  The link x -> 2x (one-word entries of one target)
@@ -1427,6 +1827,137 @@ static void clear_events(mertens_plan_s *p)
     p->prof_runs = 0;
 }
 
+// One whole run of a wheel plan on one stream.
+static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
+{
+    uint64_t launches = 0;
+    int r = 0;
+    const size_t E = p->nent;
+    cudaMemsetAsync(p->dS, 0, 2 * E * 8, s);
+    cudaMemsetAsync(p->dcarry, 0, 8, s);
+    cudaMemsetAsync(p->derr, 0, 4, s);
+    bool dense_done = p->wchunks == 0;
+    for (uint64_t b = 0; b < p->nblocks && r >= 0; ++b) {
+        const uint64_t y0 = b * p->block_len, len = wheel_block_len(p, b);
+        PhaseEvents pe, pe2;
+        WheelLaunch L;
+        L.w0 = y0 / 3;
+        L.len = len / 3;
+        L.Mloc = p->dMloc[0];
+        L.segsum = p->dsegsum[0];
+        L.segoff = p->dsegoff[0];
+        L.carry_in = p->dcarry + b;
+        L.carry_out = p->dcarry + b + 1;
+        ev_begin(p, kPhSieve, s, &pe);
+        if (p->prof) {
+            pe2.phase = kPhScan;
+            cudaEventCreate(&pe2.a);
+            cudaEventCreate(&pe2.b);
+            L.mid = pe.b;
+            L.mid2 = pe2.a;
+        }
+        r = wheel_sieve_enqueue(&p->ws, L, s);
+        if (p->prof) {
+            p->evs.push_back(pe);
+            cudaEventRecord(pe2.b, s);
+            p->evs.push_back(pe2);
+        }
+        if (r < 0)
+            break;
+        launches += r;
+        const uint64_t c0 = y0 / kWheelSegY, c1 = (y0 + len) / kWheelSegY;
+        if (!dense_done) {
+            ev_begin(p, kPhDense, s, &pe);
+            r = wheel_dense_list_enqueue(p->dMloc[0], c0, std::min(c1, p->wchunks) - c0, p->dwl,
+                                         p->dwl_cnt, s);
+            if (r < 0)
+                break;
+            launches += r;
+            if (c1 >= p->wchunks) {
+                WheelDenseArgs da;
+                da.items = p->dwitems;
+                da.nitems = p->nitems;
+                da.counter = p->dcounter_dense;
+                da.groups = p->dwgroups;
+                da.K = p->dK;
+                da.dl = p->dwl;
+                da.dl_cnt = p->dwl_cnt;
+                da.S = p->dS;
+                r = wheel_dense_enqueue(da, s);
+                if (r < 0)
+                    break;
+                launches += r;
+                dense_done = true;
+            }
+            ev_end(p, s, &pe);
+        }
+        ev_begin(p, kPhGather, s, &pe);
+        if (p->gblk[b + 1] > p->gblk[b]) {
+            WheelGatherArgs ga;
+            ga.y0 = y0;
+            ga.tiles = p->dwtiles;
+            ga.items = p->dwgitems + p->gblk[b];
+            ga.nitems = p->gblk[b + 1] - p->gblk[b];
+            ga.counter = p->dcounter_gather;
+            ga.Mloc = p->dMloc[0];
+            ga.segoff = p->dsegoff[0];
+            ga.K = p->dK;
+            ga.YC = p->dYCE;
+            ga.JL = p->dJL;
+            ga.JD = p->dJD;
+            ga.S = p->dS;
+            ga.err = p->derr;
+            ga.all_long = p->wheel_long ? 1u : 0u;
+            r = wheel_gather_enqueue(ga, s);
+            if (r < 0)
+                break;
+            launches += r;
+        }
+        WheelBlockArgs ba;
+        ba.y0 = y0;
+        ba.len = len;
+        ba.ylo = p->gend[b] + 1;
+        ba.m_ylo = magic_of(ba.ylo);
+        ba.l_ylo = magic_shift(ba.ylo);
+        ba.m_end = magic_of(y0 + len + 1);
+        ba.l_end = magic_shift(y0 + len + 1);
+        ba.kmax = p->ktile[b];
+        ba.nent = E;
+        ba.K = p->dK;
+        ba.YC = p->dYCE;
+        ba.JL = p->dJL;
+        ba.JD = p->dJD;
+        ba.S = p->dS;
+        ba.A = p->dA;
+        ba.queue = p->dqueue;
+        ba.qlen = p->dqlen;
+        ba.qcap = p->qcap;
+        ba.err = p->derr;
+        ba.Mloc = p->dMloc[0];
+        ba.segoff = p->dsegoff[0];
+        r = wheel_block_enqueue(ba, s);
+        ev_end(p, s, &pe);
+        if (r < 0)
+            break;
+        launches += r;
+    }
+    if (r >= 0) {
+        PhaseEvents pe;
+        uint64_t mx = 0;
+        for (uint64_t X : p->X)
+            mx = std::max(mx, X);
+        ev_begin(p, kPhResolve, s, &pe);
+        r = wheel_resolve_enqueue(p->dqs, (uint32_t)p->nq, mx, p->dS, p->dA, p->dR6, p->dR, s);
+        ev_end(p, s, &pe);
+    }
+    if (r < 0) {
+        set_last_error("mertens_run: launch failed: %s", cudaGetErrorString(cudaGetLastError()));
+        return MERTENS_ECUDA;
+    }
+    *out = launches + r;
+    return MERTENS_OK;
+}
+
 // Enqueues one whole run (all blocks, then resolve) forked from stream
 // `origin` onto three streams and joined back: the sieve chain (block by
 // block, two output buffers), the per-block gathered updates (each after its
@@ -1436,6 +1967,8 @@ static void clear_events(mertens_plan_s *p)
 // dense and gathered updates may interleave.  *out = kernels launched.
 static int run_enqueue(mertens_plan_s *p, cudaStream_t origin, uint64_t *out)
 {
+    if (p->wheel)
+        return wheel_run(p, origin, out);
     uint64_t launches = 0;
     int r;
     const size_t E = p->nent;
@@ -1786,7 +2319,7 @@ int mertens_result(mertens_plan_t p, size_t i, int64_t *M_n, int64_t *entries, s
     if (cudaMemcpy(&err, p->derr, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
         return MERTENS_ECUDA;
     if (p->sieves) {
-        const uint32_t st = sieve_scratch_status(&p->pt);
+        const uint32_t st = p->wheel ? wheel_sieve_status(&p->ws) : sieve_scratch_status(&p->pt);
         if (st) {
             set_last_error("mertens_result: %s", sieve_status_text(st));
             return sieve_status_code(st);
@@ -2083,6 +2616,8 @@ void mertens_destroy(mertens_plan_t p)
             cudaEventDestroy(e);
     if (p->pt.np)
         prime_table_destroy(&p->pt);
+    if (p->ws.np)
+        wheel_sieve_destroy(&p->ws);
     for (auto &a : p->allocs)
         dev_free(p->al, a.first, a.second);
     delete p;

@@ -1,0 +1,169 @@
+// The wheel form of a whole run: the sums over integers coprime to 6 only.
+//
+// Let M6(v) = sum of mu(m) over m <= v coprime to 6.  Multiplying the
+// zeta function by its Euler factors at 2 and 3 in the identity of Sec. 2
+// (arXiv:1108.0135) gives, for every v >= 1,
+//   sum over j >= 1 coprime to 6 of M6(floor(v/j)) = 1,
+// and M(v) = M6(v) - M6(v/2) - M6(v/3) + M6(v/6) (floors; every m splits
+// uniquely into a divisor of 6 times a part coprime to 6 when m is
+// squarefree).  So the sieve, the gathered terms and the dense terms of the
+// method run over a third of the integers, and a last pass turns M6 of the
+// array entries into M.
+//
+// Integers coprime to 6 are numbered w = 0, 1, 2, ...: y(w) = 3w + 1 + (w & 1)
+// (6i + 1 at w = 2i, 6i + 5 at w = 2i + 1).  phi6(v) counts those <= v.
+#pragma once
+
+#include <cstdint>
+#include <cuda_runtime.h>
+
+#include "common.cuh"
+#include "internal.h"
+
+namespace mert {
+
+// y of one segment (2048 wheel numbers): every block starts at a multiple.
+constexpr uint64_t kWheelSegY = 3ull * kSegY;
+// y of a shared-memory gather tile (32768 wheel numbers, 64 KiB of int16).
+constexpr uint64_t kWheelTileY = 3ull * kGatherTile;
+
+// Number of integers in [1, v] coprime to 6: v = 6i + r has 2i + [r >= 1] +
+// [r >= 5].
+__host__ __device__ __forceinline__ uint64_t phi6(uint64_t v)
+{
+    const uint64_t i = v / 6, r = v - 6 * i;
+    return 2 * i + (r >= 1 ? 1u : 0u) + (r >= 5 ? 1u : 0u);
+}
+
+// The same for v < 2^32 - 5: with the even part e of v + 5, e / 3 - 1.
+__host__ __device__ __forceinline__ uint32_t phi6_u32(uint32_t v)
+{
+    return ((v + 5u) & ~1u) / 3u - 1u;
+}
+
+// Index of the last wheel number <= v relative to a multiple of 6 (1 <= v <
+// 2^32): phi6(v) - 1 = floor(((v - 1) & ~1) / 3).
+__host__ __device__ __forceinline__ uint32_t wheel_index(uint32_t v)
+{
+    return ((v - 1u) & ~1u) / 3u;
+}
+
+__host__ __device__ __forceinline__ uint64_t wheel_y(uint64_t w) { return 3 * w + 1 + (w & 1); }
+
+// ---- sieve ------------------------------------------------------------------
+// Sieving primes and scratch of a wheel sieve (device arrays, primes >= 5).
+struct WheelSieve {
+    Allocator al;
+    uint32_t np = 0;            // primes in the table (2 and 3 are left out)
+    uint32_t *host_p = nullptr; // host copy
+    uint32_t *p = nullptr;      // primes
+    uint4 *pat = nullptr;       // phase copies of the small primes' pattern
+    uint4 *rec = nullptr;       // per block, see wheel_prep_kernel
+    uint2 *rec2 = nullptr;
+    uint32_t *sqcnt = nullptr, *sqlist = nullptr, *err = nullptr;
+    uint64_t max_len = 0;       // wheel numbers of the largest block
+};
+
+// One block: wheel numbers [w0, w0 + len), both multiples of kSegY.
+//   M6(y(w)) = segoff[(w - w0) >> kSegShift] + Mloc[w - w0]
+struct WheelLaunch {
+    uint64_t w0 = 0, len = 0;
+    int16_t *Mloc = nullptr;
+    int32_t *segsum = nullptr;
+    int64_t *segoff = nullptr;
+    const int64_t *carry_in = nullptr;  // device M6(y(w0) - 1)
+    int64_t *carry_out = nullptr;       // device M6 of the block's end
+    cudaEvent_t mid = nullptr, mid2 = nullptr;  // profiling: after a1, before a2
+};
+
+// Primes up to sqrt(y_max) (at least 1024) and scratch for blocks of up to
+// max_len wheel numbers; y_max < 2^54.
+int wheel_sieve_create(WheelSieve *t, const Allocator &al, uint64_t y_max, uint64_t max_len,
+                       cudaStream_t s);
+void wheel_sieve_destroy(WheelSieve *t);
+uint32_t wheel_sieve_status(WheelSieve *t);
+uint32_t wheel_primes_upto(const WheelSieve *t, uint64_t b);
+int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t s);
+bool wheel_sieve_exact(uint64_t y_max);
+
+// ---- update -------------------------------------------------------------------
+constexpr uint32_t kWheelGroup = 64;     // consecutive entries with one dense cut-off
+constexpr int kWheelDenseThreads = 256;
+enum { kDenseFloat = 0, kDenseHigh = 1, kDenseWide = 2 };
+
+struct WheelGroup {
+    uint32_t first, count;  // entries
+    uint64_t yc;            // dense cut-off
+    uint64_t kmax;          // largest k of the group (0: no one-word entry)
+};
+
+// Part `part` of `parts` of chunk c's list, for groups [g0, g1).
+struct WheelDenseItem {
+    uint32_t c, g0, g1;
+    uint32_t mode_parts;    // mode | part << 8 | parts << 16
+};
+
+struct WheelDenseArgs {
+    const WheelDenseItem *items;
+    uint32_t nitems;
+    uint32_t *counter;
+    const WheelGroup *groups;
+    const uint64_t *K;
+    const uint16_t *dl;     // kSegY offsets per chunk: mu = +1, then mu = -1
+    const uint32_t *dl_cnt; // count(+1) | count(-1) << 16
+    uint64_t *S;
+};
+
+struct WheelGatherTile {
+    uint64_t t0;            // y in [t0 + 1, t0 + len], t0 a multiple of 6
+    uint64_t m1, m2;        // division magics of t0 + 1 and t0 + len + 1
+    uint32_t len, l1, l2, pad;
+};
+
+struct WheelGatherArgs {
+    uint64_t y0;            // block start: Mloc index 0 is y0 + 1
+    const WheelGatherTile *tiles;
+    const uint4 *items;     // {tile, e0, e1, 0}
+    uint32_t nitems;
+    uint32_t *counter;
+    const int16_t *Mloc;
+    const int64_t *segoff;
+    const uint64_t *K, *YC;
+    const uint32_t *JL, *JD;
+    uint64_t *S;
+    uint32_t *err;
+    uint32_t all_long;      // 64-bit remainders for every term
+};
+
+// One block (y0, y0 + len] of the global-memory path.
+struct WheelBlockArgs {
+    uint64_t y0, len;
+    uint64_t ylo;           // first y of the global path in the block
+    uint64_t m_ylo, m_end;  // division magics of ylo and y0 + len + 1
+    uint32_t l_ylo, l_end;
+    uint64_t kmax;          // entries with k >= kmax take the block's tiles
+    uint64_t nent;
+    const uint64_t *K, *YC;
+    const uint32_t *JL, *JD;
+    uint64_t *S, *A;
+    uint4 *queue;
+    uint32_t *qlen;
+    uint32_t qcap;
+    uint32_t *err;
+    const int16_t *Mloc;
+    const int64_t *segoff;
+};
+
+int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks, uint16_t *dl,
+                             uint32_t *dl_cnt, cudaStream_t s);
+int wheel_dense_enqueue(const WheelDenseArgs &a, cudaStream_t s);
+int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s);
+int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s);
+
+struct QueryDev;
+// R6[x] = M6(floor(n/x)) from the sums S, then M in R (A: the parts of M whose
+// M6 argument lies below the array).
+int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint64_t *S,
+                          const uint64_t *A, uint64_t *R6, uint64_t *R, cudaStream_t s);
+
+}  // namespace mert

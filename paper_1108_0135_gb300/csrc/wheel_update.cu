@@ -1,0 +1,851 @@
+// Steps a3 (update) and a4 (resolve) of a whole run over the integers coprime
+// to 6 (wheel.h).
+//
+// Entry x of a target n has k = floor(n/x); its M6(k) is 1 minus the sum of
+// M6(floor(k/j)) over j >= 2 coprime to 6.  The terms with j <= floor(X/x) are
+// other entries (resolve); those with floor(X/x) < j <= jd are gathered one by
+// one; the rest, where floor(k/j) <= yc, are the dense part
+//   sum over y <= yc coprime to 6 of mu(y) (phi6(floor(k/y)) - phi6(jd))
+// (exchange the order of summation: phi6(floor(k/y)) - phi6(jd) counts the
+// j > jd coprime to 6 with floor(k/j) >= y), whose second part is
+// -M6(yc) phi6(jd).  jd = max(floor(k/(yc + 1)), floor(X/x)).
+//
+// phi6 of a quotient without the quotient: with T the integer nearest
+// k / (6y) and r = k - 6yT, |r| <= 3y,
+//   phi6(floor(k/y)) = 2T - 1 + [r >= -y] + [r >= y]
+// (6T - 1 and 6T + 1 are the wheel numbers near 6T), and the value is the same
+// for T one off as long as |r| < 5y: no wheel number lies between 6T + 1 and
+// 6T + 5.  So an estimate of k / (6y) that errs by less than 1/3 before it is
+// rounded is exact, and one 32-bit remainder and two sign bits give phi6.
+#include <algorithm>
+#include <cstdint>
+
+#include "update.h"
+#include "wheel.h"
+
+namespace mert {
+
+constexpr uint32_t kMagicBits = 0x4B400000u;  // bits of 1.5 2^23: adding it rounds a float
+constexpr float kMagicF = 12582912.0f;
+
+// ---------------------------------------------------------------------------
+// Dense list: chunk c holds the wheel numbers [c kSegY, (c + 1) kSegY), one
+// segment of the sieve; dl gets the offsets of its squarefree numbers, those
+// with mu = +1 first, read off as differences of the segment's M6.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) wheel_dense_list_kernel(const int16_t *__restrict__ Mloc,
+                                                               uint64_t c0,
+                                                               uint16_t *__restrict__ dl,
+                                                               uint32_t *__restrict__ dl_cnt)
+{
+    __shared__ uint32_t sh[33];
+    const int16_t *M = Mloc + (uint64_t)blockIdx.x * kSegY;
+    const uint4 v = reinterpret_cast<const uint4 *>(M)[threadIdx.x];
+    const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
+    int prev = threadIdx.x ? M[threadIdx.x * 8 - 1] : 0;
+    int mu[8];
+    uint32_t cnt = 0;  // +1 in the low half, -1 in the high half
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const int m = (int)(int16_t)(vw[k >> 1] >> (16 * (k & 1)));
+        mu[k] = m - prev;
+        prev = m;
+        cnt += mu[k] > 0 ? 1u : (mu[k] < 0 ? 65536u : 0u);
+    }
+    uint32_t tot;
+    const uint32_t ex = block_scan_u32(cnt, sh, &tot);
+    uint32_t ip = ex & 0xffffu, im = (tot & 0xffffu) + (ex >> 16);
+    uint16_t *d = dl + (c0 + blockIdx.x) * kSegY;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) {
+        const uint16_t o = (uint16_t)(threadIdx.x * 8 + k);
+        if (mu[k] > 0)
+            d[ip++] = o;
+        else if (mu[k] < 0)
+            d[im++] = o;
+    }
+    if (threadIdx.x == 0)
+        dl_cnt[c0 + blockIdx.x] = tot;
+}
+
+// ---------------------------------------------------------------------------
+// Dense update: a warp takes the 64 entries of a group, two per lane, against
+// the staged numbers of a chunk (shared-memory broadcasts).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t count_below(const uint16_t *a, uint32_t n, uint32_t v)
+{
+    uint32_t lo = 0, hi = n;  // number of a[i] < v
+    while (lo < hi) {
+        const uint32_t mid = (lo + hi) >> 1;
+        if (a[mid] < v)
+            lo = mid + 1;
+        else
+            hi = mid;
+    }
+    return lo;
+}
+
+// acc + the sign bit of v (as a multiply-add: the kernels' other integer work is
+// on the ALU pipe).
+__device__ __forceinline__ uint32_t add_sign(uint32_t v, uint32_t acc)
+{
+    uint32_t r;
+    asm("mad.hi.u32 %0, %1, 2, %2;" : "=r"(r) : "r"(v), "r"(acc));
+    return r;
+}
+
+// Float mode: staged {1/(6y), -6y, 6y C + y, 6y C - y}, C = kMagicBits.  The
+// estimate k (1/6y) has three roundings of 2^-24 and k/(6y) < 1.5e6 (the host's
+// rule), so it errs by less than 0.27; r + y and r - y come from the biased T
+// by one multiply-add and one add each; their sign bits and the T are summed.
+// n <= 2048 terms, so the T sum stays below 2^32.
+__device__ __forceinline__ void dense_float(const uint4 *el, uint32_t n, const float kf[2],
+                                            const uint32_t kl[2], uint64_t out[2])
+{
+    uint32_t st[2] = {0, 0}, ss[2] = {0, 0};
+#pragma unroll 4
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint4 v = el[i];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t T =
+                __float_as_uint(__fmaf_rn(kf[e], __uint_as_float(v.x), kMagicF));
+            const uint32_t r = T * v.y + kl[e];
+            st[e] += T;
+            ss[e] = add_sign(r + v.z, ss[e]);
+            ss[e] = add_sign(r + v.w, ss[e]);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        out[e] = 2ull * (uint32_t)(st[e] - n * kMagicBits) + n - ss[e];
+}
+
+// High-word mode: staged {m, -6y, y}, m = floor(2^(31 + ex)/(6y)), 2^ex <= 6y of
+// the chunk; kh the top 32 bits of k, sh the shift.  Truncations of 2^-31 and
+// at most 2^-29 and one of 2^-sh (sh >= 4) with k/(6y) < 6e7: less than 0.22.
+__device__ __forceinline__ void dense_high(const uint4 *el, uint32_t n, const uint32_t kh[2],
+                                           const uint32_t sh[2], const uint32_t kl[2],
+                                           uint64_t out[2])
+{
+    uint64_t st[2] = {0, 0};
+    uint32_t ss[2] = {0, 0};
+    const uint32_t half[2] = {1u << (sh[0] - 1u), 1u << (sh[1] - 1u)};
+#pragma unroll 4
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint4 v = el[i];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t T = (__umulhi(kh[e], v.x) + half[e]) >> sh[e];
+            const uint32_t r = T * v.y + kl[e];
+            st[e] += T;
+            ss[e] = add_sign(r + v.z, ss[e]);
+            ss[e] = add_sign(r - v.z, ss[e]);
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        out[e] = 2ull * st[e] + n - ss[e];
+}
+
+// Any k < 2^63 and y < 2^60, by 64-bit division (few terms need it).
+__device__ __forceinline__ void dense_wide(const uint16_t *off, uint32_t n, uint64_t y0,
+                                           const uint64_t k[2], uint64_t out[2])
+{
+    out[0] = out[1] = 0;
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint32_t o = off[i];
+        const uint64_t y = y0 + 3u * o + 1u + (o & 1u), d = 6u * y;
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const uint64_t t = k[e] / d, rem = k[e] - t * d;
+            out[e] += 2u * t + (rem >= y ? 1u : 0u) + (rem >= 5u * y ? 1u : 0u);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDenseArgs a)
+{
+    __shared__ uint4 s_el[kSegY];
+    __shared__ uint16_t s_off[kSegY];
+    __shared__ uint32_t s_item;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    for (;;) {
+        if (threadIdx.x == 0)
+            s_item = atomicAdd(a.counter, 1u);
+        __syncthreads();
+        if (s_item >= a.nitems)
+            break;
+        const WheelDenseItem it = a.items[s_item];
+        const uint32_t mode = it.mode_parts & 255u, part = (it.mode_parts >> 8) & 255u,
+                       parts = it.mode_parts >> 16;
+        const uint32_t cnt = a.dl_cnt[it.c];
+        const uint32_t cp = cnt & 0xffffu, cm = cnt >> 16;
+        const uint32_t p0 = cp * part / parts, m0 = cm * part / parts;
+        const uint32_t np = cp * (part + 1u) / parts - p0, nm = cm * (part + 1u) / parts - m0;
+        const uint64_t y0 = (uint64_t)it.c * kWheelSegY;
+        const uint16_t *src = a.dl + (uint64_t)it.c * kSegY;
+        // float and high-word modes: y < 3.5e8
+        const uint32_t ex = 31u - __clz((uint32_t)(6u * (uint32_t)y0 + 6u));
+        for (uint32_t i = threadIdx.x; i < np + nm; i += blockDim.x) {
+            const uint32_t o = i < np ? src[p0 + i] : src[cp + m0 + (i - np)];
+            s_off[i] = (uint16_t)o;
+            const uint32_t y = (uint32_t)y0 + 3u * o + 1u + (o & 1u), d = 6u * y;
+            if (mode == kDenseFloat) {
+                const float rf = __frcp_rn(__uint2float_rn(d));
+                const uint32_t cd = kMagicBits * d;
+                s_el[i] = make_uint4(__float_as_uint(rf), 0u - d, cd + y, cd - y);
+            } else if (mode == kDenseHigh) {
+                s_el[i] = make_uint4((uint32_t)((1ull << (31u + ex)) / d), 0u - d, y, 0u);
+            }
+        }
+        __syncthreads();
+        // one group per warp; fewer groups than warps: several warps share a
+        // group, each with its part of the staged lists
+        const uint32_t ng = it.g1 - it.g0, share = ng < nwarp ? nwarp / ng : 1u;
+        for (uint32_t t = warp; t < ng * share; t += nwarp) {
+            const WheelGroup G = a.groups[it.g0 + t % ng];
+            const uint32_t q = t / ng;
+            uint64_t k[2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t i = lane + 32u * (uint32_t)e;
+                k[e] = i < G.count ? a.K[G.first + i] : 0ull;
+            }
+            uint32_t n0 = np, n1 = nm;
+            if (G.yc < y0 + kWheelSegY) {
+                const uint32_t lim = (uint32_t)(phi6(G.yc) - (uint64_t)it.c * kSegY);
+                n0 = count_below(s_off, np, lim);
+                n1 = count_below(s_off + np, nm, lim);
+            }
+            const uint32_t f0 = n0 * q / share, f1 = np + n1 * q / share;
+            n0 = n0 * (q + 1u) / share - f0;
+            n1 = n1 * (q + 1u) / share - (f1 - np);
+            uint64_t plus[2], minus[2];
+            if (mode == kDenseFloat) {
+                const float kf[2] = {__ull2float_rn(k[0]), __ull2float_rn(k[1])};
+                const uint32_t kl[2] = {(uint32_t)k[0], (uint32_t)k[1]};
+                dense_float(s_el + f0, n0, kf, kl, plus);
+                dense_float(s_el + f1, n1, kf, kl, minus);
+            } else if (mode == kDenseHigh) {
+                uint32_t kh[2], sh[2], kl[2];
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    const uint32_t b = bitlen64(k[e]);
+                    kl[e] = (uint32_t)k[e];
+                    kh[e] = b >= 32u ? (uint32_t)(k[e] >> (b - 32u)) : (uint32_t)k[e] << (32u - b);
+                    sh[e] = ex + 31u - b;
+                    if (b == 0u || sh[e] > 31u) {  // k / (6y) rounds to 0
+                        kh[e] = 0u;
+                        sh[e] = 31u;
+                    }
+                }
+                dense_high(s_el + f0, n0, kh, sh, kl, plus);
+                dense_high(s_el + f1, n1, kh, sh, kl, minus);
+            } else {
+                dense_wide(s_off + f0, n0, y0, k, plus);
+                dense_wide(s_off + f1, n1, y0, k, minus);
+            }
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t i = lane + 32u * (uint32_t)e;
+                if (i < G.count && k[e])
+                    atomicAdd(reinterpret_cast<unsigned long long *>(a.S + G.first + i),
+                              (unsigned long long)(plus[e] - minus[e]));
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Gathered terms of a shared-memory tile: y in [t0 + 1, t0 + len], len <=
+// 98304, staged as M6(y) - M6(t0) (int16: at most 24/25 of 32768 consecutive
+// wheel numbers are squarefree) by wheel index.  A term's index is
+// phi6(floor(R/j)) - 1 with R = k - t0 j < len j: T = the integer nearest
+// R / (6j) <= 2^14 from single precision (relative error near 2^-21), then as
+// above.
+// ---------------------------------------------------------------------------
+constexpr uint32_t kGatherJ32 = 300000000u;  // 32-bit remainders below: 6j < 2^31
+constexpr uint32_t kWheelLaneTerms = 16;     // few terms: always a lane per entry
+
+// v as a float (relative error at most 2^-22) from exact 16-bit pieces.
+__device__ __forceinline__ float float_pieces(uint64_t v)
+{
+    const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
+    const float f3 = __int_as_float(0x4B000000 | (hi >> 16)) - 8388608.0f;
+    const float f2 = __int_as_float(0x4B000000 | (hi & 0xffffu)) - 8388608.0f;
+    const float f1 = __int_as_float(0x4B000000 | (lo >> 16)) - 8388608.0f;
+    const float f0 = __int_as_float(0x4B000000 | (lo & 0xffffu)) - 8388608.0f;
+    return __fmaf_rn(__fmaf_rn(f3, 65536.0f, f2), 4294967296.0f, __fmaf_rn(f1, 65536.0f, f0));
+}
+
+// Constants of a run of terms j = j0 + step i in a tile.
+struct TileStep {
+    float dRf, stepf;    // step t0 / 6, step
+    uint32_t dRt, step;  // step (6 C - t0) (mod 2^32), step
+    uint64_t dR;         // step t0
+    __device__ __forceinline__ TileStep(uint64_t t0, uint32_t st)
+        : dRf(float_pieces(t0) * ((float)st / 6.0f)), stepf((float)st),
+          dRt(st * (6u * kMagicBits - (uint32_t)t0)), step(st), dR(t0 * st)
+    {
+    }
+};
+
+// State of a run: R = k - t0 j and j of the current term.  Rf = R/6 and jf are
+// stepped from the run's start with one multiply-add each; kLong (6j beyond 32
+// bits) takes the remainder in 64 bits.
+template <bool kLong>
+struct TileRun {
+    float Rf0, jf0;
+    uint32_t Rt, j;  // R + 6 j C (mod 2^32), j
+    uint64_t R;
+    __device__ __forceinline__ TileRun(uint64_t k, uint64_t t0, uint32_t j0)
+    {
+        R = k - t0 * (uint64_t)j0;
+        Rf0 = float_pieces(R) * (1.0f / 6.0f);
+        jf0 = float_pieces(j0);
+        j = j0;
+        Rt = (uint32_t)R + kMagicBits * 6u * j0;
+    }
+    // the staged value of term i (fi = i), then on to term i + 1
+    __device__ __forceinline__ int take(const int16_t *Mt, uint32_t lim, float fi,
+                                        const TileStep &d)
+    {
+        const float Rf = __fmaf_rn(fi, -d.dRf, Rf0), jf = __fmaf_rn(fi, d.stepf, jf0);
+        float rj;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rj) : "f"(jf));
+        const uint32_t T = __float_as_uint(__fmaf_rn(Rf, rj, kMagicF));
+        uint32_t s;
+        if (kLong) {
+            const uint64_t r = R - (uint64_t)(int64_t)(int32_t)(T - kMagicBits) * 6u * j;
+            s = (uint32_t)((r + j) >> 63) + (uint32_t)((r - j) >> 63);
+            R -= d.dR;
+        } else {
+            const uint32_t r = Rt - T * (6u * j);
+            s = ((r + j) >> 31) + ((r - j) >> 31);
+            Rt += d.dRt;
+        }
+        j += d.step;
+        const uint32_t i = 2u * (T - kMagicBits) - s;
+        return Mt[i < lim ? i : lim];
+    }
+};
+
+// Terms with wheel indices [wl, wh) of one entry on one lane: the two classes
+// (even and odd indices, j in steps of 6) side by side.
+template <bool kLong>
+__device__ __forceinline__ int tile_lane(const int16_t *Mt, uint64_t k, uint64_t t0, uint32_t lim,
+                                         uint32_t wl, uint32_t wh)
+{
+    const TileStep d(t0, 6u);
+    const uint32_t we = (wl + 1u) & ~1u, wo = wl | 1u;  // first even, first odd index
+    const uint32_t ne = we < wh ? (wh - we + 1u) >> 1 : 0u, no = wo < wh ? (wh - wo + 1u) >> 1 : 0u;
+    TileRun<kLong> e(k, t0, 3u * we + 1u), o(k, t0, 3u * wo + 2u);
+    const uint32_t n = ne < no ? ne : no;
+    int acc = 0;
+    float fi = 0.0f;
+#pragma unroll 2
+    for (uint32_t i = 0; i < n; ++i, fi += 1.0f)
+        acc += e.take(Mt, lim, fi, d) + o.take(Mt, lim, fi, d);
+    if (ne > n)
+        acc += e.take(Mt, lim, fi, d);
+    if (no > n)
+        acc += o.take(Mt, lim, fi, d);
+    return acc;
+}
+
+// The same on a whole warp, lanes over consecutive indices (returns the lane's part).
+template <bool kLong>
+__device__ __forceinline__ int tile_warp(const int16_t *Mt, uint64_t k, uint64_t t0, uint32_t lim,
+                                         uint32_t wl, uint32_t wh, uint32_t lane)
+{
+    const TileStep d(t0, 96u);
+    const uint32_t w = wl + lane;
+    int acc = 0;
+    if (w < wh) {
+        TileRun<kLong> r(k, t0, 3u * w + 1u + (w & 1u));
+        const uint32_t n = (wh - w + 31u) >> 5;
+        float fi = 0.0f;
+#pragma unroll 2
+        for (uint32_t i = 0; i < n; ++i, fi += 1.0f)
+            acc += r.take(Mt, lim, fi, d);
+    }
+    return acc;
+}
+
+// M6 at wheel index i of a block.
+__device__ __forceinline__ int64_t wheel_M(const int64_t *segoff, const int16_t *Mloc, uint32_t i)
+{
+    return segoff[i >> kSegShift] + (int64_t)Mloc[i];
+}
+
+// Tiles at y <= kUniformY: 64 entries of a warp (two per lane) against the same
+// j, whose constants {1/(6j), 6j, -(6jC + j) - 1, -(6jC - j) - 1} are made 32 at a
+// time by the lanes and read back as broadcasts.  T estimates k/(6j) itself (as
+// in dense_float: k/(6j) < 1.5e6 near the tile), and with the remainder negated
+// the two sign bits add up to the index: 2T - 2 + [r >= -j] + [r >= j] less the
+// tile's first index.  An index outside [lo, lim] -- a j whose y lies beyond the
+// tile or at most yc (yc + 1 a wheel number) -- is sent to the zero after it.
+// jw: 32 uint4 of this warp; b2 = -2C - 2 - (first index) - lo.
+constexpr uint64_t kUniformY = 8400000;
+
+__device__ __forceinline__ void tile_uniform(const int16_t *Mt, uint4 *jw, const uint64_t k[2],
+                                             const uint32_t b2[2], const uint32_t lo[2],
+                                             uint32_t lim, uint32_t w0, uint32_t w1, uint32_t lane,
+                                             int acc[2])
+{
+    const float kf[2] = {__ull2float_rn(k[0]), __ull2float_rn(k[1])};
+    const uint32_t nk[2] = {0u - (uint32_t)k[0], 0u - (uint32_t)k[1]};
+    const uint32_t hi[2] = {lim + 1u - lo[0], lim + 1u - lo[1]};
+    const int16_t *Ml[2] = {Mt + lo[0], Mt + lo[1]};
+    acc[0] = acc[1] = 0;
+#pragma unroll 1
+    for (uint32_t wb = w0; wb < w1; wb += 32u) {
+        {
+            const uint32_t w = wb + lane, j = 3u * w + 1u + (w & 1u), d = 6u * j;
+            const uint32_t cd = kMagicBits * d;
+            jw[lane] = make_uint4(__float_as_uint(__frcp_rn(__uint2float_rn(d))), d,
+                                  0u - (cd + j) - 1u, 0u - (cd - j) - 1u);
+        }
+        __syncwarp();
+        const uint32_t n = min(32u, w1 - wb);
+#pragma unroll 4
+        for (uint32_t i = 0; i < n; ++i) {
+            const uint4 c = jw[i];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const uint32_t T =
+                    __float_as_uint(__fmaf_rn(kf[e], __uint_as_float(c.x), kMagicF));
+                const uint32_t nr = T * c.y + nk[e];
+                const uint32_t x = add_sign(nr + c.w, add_sign(nr + c.z, b2[e]));
+                acc[e] += Ml[e][min(2u * T + x, hi[e])];
+            }
+        }
+        __syncwarp();
+    }
+}
+
+// A work item is one tile and a range of entries of one target.  Warps take 64
+// entries at a time, two per lane, and find the ranges of wheel indices of
+// their j.  Low tiles where these ranges nearly coincide take tile_uniform;
+// otherwise, 32 entries at a time, when the counts are close (or all small)
+// every lane sums its own entry, else entries with many terms take the whole
+// warp in turn.
+__global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
+{
+    extern __shared__ __align__(16) int16_t Mt[];  // kGatherTile, a zero, j constants
+    __shared__ uint32_t s_item;
+    __shared__ int64_t s_base;
+    __shared__ int32_t s_delta[kGatherTile / kSegY];
+    __shared__ uint64_t s_mbar;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    uint4 *jw = reinterpret_cast<uint4 *>(Mt + kGatherTile + 8) + warp * 32u;
+    uint32_t staged = 0xffffffffu, phase = 0;
+    if (threadIdx.x == 0) {
+        mbar_init(&s_mbar);
+        fence_proxy_async_smem();
+    }
+    for (;;) {
+        if (threadIdx.x == 0)
+            s_item = atomicAdd(a.counter, 1u);
+        __syncthreads();
+        if (s_item >= a.nitems)
+            break;
+        const uint4 I = a.items[s_item];
+        const WheelGatherTile T = a.tiles[I.x];
+        if (I.x != staged) {
+            // one bulk asynchronous copy of the block's int16 values (whole
+            // segments), then each segment's offset added in place
+            const uint32_t o1 = (uint32_t)((T.t0 - a.y0) / 3u), n = T.len / 3u;
+            if (threadIdx.x == 0) {
+                fence_proxy_async_smem();  // earlier readers of Mt passed the barrier
+                mbar_arrive_expect(&s_mbar, n * 2u);
+                bulk_copy_g2s(Mt, a.Mloc + o1, n * 2u, &s_mbar);
+                s_base = a.segoff[o1 >> kSegShift];
+            }
+            __syncthreads();
+            if (threadIdx.x == 0)
+                Mt[n] = 0;
+            if (threadIdx.x < n / kSegY)
+                s_delta[threadIdx.x] =
+                    (int32_t)(a.segoff[(o1 >> kSegShift) + threadIdx.x] - s_base);
+            if (__syncthreads_or(!mbar_wait(&s_mbar, phase & 1u))) {
+                if (threadIdx.x == 0)
+                    atomicOr(a.err, kErrTimeout);
+                mbar_wait(&s_mbar, phase & 1u);
+                return;
+            }
+            ++phase;
+            uint32_t *Mw = reinterpret_cast<uint32_t *>(Mt);
+            for (uint32_t i = threadIdx.x; i < n / 2u; i += blockDim.x) {
+                const uint32_t v = Mw[i];
+                const int32_t dl = s_delta[(2u * i) >> kSegShift];
+                const uint32_t lo = (uint32_t)((int32_t)(int16_t)(v & 0xffffu) + dl) & 0xffffu;
+                const uint32_t hi = (uint32_t)((int32_t)(int16_t)(v >> 16) + dl);
+                Mw[i] = lo | (hi << 16);
+            }
+            staged = I.x;
+        }
+        __syncthreads();
+        const int64_t base = s_base;
+        const uint32_t lim = T.len / 3u - 1u;
+        const bool low = T.t0 + T.len <= kUniformY;
+        for (uint32_t eb = I.y + warp * 64u; eb < I.z; eb += nwarp * 64u) {
+            uint64_t k[2];
+            uint32_t wl[2], wh[2];
+            bool big = a.all_long, bound = false;  // j beyond 32-bit remainders; jlo binds
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const uint32_t e = eb + 32u * (uint32_t)h + lane;
+                k[h] = 0;
+                wl[h] = wh[h] = 0;
+                if (e < I.z) {
+                    k[h] = a.K[e];
+                    const uint64_t jd = a.JD[e], jlo = a.JL[e];
+                    const uint64_t q1 = div_magic(k[h] << 1, T.m1, T.l1);  // floor(k/(t0+1))
+                    const uint64_t q2 = div_magic(k[h] << 1, T.m2, T.l2);  // floor(k/(t0+len+1))
+                    const uint64_t t = jd < q1 ? jd : q1, b = q2 + 1u > jlo ? q2 + 1u : jlo;
+                    bound |= b != q2 + 1u;
+                    if (k[h] && t >= b) {
+                        big |= t >= kGatherJ32;
+                        wl[h] = phi6_u32((uint32_t)b - 1u);
+                        wh[h] = phi6_u32((uint32_t)t);
+                    }
+                }
+            }
+            const uint32_t c0 = wh[0] - wl[0], c1 = wh[1] - wl[1];
+            const uint32_t sum = __reduce_add_sync(0xffffffffu, c0 + c1);
+            if (sum == 0)
+                continue;
+            if (low && !__any_sync(0xffffffffu, bound || big)) {
+                const uint32_t w0 = __reduce_min_sync(0xffffffffu, min(c0 ? wl[0] : 0xffffffffu,
+                                                                       c1 ? wl[1] : 0xffffffffu));
+                const uint32_t w1 = __reduce_max_sync(0xffffffffu, max(wh[0], wh[1]));
+                // 64 (w1 - w0) terms at about 12 issue slots each against
+                // `sum` at about 21
+                if (40u * (w1 - w0) <= sum) {
+                    uint32_t lo[2], b2[2];
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t e = eb + 32u * (uint32_t)h + lane;
+                        lo[h] = lim + 1u;  // no entry: nothing counts
+                        if (k[h]) {
+                            const uint64_t yc = a.YC[e];
+                            lo[h] = yc <= T.t0 ? 0u
+                                    : yc >= T.t0 + T.len ? lim + 1u
+                                                         : phi6_u32((uint32_t)(yc - T.t0));
+                        }
+                        b2[h] = 0u - 2u * kMagicBits - 2u - (uint32_t)(T.t0 / 3u) - lo[h];
+                    }
+                    int acc[2];
+                    tile_uniform(Mt, jw, k, b2, lo, lim, w0, w1, lane, acc);
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const uint32_t cnt = h ? c1 : c0;
+                        if (cnt)
+                            atomicAdd(reinterpret_cast<unsigned long long *>(a.S + eb +
+                                                                             32u * (uint32_t)h + lane),
+                                      (unsigned long long)((int64_t)acc[h] + (int64_t)cnt * base));
+                    }
+                    continue;
+                }
+            }
+            big = __any_sync(0xffffffffu, big);
+#pragma unroll 1
+            for (uint32_t h = 0; h < 2u; ++h) {
+                const uint32_t cnt = h ? c1 : c0, wlh = h ? wl[1] : wl[0], whh = h ? wh[1] : wh[0];
+                const uint64_t kh = h ? k[1] : k[0];
+                const uint32_t e0 = eb + 32u * h;
+                const uint32_t mx = __reduce_max_sync(0xffffffffu, cnt);
+                if (mx == 0)
+                    continue;
+                const bool lanes = mx <= kWheelLaneTerms ||
+                                   16u * mx <= __reduce_add_sync(0xffffffffu, cnt);
+                if (cnt && (lanes || cnt <= kWheelLaneTerms)) {
+                    const int acc = big ? tile_lane<true>(Mt, kh, T.t0, lim, wlh, whh)
+                                        : tile_lane<false>(Mt, kh, T.t0, lim, wlh, whh);
+                    atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e0 + lane),
+                              (unsigned long long)((int64_t)acc + (int64_t)cnt * base));
+                }
+                uint32_t mask = lanes ? 0u : __ballot_sync(0xffffffffu, cnt > kWheelLaneTerms);
+                while (mask) {
+                    const int src = __ffs(mask) - 1;
+                    mask &= mask - 1;
+                    const uint32_t wls = __shfl_sync(0xffffffffu, wlh, src);
+                    const uint32_t whs = __shfl_sync(0xffffffffu, whh, src);
+                    const uint64_t ks = __shfl_sync(0xffffffffu, kh, src);
+                    const int acc = big ? tile_warp<true>(Mt, ks, T.t0, lim, wls, whs, lane)
+                                        : tile_warp<false>(Mt, ks, T.t0, lim, wls, whs, lane);
+                    const int tot = __reduce_add_sync(0xffffffffu, acc);
+                    if (lane == 0)
+                        atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e0 + src),
+                                  (unsigned long long)((int64_t)tot + (int64_t)(whs - wls) * base));
+                }
+            }
+        }
+        __syncthreads();
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Global-memory part of a block (y0, y0 + len]: one lane per entry.  Gathered
+// terms with floor(k/j) in [ylo, y0 + len] of entries with k < kmax (few: here;
+// more: posted as chunks of kSparseItem wheel indices for wheel_chunk_kernel);
+// the dense form's -M6(yc) phi6(jd) when yc is in the block; and the values
+// M6(floor(k/m)), m = 2, 3, 6, of M(k) that lie in the block when m x is
+// beyond the array (m >= floor(X/x) + 1).
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
+{
+    const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint64_t k = e < a.nent ? a.K[e] : 0ull;
+    const uint64_t yend = a.y0 + a.len;
+    uint32_t wl = 0, wh = 0;
+    if (k) {
+        const uint64_t jlo = a.JL[e], jd = a.JD[e];
+        if (k < a.kmax) {
+            const uint64_t q1 = div_magic(k << 1, a.m_ylo, a.l_ylo);  // floor(k / ylo)
+            const uint64_t q2 = div_magic(k << 1, a.m_end, a.l_end);  // floor(k / (yend + 1))
+            const uint64_t t = jd < q1 ? jd : q1, b = q2 + 1u > jlo ? q2 + 1u : jlo;
+            if (t >= b) {
+                wl = phi6_u32((uint32_t)b - 1u);
+                wh = phi6_u32((uint32_t)t);
+            }
+        }
+        const uint64_t yc = a.YC[e];
+        if (yc > a.y0 && yc <= yend)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e),
+                      (unsigned long long)(0ull - (uint64_t)wheel_M(a.segoff, a.Mloc,
+                                                                    wheel_index((uint32_t)(yc - a.y0))) *
+                                                      phi6(jd)));
+        int64_t tail = 0;
+        if (jlo <= 6u && k / 6u <= yend) {
+#pragma unroll
+            for (uint32_t m = 2; m <= 6; m += (m == 2 ? 1u : 3u)) {
+                const uint64_t y = k / m;
+                if (m >= jlo && y > a.y0 && y <= yend) {
+                    const int64_t v =
+                        wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+                    tail += m == 6 ? v : -v;
+                }
+            }
+            if (tail)
+                a.A[e] += (uint64_t)tail;
+        }
+    }
+    const uint32_t cnt = wh - wl;
+    if (cnt && cnt <= kWheelLaneTerms) {
+        int64_t acc = 0;
+#pragma unroll 4
+        for (uint32_t w = wl; w < wh; ++w) {
+            const uint64_t y = k / (3ull * w + 1u + (w & 1u));
+            acc += wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+        }
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e), (unsigned long long)acc);
+    }
+    // heavy entries: chunk records, slots taken with one atomic per warp
+    const uint32_t nch = cnt > kWheelLaneTerms ? (cnt + kSparseItem - 1) / kSparseItem : 0u;
+    uint32_t incl = nch;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t nb = __shfl_up_sync(0xffffffffu, incl, o);
+        if ((int)lane >= o)
+            incl += nb;
+    }
+    const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
+    if (total == 0)
+        return;
+    uint32_t base = 0;
+    if (lane == 31)
+        base = atomicAdd(a.qlen, total);
+    base = __shfl_sync(0xffffffffu, base, 31);
+    uint32_t slot = base + incl - nch;
+    for (uint32_t c = 0; c < nch; ++c, ++slot) {
+        const uint32_t w = wl + c * (uint32_t)kSparseItem;
+        if (slot < a.qcap)
+            a.queue[slot] = make_uint4((uint32_t)e, w, min(wh - w, (uint32_t)kSparseItem), 0u);
+        else
+            atomicOr(a.err, kErrQueue);
+    }
+}
+
+// The posted chunks, a warp each (grid-stride), lanes over consecutive indices.
+__global__ void __launch_bounds__(256) wheel_chunk_kernel(WheelBlockArgs a)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t total = min(*a.qlen, a.qcap);
+    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t q = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; q < total; q += nw) {
+        const uint4 r = a.queue[q];
+        const uint64_t k = a.K[r.x];
+        int64_t acc = 0;
+#pragma unroll 4
+        for (uint32_t i = lane; i < r.z; i += 32u) {
+            const uint32_t w = r.y + i;
+            const uint64_t y = k / (3ull * w + 1u + (w & 1u));
+            acc += wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+        }
+        acc = warp_sum_i64(acc);
+        if (lane == 0)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.S + r.x), (unsigned long long)acc);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Resolve: R6[x] = 1 - S[x] - sum over j >= 2 coprime to 6, xj <= X, of R6[xj],
+// then M[x] = R6[x] - V(2x) - V(3x) + V(6x), V(z) = R6[z] within the array (the
+// values beyond it are in A).  The smallest such j is 5, so the entries of
+// (X/5^(l+1), X/5^l] only read entries above X/5^l: level by level, every entry
+// of a level in parallel, a warp per entry where an entry has many terms.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void resolve_level(const QueryDev &Q, const uint64_t *S, uint64_t *R6,
+                                              uint64_t xlo, uint64_t xhi, uint64_t tid,
+                                              uint64_t nthreads)
+{
+    const uint64_t X = Q.X, base = Q.off;
+    if (X / xhi < 64) {
+        for (uint64_t x = xlo + tid; x <= xhi; x += nthreads) {
+            const uint32_t nw = (uint32_t)phi6(X / x);
+            uint64_t acc = 0;
+            for (uint32_t w = 1; w < nw; ++w)
+                acc += R6[base + x * wheel_y(w) - 1];
+            R6[base + x - 1] = 1ull - S[base + x - 1] - acc;
+        }
+    } else {
+        const uint32_t lane = (uint32_t)tid & 31u;
+        for (uint64_t x = xlo + (tid >> 5); x <= xhi; x += nthreads >> 5) {
+            const uint32_t nw = (uint32_t)phi6(X / x);
+            uint64_t acc = 0;
+            for (uint32_t w = 1 + lane; w < nw; w += 32)
+                acc += R6[base + x * wheel_y(w) - 1];
+            acc = warp_sum_u64(acc);
+            if (lane == 0)
+                R6[base + x - 1] = 1ull - S[base + x - 1] - acc;
+        }
+    }
+}
+
+__device__ __forceinline__ void resolve_final(const QueryDev &Q, const uint64_t *A,
+                                              const uint64_t *R6, uint64_t *R, uint64_t tid,
+                                              uint64_t nthreads)
+{
+    const uint64_t X = Q.X, base = Q.off;
+    for (uint64_t x = 1 + tid; x <= X; x += nthreads) {
+        uint64_t v = R6[base + x - 1] + A[base + x - 1];
+        if (2 * x <= X)
+            v -= R6[base + 2 * x - 1];
+        if (3 * x <= X)
+            v -= R6[base + 3 * x - 1];
+        if (6 * x <= X)
+            v += R6[base + 6 * x - 1];
+        R[base + x - 1] = v;
+    }
+}
+
+// A CTA per target, all levels.
+__global__ void __launch_bounds__(1024) wheel_resolve_kernel(const QueryDev *__restrict__ qs,
+                                                             const uint64_t *__restrict__ S,
+                                                             const uint64_t *__restrict__ A,
+                                                             uint64_t *R6, uint64_t *R)
+{
+    const QueryDev Q = qs[blockIdx.x];
+    for (uint64_t hi = Q.X; hi >= 1; hi /= 5) {
+        resolve_level(Q, S, R6, hi / 5 + 1, hi, threadIdx.x, blockDim.x);
+        __syncthreads();
+    }
+    resolve_final(Q, A, R6, R, threadIdx.x, blockDim.x);
+}
+
+// One level (the last launch: the values of M) of every target, several CTAs each.
+__global__ void __launch_bounds__(256) wheel_resolve_level_kernel(const QueryDev *__restrict__ qs,
+                                                                  const uint64_t *__restrict__ S,
+                                                                  const uint64_t *__restrict__ A,
+                                                                  uint64_t *R6, uint64_t *R,
+                                                                  uint64_t div, uint32_t last)
+{
+    const QueryDev Q = qs[blockIdx.y];
+    const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
+    const uint64_t hi = Q.X / div;
+    if (last)
+        resolve_final(Q, A, R6, R, tid, nt);
+    else if (hi)
+        resolve_level(Q, S, R6, hi / 5 + 1, hi, tid, nt);
+}
+
+// ---------------------------------------------------------------------------
+// Launchers.
+// ---------------------------------------------------------------------------
+static int sm_count()
+{
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks, uint16_t *dl,
+                             uint32_t *dl_cnt, cudaStream_t s)
+{
+    wheel_dense_list_kernel<<<(unsigned)nchunks, 256, 0, s>>>(Mloc, c0, dl, dl_cnt);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int wheel_dense_enqueue(const WheelDenseArgs &a, cudaStream_t s)
+{
+    if (a.nitems == 0)
+        return 0;
+    int per = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, wheel_dense_kernel, kWheelDenseThreads, 0);
+    const uint32_t grid = std::min<uint32_t>((uint32_t)(sm_count() * std::max(per, 1)), a.nitems);
+    cudaMemsetAsync(a.counter, 0, 4, s);
+    wheel_dense_kernel<<<grid, kWheelDenseThreads, 0, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s)
+{
+    if (a.nitems == 0)
+        return 0;
+    static std::atomic<uint64_t> attr_devs{0};
+    const int smem = kGatherTile * 2 + 16 + 16 * 32 * 16;
+    const uint64_t dbit = device_bit();
+    if (attrs_needed(attr_devs, dbit)) {
+        cudaFuncSetAttribute(wheel_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        attrs_done(attr_devs, dbit);
+    }
+    int per = 0;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, wheel_gather_kernel, 512, smem);
+    const uint32_t grid = std::min<uint32_t>((uint32_t)(sm_count() * std::max(per, 1)), a.nitems);
+    cudaMemsetAsync(a.counter, 0, 4, s);
+    wheel_gather_kernel<<<grid, 512, smem, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s)
+{
+    cudaMemsetAsync(a.qlen, 0, 4, s);
+    wheel_range_kernel<<<(unsigned)((a.nent + 255) / 256), 256, 0, s>>>(a);
+    const uint32_t grid = std::min<uint32_t>((uint32_t)sm_count() * 8u, (a.qcap + 7u) / 8u);
+    wheel_chunk_kernel<<<grid, 256, 0, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 2 : -1;
+}
+
+int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint64_t *S,
+                          const uint64_t *A, uint64_t *R6, uint64_t *R, cudaStream_t s)
+{
+    if (max_x <= 16384 || nq >= 32) {
+        wheel_resolve_kernel<<<nq, 1024, 0, s>>>(qs, S, A, R6, R);
+        return cudaGetLastError() == cudaSuccess ? 1 : -1;
+    }
+    int n = 0;
+    const dim3 grid((unsigned)std::min<uint64_t>((max_x + 255) / 256, 608), nq);
+    for (uint64_t div = 1; div <= max_x; div *= 5, ++n)
+        wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, S, A, R6, R, div, 0u);
+    wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, S, A, R6, R, 1, 1u);
+    return cudaGetLastError() == cudaSuccess ? n + 1 : -1;
+}
+
+}  // namespace mert

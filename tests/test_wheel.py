@@ -1,0 +1,82 @@
+"""The sums over integers coprime to 6 (csrc/wheel.h): CPU models of the
+identities and of the remainder rule the kernels use, and, on the GPU, whole
+runs of that form against runs of the full sums (MERTENS_SHARE=0)."""
+import math
+import random
+
+import numpy as np
+import pytest
+
+import oracle
+import paper_1108_0135_gb300 as pm
+
+
+def phi6(v):
+    i, r = divmod(v, 6)
+    return 2 * i + (r >= 1) + (r >= 5)
+
+
+def test_identities_over_integers_coprime_to_6():
+    """Sum over j coprime to 6 of M6(floor(v/j)) = 1, and M from M6."""
+    top = 3000
+    M = oracle.mertens_table(top)
+    mu = np.diff(M, prepend=0)
+    M6 = np.cumsum([int(mu[m]) if m % 2 and m % 3 else 0 for m in range(top + 1)])
+    for v in list(range(1, 200)) + [997, 1000, 2310, 3000]:
+        assert sum(M6[v // j] for j in range(1, v + 1) if math.gcd(j, 6) == 1) == 1
+        assert M[v] == M6[v] - M6[v // 2] - M6[v // 3] + M6[v // 6]
+
+
+def test_phi6_from_an_estimate_off_by_less_than_a_third():
+    """phi6(floor(k/y)) = 2T - 1 + [r >= -y] + [r >= y], r = k - 6yT, for every
+    integer T within 1/2 + 1/3 of k/(6y)."""
+    rng = random.Random(6)
+    for _ in range(20000):
+        y = rng.choice([1, 5, 7, rng.randrange(1, 50), rng.randrange(1, 10**8)])
+        k = rng.choice([rng.randrange(1, 200) * y + rng.randrange(-1, 2),
+                        rng.randrange(1, 10**15)])
+        if k < 1:
+            continue
+        # integers T with |6yT - k| < 6y (1/2 + 1/3) = 5y
+        for T in range((k - 5 * y) // (6 * y) + 1, (k + 5 * y - 1) // (6 * y) + 1):
+            r = k - 6 * y * T
+            assert 2 * T - 1 + (r >= -y) + (r >= y) == phi6(k // y), (k, y, T)
+
+
+def test_index_forms():
+    """The 32-bit forms of phi6 and of the index of the last wheel number."""
+    for v in list(range(0, 200)) + [2**31 - 1, 2**31, 2**32 - 6]:
+        assert ((v + 5) & ~1) // 3 - 1 == phi6(v)
+        if v:
+            assert ((v - 1) & ~1) // 3 == phi6(v) - 1
+    for w in range(100):
+        y = 3 * w + 1 + (w & 1)
+        assert math.gcd(y, 6) == 1 and phi6(y) == w + 1
+
+
+def _arrays(ns, u, bl):
+    plan = pm.mertens_plan(ns, u, bl)
+    try:
+        pm.mertens_run(plan)
+        return [pm.mertens_result(plan, i, entries=True)[1] for i in range(len(ns))]
+    finally:
+        pm.mertens_destroy(plan)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ns,u,bl", [
+    ([7 * 10**9 + 1], 3 * 10**5, 0),             # u near sqrt(n): bounds of floor(X/x) in low tiles
+    ([10**13 + 7], 0, 6144 * 1000),              # every dense mode; blocks of whole segments
+    ([10**13 + 7], 5 * 10**8 + 3, 10**7 + 1),    # ragged blocks, tiles cut at block ends
+    ([3 * 10**14 + 11], 0, 0),                   # blocks above the tile range
+    ([10**12, 10**12 + 10**6, 5 * 10**9 + 9, 12345, 6, 1], 0, 0),  # several targets
+])
+@pytest.mark.parametrize("quot", [None, "2"])
+def test_wheel_runs_equal_full_sums(ns, u, bl, quot, monkeypatch):
+    monkeypatch.setenv("MERTENS_SHARE", "0")
+    full = _arrays(ns, u, bl)
+    monkeypatch.delenv("MERTENS_SHARE")
+    if quot:
+        monkeypatch.setenv("MERTENS_GATHER_QUOT", quot)  # 64-bit remainders
+    for a, b in zip(full, _arrays(ns, u, bl)):
+        assert np.array_equal(a, b)
