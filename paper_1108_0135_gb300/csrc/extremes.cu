@@ -178,7 +178,7 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
     int rc = MERTENS_OK;
     int prc = prime_table_create(&pt, al, y_last, s);
     if (prc == 0)
-        prc = sieve_scratch_create(&pt, L);
+        prc = sieve_scratch_create(&pt, L, s);
     if (prc != 0)
         rc = prc == 6 ? MERTENS_ENOTSUP : (prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA);
     const uint64_t nseg = sieve_segments(L);

@@ -63,6 +63,9 @@ struct PrimeTable {
     // host copy of the primes (for counting primes <= a bound)
     uint32_t *host_p = nullptr;
     Allocator al;
+    // the device allocations behind the tables and the scratch
+    void *base = nullptr, *scratch = nullptr;
+    size_t base_bytes = 0, scratch_bytes = 0;
 };
 
 // Arguments of one sieve block (steps a1 + a2, fused).  Results:
@@ -89,7 +92,7 @@ void prime_table_destroy(PrimeTable *t);
 // Scratch of the persistent byte sieve for blocks of up to max_len y (bucket
 // storage sized from the table's primes above 2^17, and the square bit
 // array).  Optional: without it blocks take the per-tile byte kernel.
-int sieve_scratch_create(PrimeTable *t, uint64_t max_len);
+int sieve_scratch_create(PrimeTable *t, uint64_t max_len, cudaStream_t s);
 // Status bits the persistent sieve left since the last call (and clears them):
 // kErrBucket when a bucket overflowed (the block's M(y) is then wrong).
 uint32_t sieve_scratch_status(PrimeTable *t);

@@ -1668,7 +1668,7 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     if (rc == MERTENS_OK && p->sieves) {
         int prc = prime_table_create(&p->pt, p->al, std::max<uint64_t>(p->y_last, 1), nullptr);
         if (prc == 0)
-            prc = sieve_scratch_create(&p->pt, block_len);
+            prc = sieve_scratch_create(&p->pt, block_len, nullptr);
         if (prc != 0)
             rc = prc == 6 ? MERTENS_ENOTSUP : (prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA);
     }
@@ -2721,21 +2721,25 @@ static int sieve_window(uint64_t y1, uint64_t len, int8_t *mu_dev, int64_t carry
     PrimeTable pt;
     int prc = prime_table_create(&pt, al, y1 + len - 1, s);
     if (prc == 0 && len <= (1ull << 30))
-        prc = sieve_scratch_create(&pt, len);
+        prc = sieve_scratch_create(&pt, len, s);
     if (prc != 0) {
         if (pt.np)
             prime_table_destroy(&pt);
         return prc == 6 ? MERTENS_ENOTSUP : (prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA);
     }
+    // one allocation: M(y), segment sums and offsets, carries, status word
     const uint64_t nseg = sieve_segments(len);
-    int16_t *ml = (int16_t *)dev_alloc(al, (len + 2) * 2);
-    int32_t *ss = (int32_t *)dev_alloc(al, nseg * 4);
-    int64_t *so = (int64_t *)dev_alloc(al, nseg * 8);
-    int64_t *cy = (int64_t *)dev_alloc(al, 16);
-    uint32_t *er = (uint32_t *)dev_alloc(al, 4);
-    int rc = MERTENS_OK;
-    if (!ml || !ss || !so || !cy || !er)
-        rc = MERTENS_ENOMEM;
+    const auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    const size_t b_ml = up((len + 2) * 2), b_ss = up(nseg * 4), b_so = up(nseg * 8);
+    const size_t bytes = b_ml + b_ss + b_so + 256;
+    char *buf = (char *)dev_alloc(al, bytes);
+    int16_t *ml = (int16_t *)buf;
+    int32_t *ss = (int32_t *)(buf + b_ml);
+    int64_t *so = (int64_t *)(buf + b_ml + b_ss);
+    int64_t *cy = (int64_t *)(buf + b_ml + b_ss + b_so);
+    // the sieve's status word where it has one (its bits differ)
+    uint32_t *er = pt.perr ? pt.perr : (uint32_t *)(cy + 2);
+    int rc = buf ? MERTENS_OK : MERTENS_ENOMEM;
     if (rc == MERTENS_OK) {
         cudaMemcpyAsync(cy, &carry, 8, cudaMemcpyHostToDevice, s);
         cudaMemsetAsync(er, 0, 4, s);
@@ -2760,23 +2764,17 @@ static int sieve_window(uint64_t y1, uint64_t len, int8_t *mu_dev, int64_t carry
             rc = MERTENS_ECUDA;
         // the sieve's own status first: a tile it gave up on leaves garbage
         // that the int32 check below would report instead
-        if (rc == MERTENS_OK) {
-            const uint32_t st = sieve_scratch_status(&pt);
-            if (st) {
-                set_last_error("sieve: %s", sieve_status_text(st));
-                rc = sieve_status_code(st);
-            }
+        const uint32_t st = e & ~kErrMOverflow;
+        if (rc == MERTENS_OK && st) {
+            set_last_error("sieve: %s", sieve_status_text(st));
+            rc = sieve_status_code(st);
         }
         if (rc == MERTENS_OK && (e & kErrMOverflow))
             rc = MERTENS_EOVERFLOW;
     }
     if (rc == MERTENS_ECUDA)
         set_last_error("sieve: %s", cudaGetErrorString(cudaGetLastError()));
-    dev_free(al, ml, (len + 2) * 2);
-    dev_free(al, ss, nseg * 4);
-    dev_free(al, so, nseg * 8);
-    dev_free(al, cy, 16);
-    dev_free(al, er, 4);
+    dev_free(al, buf, bytes);
     prime_table_destroy(&pt);
     return rc;
 }

@@ -1336,16 +1336,17 @@ __global__ void expand_M_kernel(const int16_t *__restrict__ Mloc, const int64_t 
 // ---------------------------------------------------------------------------
 // Host side.
 // ---------------------------------------------------------------------------
+// Primes <= B (B >= 7), by a sieve of the odd numbers 2i + 1.
 static std::vector<uint32_t> host_primes(uint64_t B)
 {
-    std::vector<uint8_t> comp(B + 1, 0);
-    std::vector<uint32_t> out;
-    for (uint64_t i = 2; i <= B; ++i) {
-        if (comp[i])
+    std::vector<uint8_t> comp(B / 2 + 1, 0);
+    std::vector<uint32_t> out(1, 2u);
+    for (uint64_t q = 3; q <= B; q += 2) {
+        if (comp[q >> 1])
             continue;
-        out.push_back((uint32_t)i);
-        for (uint64_t j = i * i; j <= B; j += i)
-            comp[j] = 1;
+        out.push_back((uint32_t)q);
+        for (uint64_t j = q * q; j <= B; j += 2 * q)
+            comp[j >> 1] = 1;
     }
     return out;
 }
@@ -1360,141 +1361,107 @@ static uint64_t isqrt_u64(uint64_t v)
     return r;
 }
 
-// Odd integer nearest S log2 p (ties upward).
-static uint32_t byte_weight(uint32_t p, uint32_t S)
+// The odd integer nearest S log2 p, 2 floor(S log2(p) / 2) + 1, for S = 2, 3, 4 in
+// whole numbers: floor(log2 p), floor(log2 p^3) / 2, floor(log2 p^2).
+__device__ __forceinline__ uint32_t byte_weight(uint32_t p, uint32_t S)
 {
-    const double x = S * std::log2((double)p);
-    return 2u * (uint32_t)std::floor((x - 1.0) / 2.0 + 0.5) + 1u;
+    if (S == 2)
+        return 2u * (31u - __clz(p)) + 1u;
+    const uint64_t q = (uint64_t)p * p;
+    if (S == 4)
+        return 2u * (63u - (uint32_t)__clzll((long long)q)) + 1u;
+    const uint64_t lo = q * p, hi = __umul64hi(q, p);
+    const uint32_t l = hi ? 127u - (uint32_t)__clzll((long long)hi)
+                          : 63u - (uint32_t)__clzll((long long)lo);
+    return 2u * (l >> 1) + 1u;
 }
 
-// Host copies of the byte sieve's pre-sieve tables for weight scale S (they
-// depend on S only): built once per process and kept.
-struct BytePatterns {
-    std::vector<uint8_t> p8;     // 16 phase copies of the 2, 3, 5, 7 byte pattern
-    std::vector<uint32_t> psq;   // square flags of 4, 9, 25, 49 as a bit string
-};
-
-static const BytePatterns &byte_patterns(uint32_t S)
+// Everything a prime's records hold, from the prime alone (the host uploads
+// only the primes).
+__global__ void prime_records_kernel(uint32_t np, const uint32_t *__restrict__ primes,
+                                     uint32_t *__restrict__ lg, uint64_t *__restrict__ m,
+                                     uint8_t *__restrict__ l, uint32_t S, uint4 *__restrict__ pq,
+                                     uint4 *__restrict__ pq2, uint32_t *__restrict__ pw)
 {
-    static std::mutex mu;
-    static BytePatterns cache[5];
-    std::lock_guard<std::mutex> lk(mu);
-    BytePatterns &bp = cache[S < 5 ? S : 4];
-    if (!bp.p8.empty())
-        return bp;
-    uint32_t w[4];
+    const uint32_t t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= np)
+        return;
+    const uint32_t p = primes[t];
+    lg[t] = (uint32_t)(kLogScale * log2f((float)p) + 0.5f);
+    m[t] = magic_of(p);
+    l[t] = (uint8_t)magic_shift(p);
+    if (!S)
+        return;
+    unsigned s1 = 0, s2 = 0;
+    const uint32_t m1 = magic32_of(p, &s1);
+    const uint64_t p2 = (uint64_t)p * p;
+    const uint32_t m2 = p2 < (1ull << 30) ? magic32_of((uint32_t)p2, &s2) : 0u;
+    const uint32_t w = byte_weight(p, S);
+    pq[t] = make_uint4(p, m1, m2, s1 | (s2 << 8) | (w << 16));
+    pq2[t] = make_uint4(p, m1, m2, s1 | (s2 << 8) | (byte_weight(p, 2) << 16));
+    if (p < (1u << 17))
+        pw[t] = p | (w << 24);
+}
+
+// The pre-sieve patterns of 2, 3, 5, 7 and their squares: the 16-bit kernel's two
+// word tables; with S, the byte kernels' phase copies (copy k starts at phase k)
+// of weights at scale S, square flags as a bit string, and weights at scale 2
+// with base 1 and the flags in bit 7.
+__global__ void sieve_pattern_kernel(uint32_t *__restrict__ even, uint32_t *__restrict__ odd,
+                                     uint32_t S, uint8_t *__restrict__ pat8,
+                                     uint32_t *__restrict__ patsq, uint8_t *__restrict__ pat2)
+{
     const uint32_t small[4] = {2, 3, 5, 7};
-    for (int q = 0; q < 4; ++q)
+    const auto half = [&](uint32_t i) {  // log sum, prime count and square flag of phase i
+        uint32_t h = 0;
+        for (int q = 0; q < 4; ++q) {
+            if (i % small[q] == 0)
+                h += (uint32_t)(kLogScale * log2f((float)small[q]) + 0.5f) | kCountOne;
+            if (i % (small[q] * small[q]) == 0)
+                h |= kSquareBit;
+        }
+        return h;
+    };
+    const uint32_t n = gridDim.x * blockDim.x, t = blockIdx.x * blockDim.x + threadIdx.x;
+    for (uint32_t j = t; j < kPatternWords; j += n) {
+        even[j] = half(2 * j) | (half(2 * j + 1) << 16);
+        odd[j] = half(2 * j + 1) | (half((2 * j + 2) % kPatternPeriod) << 16);
+    }
+    if (!S)
+        return;
+    uint32_t w[4], w2[4];
+    for (int q = 0; q < 4; ++q) {
         w[q] = byte_weight(small[q], S);
-    std::vector<uint8_t> pat(kPatternPeriod);
-    std::vector<uint8_t> sqp(kPatternPeriod);
-    for (uint32_t i = 0; i < kPatternPeriod; ++i) {
-        uint32_t b = 0, f = 0;
+        w2[q] = byte_weight(small[q], 2);
+    }
+    const auto byte = [&](uint32_t i, const uint32_t *wt, uint32_t base, uint32_t flag) {
+        uint32_t b = base, f = 0;
         for (int q = 0; q < 4; ++q) {
-            if (i % small[q] == 0)
-                b += w[q];
-            if (i % (small[q] * small[q]) == 0)
-                f = 1;
+            b += i % small[q] == 0 ? wt[q] : 0u;
+            f |= i % (small[q] * small[q]) == 0 ? flag : 0u;
         }
-        pat[i] = (uint8_t)b;
-        sqp[i] = (uint8_t)f;
-    }
-    bp.p8.resize((size_t)16 * kPat8Len);
-    for (uint32_t k = 0; k < 16; ++k)
-        for (uint32_t j = 0; j < kPat8Len; ++j)
-            bp.p8[(size_t)k * kPat8Len + j] = pat[(k + j) % kPatternPeriod];
-    bp.psq.assign(kPatSqWords, 0u);
-    for (uint32_t j = 0; j < 32u * kPatSqWords; ++j)
-        if (sqp[j % kPatternPeriod])
-            bp.psq[j >> 5] |= 1u << (j & 31u);
-    return bp;
-}
-
-// Host copy of the scale-2 byte pattern (see mu_sieve_t2_kernel), 16 phase
-// copies (copy k starts at phase k), built once per process: 1 + the weights
-// of 2, 3, 5, 7, plus 128 where 4, 9, 25 or 49 divides (period 44100).
-struct T2Patterns {
-    std::vector<uint8_t> a;
-};
-
-static const T2Patterns &t2_patterns()
-{
-    static std::mutex mu;
-    static T2Patterns tp;
-    std::lock_guard<std::mutex> lk(mu);
-    if (!tp.a.empty())
-        return tp;
-    const uint32_t small[4] = {2, 3, 5, 7};
-    std::vector<uint8_t> pat(kPatternPeriod);
-    for (uint32_t i = 0; i < kPatternPeriod; ++i) {
-        uint32_t b = 1;
-        for (int q = 0; q < 4; ++q) {
-            if (i % small[q] == 0)
-                b += byte_weight(small[q], 2);
-            if (i % (small[q] * small[q]) == 0)
-                b |= 128u;
+        return b | f;
+    };
+    for (uint32_t k = 0; k < 16; ++k) {
+        for (uint32_t j = t; j < kPat8Len / 4u; j += n) {
+            uint32_t v = 0;
+            for (uint32_t b = 0; b < 4; ++b)
+                v |= byte(k + 4u * j + b, w, 0u, 0u) << (8u * b);
+            reinterpret_cast<uint32_t *>(pat8 + (size_t)k * kPat8Len)[j] = v;
         }
-        pat[i] = (uint8_t)b;
+        for (uint32_t j = t; j < kPat2Len / 4u; j += n) {
+            uint32_t v = 0;
+            for (uint32_t b = 0; b < 4; ++b)
+                v |= byte(k + 4u * j + b, w2, 1u, 128u) << (8u * b);
+            reinterpret_cast<uint32_t *>(pat2 + (size_t)k * kPat2Len)[j] = v;
+        }
     }
-    tp.a.resize((size_t)16 * kPat2Len);
-    for (uint32_t k = 0; k < 16; ++k)
-        for (uint32_t j = 0; j < kPat2Len; ++j)
-            tp.a[(size_t)k * kPat2Len + j] = pat[(k + j) % kPatternPeriod];
-    return tp;
-}
-
-// Tables of the byte sieve (see mu_sieve_byte_kernel).
-static int byte_tables_create(PrimeTable *t, const std::vector<uint32_t> &pr, cudaStream_t s)
-{
-    const size_t np = pr.size();
-    std::vector<uint4> pq(np);
-    for (size_t i = 0; i < np; ++i) {
-        const uint32_t p = pr[i];
-        unsigned s1 = 0, s2 = 0;
-        const uint32_t m1 = magic32_of(p, &s1);
-        const uint64_t p2 = (uint64_t)p * p;
-        const uint32_t m2 = p2 < (1ull << 30) ? magic32_of((uint32_t)p2, &s2) : 0u;
-        pq[i] = make_uint4(p, m1, m2, s1 | (s2 << 8) | (byte_weight(p, t->byte_scale) << 16));
+    for (uint32_t j = t; j < kPatSqWords; j += n) {
+        uint32_t v = 0;
+        for (uint32_t b = 0; b < 32; ++b)
+            v |= (half(32u * j + b) & kSquareBit ? 1u : 0u) << b;
+        patsq[j] = v;
     }
-    const BytePatterns &bp = byte_patterns(t->byte_scale);
-    const std::vector<uint8_t> &p8 = bp.p8;
-    const std::vector<uint32_t> &psq = bp.psq;
-    // p | w << 24 for the primes below 2^17
-    uint32_t nmid = 0;
-    while (nmid < np && pr[nmid] < (1u << 17))
-        ++nmid;
-    t->np_mid = nmid;
-    std::vector<uint32_t> pwv(nmid + 1, 0u);
-    for (uint32_t i = 0; i < nmid; ++i)
-        pwv[i] = pr[i] | (byte_weight(pr[i], t->byte_scale) << 24);
-    t->pw = (uint32_t *)dev_alloc(t->al, (nmid + 1) * 4);
-    if (!t->pw)
-        return 2;
-    cudaMemcpyAsync(t->pw, pwv.data(), (nmid + 1) * 4, cudaMemcpyHostToDevice, s);
-    t->pq = (uint4 *)dev_alloc(t->al, np * sizeof(uint4));
-    t->blk_r2 = (uint64_t *)dev_alloc(t->al, np * 8);
-    t->pat8 = (uint4 *)dev_alloc(t->al, p8.size());
-    t->patsq = (uint32_t *)dev_alloc(t->al, kPatSqWords * 4);
-    if (!t->pq || !t->blk_r2 || !t->pat8 || !t->patsq)
-        return 2;
-    cudaMemcpyAsync(t->pq, pq.data(), np * sizeof(uint4), cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->pat8, p8.data(), p8.size(), cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->patsq, psq.data(), kPatSqWords * 4, cudaMemcpyHostToDevice, s);
-    // scale-2 records: the same constants with w2(p) in place of w(p)
-    for (size_t i = 0; i < np; ++i)
-        pq[i].w = (pq[i].w & 0xffffu) | (byte_weight(pr[i], 2) << 16);
-    const T2Patterns &tp = t2_patterns();
-    t->pq2 = (uint4 *)dev_alloc(t->al, np * sizeof(uint4));
-    t->pat2 = (uint4 *)dev_alloc(t->al, tp.a.size());
-    t->rec = (uint4 *)dev_alloc(t->al, np * sizeof(uint4));
-    t->rec2 = (uint2 *)dev_alloc(t->al, np * sizeof(uint2));
-    if (!t->pq2 || !t->pat2 || !t->rec || !t->rec2)
-        return 2;
-    cudaMemcpyAsync(t->pq2, pq.data(), np * sizeof(uint4), cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->pat2, tp.a.data(), tp.a.size(), cudaMemcpyHostToDevice, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess)
-        return 3;
-    return 0;
 }
 
 int prime_table_create(PrimeTable *t, const Allocator &al, uint64_t y_max, cudaStream_t s,
@@ -1508,95 +1475,63 @@ int prime_table_create(PrimeTable *t, const Allocator &al, uint64_t y_max, cudaS
         return 6;
     std::vector<uint32_t> pr = host_primes(B);
     const size_t np = pr.size();
-    std::vector<uint32_t> lg(np);
-    std::vector<uint64_t> mg(np);
-    std::vector<uint8_t> sh(np);
-    for (size_t i = 0; i < np; ++i) {
-        lg[i] = (uint32_t)std::lround(kLogScale * std::log2((double)pr[i]));
-        mg[i] = magic_of(pr[i]);
-        sh[i] = (uint8_t)magic_shift(pr[i]);
-    }
-    // half-word pattern for 2,3,5,7 and 4,9,25,49, then the two word tables
-    std::vector<uint32_t> pat16(kPatternPeriod, 0);
-    const uint32_t small[4] = {2, 3, 5, 7};
-    for (uint32_t i = 0; i < kPatternPeriod; ++i) {
-        uint32_t h = 0;
-        for (int q = 0; q < 4; ++q) {
-            const uint32_t p = small[q];
-            if (i % p == 0)
-                h += lg[q] | kCountOne;
-            if (i % (p * p) == 0)
-                h |= kSquareBit;
-        }
-        pat16[i] = h;
-    }
-    std::vector<uint32_t> pe(kPatternWords), po(kPatternWords);
-    for (uint32_t j = 0; j < kPatternWords; ++j) {
-        pe[j] = pat16[2 * j] | (pat16[2 * j + 1] << 16);
-        po[j] = pat16[2 * j + 1] | (pat16[(2 * j + 2) % kPatternPeriod] << 16);
-    }
-    t->np = (uint32_t)np;
     t->host_p = (uint32_t *)malloc(np * sizeof(uint32_t));
     if (!t->host_p)
         return 2;
     memcpy(t->host_p, pr.data(), np * sizeof(uint32_t));
-    t->p = (uint32_t *)dev_alloc(al, np * 4);
-    t->lg = (uint32_t *)dev_alloc(al, np * 4);
-    t->m = (uint64_t *)dev_alloc(al, np * 8);
-    t->l = (uint8_t *)dev_alloc(al, np);
-    t->blk_r = (uint32_t *)dev_alloc(al, np * 4);
-    t->blk_qm = (uint32_t *)dev_alloc(al, np * 4);
-    t->pat_even = (uint32_t *)dev_alloc(al, kPatternWords * 4);
-    t->pat_odd = (uint32_t *)dev_alloc(al, kPatternWords * 4);
-    if (!t->p || !t->lg || !t->m || !t->l || !t->blk_r || !t->blk_qm || !t->pat_even ||
-        !t->pat_odd)
-        return 2;
-    cudaMemcpyAsync(t->p, pr.data(), np * 4, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->lg, lg.data(), np * 4, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->m, mg.data(), np * 8, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->l, sh.data(), np, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->pat_even, pe.data(), kPatternWords * 4, cudaMemcpyHostToDevice, s);
-    cudaMemcpyAsync(t->pat_odd, po.data(), kPatternWords * 4, cudaMemcpyHostToDevice, s);
-    if (cudaStreamSynchronize(s) != cudaSuccess)
-        return 3;
+    t->np = (uint32_t)np;
     // byte sieve tables: weight scale 4 below 2^42, 3 up to 2^54
-    if (with_bytes && y_max < (1ull << 54)) {
+    if (with_bytes && y_max < (1ull << 54))
         t->byte_scale = y_max < (1ull << 42) ? 4u : 3u;
-        return byte_tables_create(t, pr, s);
+    t->np_mid = prime_count_upto(t, (1u << 17) - 1u);
+    // one allocation for all tables
+    const bool by = t->byte_scale != 0;
+    for (int pass = 0; pass < 2; ++pass) {
+        size_t off = 0;
+        const auto take = [&](auto &ptr, size_t bytes) {
+            if (pass)
+                ptr = (std::remove_reference_t<decltype(ptr)>)((char *)t->base + off);
+            off += (bytes + 255) & ~(size_t)255;
+        };
+        take(t->p, np * 4);
+        take(t->lg, np * 4);
+        take(t->m, np * 8);
+        take(t->l, np);
+        take(t->blk_r, np * 4);
+        take(t->blk_qm, np * 4);
+        take(t->pat_even, kPatternWords * 4);
+        take(t->pat_odd, kPatternWords * 4);
+        if (by) {
+            take(t->pw, ((size_t)t->np_mid + 1) * 4);
+            take(t->pq, np * sizeof(uint4));
+            take(t->blk_r2, np * 8);
+            take(t->pat8, (size_t)16 * kPat8Len);
+            take(t->patsq, kPatSqWords * 4);
+            take(t->pq2, np * sizeof(uint4));
+            take(t->pat2, (size_t)16 * kPat2Len);
+            take(t->rec, np * sizeof(uint4));
+            take(t->rec2, np * sizeof(uint2));
+        }
+        if (pass == 0) {
+            t->base_bytes = off;
+            t->base = dev_alloc(al, off);
+            if (!t->base)
+                return 2;
+        }
     }
-    return 0;
+    // the upload's source is host_p, which lives as long as the table
+    cudaMemcpyAsync(t->p, t->host_p, np * 4, cudaMemcpyHostToDevice, s);
+    prime_records_kernel<<<(unsigned)((np + 127) / 128), 128, 0, s>>>(
+        t->np, t->p, t->lg, t->m, t->l, t->byte_scale, t->pq, t->pq2, t->pw);
+    sieve_pattern_kernel<<<304, 128, 0, s>>>(t->pat_even, t->pat_odd, t->byte_scale,
+                                             (uint8_t *)t->pat8, t->patsq, (uint8_t *)t->pat2);
+    return cudaStreamSynchronize(s) == cudaSuccess ? 0 : 3;
 }
 
 void prime_table_destroy(PrimeTable *t)
 {
-    const size_t np = t->np;
-    dev_free(t->al, t->p, np * 4);
-    dev_free(t->al, t->lg, np * 4);
-    dev_free(t->al, t->m, np * 8);
-    dev_free(t->al, t->l, np);
-    dev_free(t->al, t->blk_r, np * 4);
-    dev_free(t->al, t->blk_qm, np * 4);
-    dev_free(t->al, t->pat_even, kPatternWords * 4);
-    dev_free(t->al, t->pat_odd, kPatternWords * 4);
-    dev_free(t->al, t->pq, np * sizeof(uint4));
-    dev_free(t->al, t->blk_r2, np * 8);
-    dev_free(t->al, t->pat8, (size_t)16 * kPat8Len);
-    dev_free(t->al, t->patsq, kPatSqWords * 4);
-    dev_free(t->al, t->pq2, np * sizeof(uint4));
-    dev_free(t->al, t->pat2, (size_t)16 * kPat2Len);
-    dev_free(t->al, t->rec, np * sizeof(uint4));
-    dev_free(t->al, t->rec2, np * sizeof(uint2));
-    if (t->pw)
-        dev_free(t->al, t->pw, ((size_t)t->np_mid + 1) * 4);
-    if (t->scratch_len) {
-        const uint64_t ntiles = (t->scratch_len + kByteTile - 1) / kByteTile;
-        dev_free(t->al, t->bucket, ntiles * t->bucket_cap * 8);
-        dev_free(t->al, t->gsq, ntiles * (kByteTile / 8));
-        dev_free(t->al, t->perr, 4);
-        const uint64_t nt2 = (t->scratch_len + kT2MinTile - 1) / kT2MinTile;
-        dev_free(t->al, t->sqcnt, nt2 * 4);
-        dev_free(t->al, t->sqlist, nt2 * t->sq_cap * 4);
-    }
+    dev_free(t->al, t->base, t->base_bytes);
+    dev_free(t->al, t->scratch, t->scratch_bytes);
     free(t->host_p);
     *t = PrimeTable();
 }
@@ -1614,7 +1549,7 @@ uint32_t prime_count_upto(const PrimeTable *t, uint64_t b)
     return lo;
 }
 
-int sieve_scratch_create(PrimeTable *t, uint64_t max_len)
+int sieve_scratch_create(PrimeTable *t, uint64_t max_len, cudaStream_t s)
 {
     if (!t->pq || t->scratch_len || max_len == 0 || max_len > (1ull << 30))
         return 0;
@@ -1626,36 +1561,27 @@ int sieve_scratch_create(PrimeTable *t, uint64_t max_len)
     uint32_t cap = (uint32_t)(mu + 10.0 * std::sqrt(mu) + 256.0);
     cap = (cap + 31u) & ~31u;
     const uint64_t ntiles = (max_len + kByteTile - 1) / kByteTile;
-    t->bucket = (uint64_t *)dev_alloc(t->al, ntiles * cap * 8);
-    t->gsq = (uint32_t *)dev_alloc(t->al, ntiles * (kByteTile / 8));
-    t->perr = (uint32_t *)dev_alloc(t->al, 4);
-    if (!t->bucket || !t->gsq || !t->perr) {
-        dev_free(t->al, t->bucket, ntiles * cap * 8);
-        dev_free(t->al, t->gsq, ntiles * (kByteTile / 8));
-        dev_free(t->al, t->perr, 4);
-        t->bucket = nullptr;
-        t->gsq = nullptr;
-        t->perr = nullptr;
-        return 2;
-    }
     // square lists of the scale-2 kernel: the primes 8192 <= q <= P put about
     // T / (8192 ln 8192) multiples of q^2 into a tile of T y (1.3 for 96 Ki
     // y); the kernel clears its tile's count after reading it, so the counts
     // start at zero once, here
     const uint64_t nt2 = (max_len + kT2MinTile - 1) / kT2MinTile;
+    const auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    const size_t b_bucket = up(ntiles * cap * 8), b_gsq = up(ntiles * (kByteTile / 8)),
+                 b_cnt = up(nt2 * 4 + 4), b_list = up(nt2 * 64 * 4);
+    t->scratch_bytes = b_bucket + b_gsq + b_cnt + b_list;
+    t->scratch = dev_alloc(t->al, t->scratch_bytes);
+    if (!t->scratch)
+        return 2;
+    char *q = (char *)t->scratch;
+    t->bucket = (uint64_t *)q;
+    t->gsq = (uint32_t *)(q + b_bucket);
+    t->perr = (uint32_t *)(q + b_bucket + b_gsq);  // status word, then the counts
+    t->sqcnt = t->perr + 1;
+    t->sqlist = (uint32_t *)(q + b_bucket + b_gsq + b_cnt);
     t->sq_cap = 64;
-    t->sqcnt = (uint32_t *)dev_alloc(t->al, nt2 * 4);
-    t->sqlist = (uint32_t *)dev_alloc(t->al, nt2 * t->sq_cap * 4);
-    if (!t->sqcnt || !t->sqlist) {
-        dev_free(t->al, t->sqcnt, nt2 * 4);
-        dev_free(t->al, t->sqlist, nt2 * t->sq_cap * 4);
-        t->sqcnt = nullptr;
-        t->sqlist = nullptr;
-        t->sq_cap = 0;
-    } else {
-        cudaMemset(t->sqcnt, 0, nt2 * 4);
-    }
-    cudaMemset(t->perr, 0, 4);
+    if (cudaMemsetAsync(t->perr, 0, nt2 * 4 + 4, s) != cudaSuccess)
+        return 3;
     t->bucket_cap = cap;
     t->scratch_len = max_len;
     return 0;

@@ -102,7 +102,7 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
     if (rc == MERTENS_OK) {
         int prc = prime_table_create(&pt, t->al, y_max, s);
         if (prc == 0)
-            prc = sieve_scratch_create(&pt, L);
+            prc = sieve_scratch_create(&pt, L, s);
         if (prc != 0)
             rc = prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA;
     }
