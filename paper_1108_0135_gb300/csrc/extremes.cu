@@ -91,9 +91,20 @@ __host__ __device__ inline void ext_merge(Ext &e, const Ext &o)
 }
 
 constexpr int kExtThreads = 256;
-constexpr uint32_t kExtPer = 64;  // y per thread
+constexpr uint32_t kExtWarps = kExtThreads / 32;
+constexpr uint32_t kExtSegs = 4;      // segments per warp of the first pass
+constexpr uint32_t kExtScan = 304;    // CTAs of the exact pass
 
-__device__ inline Ext ext_shfl(const Ext &e, int src)
+// The scan of a block is bound by reading its int16 M(y) once (2 GB per 2^30
+// y); the exact comparison of every M(y)/sqrt(y) in 128 bits took 18.1 ms per
+// 2^30 y (instruction-bound).  So: (1) the largest and smallest M of every
+// 2048-y segment, by packed 16-bit maxima; (2) of every segment [a, b] the
+// bounds of M/sqrt(y) that these give -- a positive largest M is reached at some
+// y <= b, and no ratio of the segment is above it at y = a (a negative one:
+// the other way round) -- and the best lower bound of the block; (3) only the
+// segments whose upper bound reaches it, or that hold the block's extreme M,
+// are compared point by point.
+__device__ __forceinline__ Ext ext_shfl(const Ext &e, int src)
 {
     Ext o;
     o.mx = __shfl_down_sync(0xffffffffu, e.mx, src);
@@ -107,19 +118,9 @@ __device__ inline Ext ext_shfl(const Ext &e, int src)
     return o;
 }
 
-// One block of M(y): every CTA reduces kExtThreads * kExtPer consecutive y to
-// one record in part[blockIdx.x].
-__global__ void __launch_bounds__(kExtThreads) block_extremes_kernel(
-    uint64_t y1, uint64_t len, const int16_t *__restrict__ Mloc,
-    const int64_t *__restrict__ segoff, Ext *__restrict__ part)
+// The CTA's records into one (thread 0's return value).
+__device__ __forceinline__ Ext ext_reduce(Ext e, Ext *sh)
 {
-    __shared__ Ext sh[kExtThreads / 32];
-    Ext e;
-    ext_init(e);
-    const uint64_t i0 = ((uint64_t)blockIdx.x * kExtThreads + threadIdx.x) * kExtPer;
-    const uint64_t i1 = i0 + kExtPer < len ? i0 + kExtPer : len;
-    for (uint64_t i = i0; i < i1; ++i)
-        ext_point(e, segoff[i >> kSegShift] + (int64_t)Mloc[i], y1 + i);
     for (int o = 16; o > 0; o >>= 1) {
         const Ext q = ext_shfl(e, o);
         ext_merge(e, q);
@@ -127,28 +128,127 @@ __global__ void __launch_bounds__(kExtThreads) block_extremes_kernel(
     if ((threadIdx.x & 31) == 0)
         sh[threadIdx.x >> 5] = e;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int w = 1; w < kExtThreads / 32; ++w)
+    if (threadIdx.x == 0)
+        for (uint32_t w = 1; w < kExtWarps; ++w)
             ext_merge(e, sh[w]);
-        part[blockIdx.x] = e;
-    }
+    return e;
 }
 
-// All partial records into part[0] (one CTA, strided then a serial pass).
+// Bounds of a segment [a, b] with largest value M (smallest: of -M):
+// `reached` is at most a ratio that occurs, `limit` at least every ratio.
+__device__ __forceinline__ uint64_t ext_reached(int64_t M, uint64_t a, uint64_t b)
+{
+    return M >= 0 ? b : a;
+}
+__device__ __forceinline__ uint64_t ext_limit(int64_t M, uint64_t a, uint64_t b)
+{
+    return M >= 0 ? a : b;
+}
+
+// Pass 1: {max, min} of every segment into mm (16-bit halves), and per CTA the
+// extreme M (its segment's first y in ymx, ymn) and the best reached ratios.
+__global__ void __launch_bounds__(kExtThreads) segment_extremes_kernel(
+    uint64_t y1, uint64_t len, uint32_t nseg, const int16_t *__restrict__ Mloc,
+    const int64_t *__restrict__ segoff, uint32_t *__restrict__ mm, Ext *__restrict__ part)
+{
+    __shared__ Ext sh[kExtWarps];
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5;
+    Ext e;
+    ext_init(e);
+    for (uint32_t q = 0; q < kExtSegs; ++q) {
+        const uint32_t sg = (blockIdx.x * kExtWarps + warp) * kExtSegs + q;
+        if (sg >= nseg)
+            break;
+        const uint64_t i0 = (uint64_t)sg << kSegShift;
+        uint32_t hi = 0x80008000u, lo = 0x7fff7fffu;
+        if (i0 + kSegY <= len) {
+            const uint4 *v = reinterpret_cast<const uint4 *>(Mloc + i0);
+#pragma unroll
+            for (uint32_t r = 0; r < (uint32_t)kSegY / 256u; ++r) {
+                const uint4 x = v[r * 32u + lane];
+                hi = __vmaxs2(__vmaxs2(__vmaxs2(hi, x.x), __vmaxs2(x.y, x.z)), x.w);
+                lo = __vmins2(__vmins2(__vmins2(lo, x.x), __vmins2(x.y, x.z)), x.w);
+            }
+        } else {
+            for (uint64_t i = i0 + lane; i < len; i += 32u) {
+                const uint32_t x = (uint16_t)Mloc[i] * 0x00010001u;
+                hi = __vmaxs2(hi, x);
+                lo = __vmins2(lo, x);
+            }
+        }
+        const int mx = __reduce_max_sync(0xffffffffu, max((int)(int16_t)(hi & 0xffffu),
+                                                          (int)(int16_t)(hi >> 16)));
+        const int mn = __reduce_min_sync(0xffffffffu, min((int)(int16_t)(lo & 0xffffu),
+                                                          (int)(int16_t)(lo >> 16)));
+        if (lane == q) {
+            mm[sg] = (uint32_t)(uint16_t)mx | ((uint32_t)(uint16_t)mn << 16);
+            Ext o;
+            const uint64_t a = y1 + i0, b = y1 + min(i0 + kSegY, len) - 1;
+            o.mx = segoff[sg] + mx;
+            o.mn = segoff[sg] + mn;
+            o.ymx = o.ymn = a;
+            o.rpM = o.mx;
+            o.rpy = ext_reached(o.mx, a, b);
+            o.rnM = o.mn;
+            o.rny = ext_reached(-o.mn, a, b);
+            ext_merge(e, o);
+        }
+    }
+    e = ext_reduce(e, sh);
+    if (threadIdx.x == 0)
+        part[blockIdx.x] = e;
+}
+
+// All records into part[0] (one CTA).
 __global__ void __launch_bounds__(kExtThreads) merge_extremes_kernel(Ext *part, uint32_t n)
 {
-    __shared__ Ext sh[kExtThreads];
+    __shared__ Ext sh[kExtWarps];
     Ext e;
     ext_init(e);
     for (uint32_t i = threadIdx.x; i < n; i += kExtThreads)
         ext_merge(e, part[i]);
-    sh[threadIdx.x] = e;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int t = 1; t < kExtThreads; ++t)
-            ext_merge(e, sh[t]);
+    e = ext_reduce(e, sh);
+    if (threadIdx.x == 0)
         part[0] = e;
+}
+
+// Pass 3: the exact extremes over the segments that can hold one, given the
+// block's best record in best[0]; a record per CTA.
+__global__ void __launch_bounds__(kExtThreads) exact_extremes_kernel(
+    uint64_t y1, uint64_t len, uint32_t nseg, const int16_t *__restrict__ Mloc,
+    const int64_t *__restrict__ segoff, const uint32_t *__restrict__ mm,
+    const Ext *__restrict__ best, Ext *__restrict__ part)
+{
+    __shared__ Ext sh[kExtWarps];
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t w = (blockIdx.x * kExtThreads + threadIdx.x) >> 5, nw = gridDim.x * kExtWarps;
+    const Ext B = best[0];
+    Ext e;
+    ext_init(e);
+    for (uint32_t s0 = w * 32u; s0 < nseg; s0 += nw * 32u) {
+        const uint32_t sg = s0 + lane;
+        bool pick = false;
+        if (sg < nseg) {
+            const int64_t so = segoff[sg];
+            const int64_t mx = so + (int16_t)(mm[sg] & 0xffffu), mn = so + (int16_t)(mm[sg] >> 16);
+            const uint64_t i0 = (uint64_t)sg << kSegShift;
+            const uint64_t a = y1 + i0, b = y1 + min(i0 + kSegY, len) - 1;
+            pick = (mx == B.mx && a == B.ymx) || (mn == B.mn && a == B.ymn) ||
+                   !ratio_gt(B.rpM, B.rpy, mx, ext_limit(mx, a, b)) ||
+                   !ratio_gt(mn, ext_limit(-mn, a, b), B.rnM, B.rny);
+        }
+        for (uint32_t mask = __ballot_sync(0xffffffffu, pick); mask; mask &= mask - 1u) {
+            const uint64_t i0 = (uint64_t)(s0 + __ffs(mask) - 1u) << kSegShift;
+            const uint64_t i1 = min(i0 + kSegY, len);
+            const int64_t so = segoff[i0 >> kSegShift];
+            for (uint64_t i = i0 + lane; i < i1; i += 32u)
+                ext_point(e, so + (int64_t)Mloc[i], y1 + i);
+        }
     }
+    e = ext_reduce(e, sh);
+    if (threadIdx.x == 0)
+        part[blockIdx.x] = e;
 }
 
 }  // namespace
@@ -167,10 +267,10 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
     const uint64_t span = y_last - y_first + 1;
     const uint64_t L = std::min<uint64_t>(1ull << 30, ((span + kSegY - 1) / kSegY) * kSegY);
     const uint64_t nblocks = (span + L - 1) / L;
-    const uint64_t per_cta = (uint64_t)kExtThreads * kExtPer;
-    const uint64_t ctas = (L + per_cta - 1) / per_cta;
-    const uint64_t nparts = nblocks * ctas;
-    if (nparts >= (1ull << 32)) {
+    const uint64_t nseg = sieve_segments(L);
+    const uint64_t ctas = (nseg + kExtWarps * kExtSegs - 1) / (kExtWarps * kExtSegs);
+    const uint64_t nparts = nblocks * kExtScan;  // records of the exact passes
+    if (nblocks * ((L + 16383) / 16384) >= (1ull << 32)) {
         set_last_error("mertens_scan_extremes: interval too long");
         return MERTENS_ENOTSUP;
     }
@@ -181,13 +281,13 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
         prc = sieve_scratch_create(&pt, L, s);
     if (prc != 0)
         rc = prc == 6 ? MERTENS_ENOTSUP : (prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA);
-    const uint64_t nseg = sieve_segments(L);
     int16_t *ml = (int16_t *)dev_alloc(al, (L + 2) * 2);
     int32_t *ss = (int32_t *)dev_alloc(al, nseg * 4);
     int64_t *so = (int64_t *)dev_alloc(al, nseg * 8);
     int64_t *cy = (int64_t *)dev_alloc(al, (nblocks + 1) * 8);
     Ext *part = (Ext *)dev_alloc(al, nparts * sizeof(Ext));
-    if (rc == MERTENS_OK && (!ml || !ss || !so || !cy || !part))
+    Ext *first = (Ext *)dev_alloc(al, ctas * sizeof(Ext));  // records of a first pass
+    if (rc == MERTENS_OK && (!ml || !ss || !so || !cy || !part || !first))
         rc = MERTENS_ENOMEM;
     if (rc == MERTENS_OK) {
         cudaMemcpyAsync(cy, &carry, 8, cudaMemcpyHostToDevice, s);
@@ -202,10 +302,15 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
             Lc.carry_out = cy + b + 1;
             if (sieve_block_enqueue(&pt, Lc, s) < 0)
                 rc = MERTENS_ECUDA;
-            // every block launches all `ctas` CTAs; those past a short last
-            // block write empty records
-            block_extremes_kernel<<<(unsigned)ctas, kExtThreads, 0, s>>>(Lc.y1, Lc.len, ml, so,
-                                                                        part + b * ctas);
+            // the segment sums are no longer needed: they become the segments'
+            // {max, min}
+            const uint32_t ns = (uint32_t)sieve_segments(Lc.len);
+            const uint32_t nc = (ns + kExtWarps * kExtSegs - 1) / (kExtWarps * kExtSegs);
+            uint32_t *mm = reinterpret_cast<uint32_t *>(ss);
+            segment_extremes_kernel<<<nc, kExtThreads, 0, s>>>(Lc.y1, Lc.len, ns, ml, so, mm, first);
+            merge_extremes_kernel<<<1, kExtThreads, 0, s>>>(first, nc);
+            exact_extremes_kernel<<<kExtScan, kExtThreads, 0, s>>>(Lc.y1, Lc.len, ns, ml, so, mm,
+                                                                  first, part + b * kExtScan);
             if (cudaGetLastError() != cudaSuccess)
                 rc = MERTENS_ECUDA;
         }
@@ -246,6 +351,7 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
     dev_free(al, so, nseg * 8);
     dev_free(al, cy, (nblocks + 1) * 8);
     dev_free(al, part, nparts * sizeof(Ext));
+    dev_free(al, first, ctas * sizeof(Ext));
     if (pt.np)
         prime_table_destroy(&pt);
     return rc;
