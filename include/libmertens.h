@@ -89,10 +89,12 @@ int mertens_set_allocator(mertens_alloc_fn alloc, mertens_free_fn release, void 
  *              entries (Sec. 2); X_i >= 2^32 is MERTENS_ENOTSUP.
  *   block_len  length of a sieve block in y (Sec. 3 processes the y-axis
  *              block by block); 0 = chosen by the library.  Any value >= 1
- *              is honoured exactly.
+ *              is taken; whole runs over one-word targets round it up to a
+ *              multiple of 6144 (results do not depend on it).
  *
  * Allocates all device memory of the plan on the current device (through the
- * hook above).  Host-side work only otherwise; no kernel is launched.
+ * hook above).  Small kernels that make the plan's tables run on a stream of
+ * the library and are finished before return.
  * Errors: MERTENS_EINVAL (count = 0, bad n or u), MERTENS_ENOTSUP,
  * MERTENS_ENOMEM, MERTENS_ECUDA.  On error *out is set to NULL.
  */

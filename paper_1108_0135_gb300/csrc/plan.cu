@@ -273,7 +273,10 @@ struct mertens_plan_s {
     uint32_t *dJL = nullptr, *dJD = nullptr;
     uint64_t *dA = nullptr, *dR6 = nullptr;
     WheelGroup *dwgroups = nullptr;
-    WheelDenseItem *dwitems = nullptr;
+    uint32_t *dwpre = nullptr;
+    WheelTotals *wtotals = nullptr;
+    uint32_t wgroups = 0, wparts = 1;
+    uint64_t wdense_items = 0;   // about; the device has their number
     WheelGatherTile *dwtiles = nullptr;
     uint4 *dwgitems = nullptr;
     uint16_t *dwl = nullptr;
@@ -420,9 +423,7 @@ size_t plan_device_bytes(mertens_plan_t p)
     size_t b = 0;
     for (auto &a : p->allocs)
         b += a.second;
-    b += (size_t)p->pt.np * 25 + 2 * kPatternWords * 4 + (size_t)p->ws.np * 28 +
-         p->ws.max_len / 96 + (4u << 20);
-    return b;
+    return b + p->pt.base_bytes + p->pt.scratch_bytes;
 }
 }  // namespace mert
 
@@ -533,57 +534,50 @@ int mertens_describe(mertens_u128 n, mertens_u128 u, mertens_query_info *info)
     return MERTENS_OK;
 }
 
-// The rest of plan_create for a plan over the integers coprime to 6: K, JLO and
-// the dense cut-offs YCE of every entry are given.  Blocks are whole segments
-// (6144 y) of about block_len y.
-static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::vector<uint64_t> &K,
-                             const std::vector<uint64_t> &JLO, std::vector<uint64_t> &YC,
-                             uint64_t block_len, const mertens_tuning &tn)
+// A plan over the integers coprime to 6: targets n (one word) with sieve limits
+// us.  The entries, their dense cut-offs and the dense work items are made on
+// the device; the host lays out blocks, gather tiles and memory.  Blocks are
+// whole segments (6144 y) of about block_len y.
+static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::vector<u128> &n,
+                             const std::vector<uint64_t> &us, uint64_t block_len,
+                             const mertens_tuning &tn)
 {
-    const size_t count = p->nq, E = K.size();
-    // cut-offs common to 64 consecutive entries of a target, at most
-    // floor(k/jlo) (beyond it no term is left); jd, the last gathered j
-    std::vector<uint32_t> JL(E), JD(E);
-    std::vector<WheelGroup> groups;
-    p->ydense = p->dense_y = p->gather_j_exec = p->jmax = 0;
+    const size_t count = n.size();
+    const double dc = dense_factor(tn);
+    std::vector<WheelQuery> qs(count);
+    uint64_t E = 0, G = 0;
+    double acc = 0, ksum = 0, terms = 0, pairs = 0;
     for (size_t i = 0; i < count; ++i) {
-        const size_t o = p->off[i], X = p->X[i], ng = (X + kWheelGroup - 1) / kWheelGroup;
-        const size_t gs = groups.size();
-        groups.resize(gs + ng);
-        std::mutex mu;
-        parallel_for(ng, 256, [&](size_t glo, size_t ghi) {
-            uint64_t y_max = 0, ydense = 0, jmax = 0, dense_y = 0, exec = 0;
-            for (size_t g = glo; g < ghi; ++g) {
-                const size_t e0 = o + g * kWheelGroup, e1 = std::min(e0 + kWheelGroup, o + X);
-                uint64_t yc = UINT64_MAX;
-                for (size_t e = e0; e < e1; ++e)
-                    yc = std::min(yc, std::min(YC[e], K[e] / JLO[e]));
-                yc -= yc % 6;  // so that yc + 1 is a wheel number (tile_uniform)
-                WheelGroup &G = groups[gs + g];
-                G.first = (uint32_t)e0;
-                G.count = (uint32_t)(e1 - e0);
-                G.yc = yc;
-                G.kmax = K[e0];
-                ydense = std::max(ydense, yc);
-                dense_y += yc * (e1 - e0);
-                for (size_t e = e0; e < e1; ++e) {
-                    const uint64_t jd = std::max(K[e] / (yc + 1), JLO[e] - 1);
-                    YC[e] = yc;
-                    JL[e] = (uint32_t)JLO[e];
-                    JD[e] = (uint32_t)jd;
-                    y_max = std::max(y_max, std::max(yc, K[e] / JLO[e]));
-                    jmax = std::max(jmax, jd);
-                    exec += phi6(jd) - phi6(JLO[e] - 1);
-                }
-            }
-            std::lock_guard<std::mutex> lk(mu);
-            p->y_max = std::max(p->y_max, y_max);
-            p->ydense = std::max(p->ydense, ydense);
-            p->jmax = std::max(p->jmax, jmax);
-            p->dense_y += dense_y;
-            p->gather_j_exec += exec;
-        });
+        const uint64_t ni = (uint64_t)n[i], X = ni / us[i];
+        qs[i] = {ni, X, E, G};
+        p->n.push_back(ni);
+        p->n_hi.push_back(0);
+        p->u.push_back(us[i]);
+        p->X.push_back(X);
+        p->off.push_back(E);
+        const uint64_t ng = (X + kWheelGroup - 1) / kWheelGroup;
+        E += X;
+        G += ng;
+        // the largest y read: a direct term's, or the gathered range's of x = 1
+        p->ymax_q.push_back(std::max(isqrt64(ni), ni / (X + 1)));
+        p->y_max = std::max(p->y_max, p->ymax_q.back());
+        // no cut-off is above the first group's target value
+        const uint64_t t = ((uint64_t)(dc * std::sqrt((double)ni)) + kChunk) / kChunk * kChunk;
+        p->ydense = std::max(p->ydense, std::min(t, ni / (X + 1)));
+        const double lx = std::log((double)std::max<uint64_t>(X, 2));
+        acc += (double)ni * lx;
+        ksum += (double)ni * (lx + 1.0);
+        const double root = 2.0 * std::sqrt((double)ni * (double)X);  // sum of sqrt(k)
+        terms += root / dc / 3.0;
+        pairs += dc * root / (double)(kWheelSegY * kWheelGroup * kWheelGroupBlock) +
+                 (double)ng / kWheelGroupBlock;
     }
+    if (E >= (1ull << 32)) {
+        set_last_error("mertens_plan: more than 2^32 array entries");
+        delete p;
+        return MERTENS_ENOTSUP;
+    }
+    p->nent = E;
     p->y_first = 1;
     p->y_last = p->y_max;
     if (block_len == 0) {
@@ -601,76 +595,13 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     block_len = std::min(block_len, p->y_last);
     p->block_len = (block_len + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
     p->nblocks = (p->y_last + p->block_len - 1) / p->block_len;
-
-    // ---- dense work items ----
-    std::stable_sort(groups.begin(), groups.end(),
-                     [](const WheelGroup &a, const WheelGroup &b) { return a.yc > b.yc; });
-    std::vector<uint64_t> kmax(groups.size() + 1, 0);  // largest k of the groups from g on
-    for (size_t g = groups.size(); g-- > 0;)
-        kmax[g] = std::max(kmax[g + 1], groups[g].kmax);
     p->wchunks = (p->ydense + kWheelSegY - 1) / kWheelSegY;
-    std::vector<WheelDenseItem> ditems;
-    {
-        const size_t gpi = kWheelDenseThreads / 32;
-        double pairs = 0;
-        for (const WheelGroup &G : groups)
-            pairs += (double)(G.yc / kWheelSegY + 1);
-        // parts of a chunk's list while the items would not fill the device
-        const uint32_t parts =
-            (uint32_t)std::min(8.0, std::max(1.0, std::ceil(2400.0 * gpi / std::max(pairs, 1.0))));
-        size_t pref = groups.size();
-        for (uint64_t c = 0; c < p->wchunks; ++c) {
-            const uint64_t ys = c * kWheelSegY + 1;
-            while (pref > 0 && groups[pref - 1].yc < ys)
-                --pref;
-            // groups [0, gw) wide, [gw, gf) high-word, [gf, pref) float
-            const auto first_below = [&](double lim, bool ok) {
-                if (!ok)
-                    return pref;
-                size_t lo = 0, hi = pref;
-                while (lo < hi) {
-                    const size_t mid = (lo + hi) / 2;
-                    if ((double)kmax[mid] < lim * 6.0 * (double)ys)
-                        hi = mid;
-                    else
-                        lo = mid + 1;
-                }
-                return lo;
-            };
-            const bool small_y = ys + kWheelSegY < 350000000ull;
-            const size_t gf = first_below(1.5e6, small_y);
-            const size_t gw = std::min(gf, first_below(6.0e7, small_y && c > 0));
-            const size_t cut[4] = {0, gw, gf, pref};
-            const int mode[3] = {kDenseWide, kDenseHigh, kDenseFloat};
-            for (int m = 0; m < 3; ++m)
-                for (size_t g0 = cut[m]; g0 < cut[m + 1]; g0 += gpi)
-                    for (uint32_t q = 0; q < parts; ++q) {
-                        WheelDenseItem it;
-                        it.c = (uint32_t)c;
-                        it.g0 = (uint32_t)g0;
-                        it.g1 = (uint32_t)std::min(g0 + gpi, cut[m + 1]);
-                        it.mode_parts = (uint32_t)mode[m] | (q << 8) | (parts << 16);
-                        ditems.push_back(it);
-                    }
-        }
-    }
-    p->nitems = (uint32_t)ditems.size();
+    p->wgroups = (uint32_t)G;
+    // parts of a dense chunk's list while the items would not fill the device
+    p->wparts = (uint32_t)std::min(8.0, std::max(1.0, std::ceil(2400.0 / pairs)));
+    p->wdense_items = (uint64_t)(pairs * p->wparts * 1.1) + 64;
 
     // ---- shared-memory gather tiles ----
-    std::vector<uint64_t> ycmin(E);
-    std::vector<double> kpre(E + 1, 0.0);  // prefix sums of k over all entries
-    for (size_t e = 0; e < E; ++e)
-        kpre[e + 1] = kpre[e] + (double)K[e];
-    double acc = 0;
-    for (size_t i = 0; i < count; ++i) {
-        uint64_t run = UINT64_MAX;
-        for (uint64_t x = 0; x < p->X[i]; ++x) {
-            const size_t e = p->off[i] + x;
-            run = std::min(run, YC[e]);
-            ycmin[e] = run;
-        }
-        acc += (double)p->n[i] * std::log((double)std::max<uint64_t>(p->X[i], 2));
-    }
     {
         // Gathered terms per y near y are about (n / y^2) ln X / 3 summed over
         // the targets, 32768 (sum n ln X) / y^2 per tile: tiles of all entries
@@ -683,6 +614,11 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             ys = strtoull(e, nullptr, 10);
         p->gather_smem_end = std::min(ys, p->y_max);
     }
+    // shorter tiles while the tile range would not give every SM its CTAs
+    uint64_t tile_y = kWheelTileY;
+    while (tile_y > kWheelSegY && (double)p->gather_smem_end / (double)tile_y *
+                                          std::ceil((double)E / 1024.0) < 608.0)
+        tile_y /= 2;
     // Blocks above: tiles over the whole block for the entries with
     // k >= kt_fac y0^2 / 32768 (about kt_fac terms or more per tile; a prefix of
     // each target's entries) when they have at least kt_min terms per tile
@@ -692,205 +628,247 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         kt_fac = atof(e);
     if (const char *e = getenv("MERTENS_TILE_MIN"))
         kt_min = atof(e);
-    const double item_work =
-        std::min(2.0e5, std::max(4096.0, (double)p->gather_j_exec / 2000.0));
-    std::vector<WheelGatherTile> gtiles;
-    std::vector<uint4> gitems;
+    const double item_work = std::min(2.0e6, std::max(4096.0, terms / (456.0 * 24.0)));
+    // sum of k over the x in (a, b] of target i
+    const auto k_between = [&](size_t i, double a, double b) {
+        return (double)qs[i].n * std::log((b + 0.5) / (a + 0.5));
+    };
+    std::vector<uint2> tiles;  // {first y less one, low and high word}, {length, 0}
+    std::vector<uint4> items;
     for (uint64_t b = 0; b < p->nblocks; ++b) {
         const uint64_t y0 = b * p->block_len, blen = wheel_block_len(p, b);
-        p->gblk.push_back((uint32_t)gitems.size());
+        p->gblk.push_back((uint32_t)items.size());
         uint64_t end = y0;  // y in (y0, end] goes to tiles
         if (p->gather_smem_end > y0)
             end = std::min(y0 + blen,
                            (p->gather_smem_end + kWheelSegY - 1) / kWheelSegY * kWheelSegY);
         p->gend.push_back(end);
         uint64_t kt = UINT64_MAX;  // entries with k >= kt take this block's tiles
+        std::vector<std::pair<uint64_t, uint64_t>> ranges, all;
+        std::vector<double> ks, kall;  // sums of k of the ranges
         if (y0 >= p->gather_smem_end && kt_fac > 0) {
             const double y1 = (double)y0 + 1.0, k0 = kt_fac * y1 * y1 / kGatherTile;
-            double ksum = 0;
+            double sum = 0;
+            const uint64_t k0i = (uint64_t)std::ceil(std::min(k0, 9.2e18));
             for (size_t i = 0; i < count; ++i) {
-                const double xt = std::min((double)p->X[i], std::floor((double)p->n[i] / k0));
-                ksum += kpre[p->off[i] + (uint64_t)xt] - kpre[p->off[i]];
+                const uint64_t xt = std::min(qs[i].X, qs[i].n / k0i);
+                if (xt == 0)
+                    continue;
+                all.push_back({qs[i].off, qs[i].off + xt});
+                kall.push_back(k_between(i, 0.0, (double)xt));
+                sum += kall.back();
             }
-            if (ksum * kGatherTile / (y1 * y1) >= kt_min) {
-                kt = (uint64_t)std::ceil(k0);
+            if (sum * kGatherTile / (y1 * y1) >= kt_min) {
+                kt = k0i;
                 end = y0 + blen;
             }
         }
         p->ktile.push_back(kt);
-        const uint64_t ntile = (end - y0 + kWheelTileY - 1) / kWheelTileY;
-        std::vector<WheelGatherTile> btiles(ntile);
-        std::vector<std::vector<uint4>> bitems(ntile);
-        parallel_for(ntile, 64, [&](size_t qlo, size_t qhi) {
-            std::vector<std::pair<uint64_t, uint64_t>> ranges;
-            for (size_t q = qlo; q < qhi; ++q) {
-                const uint64_t t0 = y0 + q * kWheelTileY;
-                WheelGatherTile &T = btiles[q];
-                T.t0 = t0;
-                T.len = (uint32_t)std::min(kWheelTileY, end - t0);
-                T.m1 = magic_of(t0 + 1);
-                T.l1 = magic_shift(t0 + 1);
-                T.m2 = magic_of(t0 + T.len + 1);
-                T.l2 = magic_shift(t0 + T.len + 1);
-                T.pad = 0;
-                // entries that can have terms: per target the suffix whose
-                // cut-off lies below the tile's end (and k >= kt: a prefix);
-                // suffixes separated by short gaps are merged
+        for (uint64_t t0 = y0; t0 < end; t0 += tile_y) {
+            const uint64_t len = std::min(tile_y, end - t0);
+            if (kt == UINT64_MAX) {
+                // entries whose cut-off lies below the tile's end: all where a
+                // cut-off can be bound by floor(k/jlo), else those with
+                // dc sqrt(k of the group's first) < t0 + len + 8
                 ranges.clear();
+                ks.clear();
                 for (size_t i = 0; i < count; ++i) {
-                    const uint64_t o = p->off[i], X = p->X[i];
-                    uint64_t lo = 0, hi = X;
-                    while (lo < hi) {
-                        const uint64_t mid = (lo + hi) / 2;
-                        if (ycmin[o + mid] < t0 + T.len)
-                            hi = mid;
-                        else
-                            lo = mid + 1;
-                    }
-                    uint64_t top = X;
-                    if (kt != UINT64_MAX) {
-                        uint64_t a = 0, z = X;  // first x index with k < kt
-                        while (a < z) {
-                            const uint64_t mid = (a + z) / 2;
-                            if (K[o + mid] >= kt)
-                                a = mid + 1;
-                            else
-                                z = mid;
-                        }
-                        top = a;
-                    }
-                    if (lo >= top)
+                    const WheelQuery &Q = qs[i];
+                    const double te = (double)(t0 + len) + 8.0;
+                    uint64_t lo = 0;
+                    if (2.0 * (dc * std::sqrt((double)Q.n) + 2.0 * kChunk) < (double)us[i])
+                        lo = (uint64_t)std::min((double)Q.X, dc * dc * (double)Q.n / (te * te)) /
+                             kWheelGroup * kWheelGroup;
+                    if (lo >= Q.X)
                         continue;
-                    if (!ranges.empty() && o + lo <= ranges.back().second + 4096 &&
-                        kt == UINT64_MAX)
-                        ranges.back().second = o + top;
-                    else
-                        ranges.push_back({o + lo, o + top});
-                }
-                const double per_k = (double)T.len / 3.0 / ((double)(t0 + 1) * (double)(t0 + 1));
-                for (const auto &rg : ranges) {
-                    for (uint64_t f = rg.first; f < rg.second;) {
-                        uint64_t g = std::min<uint64_t>(f + 1024, rg.second);
-                        while (g < rg.second &&
-                               (double)(g - f) + per_k * (kpre[g] - kpre[f]) < item_work)
-                            g = std::min<uint64_t>(g + 1024, rg.second);
-                        bitems[q].push_back(make_uint4(0u, (uint32_t)f, (uint32_t)g, 0u));
-                        f = g;
+                    const double kv = k_between(i, (double)lo, (double)Q.X);
+                    if (!ranges.empty() && Q.off + lo <= ranges.back().second + 4096) {
+                        ranges.back().second = Q.off + Q.X;
+                        ks.back() += kv;
+                    } else {
+                        ranges.push_back({Q.off + lo, Q.off + Q.X});
+                        ks.push_back(kv);
                     }
                 }
             }
-        });
-        for (size_t q = 0; q < ntile; ++q) {
-            if (bitems[q].empty())
-                continue;
-            for (uint4 it : bitems[q]) {
-                it.x = (uint32_t)gtiles.size();
-                gitems.push_back(it);
+            const auto &rs = kt == UINT64_MAX ? ranges : all;
+            const auto &kv = kt == UINT64_MAX ? ks : kall;
+            const double per_k = (double)len / 3.0 / ((double)(t0 + 1) * (double)(t0 + 1));
+            const uint32_t ti = (uint32_t)(tiles.size() / 2);
+            bool any = false;
+            for (size_t r = 0; r < rs.size(); ++r) {
+                // items of equal numbers of entries, in steps of 1024, with about
+                // item_work terms and checks on the average
+                const double ne = (double)(rs[r].second - rs[r].first);
+                const double work = 2.0 * ne + per_k * kv[r];
+                const uint64_t step = (uint64_t)std::max(
+                    1024.0, std::ceil(ne / std::max(1.0, work / item_work) / 1024.0) * 1024.0);
+                for (uint64_t f = rs[r].first; f < rs[r].second; f += step) {
+                    items.push_back(make_uint4(ti, (uint32_t)f,
+                                               (uint32_t)std::min(f + step, rs[r].second), 0u));
+                    any = true;
+                }
             }
-            gtiles.push_back(btiles[q]);
+            if (any) {
+                tiles.push_back(make_uint2((uint32_t)t0, (uint32_t)(t0 >> 32)));
+                tiles.push_back(make_uint2((uint32_t)len, 0u));
+            }
         }
     }
-    p->gblk.push_back((uint32_t)gitems.size());
+    p->gblk.push_back((uint32_t)items.size());
+    // chunk records of a block's global gather: an entry with cnt > 16 terms
+    // posts ceil(cnt / kWheelItem); cnt is at most k (1/ylo - 1/(yend + 1)) / 3 + 2
+    double most = 0;
+    for (uint64_t b = 0; b < p->nblocks; ++b) {
+        const uint64_t yend = b * p->block_len + wheel_block_len(p, b), ylo = p->gend[b] + 1;
+        if (ylo > yend)
+            continue;
+        const double C =
+            ksum * (1.0 / (double)ylo - 1.0 / ((double)yend + 1.0)) / 3.0 + 2.0 * (double)E;
+        most = std::max(most, C / kWheelItem + std::min((double)E, C / 16.0));
+    }
+    p->qcap = (uint32_t)std::min(most * 1.01 + 256.0, 4.0e9);
 
-    // ---- device buffers ----
-    {
-        // chunk records of a block's global gather: an entry with cnt > 16
-        // terms posts ceil(cnt / kSparseItem); cnt is at most
-        // k (1/ylo - 1/(yend + 1)) / 3 + 2
-        double most = 0;
-        for (uint64_t b = 0; b < p->nblocks; ++b) {
-            const uint64_t y0 = b * p->block_len, yend = y0 + wheel_block_len(p, b);
-            const uint64_t ylo = p->gend[b] + 1;
-            if (ylo > yend)
-                continue;
-            const double C =
-                kpre[E] * (1.0 / (double)ylo - 1.0 / ((double)yend + 1.0)) / 3.0 + 2.0 * (double)E;
-            most = std::max(most, C / kSparseItem + std::min((double)E, C / 16.0));
-        }
-        p->qcap = (uint32_t)std::min(most * 1.01 + 256.0, 4.0e9);
-    }
+    // ---- one piece of device memory ----
     const uint64_t wlen = p->block_len / 3;
+    const uint32_t ntiles = (uint32_t)(tiles.size() / 2);
     p->serial = true;
-    p->dK = p->alloc<uint64_t>(E);
-    p->dYCE = p->alloc<uint64_t>(E);
-    p->dJL = p->alloc<uint32_t>(E);
-    p->dJD = p->alloc<uint32_t>(E);
-    p->dS = p->alloc<uint64_t>(2 * E);  // S, then A
-    p->dA = p->dS ? p->dS + E : nullptr;
-    p->dR6 = p->alloc<uint64_t>(E);
-    p->dR = p->alloc<uint64_t>(E);
-    p->dqueue = p->alloc<uint4>(p->qcap);
-    p->dMloc[0] = p->alloc<int16_t>(wlen);
-    p->dsegsum[0] = p->alloc<int32_t>(wlen / kSegY);
-    p->dsegoff[0] = p->alloc<int64_t>(wlen / kSegY);
-    p->dcarry = p->alloc<int64_t>(p->nblocks + 1);
-    p->derr = p->alloc<uint32_t>(4);  // status, chunk count, two work counters
-    p->dqlen = p->derr ? p->derr + 1 : nullptr;
-    p->dcounter_dense = p->derr ? p->derr + 2 : nullptr;
-    p->dcounter_gather = p->derr ? p->derr + 3 : nullptr;
-    p->dwgroups = p->alloc<WheelGroup>(groups.size());
-    p->dwitems = p->alloc<WheelDenseItem>(ditems.size());
-    p->dwtiles = p->alloc<WheelGatherTile>(gtiles.size());
-    p->dwgitems = p->alloc<uint4>(gitems.size());
-    p->dwl = p->alloc<uint16_t>(p->wchunks * kSegY);
-    p->dwl_cnt = p->alloc<uint32_t>(p->wchunks);
-    p->dqs = p->alloc<QueryDev>(count);
-    int rc = MERTENS_OK;
-    if (!p->dK || !p->dYCE || !p->dJL || !p->dJD || !p->dS || !p->dR6 || !p->dR || !p->dqueue ||
-        !p->dMloc[0] || !p->dsegsum[0] || !p->dsegoff[0] || !p->dcarry || !p->derr ||
-        !p->dwgroups || !p->dwitems || !p->dwtiles || !p->dwgitems || !p->dwl || !p->dwl_cnt ||
-        !p->dqs)
-        rc = MERTENS_ENOMEM;
-    if (rc == MERTENS_OK) {
-        const int prc = wheel_sieve_create(&p->ws, p->al, p->y_last, wlen, nullptr);
-        if (prc != 0)
-            rc = prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA;
-    }
-    if (rc == MERTENS_OK) {
-        // sieve updates: sum of 1/p + 1/p^2 over the primes 5 <= p <= sqrt(block
-        // end), per wheel number
-        std::vector<double> pre(p->ws.np + 1, 0.0);
-        for (uint32_t i = 0; i < p->ws.np; ++i) {
-            const double q = (double)p->ws.host_p[i];
-            pre[i + 1] = pre[i] + 1.0 / q + 1.0 / (q * q);
-        }
-        for (uint64_t b = 0; b < p->nblocks; ++b) {
-            const uint64_t len = wheel_block_len(p, b);
-            p->sieve_updates += (double)len / 3.0 *
-                                pre[wheel_primes_upto(&p->ws, isqrt64(b * p->block_len + len))];
-        }
-        std::vector<QueryDev> qs(count);
-        for (size_t i = 0; i < count; ++i) {
-            qs[i].X = p->X[i];
-            qs[i].off = p->off[i];
-        }
-        const auto up = [&](void *d, const void *h, size_t bytes) {
-            if (bytes)
-                cudaMemcpy(d, h, bytes, cudaMemcpyHostToDevice);
-            p->h2d_bytes += bytes;
+    wheel_sieve_primes(&p->ws, p->y_last);
+    const size_t ws_bytes = wheel_sieve_bytes(&p->ws, wlen);
+    const uint32_t nblk = wheel_group_blocks(p->wgroups);
+    WheelEntryArgs ea{};
+    std::vector<QueryDev> qd(count);
+    for (size_t i = 0; i < count; ++i)
+        qd[i] = {qs[i].X, qs[i].off};
+    char *base = nullptr, *ws_base = nullptr, *up = nullptr;
+    size_t up_bytes = 0, cleared = 0;
+    uint2 *d_tiles = nullptr;
+    WheelQuery *d_qs = nullptr;
+    WheelTotals *d_totals = nullptr;
+    for (int pass = 0; pass < 2; ++pass) {
+        size_t off = 0;
+        const auto take = [&](auto &ptr, size_t bytes) {
+            if (pass)
+                ptr = (std::remove_reference_t<decltype(ptr)>)(base + off);
+            off += (bytes + 255) & ~(size_t)255;
         };
-        up(p->dK, K.data(), E * 8);
-        up(p->dYCE, YC.data(), E * 8);
-        up(p->dJL, JL.data(), E * 4);
-        up(p->dJD, JD.data(), E * 4);
-        up(p->dwgroups, groups.data(), groups.size() * sizeof(WheelGroup));
-        up(p->dwitems, ditems.data(), ditems.size() * sizeof(WheelDenseItem));
-        up(p->dwtiles, gtiles.data(), gtiles.size() * sizeof(WheelGatherTile));
-        up(p->dwgitems, gitems.data(), gitems.size() * sizeof(uint4));
-        up(p->dqs, qs.data(), count * sizeof(QueryDev));
-        if (cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) != cudaSuccess ||
-            cudaGetLastError() != cudaSuccess)
-            rc = MERTENS_ECUDA;
+        take(d_totals, count * sizeof(WheelTotals) + 64);  // and four status words
+        cleared = off;
+        take(up, 0);  // uploaded with one copy
+        const size_t up0 = off;
+        take(d_qs, count * sizeof(WheelQuery));
+        take(p->dqs, count * sizeof(QueryDev));
+        take(d_tiles, tiles.size() * sizeof(uint2));
+        take(p->dwgitems, items.size() * sizeof(uint4));
+        up_bytes = off - up0;
+        take(p->dK, E * 8);
+        take(p->dYCE, E * 8);
+        take(p->dJL, E * 4);
+        take(p->dJD, E * 4);
+        take(p->dS, 2 * E * 8);  // S, then A
+        take(p->dR6, E * 8);
+        take(p->dR, E * 8);
+        take(p->dqueue, (size_t)p->qcap * sizeof(uint4));
+        take(p->dMloc[0], wlen * 2);
+        take(p->dsegsum[0], wlen / kSegY * 4);
+        take(p->dsegoff[0], wlen / kSegY * 8);
+        take(p->dcarry, (p->nblocks + 1) * 8);
+        take(p->dwgroups, (size_t)G * sizeof(WheelGroup));
+        take(p->dwpre, ((size_t)nblk + 1) * 4);
+        take(p->dwtiles, (size_t)ntiles * sizeof(WheelGatherTile));
+        take(p->dwl, p->wchunks * kSegY * 2);
+        take(p->dwl_cnt, p->wchunks * 4);
+        take(ws_base, ws_bytes);
+        if (pass == 0) {
+            base = p->alloc<char>(off);
+            if (!base) {
+                set_last_error("mertens_plan: device allocation failed");
+                mertens_destroy(p);
+                return MERTENS_ENOMEM;
+            }
+        }
     }
-    if (rc != MERTENS_OK) {
-        if (rc == MERTENS_ENOMEM)
-            set_last_error("mertens_plan: device allocation failed");
-        else
-            set_last_error("mertens_plan: CUDA error %s", cudaGetErrorString(cudaGetLastError()));
+    p->dA = p->dS + E;
+    p->wtotals = d_totals;
+    p->derr = (uint32_t *)(d_totals + count);  // status, chunk count, two work counters
+    p->dqlen = p->derr + 1;
+    p->dcounter_dense = p->derr + 2;
+    p->dcounter_gather = p->derr + 3;
+    // host image of the uploaded part (laid out as above)
+    std::vector<char> img(up_bytes);
+    const auto put = [&](const void *d, const void *h, size_t bytes) {
+        if (bytes)
+            memcpy(img.data() + ((const char *)d - up), h, bytes);
+    };
+    put(d_qs, qs.data(), count * sizeof(WheelQuery));
+    put(p->dqs, qd.data(), count * sizeof(QueryDev));
+    put(d_tiles, tiles.data(), tiles.size() * sizeof(uint2));
+    put(p->dwgitems, items.data(), items.size() * sizeof(uint4));
+    const size_t np = p->ws.host_p.size();
+    p->h2d_bytes = up_bytes + np * 4;
+    ea.qs = d_qs;
+    ea.nq = (uint32_t)count;
+    ea.ngroups = p->wgroups;
+    ea.dc = dc;
+    ea.K = p->dK;
+    ea.YC = p->dYCE;
+    ea.JL = p->dJL;
+    ea.JD = p->dJD;
+    ea.groups = p->dwgroups;
+    ea.totals = d_totals;
+    ea.parts = p->wparts;
+    ea.dpre = p->dwpre;
+    ea.tiles = p->dwtiles;
+    ea.tile_src = d_tiles;
+    ea.ntiles = ntiles;
+    // on the library's stream, finished before return
+    cudaStream_t s = alloc_stream();
+    const bool ok =
+        s && cudaMemsetAsync(base, 0, cleared, s) == cudaSuccess &&
+        cudaMemcpyAsync(up, img.data(), up_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess &&
+        wheel_entries_enqueue(ea, s) >= 0 && wheel_sieve_bind(&p->ws, ws_base, wlen, p->derr, s) == 0 &&
+        cudaMemcpyAsync(p->ws.p, p->ws.host_p.data(), np * 4, cudaMemcpyHostToDevice, s) ==
+            cudaSuccess &&
+        cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess &&
+        cudaStreamSynchronize(s) == cudaSuccess;
+    if (!ok) {
+        set_last_error("mertens_plan: CUDA error %s", cudaGetErrorString(cudaGetLastError()));
         mertens_destroy(p);
-        return rc;
+        return MERTENS_ECUDA;
+    }
+    // sieve updates: sum of 1/p + 1/p^2 over the primes 5 <= p <= sqrt(block
+    // end), per wheel number
+    double pre = 0;
+    size_t i = 0;
+    for (uint64_t b = 0; b < p->nblocks; ++b) {
+        const uint64_t len = wheel_block_len(p, b), P = isqrt64(b * p->block_len + len);
+        for (; i < np && p->ws.host_p[i] <= P; ++i) {
+            const double q = (double)p->ws.host_p[i];
+            pre += 1.0 / q + 1.0 / (q * q);
+        }
+        p->sieve_updates += (double)len / 3.0 * pre;
     }
     *out = p;
+    return MERTENS_OK;
+}
+
+// Term counts of a wheel plan's targets, read when they are asked for.
+static int wheel_counts(mertens_plan_s *p)
+{
+    if (!p->wheel || !p->direct.empty())
+        return MERTENS_OK;
+    std::vector<WheelTotals> t(p->nq);
+    if (cudaMemcpy(t.data(), p->wtotals, p->nq * sizeof(WheelTotals), cudaMemcpyDeviceToHost) !=
+        cudaSuccess)
+        return MERTENS_ECUDA;
+    for (const WheelTotals &v : t) {
+        p->direct.push_back(v.direct);
+        p->gathered.push_back(v.gathered);
+        p->terms += v.direct + v.gathered;
+        p->gather_j += v.gather_j;
+        p->gather_j_exec += v.exec;
+        p->dense_y += v.dense_y;
+    }
     return MERTENS_OK;
 }
 
@@ -960,13 +938,16 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         const char *q = getenv("MERTENS_GATHER_QUOT");
         p->wheel = !window && !table && share && !(q && q[0] == '0') && !getenv("MERTENS_OVERLAP");
         p->wheel_long = q && q[0] == '2';
+        std::vector<uint64_t> us(count);
         for (size_t i = 0; i < count && p->wheel; ++i) {
-            const uint64_t uu = u.lo ? u.lo : target_u(n128[i], ub);
-            p->wheel = n128[i] < wide_threshold() && n128[i] / uu < (1ull << 31) &&
-                       wheel_sieve_exact(uu + 2 * kWheelSegY);
+            us[i] = u.lo ? u.lo : target_u(n128[i], ub);
+            p->wheel = n128[i] < wide_threshold() && n128[i] / us[i] < (1ull << 31) &&
+                       wheel_sieve_exact(us[i] + 2 * kWheelSegY);
         }
+        if (p->wheel)
+            return plan_create_wheel(out, p, n128, us, block_len, tn);
     }
-    const bool share_dense = !window && share && !p->wheel;
+    const bool share_dense = !window && share;
     for (size_t i = 0; i < count; ++i) {
         const u128 nn = to_u128(n[i]);
         const uint64_t uu = u.lo ? u.lo : (table ? on_table_u(nn, ub, table->y_max)
@@ -1214,8 +1195,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         delete p;
         return MERTENS_ENOTSUP;
     }
-    if (p->wheel)
-        return plan_create_wheel(out, p, K, JLO, YCE, block_len, tn);
     // ---- gathered terms shared along chains x, 2x, 4x, 8x, 16x ----
     // floor(floor(n/x)/j) = floor(n/(x j)), so entry 2x's term at j' is entry
     // x's term at j = 2j'.  The link x -> 2x (one-word entries of one target)
@@ -1875,15 +1854,16 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             launches += r;
             if (c1 >= p->wchunks) {
                 WheelDenseArgs da;
-                da.items = p->dwitems;
-                da.nitems = p->nitems;
                 da.counter = p->dcounter_dense;
                 da.groups = p->dwgroups;
+                da.ngroups = p->wgroups;
+                da.parts = p->wparts;
+                da.pre = p->dwpre;
                 da.K = p->dK;
                 da.dl = p->dwl;
                 da.dl_cnt = p->dwl_cnt;
                 da.S = p->dS;
-                r = wheel_dense_enqueue(da, s);
+                r = wheel_dense_enqueue(da, p->wdense_items, s);
                 if (r < 0)
                     break;
                 launches += r;
@@ -2318,16 +2298,20 @@ int mertens_result(mertens_plan_t p, size_t i, int64_t *M_n, int64_t *entries, s
     uint32_t err = 0;
     if (cudaMemcpy(&err, p->derr, 4, cudaMemcpyDeviceToHost) != cudaSuccess)
         return MERTENS_ECUDA;
-    if (p->sieves) {
-        const uint32_t st = p->wheel ? wheel_sieve_status(&p->ws) : sieve_scratch_status(&p->pt);
+    if (p->sieves && !p->wheel) {  // a wheel plan has one status word
+        const uint32_t st = sieve_scratch_status(&p->pt);
         if (st) {
             set_last_error("mertens_result: %s", sieve_status_text(st));
             return sieve_status_code(st);
         }
     }
     if (err & kErrTimeout) {
-        set_last_error("mertens_result: a bounded wait for a bulk copy in the update gave up");
+        set_last_error("mertens_result: a bounded wait for a bulk copy gave up");
         return MERTENS_ETIMEOUT;
+    }
+    if (p->wheel && (err & kErrList)) {
+        set_last_error("mertens_result: %s", sieve_status_text(err & kErrList));
+        return MERTENS_EOVERFLOW;
     }
     if (err & kErrMOverflow) {
         set_last_error("mertens_result: |M(y)| exceeded the int32 block type");
@@ -2616,8 +2600,6 @@ void mertens_destroy(mertens_plan_t p)
             cudaEventDestroy(e);
     if (p->pt.np)
         prime_table_destroy(&p->pt);
-    if (p->ws.np)
-        wheel_sieve_destroy(&p->ws);
     for (auto &a : p->allocs)
         dev_free(p->al, a.first, a.second);
     delete p;
@@ -2627,6 +2609,8 @@ int mertens_plan_info(mertens_plan_t p, size_t i, mertens_query_info *info)
 {
     if (!p || i >= p->nq || !info)
         return MERTENS_EINVAL;
+    if (wheel_counts(p) != MERTENS_OK)
+        return MERTENS_ECUDA;
     memset(info, 0, sizeof(*info));
     info->n.lo = p->n[i];
     info->n.hi = p->n_hi[i];
@@ -2656,7 +2640,7 @@ int mertens_run_stats_get(mertens_plan_t p, mertens_run_stats *st)
     memset(st, 0, sizeof(*st));
     if (!p->ran)
         return MERTENS_ENOTREADY;
-    if (cudaEventSynchronize(p->done) != cudaSuccess)
+    if (cudaEventSynchronize(p->done) != cudaSuccess || wheel_counts(p) != MERTENS_OK)
         return MERTENS_ECUDA;
     st->blocks = p->nblocks;
     st->y_sieved = p->y_last >= p->y_first ? p->y_last - p->y_first + 1 : 0;

@@ -15,6 +15,7 @@
 #pragma once
 
 #include <cstdint>
+#include <vector>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -51,17 +52,15 @@ __host__ __device__ __forceinline__ uint32_t wheel_index(uint32_t v)
 __host__ __device__ __forceinline__ uint64_t wheel_y(uint64_t w) { return 3 * w + 1 + (w & 1); }
 
 // ---- sieve ------------------------------------------------------------------
-// Sieving primes and scratch of a wheel sieve (device arrays, primes >= 5).
+// Sieving primes and scratch of a wheel sieve (device arrays, primes >= 5), all
+// in one piece of memory of its owner.
 struct WheelSieve {
-    Allocator al;
-    uint32_t np = 0;            // primes in the table (2 and 3 are left out)
-    uint32_t *host_p = nullptr; // host copy
-    uint32_t *p = nullptr;      // primes
+    std::vector<uint32_t> host_p;  // primes 5 <= p <= P (2 and 3 are left out)
+    uint32_t *p = nullptr;         // the same on the device
     uint4 *pat = nullptr;       // phase copies of the small primes' pattern
     uint4 *rec = nullptr;       // per block, see wheel_prep_kernel
     uint2 *rec2 = nullptr;
     uint32_t *sqcnt = nullptr, *sqlist = nullptr, *err = nullptr;
-    uint64_t max_len = 0;       // wheel numbers of the largest block
 };
 
 // One block: wheel numbers [w0, w0 + len), both multiples of kSegY.
@@ -76,48 +75,93 @@ struct WheelLaunch {
     cudaEvent_t mid = nullptr, mid2 = nullptr;  // profiling: after a1, before a2
 };
 
-// Primes up to sqrt(y_max) (at least 1024) and scratch for blocks of up to
-// max_len wheel numbers; y_max < 2^54.
-int wheel_sieve_create(WheelSieve *t, const Allocator &al, uint64_t y_max, uint64_t max_len,
-                       cudaStream_t s);
-void wheel_sieve_destroy(WheelSieve *t);
-uint32_t wheel_sieve_status(WheelSieve *t);
+// Host part: the primes for blocks below y_max < 2^54 (up to its square root, at
+// least 1024).
+void wheel_sieve_primes(WheelSieve *t, uint64_t y_max);
+// Device bytes for blocks of up to max_len wheel numbers; the same memory (256-
+// byte aligned) split up, with the scratch cleared and the pattern made on `s`
+// (the caller fills t->p from t->host_p).  The kernels set kErrTimeout and
+// kErrList in *err.
+size_t wheel_sieve_bytes(const WheelSieve *t, uint64_t max_len);
+constexpr uint32_t kErrList = 4u;  // a square list overflowed its capacity
+int wheel_sieve_bind(WheelSieve *t, void *base, uint64_t max_len, uint32_t *err, cudaStream_t s);
 uint32_t wheel_primes_upto(const WheelSieve *t, uint64_t b);
 int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t s);
 bool wheel_sieve_exact(uint64_t y_max);
 
-// ---- update -------------------------------------------------------------------
-constexpr uint32_t kWheelGroup = 64;     // consecutive entries with one dense cut-off
-constexpr int kWheelDenseThreads = 256;
-enum { kDenseFloat = 0, kDenseHigh = 1, kDenseWide = 2 };
+// ---- plan -----------------------------------------------------------------------
+constexpr uint32_t kWheelGroup = 64;       // consecutive entries with one dense cut-off
+constexpr uint32_t kWheelGroupBlock = 8;   // groups of a dense work item; the first
+                                           // eight groups are items of their own (their
+                                           // k is large: more terms take a slow form)
+__host__ __device__ constexpr uint32_t wheel_group_blocks(uint32_t groups)
+{
+    return groups <= kWheelGroupBlock ? groups
+                                      : kWheelGroupBlock + (groups - 1) / kWheelGroupBlock;
+}
+// First group of group block b (b = their number: at least `groups`).
+__host__ __device__ constexpr uint32_t wheel_block_first(uint32_t b)
+{
+    return b < kWheelGroupBlock ? b : (b - kWheelGroupBlock + 1) * kWheelGroupBlock;
+}
+constexpr uint32_t kWheelItem = 256;       // wheel indices of a chunk of the global gather
+
+struct WheelQuery {
+    uint64_t n, X;
+    uint64_t off, goff;     // first entry, first group
+};
 
 struct WheelGroup {
     uint32_t first, count;  // entries
-    uint64_t yc;            // dense cut-off
-    uint64_t kmax;          // largest k of the group (0: no one-word entry)
-};
-
-// Part `part` of `parts` of chunk c's list, for groups [g0, g1).
-struct WheelDenseItem {
-    uint32_t c, g0, g1;
-    uint32_t mode_parts;    // mode | part << 8 | parts << 16
-};
-
-struct WheelDenseArgs {
-    const WheelDenseItem *items;
-    uint32_t nitems;
-    uint32_t *counter;
-    const WheelGroup *groups;
-    const uint64_t *K;
-    const uint16_t *dl;     // kSegY offsets per chunk: mu = +1, then mu = -1
-    const uint32_t *dl_cnt; // count(+1) | count(-1) << 16
-    uint64_t *S;
+    uint64_t yc;            // dense cut-off (a multiple of 6)
+    uint64_t kmax;          // largest k of the group
 };
 
 struct WheelGatherTile {
     uint64_t t0;            // y in [t0 + 1, t0 + len], t0 a multiple of 6
     uint64_t m1, m2;        // division magics of t0 + 1 and t0 + len + 1
     uint32_t len, l1, l2, pad;
+};
+
+// Totals of a target, made with the entries (WheelQuery order).
+struct WheelTotals {
+    unsigned long long direct, gathered;  // the method's terms (closed forms)
+    unsigned long long gather_j;          // gathered terms at the dense cut-offs
+    unsigned long long exec;              // those with j coprime to 6
+    unsigned long long dense_y;           // y below the cut-offs, over the entries
+};
+
+struct WheelEntryArgs {
+    const WheelQuery *qs;
+    uint32_t nq;
+    uint32_t ngroups;
+    double dc;              // dense cut-off factor
+    uint64_t *K, *YC;
+    uint32_t *JL, *JD;
+    WheelGroup *groups;
+    WheelTotals *totals;    // cleared
+    uint32_t parts;         // parts of a dense chunk's list
+    uint32_t *dpre;         // first dense item of every group block, then their number
+    WheelGatherTile *tiles;
+    const uint2 *tile_src;  // {first y / 6, len} of every tile
+    uint32_t ntiles;
+};
+// Entries, groups, totals, the dense work items' prefix sums and the gather
+// tiles' division constants of a plan.
+int wheel_entries_enqueue(const WheelEntryArgs &a, cudaStream_t s);
+
+// ---- update -------------------------------------------------------------------
+constexpr int kWheelDenseThreads = 256;
+
+struct WheelDenseArgs {
+    uint32_t *counter;
+    const WheelGroup *groups;
+    uint32_t ngroups, parts;
+    const uint32_t *pre;    // see WheelEntryArgs::dpre
+    const uint64_t *K;
+    const uint16_t *dl;     // kSegY offsets per chunk: mu = +1, then mu = -1
+    const uint32_t *dl_cnt; // count(+1) | count(-1) << 16
+    uint64_t *S;
 };
 
 struct WheelGatherArgs {
@@ -156,7 +200,7 @@ struct WheelBlockArgs {
 
 int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks, uint16_t *dl,
                              uint32_t *dl_cnt, cudaStream_t s);
-int wheel_dense_enqueue(const WheelDenseArgs &a, cudaStream_t s);
+int wheel_dense_enqueue(const WheelDenseArgs &a, uint64_t max_items, cudaStream_t s);
 int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s);
 int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s);
 

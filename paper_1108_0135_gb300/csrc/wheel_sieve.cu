@@ -27,7 +27,6 @@
 
 namespace mert {
 
-constexpr uint32_t kWErrBucket = 4u;          // a square list overflowed
 constexpr uint32_t kWPatPrimes = 3;           // table primes in the pattern: 5, 7, 11
 constexpr uint32_t kWPatPeriod = 2u * 25u * 49u * 121u;  // in w
 constexpr uint32_t kWPhases = 8;              // tile starts are even: phases 0, 2, .., 14
@@ -103,7 +102,7 @@ __global__ void wheel_prep_kernel(uint64_t I0, uint32_t np, const uint32_t *__re
             if (slot < kWSqCap)
                 list[(size_t)ti * kWSqCap + slot] = w - ti * tile;
             else
-                atomicOr(err, kWErrBucket);
+                atomicOr(err, kErrList);
         }
 }
 
@@ -519,77 +518,67 @@ bool wheel_sieve_exact(uint64_t y_max)
     return true;
 }
 
-int wheel_sieve_create(WheelSieve *t, const Allocator &al, uint64_t y_max, uint64_t max_len,
-                       cudaStream_t s)
+void wheel_sieve_primes(WheelSieve *t, uint64_t y_max)
 {
-    t->al = al;
     // the last block is rounded up to a whole segment
     const uint64_t B = sieve_bound(y_max + kWheelSegY);
     std::vector<uint8_t> comp(B / 2 + 1, 0);  // odd numbers 2i + 1
-    std::vector<uint32_t> pr;
+    t->host_p.clear();
     for (uint64_t q = 3; q <= B; q += 2) {
         if (comp[q >> 1])
             continue;
         if (q >= 5)
-            pr.push_back((uint32_t)q);
+            t->host_p.push_back((uint32_t)q);
         for (uint64_t j = q * q; j <= B; j += 2 * q)
             comp[j >> 1] = 1;
     }
-    const size_t np = pr.size();
-    t->np = (uint32_t)np;
-    t->max_len = max_len;
-    t->host_p = (uint32_t *)malloc(np * 4);
-    if (!t->host_p)
-        return 2;
-    memcpy(t->host_p, pr.data(), np * 4);
+}
+
+// Lays the arrays out from `base` (null: only counts); returns the bytes.
+static size_t wheel_layout(WheelSieve *t, size_t np, uint64_t max_len, char *base, size_t *clear)
+{
     const uint64_t nt = (max_len + kWTileSmall - 1) / kWTileSmall;
-    t->p = (uint32_t *)dev_alloc(al, np * 4);
-    t->pat = (uint4 *)dev_alloc(al, (size_t)kWPhases * kWPatLen);
-    t->rec = (uint4 *)dev_alloc(al, np * sizeof(uint4));
-    t->rec2 = (uint2 *)dev_alloc(al, np * sizeof(uint2));
-    t->sqcnt = (uint32_t *)dev_alloc(al, (nt + 1) * 4);
-    t->sqlist = (uint32_t *)dev_alloc(al, nt * kWSqCap * 4);
-    t->err = (uint32_t *)dev_alloc(al, 4);
-    if (!t->p || !t->pat || !t->rec || !t->rec2 || !t->sqcnt || !t->sqlist || !t->err)
-        return 2;
-    cudaMemcpyAsync(t->p, t->host_p, np * 4, cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(t->sqcnt, 0, (nt + 1) * 4, s);
-    cudaMemsetAsync(t->err, 0, 4, s);
+    size_t off = 0;
+    const auto take = [&](size_t bytes) {
+        char *q = base + off;
+        off += (bytes + 255) & ~(size_t)255;
+        return q;
+    };
+    char *c0 = take(nt * 4), *pat = take((size_t)kWPhases * kWPatLen), *p = take(np * 4),
+         *rec = take(np * sizeof(uint4)), *rec2 = take(np * sizeof(uint2)),
+         *list = take(nt * kWSqCap * 4);
+    if (t) {
+        t->sqcnt = (uint32_t *)c0;
+        t->pat = (uint4 *)pat;
+        t->p = (uint32_t *)p;
+        t->rec = (uint4 *)rec;
+        t->rec2 = (uint2 *)rec2;
+        t->sqlist = (uint32_t *)list;
+        *clear = nt * 4;
+    }
+    return off;
+}
+
+size_t wheel_sieve_bytes(const WheelSieve *t, uint64_t max_len)
+{
+    return wheel_layout(nullptr, t->host_p.size(), max_len, nullptr, nullptr);
+}
+
+int wheel_sieve_bind(WheelSieve *t, void *base, uint64_t max_len, uint32_t *err, cudaStream_t s)
+{
+    size_t clear = 0;
+    wheel_layout(t, t->host_p.size(), max_len, (char *)base, &clear);
+    t->err = err;
+    cudaMemsetAsync(t->sqcnt, 0, clear, s);
     wheel_pattern_kernel<<<dim3((kWPatLen + 255) / 256, kWPhases), 256, 0, s>>>((uint8_t *)t->pat);
-    return cudaStreamSynchronize(s) == cudaSuccess ? 0 : 3;
-}
-
-void wheel_sieve_destroy(WheelSieve *t)
-{
-    const size_t np = t->np;
-    const uint64_t nt = (t->max_len + kWTileSmall - 1) / kWTileSmall;
-    dev_free(t->al, t->p, np * 4);
-    dev_free(t->al, t->pat, (size_t)kWPhases * kWPatLen);
-    dev_free(t->al, t->rec, np * sizeof(uint4));
-    dev_free(t->al, t->rec2, np * sizeof(uint2));
-    dev_free(t->al, t->sqcnt, (nt + 1) * 4);
-    dev_free(t->al, t->sqlist, nt * kWSqCap * 4);
-    dev_free(t->al, t->err, 4);
-    free(t->host_p);
-    *t = WheelSieve();
-}
-
-uint32_t wheel_sieve_status(WheelSieve *t)
-{
-    if (!t->err)
-        return 0;
-    uint32_t v = 0;
-    cudaMemcpy(&v, t->err, 4, cudaMemcpyDeviceToHost);
-    if (v)
-        cudaMemset(t->err, 0, 4);
-    return v;
+    return cudaGetLastError() == cudaSuccess ? 0 : 3;
 }
 
 uint32_t wheel_primes_upto(const WheelSieve *t, uint64_t b)
 {
-    return (uint32_t)(std::upper_bound(t->host_p, t->host_p + t->np,
+    return (uint32_t)(std::upper_bound(t->host_p.begin(), t->host_p.end(),
                                        (uint32_t)std::min<uint64_t>(b, 0xffffffffu)) -
-                      t->host_p);
+                      t->host_p.begin());
 }
 
 template <uint32_t TILE, int THREADS, int MINB>

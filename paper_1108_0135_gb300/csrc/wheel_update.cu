@@ -29,6 +29,166 @@ constexpr uint32_t kMagicBits = 0x4B400000u;  // bits of 1.5 2^23: adding it rou
 constexpr float kMagicF = 12582912.0f;
 
 // ---------------------------------------------------------------------------
+// Plan: the entries of every target, a warp per group of 64 (two per lane).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint64_t isqrt_dev(uint64_t v)
+{
+    uint64_t r = (uint64_t)sqrt((double)v);
+    while (r * r > v)
+        --r;
+    while ((r + 1) * (r + 1) <= v)
+        ++r;
+    return r;
+}
+
+__device__ __forceinline__ uint64_t warp_max_u64(uint64_t v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+
+// k = floor(n/x), the first j of its gathered terms and the group's dense
+// cut-off: dc sqrt(k of the group's first entry), up to a multiple of 4096 less
+// one, within [floor(sqrt(k)), floor(k/jlo) - 1] of every entry where the group
+// has such a value (per entry otherwise), and for the group the least of these
+// and of floor(k/jlo) (beyond it no term is left), down to a multiple of 6.
+__global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g >= a.ngroups)
+        return;
+    uint32_t lo_q = 0, hi_q = a.nq;  // the last target with goff <= g
+    while (hi_q - lo_q > 1) {
+        const uint32_t mid = (lo_q + hi_q) >> 1;
+        if (a.qs[mid].goff <= g)
+            lo_q = mid;
+        else
+            hi_q = mid;
+    }
+    const WheelQuery Q = a.qs[lo_q];
+    const uint64_t x0 = (g - Q.goff) * kWheelGroup + 1;
+    const uint32_t cnt = (uint32_t)min((uint64_t)kWheelGroup, Q.X - x0 + 1);
+    const uint64_t kf = Q.n / x0;
+    uint64_t k[2], sq[2], vh[2], jlo[2], cap[2];
+    uint64_t lo = 0, nhi = 0;  // max of s, max of ~vh (= ~min)
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t i = lane + 32u * (uint32_t)h;
+        k[h] = 0;
+        if (i < cnt) {
+            const uint64_t x = x0 + i;
+            k[h] = Q.n / x;
+            sq[h] = isqrt_dev(k[h]);
+            jlo[h] = Q.X / x + 1;
+            cap[h] = k[h] / jlo[h];
+            vh[h] = jlo[h] <= k[h] / (sq[h] + 1) ? cap[h] - 1 : sq[h];
+            lo = max(lo, sq[h]);
+            nhi = max(nhi, ~vh[h]);
+        }
+    }
+    lo = warp_max_u64(lo);
+    const uint64_t hi = ~warp_max_u64(nhi);
+    uint64_t target = (uint64_t)(a.dc * sqrt((double)kf));
+    target = (target + kChunk) / kChunk * kChunk - 1;
+    uint64_t nyc = 0, yce[2];  // max of ~cut-off
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (k[h]) {
+            yce[h] = lo <= hi ? min(max(target, lo), hi) : min(max(target, sq[h]), vh[h]);
+            nyc = max(nyc, ~min(yce[h], cap[h]));
+        }
+    uint64_t yc = ~warp_max_u64(nyc);
+    yc -= yc % 6;
+    uint64_t direct = 0, gathered = 0, gather_j = 0, exec = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        if (k[h]) {
+            const uint64_t e = Q.off + x0 - 1 + lane + 32u * (uint32_t)h;
+            const uint64_t jd = max(k[h] / (yc + 1), jlo[h] - 1);
+            a.K[e] = k[h];
+            a.YC[e] = yc;
+            a.JL[e] = (uint32_t)jlo[h];
+            a.JD[e] = (uint32_t)jd;
+            direct += sq[h];
+            const uint64_t jhi = k[h] / (sq[h] + 1), jc = k[h] / (yce[h] + 1);
+            gathered += jhi >= jlo[h] ? jhi - jlo[h] + 1 : 0;
+            gather_j += jc >= jlo[h] ? jc - jlo[h] + 1 : 0;
+            exec += phi6(jd) - phi6(jlo[h] - 1);
+        }
+    direct = warp_sum_u64(direct);
+    gathered = warp_sum_u64(gathered);
+    gather_j = warp_sum_u64(gather_j);
+    exec = warp_sum_u64(exec);
+    if (lane == 0) {
+        WheelGroup G;
+        G.first = (uint32_t)(Q.off + x0 - 1);
+        G.count = cnt;
+        G.yc = yc;
+        G.kmax = kf;
+        a.groups[g] = G;
+        WheelTotals *t = a.totals + lo_q;
+        atomicAdd(&t->direct, direct);
+        atomicAdd(&t->gathered, gathered);
+        atomicAdd(&t->gather_j, gather_j);
+        atomicAdd(&t->exec, exec);
+        atomicAdd(&t->dense_y, yc * cnt);
+    }
+}
+
+// Dense work items: (group block, chunk below its largest cut-off, part of the
+// chunk's list); dpre[b] = items of the blocks before b.  One CTA.
+__global__ void __launch_bounds__(1024) wheel_dense_items_kernel(WheelEntryArgs a)
+{
+    __shared__ uint32_t sh[33];
+    const uint32_t nb = wheel_group_blocks(a.ngroups);
+    uint32_t before = 0;
+    for (uint32_t b0 = 0; b0 < nb; b0 += 1024u) {
+        const uint32_t b = b0 + threadIdx.x;
+        uint64_t yc = 0;
+        if (b < nb)
+            for (uint32_t g = wheel_block_first(b); g < min(wheel_block_first(b + 1), a.ngroups); ++g)
+                yc = max(yc, a.groups[g].yc);
+        const uint32_t c = (uint32_t)((yc + kWheelSegY - 1) / kWheelSegY) * a.parts;
+        uint32_t tot;
+        const uint32_t ex = block_scan_u32(c, sh, &tot);
+        if (b < nb)
+            a.dpre[b] = before + ex;
+        before += tot;
+    }
+    if (threadIdx.x == 0)
+        a.dpre[nb] = before;
+}
+
+__global__ void wheel_tiles_kernel(WheelEntryArgs a)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= a.ntiles)
+        return;
+    const uint2 v = a.tile_src[2 * i];
+    WheelGatherTile T;
+    T.t0 = (uint64_t)v.x | ((uint64_t)v.y << 32);
+    T.len = a.tile_src[2 * i + 1].x;
+    T.m1 = magic_of(T.t0 + 1);
+    T.l1 = magic_shift(T.t0 + 1);
+    T.m2 = magic_of(T.t0 + T.len + 1);
+    T.l2 = magic_shift(T.t0 + T.len + 1);
+    T.pad = 0;
+    a.tiles[i] = T;
+}
+
+int wheel_entries_enqueue(const WheelEntryArgs &a, cudaStream_t s)
+{
+    wheel_entries_kernel<<<(a.ngroups + 3) / 4, 128, 0, s>>>(a);
+    wheel_dense_items_kernel<<<1, 1024, 0, s>>>(a);
+    if (a.ntiles)
+        wheel_tiles_kernel<<<(a.ntiles + 127) / 128, 128, 0, s>>>(a);
+    return cudaGetLastError() == cudaSuccess ? 0 : -1;
+}
+
+// ---------------------------------------------------------------------------
 // Dense list: chunk c holds the wheel numbers [c kSegY, (c + 1) kSegY), one
 // segment of the sieve; dl gets the offsets of its squarefree numbers, those
 // with mu = +1 first, read off as differences of the segment's M6.
@@ -121,22 +281,24 @@ __device__ __forceinline__ void dense_float(const uint4 *el, uint32_t n, const f
         out[e] = 2ull * (uint32_t)(st[e] - n * kMagicBits) + n - ss[e];
 }
 
-// High-word mode: staged {m, -6y, y}, m = floor(2^(31 + ex)/(6y)), 2^ex <= 6y of
-// the chunk; kh the top 32 bits of k, sh the shift.  Truncations of 2^-31 and
-// at most 2^-29 and one of 2^-sh (sh >= 4) with k/(6y) < 6e7: less than 0.22.
+// High-word mode: staged {m, -6y, y, ex}, m = floor(2^(31 + ex)/(6y)) in [2^30,
+// 2^31), ex = floor(log2 6y); kh the top 32 bits of k (b bits), T the rounded
+// (kh m / 2^32) / 2^(ex + 31 - b).  Truncations of 2^-31 and 2^-30 and one of a
+// unit before the shift (at least 3) with k/(6y) < 6e7: less than 0.3.
 __device__ __forceinline__ void dense_high(const uint4 *el, uint32_t n, const uint32_t kh[2],
-                                           const uint32_t sh[2], const uint32_t kl[2],
+                                           const uint32_t sb[2], const uint32_t kl[2],
                                            uint64_t out[2])
 {
     uint64_t st[2] = {0, 0};
     uint32_t ss[2] = {0, 0};
-    const uint32_t half[2] = {1u << (sh[0] - 1u), 1u << (sh[1] - 1u)};
 #pragma unroll 4
     for (uint32_t i = 0; i < n; ++i) {
         const uint4 v = el[i];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const uint32_t T = (__umulhi(kh[e], v.x) + half[e]) >> sh[e];
+            // shift less one, at most 31 (k far below 6y: T = 0)
+            const uint32_t sh = min(v.w + sb[e], 31u);
+            const uint32_t T = ((__umulhi(kh[e], v.x) >> sh) + 1u) >> 1;
             const uint32_t r = T * v.y + kl[e];
             st[e] += T;
             ss[e] = add_sign(r + v.z, ss[e]);
@@ -164,48 +326,79 @@ __device__ __forceinline__ void dense_wide(const uint16_t *off, uint32_t n, uint
     }
 }
 
+// A work item is part of a chunk's list for kWheelGroupBlock groups.  Items whose
+// k/(6y) all lie below 1.5e6 (and y < 3.5e8) take the float mode; in the others
+// the y up to kmax/3.6e8 (all y from 3.5e8) take 64-bit division, the rest the
+// high-word mode.
 __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDenseArgs a)
 {
     __shared__ uint4 s_el[kSegY];
     __shared__ uint16_t s_off[kSegY];
-    __shared__ uint32_t s_item;
+    __shared__ uint32_t s_item, s_block;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
+    const uint32_t nb = wheel_group_blocks(a.ngroups);
+    const uint32_t nitems = a.pre[nb];
     for (;;) {
-        if (threadIdx.x == 0)
-            s_item = atomicAdd(a.counter, 1u);
+        if (warp == 0) {
+            uint32_t it = 0;
+            if (lane == 0)
+                it = atomicAdd(a.counter, 1u);
+            it = __shfl_sync(0xffffffffu, it, 0);
+            // the last group block with pre <= it, 32 candidates at a time
+            uint32_t lo = 0, hi = nb;
+            while (it < nitems && hi - lo > 1u) {
+                const uint32_t step = (hi - lo + 31u) / 32u, p = lo + lane * step;
+                const uint32_t le = __popc(__ballot_sync(0xffffffffu, p < hi && a.pre[p] <= it));
+                hi = min(hi, lo + le * step);
+                lo += (le - 1u) * step;
+            }
+            if (lane == 0) {
+                s_item = it;
+                s_block = lo;
+            }
+        }
         __syncthreads();
-        if (s_item >= a.nitems)
+        if (s_item >= nitems)
             break;
-        const WheelDenseItem it = a.items[s_item];
-        const uint32_t mode = it.mode_parts & 255u, part = (it.mode_parts >> 8) & 255u,
-                       parts = it.mode_parts >> 16;
-        const uint32_t cnt = a.dl_cnt[it.c];
+        const uint32_t g0 = wheel_block_first(s_block);
+        const uint32_t ng = min(wheel_block_first(s_block + 1), a.ngroups) - g0;
+        const uint32_t rel = s_item - a.pre[s_block];
+        const uint32_t c = rel / a.parts, part = rel % a.parts;
+        uint64_t kmax = 0;
+        for (uint32_t g = 0; g < ng; ++g)
+            kmax = max(kmax, a.groups[g0 + g].kmax);
+        const uint64_t y0 = (uint64_t)c * kWheelSegY;
+        const bool small_y = y0 + kWheelSegY < 350000000u;
+        const bool fl = small_y && kmax < 9000000ull * (y0 + 1);
+        const uint32_t cnt = a.dl_cnt[c];
         const uint32_t cp = cnt & 0xffffu, cm = cnt >> 16;
-        const uint32_t p0 = cp * part / parts, m0 = cm * part / parts;
-        const uint32_t np = cp * (part + 1u) / parts - p0, nm = cm * (part + 1u) / parts - m0;
-        const uint64_t y0 = (uint64_t)it.c * kWheelSegY;
-        const uint16_t *src = a.dl + (uint64_t)it.c * kSegY;
-        // float and high-word modes: y < 3.5e8
-        const uint32_t ex = 31u - __clz((uint32_t)(6u * (uint32_t)y0 + 6u));
+        const uint32_t p0 = cp * part / a.parts, m0 = cm * part / a.parts;
+        const uint32_t np = cp * (part + 1u) / a.parts - p0, nm = cm * (part + 1u) / a.parts - m0;
+        const uint16_t *src = a.dl + (uint64_t)c * kSegY;
         for (uint32_t i = threadIdx.x; i < np + nm; i += blockDim.x) {
             const uint32_t o = i < np ? src[p0 + i] : src[cp + m0 + (i - np)];
             s_off[i] = (uint16_t)o;
+            if (!small_y)
+                continue;
             const uint32_t y = (uint32_t)y0 + 3u * o + 1u + (o & 1u), d = 6u * y;
-            if (mode == kDenseFloat) {
+            if (fl) {
                 const float rf = __frcp_rn(__uint2float_rn(d));
                 const uint32_t cd = kMagicBits * d;
                 s_el[i] = make_uint4(__float_as_uint(rf), 0u - d, cd + y, cd - y);
-            } else if (mode == kDenseHigh) {
-                s_el[i] = make_uint4((uint32_t)((1ull << (31u + ex)) / d), 0u - d, y, 0u);
+            } else {
+                const uint32_t ex = 31u - __clz(d);
+                s_el[i] = make_uint4((uint32_t)((1ull << (31u + ex)) / d), 0u - d, y, ex);
             }
         }
         __syncthreads();
         // one group per warp; fewer groups than warps: several warps share a
         // group, each with its part of the staged lists
-        const uint32_t ng = it.g1 - it.g0, share = ng < nwarp ? nwarp / ng : 1u;
+        const uint32_t share = nwarp / ng;
         for (uint32_t t = warp; t < ng * share; t += nwarp) {
-            const WheelGroup G = a.groups[it.g0 + t % ng];
+            const WheelGroup G = a.groups[g0 + t % ng];
             const uint32_t q = t / ng;
+            if (G.yc <= y0)
+                continue;
             uint64_t k[2];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
@@ -214,45 +407,56 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
             }
             uint32_t n0 = np, n1 = nm;
             if (G.yc < y0 + kWheelSegY) {
-                const uint32_t lim = (uint32_t)(phi6(G.yc) - (uint64_t)it.c * kSegY);
+                const uint32_t lim = (uint32_t)(phi6(G.yc) - (uint64_t)c * kSegY);
                 n0 = count_below(s_off, np, lim);
                 n1 = count_below(s_off + np, nm, lim);
             }
             const uint32_t f0 = n0 * q / share, f1 = np + n1 * q / share;
             n0 = n0 * (q + 1u) / share - f0;
             n1 = n1 * (q + 1u) / share - (f1 - np);
-            uint64_t plus[2], minus[2];
-            if (mode == kDenseFloat) {
+            uint64_t sum[2], part2[2];
+            if (fl) {
                 const float kf[2] = {__ull2float_rn(k[0]), __ull2float_rn(k[1])};
                 const uint32_t kl[2] = {(uint32_t)k[0], (uint32_t)k[1]};
-                dense_float(s_el + f0, n0, kf, kl, plus);
-                dense_float(s_el + f1, n1, kf, kl, minus);
-            } else if (mode == kDenseHigh) {
-                uint32_t kh[2], sh[2], kl[2];
+                dense_float(s_el + f0, n0, kf, kl, sum);
+                dense_float(s_el + f1, n1, kf, kl, part2);
+                sum[0] -= part2[0];
+                sum[1] -= part2[1];
+            } else {
+                const uint64_t yw = small_y ? G.kmax / 360000000ull : UINT64_MAX;
+                uint32_t w0 = 0, w1 = 0;  // terms by division
+                if (yw > y0) {
+                    const uint32_t lim =
+                        yw >= y0 + kWheelSegY ? 0xffffu
+                                              : (uint32_t)(phi6(yw) - (uint64_t)c * kSegY);
+                    w0 = count_below(s_off + f0, n0, lim);
+                    w1 = count_below(s_off + f1, n1, lim);
+                }
+                uint32_t kh[2], sb[2], kl[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const uint32_t b = bitlen64(k[e]);
                     kl[e] = (uint32_t)k[e];
-                    kh[e] = b >= 32u ? (uint32_t)(k[e] >> (b - 32u)) : (uint32_t)k[e] << (32u - b);
-                    sh[e] = ex + 31u - b;
-                    if (b == 0u || sh[e] > 31u) {  // k / (6y) rounds to 0
-                        kh[e] = 0u;
-                        sh[e] = 31u;
-                    }
+                    kh[e] = b >= 32u ? (uint32_t)(k[e] >> (b - 32u)) : (uint32_t)k[e] << ((32u - b) & 31u);
+                    sb[e] = 30u - b;
                 }
-                dense_high(s_el + f0, n0, kh, sh, kl, plus);
-                dense_high(s_el + f1, n1, kh, sh, kl, minus);
-            } else {
-                dense_wide(s_off + f0, n0, y0, k, plus);
-                dense_wide(s_off + f1, n1, y0, k, minus);
+                dense_wide(s_off + f0, w0, y0, k, sum);
+                dense_wide(s_off + f1, w1, y0, k, part2);
+                sum[0] -= part2[0];
+                sum[1] -= part2[1];
+                dense_high(s_el + f0 + w0, n0 - w0, kh, sb, kl, part2);
+                sum[0] += part2[0];
+                sum[1] += part2[1];
+                dense_high(s_el + f1 + w1, n1 - w1, kh, sb, kl, part2);
+                sum[0] -= part2[0];
+                sum[1] -= part2[1];
             }
 #pragma unroll
-            for (int e = 0; e < 2; ++e) {
-                const uint32_t i = lane + 32u * (uint32_t)e;
-                if (i < G.count && k[e])
-                    atomicAdd(reinterpret_cast<unsigned long long *>(a.S + G.first + i),
-                              (unsigned long long)(plus[e] - minus[e]));
-            }
+            for (int e = 0; e < 2; ++e)
+                if (k[e])
+                    atomicAdd(reinterpret_cast<unsigned long long *>(a.S + G.first + lane +
+                                                                     32u * (uint32_t)e),
+                              (unsigned long long)sum[e]);
         }
         __syncthreads();
     }
@@ -591,7 +795,7 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
 // ---------------------------------------------------------------------------
 // Global-memory part of a block (y0, y0 + len]: one lane per entry.  Gathered
 // terms with floor(k/j) in [ylo, y0 + len] of entries with k < kmax (few: here;
-// more: posted as chunks of kSparseItem wheel indices for wheel_chunk_kernel);
+// more: posted as chunks of kWheelItem wheel indices for wheel_chunk_kernel);
 // the dense form's -M6(yc) phi6(jd) when yc is in the block; and the values
 // M6(floor(k/m)), m = 2, 3, 6, of M(k) that lie in the block when m x is
 // beyond the array (m >= floor(X/x) + 1).
@@ -646,7 +850,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
         atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e), (unsigned long long)acc);
     }
     // heavy entries: chunk records, slots taken with one atomic per warp
-    const uint32_t nch = cnt > kWheelLaneTerms ? (cnt + kSparseItem - 1) / kSparseItem : 0u;
+    const uint32_t nch = cnt > kWheelLaneTerms ? (cnt + kWheelItem - 1) / kWheelItem : 0u;
     uint32_t incl = nch;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -663,9 +867,9 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
     base = __shfl_sync(0xffffffffu, base, 31);
     uint32_t slot = base + incl - nch;
     for (uint32_t c = 0; c < nch; ++c, ++slot) {
-        const uint32_t w = wl + c * (uint32_t)kSparseItem;
+        const uint32_t w = wl + c * kWheelItem;
         if (slot < a.qcap)
-            a.queue[slot] = make_uint4((uint32_t)e, w, min(wh - w, (uint32_t)kSparseItem), 0u);
+            a.queue[slot] = make_uint4((uint32_t)e, w, min(wh - w, kWheelItem), 0u);
         else
             atomicOr(a.err, kErrQueue);
     }
@@ -793,13 +997,11 @@ int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks,
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-int wheel_dense_enqueue(const WheelDenseArgs &a, cudaStream_t s)
+int wheel_dense_enqueue(const WheelDenseArgs &a, uint64_t max_items, cudaStream_t s)
 {
-    if (a.nitems == 0)
-        return 0;
     int per = 0;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, wheel_dense_kernel, kWheelDenseThreads, 0);
-    const uint32_t grid = std::min<uint32_t>((uint32_t)(sm_count() * std::max(per, 1)), a.nitems);
+    const uint32_t grid = (uint32_t)std::min<uint64_t>((uint64_t)(sm_count() * std::max(per, 1)), max_items);
     cudaMemsetAsync(a.counter, 0, 4, s);
     wheel_dense_kernel<<<grid, kWheelDenseThreads, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
