@@ -102,12 +102,12 @@ int mertens_plan(mertens_plan_t *out, const mertens_u128 *n, size_t count,
                  mertens_u128 u, uint64_t block_len);
 
 /*
- * Resident M(y) table.  The sieve's output (steps a1 + a2: M(y) for
- * 1 <= y <= y_max) is computed once and kept in device memory (about
- * 2 bytes per y), together with what the update needs independently of the
- * target for all n <= n_max (the divisor magics and the squarefree list of
- * the dense form).  Plans made on it read M(y) from the table for every sieve
- * block that ends at or below y_max and sieve only the blocks above it; their
+ * Resident M(y) table.  The sieve's output for 1 <= y <= y_max (steps a1 +
+ * a2, over the y coprime to 6, from which M(y) follows) is computed once and
+ * kept in device memory (about 0.67 bytes per y), together with what the
+ * update needs independently of the target for all n <= n_max (the squarefree
+ * list of the dense form).  Plans made on it read M(y) from the table for every
+ * sieve block that ends at or below y_max and sieve only the blocks above it; their
  * sieve limit u is at least min(n, y_max + 1) (the table's part of the sieve
  * costs nothing and the update's terms fall as 1/sqrt(u)) and at least the
  * automatic limit of a sieving plan for the same targets; a target

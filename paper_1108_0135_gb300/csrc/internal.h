@@ -146,26 +146,21 @@ inline uint64_t dense_chunks(uint64_t ydense) { return ydense / kChunk + 1; }
 
 }  // namespace mert
 
-// A resident M(y) table (mertens_table_create): M(y) for 1 <= y <= y_max in
-// the sieve's block layout (int16 relative to the 2048-y segment, int64
-// segment offsets, both indexed from y = 1), and the query-independent parts
-// of the update for targets up to n_max: divisor magics for d < mg_n and the
-// squarefree dense list for y <= ydense.
+// A resident table (mertens_table_create) in the form of wheel.h: M6(y) for the
+// y <= y_cov (y_max up to whole segments) coprime to 6, in the sieve's layout
+// (int16 relative to the 2048-number segment, int64 segment offsets), and the
+// dense list of the squarefree ones up to ydense.
 struct mertens_table_s {
     mert::Allocator al;
     int device = 0;
-    uint64_t y_max = 0;
+    uint64_t y_max = 0, y_cov = 0;
     uint64_t n_max_lo = 0, n_max_hi = 0;
-    uint64_t ydense = 0, mg_n = 0;
+    uint64_t ydense = 0;
     int16_t *Mloc = nullptr;
     int64_t *segoff = nullptr;
-    uint64_t *MG = nullptr, *dl_m = nullptr;
-    uint16_t *dl_yo = nullptr;
-    uint2 *dl_cnt = nullptr;
+    uint16_t *dl = nullptr;
+    uint32_t *dl_cnt = nullptr;
     size_t bytes = 0;
     std::vector<std::pair<void *, size_t>> allocs;
 };
 
-namespace mert {
-
-}  // namespace mert

@@ -263,6 +263,7 @@ struct mertens_plan_s {
     // entries with k >= 2^63 (targets n >= 2^63) and the wide kernel's
     // grid width per block (0: no terms in the block)
     std::vector<WideEntry> wide;
+    std::vector<uint64_t> wide_direct, wide_gathered;  // their terms, per target (wheel plans)
     WideEntry *dwide = nullptr;
     std::vector<uint32_t> wide_grid;
     bool mg_built = false;
@@ -534,40 +535,98 @@ int mertens_describe(mertens_u128 n, mertens_u128 u, mertens_query_info *info)
     return MERTENS_OK;
 }
 
-// A plan over the integers coprime to 6: targets n (one word) with sieve limits
-// us.  The entries, their dense cut-offs and the dense work items are made on
+// The dense cut-off (at most, over the entries) that the planner sets for the
+// first 64 entries of target n: what a table's squarefree list has to reach.
+static uint64_t first_cutoff(u128 n, uint64_t X, double dc, u128 wide_from)
+{
+    const uint64_t cnt = std::min<uint64_t>(64, X);
+    uint64_t lo = 0, hi = UINT64_MAX, kf = 0, top = 0;
+    std::vector<std::pair<uint64_t, uint64_t>> v;  // floor(sqrt(k)), the largest cut-off
+    bool wide = false;
+    for (uint64_t x = 1; x <= cnt; ++x) {
+        if (n / x >= wide_from) {
+            wide = true;
+            continue;
+        }
+        const uint64_t k = (uint64_t)(n / x), s = isqrt64(k), jlo = X / x + 1;
+        const uint64_t vh = jlo <= k / (s + 1) ? k / jlo - 1 : s;
+        kf = std::max(kf, k);
+        lo = std::max(lo, s);
+        hi = std::min(hi, vh);
+        v.push_back({s, vh});
+    }
+    const uint64_t t =
+        ((uint64_t)(dc * std::sqrt((double)kf)) + kChunk) / kChunk * kChunk - 1;
+    if (!wide && lo <= hi)
+        return std::min(std::max(t, lo), hi);
+    for (const auto &e : v)
+        top = std::max(top, std::min(std::max(t, e.first), e.second));
+    return top;
+}
+
+// A plan over the integers coprime to 6: targets n with sieve limits us, on a
+// resident table or not.  The entries, their dense cut-offs and the dense work items are made on
 // the device; the host lays out blocks, gather tiles and memory.  Blocks are
 // whole segments (6144 y) of about block_len y.
 static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::vector<u128> &n,
                              const std::vector<uint64_t> &us, uint64_t block_len,
-                             const mertens_tuning &tn)
+                             const mertens_tuning &tn, mertens_table_s *table)
 {
     const size_t count = n.size();
     const double dc = dense_factor(tn);
+    const u128 wide_from = wide_threshold();
     std::vector<WheelQuery> qs(count);
-    uint64_t E = 0, G = 0;
+    uint64_t E = 0, G = 0, cut = 0;
     double acc = 0, ksum = 0, terms = 0, pairs = 0;
     for (size_t i = 0; i < count; ++i) {
-        const uint64_t ni = (uint64_t)n[i], X = ni / us[i];
-        qs[i] = {ni, X, E, G};
-        p->n.push_back(ni);
-        p->n_hi.push_back(0);
+        const uint64_t X = (uint64_t)(n[i] / us[i]);
+        qs[i] = {(uint64_t)n[i], (uint64_t)(n[i] >> 64), X, E, G};
+        p->n.push_back(qs[i].n);
+        p->n_hi.push_back(qs[i].n_hi);
         p->u.push_back(us[i]);
         p->X.push_back(X);
         p->off.push_back(E);
+        p->wide_direct.push_back(0);
+        p->wide_gathered.push_back(0);
         const uint64_t ng = (X + kWheelGroup - 1) / kWheelGroup;
-        E += X;
         G += ng;
+        if (table && n[i] <= table->y_max && X == 1) {
+            // M(n) is in the table: one entry, no terms, read after resolve
+            p->lookups.push_back(E);
+            p->lookups.push_back(qs[i].n);
+            p->ymax_q.push_back(0);
+            qs[i].n = 0;
+            E += X;
+            continue;
+        }
+        for (uint64_t x = 1; x <= X && n[i] / x >= wide_from; ++x) {
+            const u128 k = n[i] / x;
+            WideEntry W;
+            W.k_lo = (uint64_t)k;
+            W.k_hi = (uint64_t)(k >> 64);
+            W.s = isqrt128(k);
+            W.jlo = X / x + 1;
+            W.jhi = (uint64_t)(k / ((u128)W.s + 1));
+            W.e = E + x - 1;
+            p->wide.push_back(W);
+            p->wide_direct.back() += W.s;
+            p->wide_gathered.back() += W.jhi >= W.jlo ? W.jhi - W.jlo + 1 : 0;
+        }
+        if (table)
+            cut = std::max(cut, first_cutoff(n[i], X, dc, wide_from));
+        E += X;
         // the largest y read: a direct term's, or the gathered range's of x = 1
-        p->ymax_q.push_back(std::max(isqrt64(ni), ni / (X + 1)));
+        const uint64_t yg = (uint64_t)(n[i] / ((u128)X + 1));
+        p->ymax_q.push_back(std::max(isqrt128(n[i]), yg));
         p->y_max = std::max(p->y_max, p->ymax_q.back());
         // no cut-off is above the first group's target value
-        const uint64_t t = ((uint64_t)(dc * std::sqrt((double)ni)) + kChunk) / kChunk * kChunk;
-        p->ydense = std::max(p->ydense, std::min(t, ni / (X + 1)));
+        const double nd = (double)n[i], kf = std::min(nd, (double)wide_from);
+        const uint64_t t = ((uint64_t)(dc * std::sqrt(kf)) + kChunk) / kChunk * kChunk;
+        p->ydense = std::max(p->ydense, std::min(t, yg));
         const double lx = std::log((double)std::max<uint64_t>(X, 2));
-        acc += (double)ni * lx;
-        ksum += (double)ni * (lx + 1.0);
-        const double root = 2.0 * std::sqrt((double)ni * (double)X);  // sum of sqrt(k)
+        acc += nd * lx;
+        ksum += nd * (lx + 1.0);
+        const double root = 2.0 * std::sqrt(nd * (double)X);  // sum of sqrt(k)
         terms += root / dc / 3.0;
         pairs += dc * root / (double)(kWheelSegY * kWheelGroup * kWheelGroupBlock) +
                  (double)ng / kWheelGroupBlock;
@@ -578,8 +637,25 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         return MERTENS_ENOTSUP;
     }
     p->nent = E;
+    p->y_max = std::max<uint64_t>(p->y_max, 1);
     p->y_first = 1;
     p->y_last = p->y_max;
+    p->table = table;
+    if (table) {
+        if (block_len == 0)
+            block_len = 1ull << 30;
+        if (block_len % kSegY) {
+            set_last_error("mertens_plan_on_table: block_len must be a multiple of %d", kSegY);
+            delete p;
+            return MERTENS_EINVAL;
+        }
+        if (cut > table->ydense) {
+            set_last_error("mertens_plan_on_table: the targets need dense cut-offs beyond the "
+                           "table");
+            delete p;
+            return MERTENS_ENOTSUP;
+        }
+    }
     if (block_len == 0) {
         // one block when it fits 2^28 y, else 2^28 (up to 2^36 y) or 2^30 y blocks
         uint64_t cap = p->y_last > (1ull << 36) ? (1ull << 30) : (1ull << 28);
@@ -593,6 +669,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         return MERTENS_EINVAL;
     }
     block_len = std::min(block_len, p->y_last);
+    // a plan on a table sieves only the blocks that end above it
+    p->sieves = !table || p->y_last > table->y_max;
     p->block_len = (block_len + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
     p->nblocks = (p->y_last + p->block_len - 1) / p->block_len;
     p->wchunks = (p->ydense + kWheelSegY - 1) / kWheelSegY;
@@ -631,7 +709,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     const double item_work = std::min(2.0e6, std::max(4096.0, terms / (456.0 * 24.0)));
     // sum of k over the x in (a, b] of target i
     const auto k_between = [&](size_t i, double a, double b) {
-        return (double)qs[i].n * std::log((b + 0.5) / (a + 0.5));
+        return (double)n[i] * std::log((b + 0.5) / (a + 0.5));
     };
     std::vector<uint2> tiles;  // {first y less one, low and high word}, {length, 0}
     std::vector<uint4> items;
@@ -651,7 +729,9 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             double sum = 0;
             const uint64_t k0i = (uint64_t)std::ceil(std::min(k0, 9.2e18));
             for (size_t i = 0; i < count; ++i) {
-                const uint64_t xt = std::min(qs[i].X, qs[i].n / k0i);
+                if (!qs[i].n && !qs[i].n_hi)
+                    continue;
+                const uint64_t xt = (uint64_t)std::min<u128>(qs[i].X, n[i] / k0i);
                 if (xt == 0)
                     continue;
                 all.push_back({qs[i].off, qs[i].off + xt});
@@ -674,10 +754,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
                 ks.clear();
                 for (size_t i = 0; i < count; ++i) {
                     const WheelQuery &Q = qs[i];
-                    const double te = (double)(t0 + len) + 8.0;
+                    if (!Q.n && !Q.n_hi)
+                        continue;
+                    const double nd = (double)n[i], te = (double)(t0 + len) + 8.0;
                     uint64_t lo = 0;
-                    if (2.0 * (dc * std::sqrt((double)Q.n) + 2.0 * kChunk) < (double)us[i])
-                        lo = (uint64_t)std::min((double)Q.X, dc * dc * (double)Q.n / (te * te)) /
+                    if (2.0 * (dc * std::sqrt(nd) + 2.0 * kChunk) < (double)us[i])
+                        lo = (uint64_t)std::min((double)Q.X, dc * dc * nd / (te * te)) /
                              kWheelGroup * kWheelGroup;
                     if (lo >= Q.X)
                         continue;
@@ -733,8 +815,9 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     const uint64_t wlen = p->block_len / 3;
     const uint32_t ntiles = (uint32_t)(tiles.size() / 2);
     p->serial = true;
-    wheel_sieve_primes(&p->ws, p->y_last);
-    const size_t ws_bytes = wheel_sieve_bytes(&p->ws, wlen);
+    if (p->sieves)
+        wheel_sieve_primes(&p->ws, p->y_last);
+    const size_t ws_bytes = p->sieves ? wheel_sieve_bytes(&p->ws, wlen) : 0;
     const uint32_t nblk = wheel_group_blocks(p->wgroups);
     WheelEntryArgs ea{};
     std::vector<QueryDev> qd(count);
@@ -760,6 +843,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         take(p->dqs, count * sizeof(QueryDev));
         take(d_tiles, tiles.size() * sizeof(uint2));
         take(p->dwgitems, items.size() * sizeof(uint4));
+        take(p->dwide, p->wide.size() * sizeof(WideEntry));
+        take(p->dlook, p->lookups.size() * 8);
         up_bytes = off - up0;
         take(p->dK, E * 8);
         take(p->dYCE, E * 8);
@@ -769,15 +854,19 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         take(p->dR6, E * 8);
         take(p->dR, E * 8);
         take(p->dqueue, (size_t)p->qcap * sizeof(uint4));
-        take(p->dMloc[0], wlen * 2);
-        take(p->dsegsum[0], wlen / kSegY * 4);
-        take(p->dsegoff[0], wlen / kSegY * 8);
+        if (p->sieves) {
+            take(p->dMloc[0], wlen * 2);
+            take(p->dsegsum[0], wlen / kSegY * 4);
+            take(p->dsegoff[0], wlen / kSegY * 8);
+        }
         take(p->dcarry, (p->nblocks + 1) * 8);
         take(p->dwgroups, (size_t)G * sizeof(WheelGroup));
         take(p->dwpre, ((size_t)nblk + 1) * 4);
         take(p->dwtiles, (size_t)ntiles * sizeof(WheelGatherTile));
-        take(p->dwl, p->wchunks * kSegY * 2);
-        take(p->dwl_cnt, p->wchunks * 4);
+        if (!table) {
+            take(p->dwl, p->wchunks * kSegY * 2);
+            take(p->dwl_cnt, p->wchunks * 4);
+        }
         take(ws_base, ws_bytes);
         if (pass == 0) {
             base = p->alloc<char>(off);
@@ -787,6 +876,10 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
                 return MERTENS_ENOMEM;
             }
         }
+    }
+    if (table) {
+        p->dwl = table->dl;
+        p->dwl_cnt = table->dl_cnt;
     }
     p->dA = p->dS + E;
     p->wtotals = d_totals;
@@ -804,12 +897,15 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     put(p->dqs, qd.data(), count * sizeof(QueryDev));
     put(d_tiles, tiles.data(), tiles.size() * sizeof(uint2));
     put(p->dwgitems, items.data(), items.size() * sizeof(uint4));
+    put(p->dwide, p->wide.data(), p->wide.size() * sizeof(WideEntry));
+    put(p->dlook, p->lookups.data(), p->lookups.size() * 8);
     const size_t np = p->ws.host_p.size();
     p->h2d_bytes = up_bytes + np * 4;
     ea.qs = d_qs;
     ea.nq = (uint32_t)count;
     ea.ngroups = p->wgroups;
     ea.dc = dc;
+    ea.wide_from = (uint64_t)wide_from;
     ea.K = p->dK;
     ea.YC = p->dYCE;
     ea.JL = p->dJL;
@@ -821,14 +917,17 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     ea.tiles = p->dwtiles;
     ea.tile_src = d_tiles;
     ea.ntiles = ntiles;
-    // on the library's stream, finished before return
-    cudaStream_t s = alloc_stream();
+    // on the library's stream (with an allocation hook on the default stream, to
+    // which its memory belongs), finished before return
+    cudaStream_t s = p->al.alloc ? nullptr : alloc_stream();
     const bool ok =
-        s && cudaMemsetAsync(base, 0, cleared, s) == cudaSuccess &&
+        (s || p->al.alloc) && cudaMemsetAsync(base, 0, cleared, s) == cudaSuccess &&
         cudaMemcpyAsync(up, img.data(), up_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess &&
-        wheel_entries_enqueue(ea, s) >= 0 && wheel_sieve_bind(&p->ws, ws_base, wlen, p->derr, s) == 0 &&
-        cudaMemcpyAsync(p->ws.p, p->ws.host_p.data(), np * 4, cudaMemcpyHostToDevice, s) ==
-            cudaSuccess &&
+        wheel_entries_enqueue(ea, s) >= 0 &&
+        (!p->sieves ||
+         (wheel_sieve_bind(&p->ws, ws_base, wlen, p->derr, s) == 0 &&
+          cudaMemcpyAsync(p->ws.p, p->ws.host_p.data(), np * 4, cudaMemcpyHostToDevice, s) ==
+              cudaSuccess)) &&
         cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess &&
         cudaStreamSynchronize(s) == cudaSuccess;
     if (!ok) {
@@ -842,6 +941,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     size_t i = 0;
     for (uint64_t b = 0; b < p->nblocks; ++b) {
         const uint64_t len = wheel_block_len(p, b), P = isqrt64(b * p->block_len + len);
+        if (table && b * p->block_len + len <= table->y_cov)
+            continue;  // read from the table
         for (; i < np && p->ws.host_p[i] <= P; ++i) {
             const double q = (double)p->ws.host_p[i];
             pre += 1.0 / q + 1.0 / (q * q);
@@ -861,10 +962,11 @@ static int wheel_counts(mertens_plan_s *p)
     if (cudaMemcpy(t.data(), p->wtotals, p->nq * sizeof(WheelTotals), cudaMemcpyDeviceToHost) !=
         cudaSuccess)
         return MERTENS_ECUDA;
-    for (const WheelTotals &v : t) {
-        p->direct.push_back(v.direct);
-        p->gathered.push_back(v.gathered);
-        p->terms += v.direct + v.gathered;
+    for (size_t i = 0; i < p->nq; ++i) {
+        const WheelTotals &v = t[i];
+        p->direct.push_back(v.direct + p->wide_direct[i]);
+        p->gathered.push_back(v.gathered + p->wide_gathered[i]);
+        p->terms += p->direct[i] + p->gathered[i];
         p->gather_j += v.gather_j;
         p->gather_j_exec += v.exec;
         p->dense_y += v.dense_y;
@@ -930,28 +1032,30 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     std::vector<Group> groups;
     const char *share_env = getenv("MERTENS_SHARE");
     const bool share = !(share_env && share_env[0] == '0');
-    // whole runs of one-word targets take the sums over integers coprime to 6
-    // (window plans return sums over all y; MERTENS_SHARE=0 and
-    // MERTENS_GATHER_QUOT=0 keep the full sums, MERTENS_OVERLAP the three-stream
-    // schedule, which is the full path's)
+    // whole runs take the sums over integers coprime to 6; window plans return
+    // sums over all y, and MERTENS_SHARE=0, MERTENS_GATHER_QUOT=0 and
+    // MERTENS_OVERLAP (three streams) keep the full sums where there is no table
     {
         const char *q = getenv("MERTENS_GATHER_QUOT");
-        p->wheel = !window && !table && share && !(q && q[0] == '0') && !getenv("MERTENS_OVERLAP");
+        p->wheel = !window && (table || (share && !(q && q[0] == '0') && !getenv("MERTENS_OVERLAP")));
         p->wheel_long = q && q[0] == '2';
         std::vector<uint64_t> us(count);
         for (size_t i = 0; i < count && p->wheel; ++i) {
-            us[i] = u.lo ? u.lo : target_u(n128[i], ub);
-            p->wheel = n128[i] < wide_threshold() && n128[i] / us[i] < (1ull << 31) &&
-                       wheel_sieve_exact(us[i] + 2 * kWheelSegY);
+            us[i] = u.lo ? u.lo : (table ? on_table_u(n128[i], ub, table->y_max)
+                                         : target_u(n128[i], ub));
+            p->wheel = n128[i] / us[i] < 0xfffffff0u && wheel_sieve_exact(us[i] + 2 * kWheelSegY);
         }
         if (p->wheel)
-            return plan_create_wheel(out, p, n128, us, block_len, tn);
+            return plan_create_wheel(out, p, n128, us, block_len, tn, table);
+        if (table) {
+            set_last_error("mertens_plan_on_table: sieve limits beyond 2^54 or 2^32 - 16 entries");
+            delete p;
+            return MERTENS_ENOTSUP;
+        }
     }
-    const bool share_dense = !window && share;
     for (size_t i = 0; i < count; ++i) {
         const u128 nn = to_u128(n[i]);
-        const uint64_t uu = u.lo ? u.lo : (table ? on_table_u(nn, ub, table->y_max)
-                                                 : target_u(nn, ub));
+        const uint64_t uu = u.lo ? u.lo : target_u(nn, ub);
         const uint64_t X = (uint64_t)(nn / uu);
         p->n.push_back((uint64_t)nn);
         p->n_hi.push_back((uint64_t)(nn >> 64));
@@ -959,33 +1063,8 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         p->X.push_back(X);
         p->off.push_back(K.size());
         uint64_t d = 0, g = 0, ymq = 0;
-        if (table && nn <= table->y_max && X == 1) {
-            // M(n) is in the table: one entry, no terms, read after resolve
-            p->lookups.push_back(K.size());
-            p->lookups.push_back((uint64_t)nn);
-            K.push_back(0);
-            JLO.push_back(1);
-            YCE.push_back(0);
-            JC0.push_back(0);
-            Group G;
-            G.first = (uint32_t)(K.size() - 1);
-            G.count = 1;
-            G.pred = 1;
-            G.emit = 0;
-            G.yc = 0;
-            G.olo = 0;
-            G.x0 = 1;
-            G.stride = 1;
-            groups.push_back(G);
-            p->direct.push_back(0);
-            p->gathered.push_back(0);
-            p->ymax_q.push_back(0);
-            continue;
-        }
         // blocks of 64 consecutive x share a dense cut-off; each is two groups
-        // of 32 (odd x, even x), so the entries x/2 of an even group lie in
-        // one earlier block and share its cut-off (the dense form's sharing)
-        const size_t gstart = groups.size();  // this target's groups: two per block
+        // of 32
         std::vector<uint64_t> S_(64), VH(64);
         std::vector<uint8_t> WD(64);
         const u128 wide_from = wide_threshold();
@@ -1059,10 +1138,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
             Group G;
             G.first = (uint32_t)(K.size() - cnt);
             G.count = cnt;
-            G.emit = 0;
-            G.olo = 0;
-            G.x0 = (uint32_t)x0;
-            G.stride = 1;
             if (any_wide) {
                 // per-entry cut-offs; the two-word entries take none
                 G.pred = 1;
@@ -1088,18 +1163,13 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
                     G.yc = std::max(G.yc, yc);
                 }
             }
-            {
-                // the block as two stride-2 groups (odd x, then even x)
-                Group H = G;
-                H.stride = 2;
-                H.count = (cnt + 1) / 2;
+            Group H = G;
+            H.count = std::min(cnt, 32u);
+            groups.push_back(H);
+            if (cnt > 32) {
+                H.first = G.first + 32;
+                H.count = cnt - 32;
                 groups.push_back(H);
-                if (cnt > 1) {
-                    H.first = G.first + 1;
-                    H.x0 = G.x0 + 1;
-                    H.count = cnt / 2;
-                    groups.push_back(H);
-                }
             }
         }
         {
@@ -1145,42 +1215,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
                 p->dense_y += P.dense_y;
                 p->gather_j += P.gather_j;
                 g += P.g;
-            }
-        }
-        // ---- the dense form's terms shared between entries x and 2x ----
-        // mu(y) floor(floor(n/2x)/y) = -mu(2y) floor(floor(n/x)/2y) for odd y,
-        // and the even squarefree y' <= yc_x are exactly 2y for the odd
-        // squarefree y <= floor(yc_x/2).  So the even group of block M
-        // (x = 64M + 2, ..., whose x/2 = 32M + 1, ... lie in block M/2) leaves
-        // out its odd y <= b = floor(yc/2) of that block's common cut-off when
-        // b is within every one of its entries' cut-offs, and those x/2 add
-        // minus their even-y sums to it.  Not in window plans (their dense
-        // part is cut to the window's y, which 2y can leave).
-        if (share_dense) {
-            const size_t nblk = (X + 63) / 64;
-            for (size_t M = 0; M < nblk; ++M) {
-                const size_t gr = gstart + 2 * M + 1;  // even group of block M
-                if (64 * M + 2 > X || gr >= groups.size())
-                    continue;
-                Group &R = groups[gr];
-                const Group &Sg = groups[gstart + 2 * (M / 2)];
-                if (Sg.pred || Sg.yc < 2)
-                    continue;
-                const uint64_t b = Sg.yc / 2;
-                bool ok = true;
-                for (uint32_t t = 0; t < R.count && ok; ++t) {
-                    const size_t e = (size_t)R.first + 2 * t;
-                    ok = K[e] != 0 && b <= YCE[e];
-                }
-                if (!ok)
-                    continue;
-                R.olo = b;
-                p->dense_odd_skip += (b + 1) / 2 * (uint64_t)R.count;
-                for (uint32_t t = 0; t < R.count; ++t) {
-                    const uint64_t xs = 32 * M + 1 + t;       // source x
-                    const uint64_t o = xs - (64 * (M / 2) + 1);  // offset in its block
-                    groups[gstart + 2 * (M / 2) + (o & 1)].emit |= 1u << (o >> 1);
-                }
             }
         }
         p->direct.push_back(d);
@@ -1243,16 +1277,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
             if (K[e2] && JC0[e2] >= JOWN[e2])
                 p->gather_j_exec += JC0[e2] - JOWN[e2] + 1;
     }
-    p->table = table;
-    if (table) {
-        if (block_len == 0)
-            block_len = 1ull << 30;
-        if (block_len % kSegY) {
-            set_last_error("mertens_plan_on_table: block_len must be a multiple of %d", kSegY);
-            delete p;
-            return MERTENS_EINVAL;
-        }
-    }
     p->window = window;
     p->y_first = window ? w_first : 1;
     p->y_last = window ? std::min(w_last, p->y_max) : p->y_max;
@@ -1292,13 +1316,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         else if (e[0] == '2')
             p->gquot = 2;
     }
-    if (table && (p->ydense > table->ydense || p->mg_n > table->mg_n)) {
-        set_last_error("mertens_plan_on_table: the targets need dense cut-offs or divisors "
-                       "beyond the table");
-        delete p;
-        return MERTENS_ENOTSUP;
-    }
-
     // ---- dense work items: groups sorted by cut-off, chunk ranges ----
     std::vector<uint32_t> order(groups.size());
     for (size_t i = 0; i < order.size(); ++i)
@@ -1577,43 +1594,25 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     const uint64_t nseg = sieve_segments(L);
     // One stream by default: on GB300 the three-stream schedule measured
     // slower (the sieve and the updates contend for the same SM resources);
-    // MERTENS_OVERLAP=1 selects it.  Plans on a table have no sieve.
-    p->serial = getenv("MERTENS_OVERLAP") == nullptr || p->nblocks == 1 || table;
-    // a plan on a table sieves only the blocks that end above the table
-    p->sieves = !table || p->y_last > table->y_max;
-    if (table) {
-        // the table's M(y) blocks are addressed per block at run time
-        p->dmu_aux = nullptr;
-        p->dMG = table->MG;
-        p->ddl_m = table->dl_m;
-        p->ddl_yo = table->dl_yo;
-        p->ddl_cnt = table->dl_cnt;
-        p->mg_built = true;
-        if (!p->lookups.empty())
-            p->dlook = p->alloc<uint64_t>(p->lookups.size());
-    }
-    if (p->sieves) {
-        if (!table)
-            p->dmu_aux = p->alloc<int8_t>(p->ydense + 16);
-        const int nbuf = p->serial ? 1 : 2;
-        for (int i = 0; i < 2; ++i) {
-            if (i < nbuf) {
-                p->dMloc[i] = p->alloc<int16_t>(L + 16);  // tiles copy whole 16-byte units
-                p->dsegsum[i] = p->alloc<int32_t>(nseg);
-                p->dsegoff[i] = p->alloc<int64_t>(nseg);
-            } else {
-                p->dMloc[i] = p->dMloc[0];
-                p->dsegsum[i] = p->dsegsum[0];
-                p->dsegoff[i] = p->dsegoff[0];
-            }
-        }
-        if (!table) {
-            p->dMG = p->alloc<uint64_t>(p->mg_n + 1);
-            p->ddl_m = p->alloc<uint64_t>(nchunks * kChunkCapPad);
-            p->ddl_yo = p->alloc<uint16_t>(nchunks * kChunkCapPad);
-            p->ddl_cnt = p->alloc<uint2>(nchunks);
+    // MERTENS_OVERLAP=1 selects it.
+    p->serial = getenv("MERTENS_OVERLAP") == nullptr || p->nblocks == 1;
+    p->dmu_aux = p->alloc<int8_t>(p->ydense + 16);
+    const int nbuf = p->serial ? 1 : 2;
+    for (int i = 0; i < 2; ++i) {
+        if (i < nbuf) {
+            p->dMloc[i] = p->alloc<int16_t>(L + 16);  // tiles copy whole 16-byte units
+            p->dsegsum[i] = p->alloc<int32_t>(nseg);
+            p->dsegoff[i] = p->alloc<int64_t>(nseg);
+        } else {
+            p->dMloc[i] = p->dMloc[0];
+            p->dsegsum[i] = p->dsegsum[0];
+            p->dsegoff[i] = p->dsegoff[0];
         }
     }
+    p->dMG = p->alloc<uint64_t>(p->mg_n + 1);
+    p->ddl_m = p->alloc<uint64_t>(nchunks * kChunkCapPad);
+    p->ddl_yo = p->alloc<uint16_t>(nchunks * kChunkCapPad);
+    p->ddl_cnt = p->alloc<uint2>(nchunks);
     p->dcarry = p->alloc<int64_t>(p->nblocks + 1);
     p->dgtiles = p->alloc<GatherTile>(gtiles.size() + 1);
     p->dgitems = p->alloc<GatherItem>(gitems.size() + 1);
@@ -1634,24 +1633,22 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
             rc = MERTENS_ENOMEM;
     bool any_null = !p->dK || !p->dJLO || !p->dEMIT || !p->dJC0 || !p->dJCUR || !p->dYCE || !p->dqueue ||
                     !p->dqlen || !p->dS || !p->dR ||
-                    (!table && !p->dmu_aux) ||
-                    (p->sieves && (!p->dMloc[0] || !p->dsegsum[0] || !p->dsegoff[0] ||
-                                   !p->dMloc[1] || !p->dsegsum[1] || !p->dsegoff[1])) ||
-                    (!p->lookups.empty() && !p->dlook) || !p->dgtiles ||
+                    !p->dmu_aux || !p->dMloc[0] || !p->dsegsum[0] || !p->dsegoff[0] ||
+                    !p->dMloc[1] || !p->dsegsum[1] || !p->dsegoff[1] || !p->dgtiles ||
                     !p->dcounter_dense || !p->dcounter_gather ||
                     !p->dgitems || !p->dcarry || !p->derr || !p->dcounter || !p->dMG ||
                     !p->ddl_m || !p->ddl_yo || !p->ddl_cnt || !p->dgroups || !p->ditems ||
                     !p->dqs || (!p->wide.empty() && !p->dwide) || (window && !p->dcoef);
     if (any_null)
         rc = MERTENS_ENOMEM;
-    if (rc == MERTENS_OK && p->sieves) {
+    if (rc == MERTENS_OK) {
         int prc = prime_table_create(&p->pt, p->al, std::max<uint64_t>(p->y_last, 1), nullptr);
         if (prc == 0)
             prc = sieve_scratch_create(&p->pt, block_len, nullptr);
         if (prc != 0)
             rc = prc == 6 ? MERTENS_ENOTSUP : (prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA);
     }
-    if (rc == MERTENS_OK && p->sieves) {
+    if (rc == MERTENS_OK) {
         // algorithmic sieve updates: each block of length len sieved with the
         // primes p <= max(7, sqrt(block end)) costs len * sum (1/p + 1/p^2)
         std::vector<double> pre(p->pt.np + 1, 0.0);
@@ -1662,8 +1659,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         for (uint64_t b = 0; b < p->nblocks; ++b) {
             uint64_t y1, y2;
             block_range(p, b, &y1, &y2);
-            if (table && y2 <= table->y_max)
-                continue;  // read from the table
             const uint64_t P = std::max<uint64_t>(7, isqrt64(y2));
             p->sieve_updates += (double)(y2 - y1 + 1) * pre[prime_count_upto(&p->pt, P)];
         }
@@ -1686,9 +1681,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         cudaMemcpy(p->dqs, qs.data(), count * sizeof(QueryDev), cudaMemcpyHostToDevice);
         if (!p->wide.empty())
             cudaMemcpy(p->dwide, p->wide.data(), p->wide.size() * sizeof(WideEntry),
-                       cudaMemcpyHostToDevice);
-        if (!p->lookups.empty())
-            cudaMemcpy(p->dlook, p->lookups.data(), p->lookups.size() * 8,
                        cudaMemcpyHostToDevice);
         if (window)
             cudaMemcpy(p->dcoef, p->coef.data(), E * 8, cudaMemcpyHostToDevice);
@@ -1812,64 +1804,85 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
     uint64_t launches = 0;
     int r = 0;
     const size_t E = p->nent;
+    const mertens_table_s *tab = p->table;
     cudaMemsetAsync(p->dS, 0, 2 * E * 8, s);
     cudaMemsetAsync(p->dcarry, 0, 8, s);
     cudaMemsetAsync(p->derr, 0, 4, s);
+    WheelDenseArgs da;
+    da.counter = p->dcounter_dense;
+    da.groups = p->dwgroups;
+    da.ngroups = p->wgroups;
+    da.parts = p->wparts;
+    da.pre = p->dwpre;
+    da.K = p->dK;
+    da.dl = p->dwl;
+    da.dl_cnt = p->dwl_cnt;
+    da.S = p->dS;
     bool dense_done = p->wchunks == 0;
+    if (tab && !dense_done) {
+        // the squarefree list is the table's: the dense part needs no block
+        PhaseEvents pe;
+        ev_begin(p, kPhDense, s, &pe);
+        r = wheel_dense_enqueue(da, p->wdense_items, s);
+        ev_end(p, s, &pe);
+        launches += r > 0 ? r : 0;
+        dense_done = true;
+    }
+    bool after_table = false;  // the block before was read from the table
     for (uint64_t b = 0; b < p->nblocks && r >= 0; ++b) {
         const uint64_t y0 = b * p->block_len, len = wheel_block_len(p, b);
+        const bool from_table = tab && y0 + len <= tab->y_cov;
+        const int16_t *Mb = from_table ? tab->Mloc + y0 / 3 : p->dMloc[0];
+        const int64_t *Sb = from_table ? tab->segoff + y0 / kWheelSegY : p->dsegoff[0];
         PhaseEvents pe, pe2;
-        WheelLaunch L;
-        L.w0 = y0 / 3;
-        L.len = len / 3;
-        L.Mloc = p->dMloc[0];
-        L.segsum = p->dsegsum[0];
-        L.segoff = p->dsegoff[0];
-        L.carry_in = p->dcarry + b;
-        L.carry_out = p->dcarry + b + 1;
-        ev_begin(p, kPhSieve, s, &pe);
-        if (p->prof) {
-            pe2.phase = kPhScan;
-            cudaEventCreate(&pe2.a);
-            cudaEventCreate(&pe2.b);
-            L.mid = pe.b;
-            L.mid2 = pe2.a;
-        }
-        r = wheel_sieve_enqueue(&p->ws, L, s);
-        if (p->prof) {
-            p->evs.push_back(pe);
-            cudaEventRecord(pe2.b, s);
-            p->evs.push_back(pe2);
-        }
-        if (r < 0)
-            break;
-        launches += r;
-        const uint64_t c0 = y0 / kWheelSegY, c1 = (y0 + len) / kWheelSegY;
-        if (!dense_done) {
-            ev_begin(p, kPhDense, s, &pe);
-            r = wheel_dense_list_enqueue(p->dMloc[0], c0, std::min(c1, p->wchunks) - c0, p->dwl,
-                                         p->dwl_cnt, s);
-            if (r < 0)
-                break;
-            launches += r;
-            if (c1 >= p->wchunks) {
-                WheelDenseArgs da;
-                da.counter = p->dcounter_dense;
-                da.groups = p->dwgroups;
-                da.ngroups = p->wgroups;
-                da.parts = p->wparts;
-                da.pre = p->dwpre;
-                da.K = p->dK;
-                da.dl = p->dwl;
-                da.dl_cnt = p->dwl_cnt;
-                da.S = p->dS;
-                r = wheel_dense_enqueue(da, p->wdense_items, s);
+        if (!from_table) {
+            if (after_table) {
+                r = wheel_carry_at_enqueue(tab->Mloc, tab->segoff, y0, p->dcarry + b, s);
                 if (r < 0)
                     break;
                 launches += r;
+            }
+            WheelLaunch L;
+            L.w0 = y0 / 3;
+            L.len = len / 3;
+            L.Mloc = p->dMloc[0];
+            L.segsum = p->dsegsum[0];
+            L.segoff = p->dsegoff[0];
+            L.carry_in = p->dcarry + b;
+            L.carry_out = p->dcarry + b + 1;
+            ev_begin(p, kPhSieve, s, &pe);
+            if (p->prof) {
+                pe2.phase = kPhScan;
+                cudaEventCreate(&pe2.a);
+                cudaEventCreate(&pe2.b);
+                L.mid = pe.b;
+                L.mid2 = pe2.a;
+            }
+            r = wheel_sieve_enqueue(&p->ws, L, s);
+            if (p->prof) {
+                p->evs.push_back(pe);
+                cudaEventRecord(pe2.b, s);
+                p->evs.push_back(pe2);
+            }
+            if (r < 0)
+                break;
+            launches += r;
+        }
+        after_table = from_table;
+        const uint64_t c0 = y0 / kWheelSegY, c1 = (y0 + len) / kWheelSegY;
+        if (!dense_done) {
+            ev_begin(p, kPhDense, s, &pe);
+            r = wheel_dense_list_enqueue(Mb, c0, std::min(c1, p->wchunks) - c0, p->dwl, p->dwl_cnt,
+                                         s);
+            launches += r > 0 ? r : 0;
+            if (r >= 0 && c1 >= p->wchunks) {
+                r = wheel_dense_enqueue(da, p->wdense_items, s);
+                launches += r > 0 ? r : 0;
                 dense_done = true;
             }
             ev_end(p, s, &pe);
+            if (r < 0)
+                break;
         }
         ev_begin(p, kPhGather, s, &pe);
         if (p->gblk[b + 1] > p->gblk[b]) {
@@ -1879,8 +1892,8 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             ga.items = p->dwgitems + p->gblk[b];
             ga.nitems = p->gblk[b + 1] - p->gblk[b];
             ga.counter = p->dcounter_gather;
-            ga.Mloc = p->dMloc[0];
-            ga.segoff = p->dsegoff[0];
+            ga.Mloc = Mb;
+            ga.segoff = Sb;
             ga.K = p->dK;
             ga.YC = p->dYCE;
             ga.JL = p->dJL;
@@ -1913,9 +1926,27 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
         ba.qlen = p->dqlen;
         ba.qcap = p->qcap;
         ba.err = p->derr;
-        ba.Mloc = p->dMloc[0];
-        ba.segoff = p->dsegoff[0];
+        ba.Mloc = Mb;
+        ba.segoff = Sb;
         r = wheel_block_enqueue(ba, s);
+        if (r >= 0 && !p->wide.empty()) {
+            launches += r;
+            WheelWideArgs wa;
+            wa.W = p->dwide;
+            wa.y0 = y0;
+            wa.len = len;
+            wa.Mloc = Mb;
+            wa.segoff = Sb;
+            wa.S = p->dS;
+            wa.A = p->dA;
+            uint64_t units = 0;
+            for (const WideEntry &W : p->wide) {
+                uint64_t nd, wj, ng;
+                wheel_wide_units(W, y0, len, &nd, &wj, &ng);
+                units = std::max(units, nd + ng);
+            }
+            r = wheel_wide_enqueue(wa, (uint32_t)p->wide.size(), units, s);
+        }
         ev_end(p, s, &pe);
         if (r < 0)
             break;
@@ -1928,6 +1959,11 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             mx = std::max(mx, X);
         ev_begin(p, kPhResolve, s, &pe);
         r = wheel_resolve_enqueue(p->dqs, (uint32_t)p->nq, mx, p->dS, p->dA, p->dR6, p->dR, s);
+        if (r >= 0 && !p->lookups.empty()) {
+            const int r2 = wheel_lookup_enqueue(p->dlook, (uint32_t)(p->lookups.size() / 2),
+                                                tab->Mloc, tab->segoff, p->dR, s);
+            r = r2 < 0 ? r2 : r + r2;
+        }
         ev_end(p, s, &pe);
     }
     if (r < 0) {
@@ -1964,10 +2000,9 @@ static int run_enqueue(mertens_plan_s *p, cudaStream_t origin, uint64_t *out)
     }
     cudaMemsetAsync(p->dS, 0, E * 8, su);
     cudaMemcpyAsync(p->dJCUR, p->dJC0, E * 8, cudaMemcpyDeviceToDevice, su);
-    const mertens_table_s *tab = p->table;
     cudaMemsetAsync(p->dcarry, 0, 8 * (p->nblocks + 1), ss);
     cudaMemsetAsync(p->derr, 0, 4, su);
-    if (p->window && p->y_first <= p->ydense && !tab)
+    if (p->window && p->y_first <= p->ydense)
         cudaMemsetAsync(p->dmu_aux, 0, p->ydense + 1, ss);  // mu outside the window: none
     if (!p->mg_built) {
         r = magic_table_enqueue(p->dMG, p->mg_n, su);
@@ -1986,51 +2021,16 @@ static int run_enqueue(mertens_plan_s *p, cudaStream_t origin, uint64_t *out)
         // window's end); a window above Y_dense has none
         bool dense_done = p->y_first > p->ydense;
         const uint64_t dense_at = std::min(p->ydense, p->y_last);
-        if (tab && !dense_done) {
-            // the squarefree list is the table's: the dense part needs no block
-            PhaseEvents pe;
-            ev_begin(p, kPhDense, su, &pe);
-            DenseArgs da;
-            da.items = p->ditems;
-            da.nitems = p->nitems;
-            da.counter = p->dcounter_dense;
-            da.groups = p->dgroups;
-            da.K = p->dK;
-            da.YCE = p->dYCE;
-            da.dl_m = p->ddl_m;
-            da.dl_yo = p->ddl_yo;
-            da.dl_cnt = p->ddl_cnt;
-            da.S = p->dS;
-            da.ctas_per_sm = 0;
-            r = dense_update_enqueue(da, su);
-            ev_end(p, su, &pe);
-            if (r < 0)
-                goto fail;
-            launches += r;
-            dense_done = true;
-        }
         for (uint64_t b = 0; b < p->nblocks; ++b) {
             uint64_t y1, y2;
             block_range(p, b, &y1, &y2);
             const int buf = (int)(b & 1);
-            // M(y) of the block: the table's where it covers the whole block,
-            // else the plan's buffer (sieved below)
-            const bool from_table = tab && y2 <= tab->y_max;
-            const int16_t *Mb = from_table ? tab->Mloc + (y1 - 1) : p->dMloc[buf];
-            const int64_t *Sb =
-                from_table ? tab->segoff + ((y1 - 1) >> kSegShift) : p->dsegoff[buf];
+            const int16_t *Mb = p->dMloc[buf];
+            const int64_t *Sb = p->dsegoff[buf];
             if (!serial && b >= 2)
                 cudaStreamWaitEvent(ss, p->ev_upd[b - 2], 0);
             cudaStream_t s = ss;
-            if (tab && !from_table && y1 > 1 && y1 - 1 <= tab->y_max) {
-                // the first sieved block above the table: its carry M(y1 - 1)
-                // is the table's
-                r = carry_from_table_enqueue(tab->Mloc, tab->segoff, y1 - 1, p->dcarry + b, ss);
-                if (r < 0)
-                    goto fail;
-                launches += r;
-            }
-            if (!from_table) {
+            {
                 SieveLaunch L;
                 L.y1 = y1;
                 L.len = y2 - y1 + 1;
@@ -2183,11 +2183,6 @@ static int run_enqueue(mertens_plan_s *p, cudaStream_t origin, uint64_t *out)
             PhaseEvents pe;
             ev_begin(p, kPhResolve, su, &pe);
             r = resolve_enqueue(p->dqs, (uint32_t)p->nq, p->dS, p->dK, p->dR, su);
-            if (r >= 0 && !p->lookups.empty()) {
-                const int r2 = table_lookup_enqueue(p->dlook, (uint32_t)(p->lookups.size() / 2),
-                                                    tab->Mloc, tab->segoff, p->dR, su);
-                r = r2 < 0 ? r2 : r + r2;
-            }
             ev_end(p, su, &pe);
             if (r < 0)
                 goto fail;
@@ -2650,7 +2645,7 @@ int mertens_run_stats_get(mertens_plan_t p, mertens_run_stats *st)
         for (uint64_t b = 0; b < p->nblocks; ++b) {
             uint64_t y1, y2;
             block_range(p, b, &y1, &y2);
-            if (y2 > p->table->y_max)
+            if (y2 > p->table->y_cov)
                 st->y_sieved += y2 - y1 + 1;
         }
     }

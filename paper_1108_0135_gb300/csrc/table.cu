@@ -1,9 +1,9 @@
-// Resident M(y) table: the sieve (steps a1 + a2) run once over [1, y_max]
-// and kept in device memory, together with the parts of the update that do
-// not depend on the target (the divisor magics and the squarefree dense
-// list).  Plans made on a table (mertens_plan_on_table) read M(y) from it and
-// run only the update and resolve.  The paper sieves per target (Sec. 3);
-// keeping the sieve's output resident is what lets many queries share it.
+// Resident M(y) table: the sieve (steps a1 + a2, in the form of wheel.h) run
+// once up to y_max and kept in device memory (0.67 bytes per y), together with
+// the part of the update that does not depend on the target (the dense list of
+// squarefree numbers).  Plans made on a table (mertens_plan_on_table) read M6(y)
+// from it and run only the update and resolve.  The paper sieves per target
+// (Sec. 3); keeping the sieve's output resident lets many queries share it.
 #include <algorithm>
 #include <cmath>
 #include <cstring>
@@ -12,6 +12,7 @@
 #include "common.cuh"
 #include "internal.h"
 #include "update.h"
+#include "wheel.h"
 
 namespace mert {
 double plan_dense_factor();
@@ -73,82 +74,69 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
     const u128 nm = ((u128)n_max.hi << 64) | n_max.lo;
     const uint64_t r = isqrt_u128(nm);
     // the planner's dense cut-offs stay below the chunk-aligned dc sqrt(n)
-    // (or sqrt(n) itself); their quotients k/(yc+1) below sqrt(n)
+    // (or sqrt(n) itself)
     const double dc = plan_dense_factor();
     uint64_t yd = (uint64_t)(std::max(dc, 1.0) * std::sqrt((double)nm)) + 2 * kChunk;
     yd = ((yd + kChunk - 1) / kChunk) * kChunk - 1;
     t->ydense = std::min(yd, y_max);
-    t->mg_n = std::max(t->ydense, r) + 2;
-
-    const uint64_t nseg = sieve_segments(y_max);
-    const uint64_t nchunks = dense_chunks(t->ydense);
-    t->Mloc = table_alloc<int16_t>(t, y_max + 16);  // gather tiles copy whole 16-byte units
+    // M6 of the integers coprime to 6 up to whole segments of 6144 y, and the
+    // dense list of the first nchunks of them
+    t->y_cov = (y_max + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
+    const uint64_t nseg = t->y_cov / kWheelSegY;
+    const uint64_t nchunks = (t->ydense + kWheelSegY - 1) / kWheelSegY;
+    t->Mloc = table_alloc<int16_t>(t, nseg * kSegY);
     t->segoff = table_alloc<int64_t>(t, nseg);
-    t->MG = table_alloc<uint64_t>(t, t->mg_n + 1);
-    t->dl_m = table_alloc<uint64_t>(t, nchunks * kChunkCapPad);
-    t->dl_yo = table_alloc<uint16_t>(t, nchunks * kChunkCapPad);
-    t->dl_cnt = table_alloc<uint2>(t, nchunks);
-    // scratch of the build
-    const uint64_t L = std::min<uint64_t>(1ull << 30, ((y_max + kSegY - 1) / kSegY) * kSegY);
-    const uint64_t nblocks = (y_max + L - 1) / L;
-    int8_t *mu = (int8_t *)dev_alloc(t->al, t->ydense + 16);
-    int32_t *segsum = (int32_t *)dev_alloc(t->al, sieve_segments(L) * 4);
-    int64_t *carry = (int64_t *)dev_alloc(t->al, (nblocks + 1) * 8);
-    int rc = MERTENS_OK;
-    if (!t->Mloc || !t->segoff || !t->MG || !t->dl_m || !t->dl_yo || !t->dl_cnt || !mu ||
-        !segsum || !carry)
-        rc = MERTENS_ENOMEM;
-    PrimeTable pt;
+    t->dl = table_alloc<uint16_t>(t, nchunks * kSegY);
+    t->dl_cnt = table_alloc<uint32_t>(t, nchunks);
+    // scratch of the build: sieve tables, segment sums, carries, status word
+    const uint64_t L = std::min<uint64_t>((1ull << 30) / kWheelSegY * kWheelSegY, t->y_cov);
+    const uint64_t nblocks = (t->y_cov + L - 1) / L;
+    WheelSieve ws;
+    wheel_sieve_primes(&ws, y_max);
+    const auto up = [](size_t v) { return (v + 255) & ~(size_t)255; };
+    const size_t b_ws = up(wheel_sieve_bytes(&ws, L / 3)), b_sum = up(L / kWheelSegY * 4),
+                 b_cy = up((nblocks + 1) * 8), bytes = b_ws + b_sum + b_cy + 256;
+    char *buf = (char *)dev_alloc(t->al, bytes);
+    int rc = t->Mloc && t->segoff && t->dl && t->dl_cnt && buf ? MERTENS_OK : MERTENS_ENOMEM;
     if (rc == MERTENS_OK) {
-        int prc = prime_table_create(&pt, t->al, y_max, s);
-        if (prc == 0)
-            prc = sieve_scratch_create(&pt, L, s);
-        if (prc != 0)
-            rc = prc == 2 ? MERTENS_ENOMEM : MERTENS_ECUDA;
-    }
-    if (rc == MERTENS_OK) {
-        cudaMemsetAsync(carry, 0, (nblocks + 1) * 8, s);
-        cudaMemsetAsync(mu, 0, t->ydense + 16, s);
+        int32_t *segsum = (int32_t *)(buf + b_ws);
+        int64_t *carry = (int64_t *)(buf + b_ws + b_sum);
+        uint32_t *err = (uint32_t *)(buf + b_ws + b_sum + b_cy);
+        cudaMemsetAsync(carry, 0, 8, s);
+        cudaMemsetAsync(err, 0, 4, s);
+        if (wheel_sieve_bind(&ws, buf, L / 3, err, s) != 0)
+            rc = MERTENS_ECUDA;
+        cudaMemcpyAsync(ws.p, ws.host_p.data(), ws.host_p.size() * 4, cudaMemcpyHostToDevice, s);
         for (uint64_t b = 0; b < nblocks && rc == MERTENS_OK; ++b) {
-            const uint64_t y1 = 1 + b * L;
-            const uint64_t y2 = std::min(y1 + L - 1, y_max);
-            SieveLaunch Lc;
-            Lc.y1 = y1;
-            Lc.len = y2 - y1 + 1;
-            Lc.Mloc = t->Mloc + (y1 - 1);
+            const uint64_t y0 = b * L;
+            WheelLaunch Lc;
+            Lc.w0 = y0 / 3;
+            Lc.len = std::min(L, t->y_cov - y0) / 3;
+            Lc.Mloc = t->Mloc + y0 / 3;
             Lc.segsum = segsum;
-            Lc.segoff = t->segoff + ((y1 - 1) >> kSegShift);
+            Lc.segoff = t->segoff + y0 / kWheelSegY;
             Lc.carry_in = carry + b;
             Lc.carry_out = carry + b + 1;
-            Lc.mu_out = y1 <= t->ydense ? mu : nullptr;
-            Lc.mu_base = 1;
-            Lc.mu_end = t->ydense;
-            if (sieve_block_enqueue(&pt, Lc, s) < 0)
+            if (wheel_sieve_enqueue(&ws, Lc, s) < 0)
                 rc = MERTENS_ECUDA;
         }
-        if (rc == MERTENS_OK && (magic_table_enqueue(t->MG, t->mg_n, s) < 0 ||
-                                 dense_list_enqueue(mu, t->ydense, t->MG, t->dl_m, t->dl_yo,
-                                                    t->dl_cnt, s) < 0))
+        if (rc == MERTENS_OK &&
+            wheel_dense_list_enqueue(t->Mloc, 0, nchunks, t->dl, t->dl_cnt, s) < 0)
             rc = MERTENS_ECUDA;
-        if (cudaStreamSynchronize(s) != cudaSuccess)
+        uint32_t st = 0;
+        if (cudaMemcpyAsync(&st, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+            cudaStreamSynchronize(s) != cudaSuccess)
             rc = MERTENS_ECUDA;
-        if (rc == MERTENS_OK) {
-            const uint32_t st = sieve_scratch_status(&pt);
-            if (st) {
-                set_last_error("mertens_table_create: %s", sieve_status_text(st));
-                rc = sieve_status_code(st);
-            }
+        if (rc == MERTENS_OK && st) {
+            set_last_error("mertens_table_create: %s", sieve_status_text(st));
+            rc = sieve_status_code(st);
         }
     }
     if (rc == MERTENS_ECUDA)
         set_last_error("mertens_table_create: %s", cudaGetErrorString(cudaGetLastError()));
     else if (rc == MERTENS_ENOMEM)
         set_last_error("mertens_table_create: device allocation failed");
-    if (pt.np)
-        prime_table_destroy(&pt);
-    dev_free(t->al, mu, t->ydense + 16);
-    dev_free(t->al, segsum, sieve_segments(L) * 4);
-    dev_free(t->al, carry, (nblocks + 1) * 8);
+    dev_free(t->al, buf, bytes);
     if (rc != MERTENS_OK) {
         mertens_table_destroy(t);
         return rc;

@@ -37,9 +37,9 @@ __global__ void magic_table_kernel(uint64_t *__restrict__ MG, uint64_t nd)
 }
 
 // Squarefree list of one chunk of kChunk y values (y <= ydense): the magics
-// and offsets y - chunk start, in increasing y, in four parts -- mu = +1 and
-// odd y, +1 and even y, -1 and odd y, -1 and even y -- each from an even
-// index; dl_cnt = {n0 | n1 << 16, n2 | n3 << 16}.  256 threads x 16 y.
+// and offsets y - chunk start, in increasing y, those with mu = +1, then from an
+// even index those with mu = -1; dl_cnt = {count(+1), count(-1)}.  256 threads x
+// 16 y.
 __device__ __forceinline__ uint32_t even_up(uint32_t v) { return (v + 1u) & ~1u; }
 
 __global__ void __launch_bounds__(256) dense_list_kernel(const int8_t *__restrict__ mu_aux,
@@ -53,36 +53,29 @@ __global__ void __launch_bounds__(256) dense_list_kernel(const int8_t *__restric
     const uint64_t c = blockIdx.x;
     const uint64_t cb = c * kChunk;
     int8_t mv[16];
-    uint32_t cp = 0, cm = 0;  // per thread: counts of the parts, 16-bit fields (odd | even << 16)
+    uint32_t cnt = 0;  // +1 in the low half, -1 in the high half
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const uint64_t y = cb + threadIdx.x * 16 + k;
         mv[k] = (y >= 1 && y <= ydense) ? mu_aux[y - 1] : (int8_t)0;
-        const uint32_t f = (k & 1) ? 1u : 65536u;  // y even when k is (cb and 16 t are even)
-        cp += mv[k] > 0 ? f : 0u;
-        cm += mv[k] < 0 ? f : 0u;
+        cnt += mv[k] > 0 ? 1u : (mv[k] < 0 ? 65536u : 0u);
     }
-    uint32_t totp, totm;
-    const uint32_t ip = block_scan_u32(cp, sh, &totp);  // no field exceeds 2048
-    const uint32_t im = block_scan_u32(cm, sh, &totm);
-    const uint32_t n0 = totp & 0xffffu, n1 = totp >> 16, n2 = totm & 0xffffu;
-    const uint32_t b1 = even_up(n0), b2 = b1 + even_up(n1), b3 = b2 + even_up(n2);
-    uint32_t i0 = ip & 0xffffu, i1 = b1 + (ip >> 16), i2 = b2 + (im & 0xffffu),
-             i3 = b3 + (im >> 16);
+    uint32_t tot;
+    const uint32_t ex = block_scan_u32(cnt, sh, &tot);
+    uint32_t ip = ex & 0xffffu, im = even_up(tot & 0xffffu) + (ex >> 16);
     uint64_t *dm = dl_m + c * kChunkCapPad;
     uint16_t *dy = dl_yo + c * kChunkCapPad;
 #pragma unroll
     for (int k = 0; k < 16; ++k) {
         const uint32_t o = threadIdx.x * 16 + k;
-        const uint64_t y = cb + o;
         if (mv[k] != 0) {
-            const uint32_t i = mv[k] > 0 ? ((k & 1) ? i0++ : i1++) : ((k & 1) ? i2++ : i3++);
-            dm[i] = MG[y];
+            const uint32_t i = mv[k] > 0 ? ip++ : im++;
+            dm[i] = MG[cb + o];
             dy[i] = (uint16_t)o;
         }
     }
     if (threadIdx.x == 0)
-        dl_cnt[c] = make_uint2(totp, totm);
+        dl_cnt[c] = make_uint2(tot & 0xffffu, tot >> 16);
 }
 
 // ---------------------------------------------------------------------------
@@ -122,20 +115,6 @@ __device__ __forceinline__ uint64_t quot_sum_uniform(uint64_t k2, const uint64_t
     return (a0 + a1) + (a2 + a3);
 }
 
-// The same over mp[s0 .. s0 + n): a first odd element alone, then from an
-// even index (mp itself starts at an even index).
-__device__ __forceinline__ uint64_t quot_sum_uniform_at(uint64_t k2, const uint64_t *mp,
-                                                        uint32_t s0, uint32_t n, unsigned l)
-{
-    uint64_t a = 0;
-    if ((s0 & 1u) && n) {
-        a = div_magic(k2, mp[s0], l);
-        ++s0;
-        --n;
-    }
-    return a + quot_sum_uniform(k2, mp + s0, n, l);
-}
-
 // Same with a per-term shift (chunk 0) and/or a per-lane cut-off y <= ycl.
 __device__ __forceinline__ uint64_t quot_sum_general(uint64_t k2, const uint64_t *mp,
                                                      const uint16_t *yp, uint32_t n, uint64_t cb,
@@ -169,8 +148,7 @@ __global__ void __launch_bounds__(kDenseThreads) dense_update_kernel(DenseArgs a
         const DenseItem d = a.items[it];
         for (uint32_t c = d.c0; c < d.c1; ++c) {
             const uint2 cnt = a.dl_cnt[c];
-            const uint32_t tot = even_up(cnt.x & 0xffffu) + even_up(cnt.x >> 16) +
-                                 even_up(cnt.y & 0xffffu) + (cnt.y >> 16);
+            const uint32_t tot = even_up(cnt.x) + cnt.y;
             const uint64_t *src = a.dl_m + (uint64_t)c * kChunkCapPad;
             const uint16_t *ysrc = a.dl_yo + (uint64_t)c * kChunkCapPad;
             uint64_t *dst = s_m + (c - d.c0) * kChunkCapPad;
@@ -186,66 +164,34 @@ __global__ void __launch_bounds__(kDenseThreads) dense_update_kernel(DenseArgs a
         for (uint32_t g = d.g0 + warp; g < d.g1; g += nwarp) {
             const Group G = a.groups[g];
             const bool act = (uint32_t)lane < G.count;
-            const uint64_t e = (uint64_t)G.first + (uint64_t)G.stride * lane;
+            const uint64_t e = (uint64_t)G.first + lane;
             const uint64_t k2 = act ? (a.K[e] << 1) : 0ull;
             const uint64_t ycl = G.pred ? (act ? a.YCE[e] : 0ull) : G.yc;
-            uint64_t acc_o = 0, acc_e = 0;  // odd-y and even-y parts, mod 2^64
+            uint64_t acc = 0;  // mod 2^64
             for (uint32_t c = d.c0; c < d.c1; ++c) {
                 const uint64_t cb = (uint64_t)c * kChunk;
                 if (cb > G.yc)
                     break;
                 const uint2 cnt = s_cnt[c - d.c0];
-                // parts: [lo, hi) index ranges of +odd, +even, -odd, -even
-                uint32_t n[4] = {cnt.x & 0xffffu, cnt.x >> 16, cnt.y & 0xffffu, cnt.y >> 16};
-                uint32_t base[4];
-                base[0] = 0;
-                base[1] = even_up(n[0]);
-                base[2] = base[1] + even_up(n[1]);
-                base[3] = base[2] + even_up(n[2]);
+                uint32_t np = cnt.x, nm = cnt.y;
+                const uint32_t bm = even_up(cnt.x);
                 const uint64_t *mp = s_m + (c - d.c0) * kChunkCapPad;
                 const uint16_t *yp = s_yo + (c - d.c0) * kChunkCapPad;
                 if (cb + kChunk - 1 > G.yc) {
                     const uint32_t lim = (uint32_t)(G.yc - cb);
-#pragma unroll
-                    for (int q = 0; q < 4; ++q)
-                        n[q] = upper_bound_u16(yp + base[q], n[q], lim);
-                }
-                // odd y <= olo come from entry x/2 (the group's lower bound)
-                uint32_t skip[4] = {0, 0, 0, 0};
-                if (G.olo >= cb) {
-                    if (G.olo >= cb + kChunk - 1) {
-                        skip[0] = n[0];
-                        skip[2] = n[2];
-                    } else {
-                        const uint32_t lo = (uint32_t)(G.olo - cb);
-                        skip[0] = upper_bound_u16(yp + base[0], n[0], lo);
-                        skip[2] = upper_bound_u16(yp + base[2], n[2], lo);
-                    }
+                    np = upper_bound_u16(yp, np, lim);
+                    nm = upper_bound_u16(yp + bm, nm, lim);
                 }
                 const unsigned l = magic_shift((c + 1) * (uint64_t)kChunk - 1);
-                uint64_t part[4];
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    const uint32_t s0 = skip[q], cntq = n[q] > s0 ? n[q] - s0 : 0u;
-                    if (c == 0 || G.pred)
-                        part[q] = quot_sum_general(k2, mp + base[q] + s0, yp + base[q] + s0, cntq,
-                                                   cb, l, c == 0, ycl);
-                    else
-                        part[q] = quot_sum_uniform_at(k2, mp + base[q], s0, cntq, l);
-                }
-                acc_o += part[0] - part[2];
-                acc_e += part[1] - part[3];
+                if (c == 0 || G.pred)
+                    acc += quot_sum_general(k2, mp, yp, np, cb, l, c == 0, ycl) -
+                           quot_sum_general(k2, mp + bm, yp + bm, nm, cb, l, c == 0, ycl);
+                else
+                    acc += quot_sum_uniform(k2, mp, np, l) - quot_sum_uniform(k2, mp + bm, nm, l);
             }
-            if (act) {
+            if (act)
                 atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e),
-                          (unsigned long long)(acc_o + acc_e));
-                if ((G.emit >> lane) & 1u) {
-                    // entry 2x: its odd y' = y/2 terms are minus these
-                    const uint64_t x = (uint64_t)G.x0 + (uint64_t)G.stride * lane;
-                    atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e + x),
-                              (unsigned long long)(0ull - acc_e));
-                }
-            }
+                          (unsigned long long)acc);
         }
         __syncthreads();
     }
@@ -974,40 +920,6 @@ __global__ void __launch_bounds__(kWideThreads) wide_update_kernel(WideArgs a)
         if (t)
             atomicAdd(reinterpret_cast<unsigned long long *>(a.S + W.e), (unsigned long long)t);
     }
-}
-
-__global__ void table_lookup_kernel(const uint64_t *__restrict__ pairs, uint32_t count,
-                                    const int16_t *__restrict__ Mloc,
-                                    const int64_t *__restrict__ segoff, uint64_t *__restrict__ R)
-{
-    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= count)
-        return;
-    const uint64_t y = pairs[2 * i + 1];
-    R[pairs[2 * i]] = (uint64_t)(segoff[(y - 1) >> kSegShift] + (int64_t)Mloc[y - 1]);
-}
-
-__global__ void carry_from_table_kernel(const int16_t *__restrict__ Mloc,
-                                        const int64_t *__restrict__ segoff, uint64_t y,
-                                        int64_t *__restrict__ out)
-{
-    *out = segoff[(y - 1) >> kSegShift] + (int64_t)Mloc[y - 1];
-}
-
-int carry_from_table_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y,
-                             int64_t *out, cudaStream_t s)
-{
-    carry_from_table_kernel<<<1, 1, 0, s>>>(Mloc, segoff, y, out);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
-}
-
-int table_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
-                         const int64_t *segoff, uint64_t *R, cudaStream_t s)
-{
-    if (count == 0)
-        return 0;
-    table_lookup_kernel<<<(count + 255) / 256, 256, 0, s>>>(pairs, count, Mloc, segoff, R);
-    return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
 int wide_update_enqueue(const WideArgs &a, uint32_t nw, uint32_t grid_x, cudaStream_t s)

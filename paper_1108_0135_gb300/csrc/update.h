@@ -7,9 +7,9 @@
 namespace mert {
 
 // Chunks staged per dense work item, threads per dense CTA, and the padded
-// per-chunk capacity of the squarefree list (four parts -- mu = +1 odd y,
-// +1 even, -1 odd, -1 even -- each starting at an even index so that they
-// can be read 16 bytes at a time; at most 3072 squarefree y per chunk).
+// per-chunk capacity of the squarefree list (two parts -- mu = +1, mu = -1 --
+// each starting at an even index so that they can be read 16 bytes at a time;
+// at most 3072 squarefree y per chunk).
 constexpr int kDenseChunks = 2;
 constexpr int kDenseThreads = 256;
 constexpr int kChunkCapPad = 3076;
@@ -18,20 +18,13 @@ constexpr int kChunkCapPad = 3076;
 // one target (update.cu): the level sums the kernels produce per entry.
 constexpr uint32_t kShareLevels = 4;
 
-// Up to 32 entries of one target, e = first + stride * lane (x = x0 +
-// stride * lane), sharing one dense cut-off yc (pred = 0), or with a cut-off
-// per entry in YCE (pred = 1; yc = their maximum).  Odd y <= olo are left
-// out of their sums (0: none): those terms come from the entries x/2, whose
-// lanes in `emit` add minus their even-y sums to entry 2x (update.cu).
+// Up to 32 consecutive entries of one target sharing one dense cut-off yc
+// (pred = 0), or with a cut-off per entry in YCE (pred = 1; yc = their maximum).
 struct Group {
     uint32_t first;
     uint32_t count;   // entries in the group (1..32)
     uint32_t pred;
-    uint32_t emit;    // lanes that add their even-y sum to entry 2x
     uint64_t yc;
-    uint64_t olo;
-    uint32_t x0;
-    uint32_t stride;  // 1 or 2
 };
 
 // Dense work item: chunks [c0, c1) for the groups [g0, g1) of the sorted
@@ -164,12 +157,6 @@ __host__ __device__ inline void wide_ranges(const WideEntry &W, uint64_t y1, uin
 }
 
 int magic_table_enqueue(uint64_t *MG, uint64_t nd, cudaStream_t s);
-// R[pairs[2i]] = M(pairs[2i+1]) from a resident table (i < count).
-int table_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
-                         const int64_t *segoff, uint64_t *R, cudaStream_t s);
-// *out = M(y) from a resident table (1 <= y <= its y_max).
-int carry_from_table_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y,
-                             int64_t *out, cudaStream_t s);
 int wide_update_enqueue(const WideArgs &a, uint32_t nw, uint32_t grid_x, cudaStream_t s);
 int dense_list_enqueue(const int8_t *mu_aux, uint64_t ydense, const uint64_t *MG, uint64_t *dl_m,
                        uint16_t *dl_yo, uint2 *dl_cnt, cudaStream_t s);

@@ -106,8 +106,9 @@ __host__ __device__ constexpr uint32_t wheel_block_first(uint32_t b)
 }
 constexpr uint32_t kWheelItem = 256;       // wheel indices of a chunk of the global gather
 
+// A target; n = 0: its value is read from a table (one entry, no terms).
 struct WheelQuery {
-    uint64_t n, X;
+    uint64_t n, n_hi, X;
     uint64_t off, goff;     // first entry, first group
 };
 
@@ -136,6 +137,7 @@ struct WheelEntryArgs {
     uint32_t nq;
     uint32_t ngroups;
     double dc;              // dense cut-off factor
+    uint64_t wide_from;     // entries with k at or above: two-word ones (k = 0 here)
     uint64_t *K, *YC;
     uint32_t *JL, *JD;
     WheelGroup *groups;
@@ -203,6 +205,32 @@ int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks,
 int wheel_dense_enqueue(const WheelDenseArgs &a, uint64_t max_items, cudaStream_t s);
 int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s);
 int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s);
+
+// Entries with k >= 2^63 (k = 0 in the arrays above), with 128-bit quotients: the
+// direct terms M6(y) (phi6(floor(k/y)) - phi6(floor(k/(y+1)))) of the y <= s, which
+// telescope over the y between two wheel numbers, and the gathered terms j in
+// [jlo, jhi] coprime to 6 (update.h's WheelEntry fields); and the values of M
+// with an argument floor(k/m) in the block, m = 2, 3, 6.
+struct WideEntry;
+struct WheelWideArgs {
+    const WideEntry *W;
+    uint64_t y0, len;
+    const int16_t *Mloc;
+    const int64_t *segoff;
+    uint64_t *S, *A;
+};
+// Terms of entry W in the block (y0, y0 + len]: `direct` wheel numbers, then the
+// wheel indices [wj, wj + gathered).
+void wheel_wide_units(const WideEntry &W, uint64_t y0, uint64_t len, uint64_t *direct,
+                      uint64_t *wj, uint64_t *gathered);
+int wheel_wide_enqueue(const WheelWideArgs &a, uint32_t nw, uint64_t units, cudaStream_t s);
+
+// Reads of a resident table (Mloc and segoff from y = 0 on): M(y) of (entry, y)
+// pairs into R; M6(y0) into *out (y0 a multiple of a segment, > 0).
+int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
+                         const int64_t *segoff, uint64_t *R, cudaStream_t s);
+int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y0, int64_t *out,
+                           cudaStream_t s);
 
 struct QueryDev;
 // R6[x] = M6(floor(n/x)) from the sums S, then M in R (A: the parts of M whose

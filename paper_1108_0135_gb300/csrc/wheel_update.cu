@@ -50,7 +50,7 @@ __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v)
 }
 
 // k = floor(n/x), the first j of its gathered terms and the group's dense
-// cut-off: dc sqrt(k of the group's first entry), up to a multiple of 4096 less
+// cut-off: dc sqrt(k of the group's first one-word entry), up to a multiple of 4096 less
 // one, within [floor(sqrt(k)), floor(k/jlo) - 1] of every entry where the group
 // has such a value (per entry otherwise), and for the group the least of these
 // and of floor(k/jlo) (beyond it no term is left), down to a multiple of 6.
@@ -71,24 +71,40 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
     const WheelQuery Q = a.qs[lo_q];
     const uint64_t x0 = (g - Q.goff) * kWheelGroup + 1;
     const uint32_t cnt = (uint32_t)min((uint64_t)kWheelGroup, Q.X - x0 + 1);
-    const uint64_t kf = Q.n / x0;
     uint64_t k[2], sq[2], vh[2], jlo[2], cap[2];
-    uint64_t lo = 0, nhi = 0;  // max of s, max of ~vh (= ~min)
+    uint64_t lo = 0, nhi = 0, kf = 0;  // max of s, max of ~vh (= ~min), largest k
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
         k[h] = 0;
         if (i < cnt) {
             const uint64_t x = x0 + i;
-            k[h] = Q.n / x;
-            sq[h] = isqrt_dev(k[h]);
-            jlo[h] = Q.X / x + 1;
-            cap[h] = k[h] / jlo[h];
-            vh[h] = jlo[h] <= k[h] / (sq[h] + 1) ? cap[h] - 1 : sq[h];
-            lo = max(lo, sq[h]);
-            nhi = max(nhi, ~vh[h]);
+            if (Q.n_hi) {
+                const unsigned __int128 kk = (((unsigned __int128)Q.n_hi << 64) | Q.n) / x;
+                k[h] = kk < a.wide_from ? (uint64_t)kk : 0;
+            } else {
+                k[h] = Q.n / x;
+                if (k[h] >= a.wide_from)
+                    k[h] = 0;
+            }
+            if (k[h]) {
+                kf = max(kf, k[h]);
+                sq[h] = isqrt_dev(k[h]);
+                jlo[h] = Q.X / x + 1;
+                cap[h] = k[h] / jlo[h];
+                vh[h] = jlo[h] <= k[h] / (sq[h] + 1) ? cap[h] - 1 : sq[h];
+                lo = max(lo, sq[h]);
+                nhi = max(nhi, ~vh[h]);
+            } else {
+                const uint64_t e = Q.off + x - 1;
+                a.K[e] = 0;
+                a.YC[e] = 0;
+                a.JL[e] = 1;
+                a.JD[e] = 0;
+            }
         }
     }
+    kf = warp_max_u64(kf);
     lo = warp_max_u64(lo);
     const uint64_t hi = ~warp_max_u64(nhi);
     uint64_t target = (uint64_t)(a.dc * sqrt((double)kf));
@@ -100,7 +116,7 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
             yce[h] = lo <= hi ? min(max(target, lo), hi) : min(max(target, sq[h]), vh[h]);
             nyc = max(nyc, ~min(yce[h], cap[h]));
         }
-    uint64_t yc = ~warp_max_u64(nyc);
+    uint64_t yc = kf ? ~warp_max_u64(nyc) : 0;
     yc -= yc % 6;
     uint64_t direct = 0, gathered = 0, gather_j = 0, exec = 0;
 #pragma unroll
@@ -898,6 +914,116 @@ __global__ void __launch_bounds__(256) wheel_chunk_kernel(WheelBlockArgs a)
 }
 
 // ---------------------------------------------------------------------------
+// Two-word entries (grid.y of them), the block's terms numbered as one range,
+// kWidePer consecutive ones per thread; sums mod 2^64.
+// ---------------------------------------------------------------------------
+typedef unsigned __int128 u128d;
+
+// phi6(floor(k/y)) mod 2^64.
+__device__ __forceinline__ uint64_t phi6_quot(u128d k, uint64_t y)
+{
+    const u128d d = (u128d)6u * y, t = k / d, rem = k - t * d;
+    return 2u * (uint64_t)t + (rem >= y ? 1u : 0u) + (rem >= (u128d)5u * y ? 1u : 0u);
+}
+
+__host__ __device__ inline void wide_units(const WideEntry &W, uint64_t y0, uint64_t len,
+                                           uint64_t *direct, uint64_t *wj, uint64_t *gathered)
+{
+    const unsigned __int128 k = ((unsigned __int128)W.k_hi << 64) | W.k_lo;
+    const uint64_t yend = y0 + len, top = W.s < yend ? W.s : yend;
+    *direct = top > y0 ? phi6(top) - phi6(y0) : 0;
+    // j with floor(k/j) in (y0, yend]
+    const unsigned __int128 q2 = k / ((unsigned __int128)yend + 1) + 1;
+    const unsigned __int128 q1 = k / ((unsigned __int128)y0 + 1);
+    const uint64_t b = q2 > W.jlo ? (q2 > W.jhi ? W.jhi + 1 : (uint64_t)q2) : W.jlo;
+    const uint64_t t = q1 < W.jhi ? (uint64_t)q1 : W.jhi;
+    *wj = b <= t ? phi6(b - 1) : 0;
+    *gathered = b <= t ? phi6(t) - *wj : 0;
+}
+
+void wheel_wide_units(const WideEntry &W, uint64_t y0, uint64_t len, uint64_t *direct,
+                      uint64_t *wj, uint64_t *gathered)
+{
+    wide_units(W, y0, len, direct, wj, gathered);
+}
+
+__global__ void __launch_bounds__(kWideThreads) wheel_wide_kernel(WheelWideArgs a)
+{
+    __shared__ uint64_t red[kWideThreads / 32];
+    const WideEntry W = a.W[blockIdx.y];
+    const u128d k = ((u128d)W.k_hi << 64) | W.k_lo;
+    uint64_t nd, wj, ng;
+    wide_units(W, a.y0, a.len, &nd, &wj, &ng);
+    const uint64_t units = nd + ng;
+    const uint64_t u0 = (uint64_t)blockIdx.x * kWideUnitsPerCta + (uint64_t)threadIdx.x * kWidePer;
+    const uint64_t u1 = u0 + kWidePer < units ? u0 + kWidePer : units;
+    uint64_t acc = 0, u = u0;
+    if (u < u1 && u < nd) {
+        // direct: wheel number w0 + u and the y up to the next one (or s)
+        const uint64_t w0 = a.y0 / 3;
+        uint64_t p = phi6_quot(k, wheel_y(w0 + u));
+        for (const uint64_t ue = u1 < nd ? u1 : nd; u < ue; ++u) {
+            const uint64_t yn = wheel_y(w0 + u + 1);
+            const uint64_t pn = phi6_quot(k, yn <= W.s ? yn : W.s + 1);
+            acc += (uint64_t)wheel_M(a.segoff, a.Mloc, (uint32_t)u) * (p - pn);
+            p = pn;
+        }
+    }
+    for (; u < u1; ++u) {
+        const uint64_t j = wheel_y(wj + (u - nd));
+        acc += (uint64_t)wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)((uint64_t)(k / j) - a.y0)));
+    }
+    acc = warp_sum_u64(acc);
+    if ((threadIdx.x & 31) == 0)
+        red[threadIdx.x >> 5] = acc;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        uint64_t t = 0;
+        for (int w = 0; w < kWideThreads / 32; ++w)
+            t += red[w];
+        if (t)
+            atomicAdd(reinterpret_cast<unsigned long long *>(a.S + W.e), (unsigned long long)t);
+        if (blockIdx.x == 0 && W.jlo <= 6u) {
+            int64_t tail = 0;
+            for (uint32_t m = 2; m <= 6; m += (m == 2 ? 1u : 3u)) {
+                const u128d y = k / m;
+                if (m >= W.jlo && y > a.y0 && y <= a.y0 + a.len) {
+                    const int64_t v = wheel_M(a.segoff, a.Mloc,
+                                              wheel_index((uint32_t)((uint64_t)y - a.y0)));
+                    tail += m == 6 ? v : -v;
+                }
+            }
+            a.A[W.e] += (uint64_t)tail;
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Resident tables.
+// ---------------------------------------------------------------------------
+__global__ void wheel_lookup_kernel(const uint64_t *__restrict__ pairs, uint32_t count,
+                                    const int16_t *__restrict__ Mloc,
+                                    const int64_t *__restrict__ segoff, uint64_t *__restrict__ R)
+{
+    const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= count)
+        return;
+    const uint64_t y = pairs[2 * i + 1];
+    const auto M6 = [&](uint64_t v) -> int64_t {
+        const uint64_t w = phi6(v);
+        return w ? segoff[(w - 1) >> kSegShift] + (int64_t)Mloc[w - 1] : 0;
+    };
+    R[pairs[2 * i]] = (uint64_t)(M6(y) - M6(y / 2) - M6(y / 3) + M6(y / 6));
+}
+
+__global__ void wheel_carry_at_kernel(const int16_t *__restrict__ Mloc,
+                                      const int64_t *__restrict__ segoff, uint64_t w,
+                                      int64_t *__restrict__ out)
+{
+    *out = segoff[w >> kSegShift] + (int64_t)Mloc[w];
+}
+
+// ---------------------------------------------------------------------------
 // Resolve: R6[x] = 1 - S[x] - sum over j >= 2 coprime to 6, xj <= X, of R6[xj],
 // then M[x] = R6[x] - V(2x) - V(3x) + V(6x), V(z) = R6[z] within the array (the
 // values beyond it are in A).  The smallest such j is 5, so the entries of
@@ -1033,6 +1159,36 @@ int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s)
     const uint32_t grid = std::min<uint32_t>((uint32_t)sm_count() * 8u, (a.qcap + 7u) / 8u);
     wheel_chunk_kernel<<<grid, 256, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? 2 : -1;
+}
+
+int wheel_wide_enqueue(const WheelWideArgs &a, uint32_t nw, uint64_t units, cudaStream_t s)
+{
+    if (nw == 0)
+        return 0;
+    const uint64_t gx = std::max<uint64_t>(1, (units + kWideUnitsPerCta - 1) / kWideUnitsPerCta);
+    int n = 0;
+    for (uint32_t w = 0; w < nw; w += 65535u, ++n) {  // grid.y is 16 bits
+        WheelWideArgs b = a;
+        b.W += w;
+        wheel_wide_kernel<<<dim3((unsigned)gx, std::min(nw - w, 65535u)), kWideThreads, 0, s>>>(b);
+    }
+    return cudaGetLastError() == cudaSuccess ? n : -1;
+}
+
+int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
+                         const int64_t *segoff, uint64_t *R, cudaStream_t s)
+{
+    if (count == 0)
+        return 0;
+    wheel_lookup_kernel<<<(count + 127) / 128, 128, 0, s>>>(pairs, count, Mloc, segoff, R);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
+}
+
+int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y0, int64_t *out,
+                           cudaStream_t s)
+{
+    wheel_carry_at_kernel<<<1, 1, 0, s>>>(Mloc, segoff, y0 / 3 - 1, out);
+    return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
 int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint64_t *S,
