@@ -748,8 +748,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             const uint64_t len = std::min(tile_y, end - t0);
             if (kt == UINT64_MAX) {
                 // entries whose cut-off lies below the tile's end: all where a
-                // cut-off can be bound by floor(k/jlo), else those with
-                // dc sqrt(k of the group's first) < t0 + len + 8
+                // cut-off can be bound by floor(k/jlo), else those of the groups
+                // with dc sqrt(k of the group's last) < t0 + len + 8
                 ranges.clear();
                 ks.clear();
                 for (size_t i = 0; i < count; ++i) {
@@ -759,7 +759,9 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
                     const double nd = (double)n[i], te = (double)(t0 + len) + 8.0;
                     uint64_t lo = 0;
                     if (2.0 * (dc * std::sqrt(nd) + 2.0 * kChunk) < (double)us[i])
-                        lo = (uint64_t)std::min((double)Q.X, dc * dc * nd / (te * te)) /
+                        lo = (uint64_t)std::max(0.0, std::min((double)Q.X + kWheelGroup,
+                                                              dc * dc * nd / (te * te)) -
+                                                         (double)kWheelGroup) /
                              kWheelGroup * kWheelGroup;
                     if (lo >= Q.X)
                         continue;

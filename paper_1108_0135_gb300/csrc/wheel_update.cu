@@ -10,13 +10,13 @@
 // j > jd coprime to 6 with floor(k/j) >= y), whose second part is
 // -M6(yc) phi6(jd).  jd = max(floor(k/(yc + 1)), floor(X/x)).
 //
-// phi6 of a quotient without the quotient: with T the integer nearest
-// k / (6y) and r = k - 6yT, |r| <= 3y,
-//   phi6(floor(k/y)) = 2T - 1 + [r >= -y] + [r >= y]
-// (6T - 1 and 6T + 1 are the wheel numbers near 6T), and the value is the same
-// for T one off as long as |r| < 5y: no wheel number lies between 6T + 1 and
-// 6T + 5.  So an estimate of k / (6y) that errs by less than 1/3 before it is
-// rounded is exact, and one 32-bit remainder and two sign bits give phi6.
+// phi6 of a quotient without the quotient: with Y(w) = 3w + 1 + (w & 1) =
+// (3w + 1) | 1 the wheel numbers and T near k / (3y),
+//   phi6(floor(k/y)) = T + [k >= y Y(T)]
+// whenever Y(T - 1) <= k/y < Y(T + 1), which holds for -1/3 <= k/(3y) - T < 4/3
+// (T even: 3T - 1 <= k/y < 3T + 5, T odd: 3T - 2 <= k/y < 3T + 4).  So the floor
+// of an estimate of k/(3y) that errs by less than 1/3 is exact, and one 32-bit
+// multiply-subtract and its sign bit give phi6.
 #include <algorithm>
 #include <cstdint>
 
@@ -25,8 +25,16 @@
 
 namespace mert {
 
-constexpr uint32_t kMagicBits = 0x4B400000u;  // bits of 1.5 2^23: adding it rounds a float
+// A float estimate plus 1.5 2^23, rounded down, has the bits kMagicBits + its
+// floor.
+constexpr uint32_t kMagicBits = 0x4B400000u;
 constexpr float kMagicF = 12582912.0f;
+
+// Y(T) from the biased bits.
+__device__ __forceinline__ uint32_t wheel_of_bits(uint32_t bits)
+{
+    return (3u * bits + (1u - 3u * kMagicBits)) | 1u;
+}
 
 // ---------------------------------------------------------------------------
 // Plan: the entries of every target, a warp per group of 64 (two per lane).
@@ -50,10 +58,14 @@ __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v)
 }
 
 // k = floor(n/x), the first j of its gathered terms and the group's dense
-// cut-off: dc sqrt(k of the group's first one-word entry), up to a multiple of 4096 less
-// one, within [floor(sqrt(k)), floor(k/jlo) - 1] of every entry where the group
-// has such a value (per entry otherwise), and for the group the least of these
-// and of floor(k/jlo) (beyond it no term is left), down to a multiple of 6.
+// cut-off: dc sqrt(mean k of the group), at most floor(k/jlo) of every entry
+// (beyond it no term is left), down to a multiple of 6.  Any cut-off gives the
+// same sums; a dense y costs the whole group one term per entry, a gathered j
+// only its own, so the mean of k balances them (with the first entry's k, the
+// first group had four times the dense terms: 14% of all at n = 10^13).  jd stays
+// below 2^32.  The totals' gather_j counts the gathered terms of the full sums'
+// cut-offs (dc sqrt(k of the first one-word entry), up to a multiple of 4096 less
+// one, within [floor(sqrt(k)), floor(k/jlo) - 1]).
 __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
 {
     const uint32_t lane = threadIdx.x & 31u;
@@ -73,6 +85,7 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
     const uint32_t cnt = (uint32_t)min((uint64_t)kWheelGroup, Q.X - x0 + 1);
     uint64_t k[2], sq[2], vh[2], jlo[2], cap[2];
     uint64_t lo = 0, nhi = 0, kf = 0;  // max of s, max of ~vh (= ~min), largest k
+    float ksum = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
@@ -89,6 +102,7 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
             }
             if (k[h]) {
                 kf = max(kf, k[h]);
+                ksum += (float)k[h];
                 sq[h] = isqrt_dev(k[h]);
                 jlo[h] = Q.X / x + 1;
                 cap[h] = k[h] / jlo[h];
@@ -105,6 +119,10 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
         }
     }
     kf = warp_max_u64(kf);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
+    const uint64_t mean = max((uint64_t)(a.dc * sqrt((double)ksum / cnt)), kf / (uint64_t)4000000000u);
     lo = warp_max_u64(lo);
     const uint64_t hi = ~warp_max_u64(nhi);
     uint64_t target = (uint64_t)(a.dc * sqrt((double)kf));
@@ -114,7 +132,7 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
     for (int h = 0; h < 2; ++h)
         if (k[h]) {
             yce[h] = lo <= hi ? min(max(target, lo), hi) : min(max(target, sq[h]), vh[h]);
-            nyc = max(nyc, ~min(yce[h], cap[h]));
+            nyc = max(nyc, ~min(mean, cap[h]));
         }
     uint64_t yc = kf ? ~warp_max_u64(nyc) : 0;
     yc -= yc % 6;
@@ -261,47 +279,34 @@ __device__ __forceinline__ uint32_t count_below(const uint16_t *a, uint32_t n, u
     return lo;
 }
 
-// acc + the sign bit of v (as a multiply-add: the kernels' other integer work is
-// on the ALU pipe).
-__device__ __forceinline__ uint32_t add_sign(uint32_t v, uint32_t acc)
-{
-    uint32_t r;
-    asm("mad.hi.u32 %0, %1, 2, %2;" : "=r"(r) : "r"(v), "r"(acc));
-    return r;
-}
-
-// Float mode: staged {1/(6y), -6y, 6y C + y, 6y C - y}, C = kMagicBits.  The
-// estimate k (1/6y) has three roundings of 2^-24 and k/(6y) < 1.5e6 (the host's
-// rule), so it errs by less than 0.27; r + y and r - y come from the biased T
-// by one multiply-add and one add each; their sign bits and the T are summed.
-// n <= 2048 terms, so the T sum stays below 2^32.
-__device__ __forceinline__ void dense_float(const uint4 *el, uint32_t n, const float kf[2],
+// Float mode: staged {1/(3y), -y}.  The estimate k (1/3y) has roundings of 2^-24
+// in k, in the reciprocal and, from 3y = 2^24 on, in 3y: it errs by less than 1/3
+// for k/(3y) < 2.06e6, or 1.8e6 there (the kernel's rule; n <= 2048 terms, so the
+// sum of the T stays below 2^32).
+__device__ __forceinline__ void dense_float(const uint2 *el, uint32_t n, const float kf[2],
                                             const uint32_t kl[2], uint64_t out[2])
 {
     uint32_t st[2] = {0, 0}, ss[2] = {0, 0};
 #pragma unroll 4
     for (uint32_t i = 0; i < n; ++i) {
-        const uint4 v = el[i];
+        const uint2 v = el[i];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            const uint32_t T =
-                __float_as_uint(__fmaf_rn(kf[e], __uint_as_float(v.x), kMagicF));
-            const uint32_t r = T * v.y + kl[e];
+            const uint32_t T = __float_as_uint(__fmaf_rd(kf[e], __uint_as_float(v.x), kMagicF));
+            ss[e] += (wheel_of_bits(T) * v.y + kl[e]) >> 31;
             st[e] += T;
-            ss[e] = add_sign(r + v.z, ss[e]);
-            ss[e] = add_sign(r + v.w, ss[e]);
         }
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e)
-        out[e] = 2ull * (uint32_t)(st[e] - n * kMagicBits) + n - ss[e];
+        out[e] = (uint64_t)(uint32_t)(st[e] - n * kMagicBits) + n - ss[e];
 }
 
-// High-word mode: staged {m, -6y, y, ex}, m = floor(2^(31 + ex)/(6y)) in [2^30,
-// 2^31), ex = floor(log2 6y); kh the top 32 bits of k (b bits), T the rounded
+// High-word mode: staged {m, -y}, m = floor(2^(31 + ex)/(3y)) in [2^30, 2^31),
+// ex = floor(log2 3y); kh the top 32 bits of k (b bits), T the floor of
 // (kh m / 2^32) / 2^(ex + 31 - b).  Truncations of 2^-31 and 2^-30 and one of a
-// unit before the shift (at least 3) with k/(6y) < 6e7: less than 0.3.
-__device__ __forceinline__ void dense_high(const uint4 *el, uint32_t n, const uint32_t kh[2],
+// unit before the shift (at least 4) with k/(3y) < 6e7: less than 0.15.
+__device__ __forceinline__ void dense_high(const uint2 *el, uint32_t n, const uint32_t kh[2],
                                            const uint32_t sb[2], const uint32_t kl[2],
                                            uint64_t out[2])
 {
@@ -309,21 +314,50 @@ __device__ __forceinline__ void dense_high(const uint4 *el, uint32_t n, const ui
     uint32_t ss[2] = {0, 0};
 #pragma unroll 4
     for (uint32_t i = 0; i < n; ++i) {
-        const uint4 v = el[i];
+        const uint2 v = el[i];
+        const uint32_t ex = 31u - __clz(0u - 3u * v.y);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
-            // shift less one, at most 31 (k far below 6y: T = 0)
-            const uint32_t sh = min(v.w + sb[e], 31u);
-            const uint32_t T = ((__umulhi(kh[e], v.x) >> sh) + 1u) >> 1;
-            const uint32_t r = T * v.y + kl[e];
+            // at most 31 (k far below 3y: T = 0)
+            const uint32_t T = __umulhi(kh[e], v.x) >> min(ex + sb[e], 31u);
+            ss[e] += (((3u * T + 1u) | 1u) * v.y + kl[e]) >> 31;
             st[e] += T;
-            ss[e] = add_sign(r + v.z, ss[e]);
-            ss[e] = add_sign(r - v.z, ss[e]);
         }
     }
 #pragma unroll
     for (int e = 0; e < 2; ++e)
-        out[e] = 2ull * st[e] + n - ss[e];
+        out[e] = st[e] + n - ss[e];
+}
+
+// Two steps, k/(3y) < 3e14, from the same staged values: q1 from the high words as
+// above but in 64 bits (at most 3.3e-9 k/(3y) + 1 below k/(3y)), then the float
+// mode's estimate for the rest k - 3y q1 < 2^35 (its quotient below 1e6).
+__device__ __forceinline__ void dense_two(const uint2 *el, uint32_t n, const uint64_t k[2],
+                                          const uint32_t kh[2], const uint32_t sb[2],
+                                          uint64_t out[2])
+{
+    uint64_t st[2] = {0, 0};
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint2 v = el[i];
+        const uint32_t d = 0u - 3u * v.y, ex = 31u - __clz(d);
+        const float rf = __uint2float_rn(v.x) * __uint_as_float((96u - ex) << 23);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const uint32_t h = __umulhi(kh[e], v.x);
+            const int sh = (int)(ex + sb[e]);
+            const uint64_t q1 = sh >= 0 ? (uint64_t)(h >> min(sh, 31)) : (uint64_t)h << -sh;
+            const uint64_t r1 = k[e] - q1 * d;
+            const float rh = __uint_as_float(0x4B000000u | (uint32_t)(r1 >> 16)) - 8388608.0f;
+            const float rl = __uint_as_float(0x4B000000u | ((uint32_t)r1 & 0xffffu)) - 8388608.0f;
+            const uint32_t T2 =
+                __float_as_uint(__fmaf_rd(__fmaf_rn(rh, 65536.0f, rl), rf, kMagicF)) - kMagicBits;
+            const uint64_t T = q1 + T2;
+            st[e] += T + 1u -
+                     ((((3u * (uint32_t)T + 1u) | 1u) * v.y + (uint32_t)k[e]) >> 31);
+        }
+    }
+    out[0] = st[0];
+    out[1] = st[1];
 }
 
 // Any k < 2^63 and y < 2^60, by 64-bit division (few terms need it).
@@ -343,12 +377,12 @@ __device__ __forceinline__ void dense_wide(const uint16_t *off, uint32_t n, uint
 }
 
 // A work item is part of a chunk's list for kWheelGroupBlock groups.  Items whose
-// k/(6y) all lie below 1.5e6 (and y < 3.5e8) take the float mode; in the others
-// the y up to kmax/3.6e8 (all y from 3.5e8) take 64-bit division, the rest the
-// high-word mode.
+// k/(3y) all lie below the float mode's bound (and y < 3.5e8) take it; in the
+// others the y up to kmax/9e14 (all y from 3.5e8) take 64-bit division, those up
+// to kmax/1.8e8 the two-step mode, the rest the high-word mode.
 __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDenseArgs a)
 {
-    __shared__ uint4 s_el[kSegY];
+    __shared__ uint2 s_el[kSegY];
     __shared__ uint16_t s_off[kSegY];
     __shared__ uint32_t s_item, s_block;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -385,7 +419,8 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
             kmax = max(kmax, a.groups[g0 + g].kmax);
         const uint64_t y0 = (uint64_t)c * kWheelSegY;
         const bool small_y = y0 + kWheelSegY < 350000000u;
-        const bool fl = small_y && kmax < 9000000ull * (y0 + 1);
+        const bool fl =
+            small_y && kmax < (y0 + kWheelSegY < 5500000u ? 6200000ull : 5400000ull) * (y0 + 1);
         const uint32_t cnt = a.dl_cnt[c];
         const uint32_t cp = cnt & 0xffffu, cm = cnt >> 16;
         const uint32_t p0 = cp * part / a.parts, m0 = cm * part / a.parts;
@@ -396,15 +431,11 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
             s_off[i] = (uint16_t)o;
             if (!small_y)
                 continue;
-            const uint32_t y = (uint32_t)y0 + 3u * o + 1u + (o & 1u), d = 6u * y;
-            if (fl) {
-                const float rf = __frcp_rn(__uint2float_rn(d));
-                const uint32_t cd = kMagicBits * d;
-                s_el[i] = make_uint4(__float_as_uint(rf), 0u - d, cd + y, cd - y);
-            } else {
-                const uint32_t ex = 31u - __clz(d);
-                s_el[i] = make_uint4((uint32_t)((1ull << (31u + ex)) / d), 0u - d, y, ex);
-            }
+            const uint32_t y = (uint32_t)y0 + 3u * o + 1u + (o & 1u), d = 3u * y;
+            const uint32_t ex = 31u - __clz(d);
+            s_el[i] = make_uint2(fl ? __float_as_uint(__frcp_rn(__uint2float_rn(d)))
+                                    : (uint32_t)((1ull << (31u + ex)) / d),
+                                 0u - y);
         }
         __syncthreads();
         // one group per warp; fewer groups than warps: several warps share a
@@ -439,33 +470,47 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
                 sum[0] -= part2[0];
                 sum[1] -= part2[1];
             } else {
-                const uint64_t yw = small_y ? G.kmax / 360000000ull : UINT64_MAX;
-                uint32_t w0 = 0, w1 = 0;  // terms by division
-                if (yw > y0) {
-                    const uint32_t lim =
-                        yw >= y0 + kWheelSegY ? 0xffffu
-                                              : (uint32_t)(phi6(yw) - (uint64_t)c * kSegY);
-                    w0 = count_below(s_off + f0, n0, lim);
-                    w1 = count_below(s_off + f1, n1, lim);
-                }
+                // terms with y <= yl of a list
+                const auto upto = [&](const uint16_t *off, uint32_t n, uint64_t yl) -> uint32_t {
+                    if (yl <= y0)
+                        return 0;
+                    if (yl >= y0 + kWheelSegY)
+                        return n;
+                    return count_below(off, n, (uint32_t)(phi6(yl) - (uint64_t)c * kSegY));
+                };
+                const uint64_t yd = small_y ? G.kmax / 900000000000000ull : UINT64_MAX;
+                const uint64_t yt = small_y ? G.kmax / 180000000ull : UINT64_MAX;
                 uint32_t kh[2], sb[2], kl[2];
 #pragma unroll
                 for (int e = 0; e < 2; ++e) {
                     const uint32_t b = bitlen64(k[e]);
                     kl[e] = (uint32_t)k[e];
-                    kh[e] = b >= 32u ? (uint32_t)(k[e] >> (b - 32u)) : (uint32_t)k[e] << ((32u - b) & 31u);
-                    sb[e] = 30u - b;
+                    kh[e] = b >= 32u ? (uint32_t)(k[e] >> (b - 32u))
+                                     : (uint32_t)k[e] << ((32u - b) & 31u);
+                    sb[e] = 31u - b;
                 }
-                dense_wide(s_off + f0, w0, y0, k, sum);
-                dense_wide(s_off + f1, w1, y0, k, part2);
-                sum[0] -= part2[0];
-                sum[1] -= part2[1];
-                dense_high(s_el + f0 + w0, n0 - w0, kh, sb, kl, part2);
-                sum[0] += part2[0];
-                sum[1] += part2[1];
-                dense_high(s_el + f1 + w1, n1 - w1, kh, sb, kl, part2);
-                sum[0] -= part2[0];
-                sum[1] -= part2[1];
+                sum[0] = sum[1] = 0;
+#pragma unroll 1
+                for (uint32_t l = 0; l < 2u; ++l) {  // mu = +1, then -1
+                    const uint32_t f = l ? f1 : f0, n = l ? n1 : n0;
+                    const uint32_t nd = upto(s_off + f, n, yd), nt = upto(s_off + f, n, yt);
+                    uint64_t t[2] = {0, 0};
+                    if (nd) {
+                        dense_wide(s_off + f, nd, y0, k, part2);
+                        t[0] += part2[0];
+                        t[1] += part2[1];
+                    }
+                    if (nt > nd) {
+                        dense_two(s_el + f + nd, nt - nd, k, kh, sb, part2);
+                        t[0] += part2[0];
+                        t[1] += part2[1];
+                    }
+                    dense_high(s_el + f + nt, n - nt, kh, sb, kl, part2);
+                    t[0] += part2[0];
+                    t[1] += part2[1];
+                    sum[0] += l ? 0u - t[0] : t[0];
+                    sum[1] += l ? 0u - t[1] : t[1];
+                }
             }
 #pragma unroll
             for (int e = 0; e < 2; ++e)
@@ -482,11 +527,10 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
 // Gathered terms of a shared-memory tile: y in [t0 + 1, t0 + len], len <=
 // 98304, staged as M6(y) - M6(t0) (int16: at most 24/25 of 32768 consecutive
 // wheel numbers are squarefree) by wheel index.  A term's index is
-// phi6(floor(R/j)) - 1 with R = k - t0 j < len j: T = the integer nearest
-// R / (6j) <= 2^14 from single precision (relative error near 2^-21), then as
-// above.
+// phi6(floor(R/j)) - 1 with R = k - t0 j < len j: T = floor of R / (3j) <= 2^15
+// from single precision (relative error near 2^-21), then as above.
 // ---------------------------------------------------------------------------
-constexpr uint32_t kGatherJ32 = 300000000u;  // 32-bit remainders below: 6j < 2^31
+constexpr uint32_t kGatherJ32 = 300000000u;  // 32-bit remainders below: 5j < 2^31
 constexpr uint32_t kWheelLaneTerms = 16;     // few terms: always a lane per entry
 
 // v as a float (relative error at most 2^-22) from exact 16-bit pieces.
@@ -502,31 +546,31 @@ __device__ __forceinline__ float float_pieces(uint64_t v)
 
 // Constants of a run of terms j = j0 + step i in a tile.
 struct TileStep {
-    float dRf, stepf;    // step t0 / 6, step
-    uint32_t dRt, step;  // step (6 C - t0) (mod 2^32), step
+    float dRf, stepf;    // step t0 / 3, step
+    uint32_t dR32, step; // step t0 (mod 2^32), step
     uint64_t dR;         // step t0
     __device__ __forceinline__ TileStep(uint64_t t0, uint32_t st)
-        : dRf(float_pieces(t0) * ((float)st / 6.0f)), stepf((float)st),
-          dRt(st * (6u * kMagicBits - (uint32_t)t0)), step(st), dR(t0 * st)
+        : dRf(float_pieces(t0) * ((float)st / 3.0f)), stepf((float)st), dR32((uint32_t)t0 * st),
+          step(st), dR(t0 * st)
     {
     }
 };
 
-// State of a run: R = k - t0 j and j of the current term.  Rf = R/6 and jf are
-// stepped from the run's start with one multiply-add each; kLong (6j beyond 32
+// State of a run: R = k - t0 j and j of the current term.  Rf = R/3 and jf are
+// stepped from the run's start with one multiply-add each; kLong (5j beyond 32
 // bits) takes the remainder in 64 bits.
 template <bool kLong>
 struct TileRun {
     float Rf0, jf0;
-    uint32_t Rt, j;  // R + 6 j C (mod 2^32), j
+    uint32_t nR, j;  // -R - 1 (mod 2^32), j
     uint64_t R;
     __device__ __forceinline__ TileRun(uint64_t k, uint64_t t0, uint32_t j0)
     {
         R = k - t0 * (uint64_t)j0;
-        Rf0 = float_pieces(R) * (1.0f / 6.0f);
+        Rf0 = float_pieces(R) * (1.0f / 3.0f);
         jf0 = float_pieces(j0);
         j = j0;
-        Rt = (uint32_t)R + kMagicBits * 6u * j0;
+        nR = ~(uint32_t)R;
     }
     // the staged value of term i (fi = i), then on to term i + 1
     __device__ __forceinline__ int take(const int16_t *Mt, uint32_t lim, float fi,
@@ -535,19 +579,17 @@ struct TileRun {
         const float Rf = __fmaf_rn(fi, -d.dRf, Rf0), jf = __fmaf_rn(fi, d.stepf, jf0);
         float rj;
         asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(rj) : "f"(jf));
-        const uint32_t T = __float_as_uint(__fmaf_rn(Rf, rj, kMagicF));
-        uint32_t s;
+        const uint32_t T = __float_as_uint(__fmaf_rd(Rf, rj, kMagicF));
+        const uint32_t W = wheel_of_bits(T);
+        uint32_t i;  // T - 1 + [R >= j W]
         if (kLong) {
-            const uint64_t r = R - (uint64_t)(int64_t)(int32_t)(T - kMagicBits) * 6u * j;
-            s = (uint32_t)((r + j) >> 63) + (uint32_t)((r - j) >> 63);
+            i = T - kMagicBits - (uint32_t)((R - (uint64_t)(int64_t)(int32_t)W * j) >> 63);
             R -= d.dR;
         } else {
-            const uint32_t r = Rt - T * (6u * j);
-            s = ((r + j) >> 31) + ((r - j) >> 31);
-            Rt += d.dRt;
+            i = T - (kMagicBits + 1u) + ((W * j + nR) >> 31);
+            nR += d.dR32;
         }
         j += d.step;
-        const uint32_t i = 2u * (T - kMagicBits) - s;
         return Mt[i < lim ? i : lim];
     }
 };
@@ -601,45 +643,43 @@ __device__ __forceinline__ int64_t wheel_M(const int64_t *segoff, const int16_t 
 }
 
 // Tiles at y <= kUniformY: 64 entries of a warp (two per lane) against the same
-// j, whose constants {1/(6j), 6j, -(6jC + j) - 1, -(6jC - j) - 1} are made 32 at a
-// time by the lanes and read back as broadcasts.  T estimates k/(6j) itself (as
-// in dense_float: k/(6j) < 1.5e6 near the tile), and with the remainder negated
-// the two sign bits add up to the index: 2T - 2 + [r >= -j] + [r >= j] less the
-// tile's first index.  An index outside [lo, lim] -- a j whose y lies beyond the
-// tile or at most yc (yc + 1 a wheel number) -- is sent to the zero after it.
-// jw: 32 uint4 of this warp; b2 = -2C - 2 - (first index) - lo.
-constexpr uint64_t kUniformY = 8400000;
+// j, whose constants {1/(3j), j} are made 32 at a time by the lanes and read back
+// as broadcasts.  T estimates k/(3j) itself (3j < 2^24 here, so two roundings of
+// 2^-24, and k/(3j) < 2.6e6 for 5% beyond the tile), and the sign bit of
+// j Y(T) - k - 1 completes the index T - 1 + [k >= j Y(T)] less the tile's first
+// one.  An index outside [lo, lim] -- a j whose y lies beyond the tile or at most
+// yc (yc + 1 a wheel number) -- is sent to the zero after it.  jw: 32 uint2 of
+// this warp; b2 = -C - 1 - (first index) - lo.
+constexpr uint64_t kUniformY = 7400000;
+constexpr uint32_t kUniformW = 1860000;  // 3j < 2^24
 
-__device__ __forceinline__ void tile_uniform(const int16_t *Mt, uint4 *jw, const uint64_t k[2],
+__device__ __forceinline__ void tile_uniform(const int16_t *Mt, uint2 *jw, const uint64_t k[2],
                                              const uint32_t b2[2], const uint32_t lo[2],
                                              uint32_t lim, uint32_t w0, uint32_t w1, uint32_t lane,
                                              int acc[2])
 {
     const float kf[2] = {__ull2float_rn(k[0]), __ull2float_rn(k[1])};
-    const uint32_t nk[2] = {0u - (uint32_t)k[0], 0u - (uint32_t)k[1]};
+    const uint32_t nk[2] = {~(uint32_t)k[0], ~(uint32_t)k[1]};
     const uint32_t hi[2] = {lim + 1u - lo[0], lim + 1u - lo[1]};
     const int16_t *Ml[2] = {Mt + lo[0], Mt + lo[1]};
     acc[0] = acc[1] = 0;
 #pragma unroll 1
     for (uint32_t wb = w0; wb < w1; wb += 32u) {
         {
-            const uint32_t w = wb + lane, j = 3u * w + 1u + (w & 1u), d = 6u * j;
-            const uint32_t cd = kMagicBits * d;
-            jw[lane] = make_uint4(__float_as_uint(__frcp_rn(__uint2float_rn(d))), d,
-                                  0u - (cd + j) - 1u, 0u - (cd - j) - 1u);
+            const uint32_t w = wb + lane, j = 3u * w + 1u + (w & 1u);
+            jw[lane] = make_uint2(__float_as_uint(__frcp_rn(__uint2float_rn(3u * j))), j);
         }
         __syncwarp();
         const uint32_t n = min(32u, w1 - wb);
 #pragma unroll 4
         for (uint32_t i = 0; i < n; ++i) {
-            const uint4 c = jw[i];
+            const uint2 c = jw[i];
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const uint32_t T =
-                    __float_as_uint(__fmaf_rn(kf[e], __uint_as_float(c.x), kMagicF));
-                const uint32_t nr = T * c.y + nk[e];
-                const uint32_t x = add_sign(nr + c.w, add_sign(nr + c.z, b2[e]));
-                acc[e] += Ml[e][min(2u * T + x, hi[e])];
+                    __float_as_uint(__fmaf_rd(kf[e], __uint_as_float(c.x), kMagicF));
+                const uint32_t x = T + b2[e] + ((wheel_of_bits(T) * c.y + nk[e]) >> 31);
+                acc[e] += Ml[e][min(x, hi[e])];
             }
         }
         __syncwarp();
@@ -660,7 +700,7 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
     __shared__ int32_t s_delta[kGatherTile / kSegY];
     __shared__ uint64_t s_mbar;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
-    uint4 *jw = reinterpret_cast<uint4 *>(Mt + kGatherTile + 8) + warp * 32u;
+    uint2 *jw = reinterpret_cast<uint2 *>(Mt + kGatherTile + 8) + warp * 32u;
     uint32_t staged = 0xffffffffu, phase = 0;
     if (threadIdx.x == 0) {
         mbar_init(&s_mbar);
@@ -742,9 +782,9 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                 const uint32_t w0 = __reduce_min_sync(0xffffffffu, min(c0 ? wl[0] : 0xffffffffu,
                                                                        c1 ? wl[1] : 0xffffffffu));
                 const uint32_t w1 = __reduce_max_sync(0xffffffffu, max(wh[0], wh[1]));
-                // 64 (w1 - w0) terms at about 12 issue slots each against
-                // `sum` at about 21
-                if (40u * (w1 - w0) <= sum) {
+                // 64 (w1 - w0) terms at about 11 issue slots each against
+                // `sum` at about 18
+                if (40u * (w1 - w0) <= sum && w1 < kUniformW) {
                     uint32_t lo[2], b2[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -756,7 +796,7 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                                     : yc >= T.t0 + T.len ? lim + 1u
                                                          : phi6_u32((uint32_t)(yc - T.t0));
                         }
-                        b2[h] = 0u - 2u * kMagicBits - 2u - (uint32_t)(T.t0 / 3u) - lo[h];
+                        b2[h] = 0u - kMagicBits - 1u - (uint32_t)(T.t0 / 3u) - lo[h];
                     }
                     int acc[2];
                     tile_uniform(Mt, jw, k, b2, lo, lim, w0, w1, lane, acc);
@@ -1138,7 +1178,7 @@ int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s)
     if (a.nitems == 0)
         return 0;
     static std::atomic<uint64_t> attr_devs{0};
-    const int smem = kGatherTile * 2 + 16 + 16 * 32 * 16;
+    const int smem = kGatherTile * 2 + 16 + 16 * 32 * 8;
     const uint64_t dbit = device_bit();
     if (attrs_needed(attr_devs, dbit)) {
         cudaFuncSetAttribute(wheel_gather_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

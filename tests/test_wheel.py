@@ -27,9 +27,9 @@ def test_identities_over_integers_coprime_to_6():
         assert M[v] == M6[v] - M6[v // 2] - M6[v // 3] + M6[v // 6]
 
 
-def test_phi6_from_an_estimate_off_by_less_than_a_third():
-    """phi6(floor(k/y)) = 2T - 1 + [r >= -y] + [r >= y], r = k - 6yT, for every
-    integer T within 1/2 + 1/3 of k/(6y)."""
+def test_phi6_from_the_floor_of_an_estimate():
+    """phi6(floor(k/y)) = T + [k >= y Y(T)], Y(T) = (3T + 1) | 1, for the floor T
+    of any estimate of k/(3y) that errs by less than 1/3."""
     rng = random.Random(6)
     for _ in range(20000):
         y = rng.choice([1, 5, 7, rng.randrange(1, 50), rng.randrange(1, 10**8)])
@@ -37,10 +37,24 @@ def test_phi6_from_an_estimate_off_by_less_than_a_third():
                         rng.randrange(1, 10**15)])
         if k < 1:
             continue
-        # integers T with |6yT - k| < 6y (1/2 + 1/3) = 5y
-        for T in range((k - 5 * y) // (6 * y) + 1, (k + 5 * y - 1) // (6 * y) + 1):
-            r = k - 6 * y * T
-            assert 2 * T - 1 + (r >= -y) + (r >= y) == phi6(k // y), (k, y, T)
+        # floors of k/(3y) - 1/3 < v < k/(3y) + 1/3
+        for T in {(k - y) // (3 * y), k // (3 * y), -(-(k + y) // (3 * y)) - 1}:
+            if T >= 0:
+                assert T + (k >= y * ((3 * T + 1) | 1)) == phi6(k // y), (k, y, T)
+
+
+def test_float_estimate_of_the_dense_terms():
+    """The float modes' estimate, k (1/3y) with every operation in single
+    precision (the sum with 1.5 2^23 is exact before it is rounded down), errs by
+    less than 1/3 up to the bounds the kernels use."""
+    rng = random.Random(7)
+    f = np.float32
+    for bound, ylo, yhi in ((2_600_000 / 1.05, 5, 5_590_000), (1_800_000, 5_590_000, 350_000_000)):
+        for _ in range(20000):
+            y = rng.randrange(ylo, yhi)
+            k = rng.randrange(1, int(3 * y * bound) + 1)
+            kf, rf = float(f(k)), float(f(1.0) / f(3 * y))
+            assert abs(kf * rf - k / (3 * y)) < 1 / 3
 
 
 def test_index_forms():
