@@ -89,8 +89,9 @@ int mertens_set_allocator(mertens_alloc_fn alloc, mertens_free_fn release, void 
  *              entries (Sec. 2); X_i >= 2^32 is MERTENS_ENOTSUP.
  *   block_len  length of a sieve block in y (Sec. 3 processes the y-axis
  *              block by block); 0 = chosen by the library.  Any value >= 1
- *              is taken; whole runs over one-word targets round it up to a
- *              multiple of 6144 (results do not depend on it).
+ *              is taken; whole runs, whose M(y) takes a third of the memory
+ *              per y of a window plan's, make blocks of three times block_len,
+ *              up to a multiple of 6144 (results do not depend on it).
  *
  * Allocates all device memory of the plan on the current device (through the
  * hook above).  Small kernels that make the plan's tables run on a stream of

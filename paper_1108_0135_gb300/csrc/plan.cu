@@ -272,6 +272,7 @@ struct mertens_plan_s {
     bool wheel_long = false;     // 64-bit remainders for every gathered term
     WheelSieve ws;
     uint32_t *dJL = nullptr, *dJD = nullptr;
+    uint32_t *dplace = nullptr;  // entries' places (several targets)
     uint64_t *dA = nullptr, *dR6 = nullptr;
     WheelGroup *dwgroups = nullptr;
     uint32_t *dwpre = nullptr;
@@ -580,7 +581,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     double acc = 0, ksum = 0, terms = 0, pairs = 0;
     for (size_t i = 0; i < count; ++i) {
         const uint64_t X = (uint64_t)(n[i] / us[i]);
-        qs[i] = {(uint64_t)n[i], (uint64_t)(n[i] >> 64), X, E, G};
+        qs[i] = {(uint64_t)n[i], (uint64_t)(n[i] >> 64), X, E, G, 0};
         p->n.push_back(qs[i].n);
         p->n_hi.push_back(qs[i].n_hi);
         p->u.push_back(us[i]);
@@ -637,6 +638,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         return MERTENS_ENOTSUP;
     }
     p->nent = E;
+    // several one-word targets: entries in order of k (E count divisions on the
+    // device); otherwise target by target
+    const bool sorted = count > 1 && p->wide.empty() && (double)E * (double)count < 4.0e9;
+    for (size_t i = 0, l = 0; i < count; ++i)
+        if (!qs[i].n && !qs[i].n_hi)
+            qs[i].place = E - p->lookups.size() / 2 + l++;
     p->y_max = std::max<uint64_t>(p->y_max, 1);
     p->y_first = 1;
     p->y_last = p->y_max;
@@ -668,13 +675,22 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         delete p;
         return MERTENS_EINVAL;
     }
-    block_len = std::min(block_len, p->y_last);
+    // a block's M6 takes a third of the memory of block_len y in the full form, so
+    // three times as many y make a block (fewer launches: 48.9 -> 45.2 ms at
+    // n = 10^16 with 2^28-y blocks)
+    block_len = std::min(std::min<uint64_t>(3 * block_len, 3ull << 30), p->y_last);
     // a plan on a table sieves only the blocks that end above it
     p->sieves = !table || p->y_last > table->y_max;
     p->block_len = (block_len + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
+    if (table) {
+        // equal blocks up to the table's end, so that no block of its size is
+        // half in the table
+        const uint64_t m = (table->y_cov + p->block_len - 1) / p->block_len;
+        p->block_len = std::max(kWheelSegY, table->y_cov / m / kWheelSegY * kWheelSegY);
+    }
     p->nblocks = (p->y_last + p->block_len - 1) / p->block_len;
     p->wchunks = (p->ydense + kWheelSegY - 1) / kWheelSegY;
-    p->wgroups = (uint32_t)G;
+    p->wgroups = (uint32_t)((E + kWheelGroup - 1) / kWheelGroup);
     // parts of a dense chunk's list while the items would not fill the device
     p->wparts = (uint32_t)std::min(8.0, std::max(1.0, std::ceil(2400.0 / pairs)));
     p->wdense_items = (uint64_t)(pairs * p->wparts * 1.1) + 64;
@@ -692,112 +708,120 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             ys = strtoull(e, nullptr, 10);
         p->gather_smem_end = std::min(ys, p->y_max);
     }
-    // shorter tiles while the tile range would not give every SM its CTAs
-    uint64_t tile_y = kWheelTileY;
-    while (tile_y > kWheelSegY && (double)p->gather_smem_end / (double)tile_y *
-                                          std::ceil((double)E / 1024.0) < 608.0)
-        tile_y /= 2;
-    // Blocks above: tiles over the whole block for the entries with
-    // k >= kt_fac y0^2 / 32768 (about kt_fac terms or more per tile; a prefix of
-    // each target's entries) when they have at least kt_min terms per tile
-    // together; the global path takes the others.
+    // Above it, to the end of each block: tiles for the entries with
+    // k >= kt_fac y^2 / 32768 at its first such y (about kt_fac terms or more per
+    // tile there; a prefix of each target's entries) when they have at least
+    // kt_min terms per tile together; the global path takes the others.
     double kt_fac = 1.0, kt_min = 700.0;
     if (const char *e = getenv("MERTENS_TILE_KT"))
         kt_fac = atof(e);
     if (const char *e = getenv("MERTENS_TILE_MIN"))
         kt_min = atof(e);
+    // an item: about item_work terms and checks, at least 1024 entries; tiles are
+    // halved (to one segment at least) while 1024 entries hold more than item_max
+    // terms -- the low tiles hold most terms of all, and the device waited for
+    // their few items (0.79 ms at n = 10^13)
     const double item_work = std::min(2.0e6, std::max(4096.0, terms / (456.0 * 24.0)));
+    const double item_max = std::max(8192.0, terms / (456.0 * 4.0));
+    double yc_min = 1e300;  // about the least dense cut-off
+    for (size_t i = 0; i < count; ++i)
+        if (qs[i].n || qs[i].n_hi)
+            yc_min = std::min(yc_min, dc * std::sqrt((double)n[i] / (double)qs[i].X));
     // sum of k over the x in (a, b] of target i
     const auto k_between = [&](size_t i, double a, double b) {
         return (double)n[i] * std::log((b + 0.5) / (a + 0.5));
     };
     std::vector<uint2> tiles;  // {first y less one, low and high word}, {length, 0}
     std::vector<uint4> items;
+    struct Range {
+        uint64_t e0, e1;
+        double ksum;
+    };
+    Range range{0, 0, 0.0};
+    bool bound = count > 1 && !sorted;  // a cut-off can be bound by floor(k/jlo)
+    for (size_t i = 0; i < count; ++i)
+        if (qs[i].n || qs[i].n_hi)
+            bound = bound || 2.0 * (dc * std::sqrt((double)n[i]) + 2.0 * kChunk) >= (double)us[i];
+    // the places with k < kt (before them all others), their sum of k
+    const auto k_below = [&](double kt) {
+        range = {0, sorted ? E - p->lookups.size() / 2 : E, 0.0};
+        for (size_t i = 0; i < count; ++i) {
+            if (!qs[i].n && !qs[i].n_hi)
+                continue;
+            const double lo = std::min((double)qs[i].X, std::floor((double)n[i] / kt));
+            range.e0 += (uint64_t)lo;
+            range.ksum += k_between(i, lo, (double)qs[i].X);
+        }
+    };
+    // places whose cut-off lies below te: all where a cut-off can be bound by
+    // floor(k/jlo), else from the group of the first with dc sqrt(k) < te + 8
+    const auto below = [&](uint64_t te) {
+        const double t = ((double)te + 8.0) / dc;
+        k_below(bound ? 1e300 : t * t);
+        range.e0 = std::max<uint64_t>(range.e0, kWheelGroup) - kWheelGroup;
+        range.e0 -= range.e0 % kWheelGroup;
+    };
+    // the tile (t0, t0 + len] with the current range; false: too many terms in
+    // 1024 entries of it
+    const auto add_tile = [&](uint64_t t0, uint64_t len, bool may_split) {
+        if (range.e0 >= range.e1)
+            return true;
+        const double terms =
+            (1.0 / std::max((double)t0 + 1.0, std::min(yc_min, (double)(t0 + len))) -
+             1.0 / ((double)(t0 + len) + 1.0)) / 3.0 * range.ksum;
+        const double ne = (double)(range.e1 - range.e0), work = 2.0 * ne + terms;
+        if (may_split && terms > item_max * std::ceil(ne / 1024.0))
+            return false;
+        const uint64_t step = (uint64_t)std::max(
+            1024.0, std::ceil(ne / std::max(1.0, work / item_work) / 1024.0) * 1024.0);
+        for (uint64_t f = range.e0; f < range.e1; f += step)
+            items.push_back(make_uint4((uint32_t)(tiles.size() / 2), (uint32_t)f,
+                                       (uint32_t)std::min(f + step, range.e1), 0u));
+        tiles.push_back(make_uint2((uint32_t)t0, (uint32_t)(t0 >> 32)));
+        tiles.push_back(make_uint2((uint32_t)len, 0u));
+        return true;
+    };
     for (uint64_t b = 0; b < p->nblocks; ++b) {
-        const uint64_t y0 = b * p->block_len, blen = wheel_block_len(p, b);
+        const uint64_t y0 = b * p->block_len, yend = y0 + wheel_block_len(p, b);
         p->gblk.push_back((uint32_t)items.size());
-        uint64_t end = y0;  // y in (y0, end] goes to tiles
+        uint64_t end = y0;  // y in (y0, end] goes to tiles of all entries
         if (p->gather_smem_end > y0)
-            end = std::min(y0 + blen,
-                           (p->gather_smem_end + kWheelSegY - 1) / kWheelSegY * kWheelSegY);
+            end = std::min(yend, (p->gather_smem_end + kWheelSegY - 1) / kWheelSegY * kWheelSegY);
         p->gend.push_back(end);
-        uint64_t kt = UINT64_MAX;  // entries with k >= kt take this block's tiles
-        std::vector<std::pair<uint64_t, uint64_t>> ranges, all;
-        std::vector<double> ks, kall;  // sums of k of the ranges
-        if (y0 >= p->gather_smem_end && kt_fac > 0) {
-            const double y1 = (double)y0 + 1.0, k0 = kt_fac * y1 * y1 / kGatherTile;
-            double sum = 0;
+        uint64_t len = 0;
+        for (uint64_t t0 = y0; t0 < end; t0 += len) {
+            len = std::min(kWheelTileY, end - t0);
+            for (;;) {
+                below(t0 + len);
+                const uint64_t half = (len / 2 + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
+                if (add_tile(t0, len, half < len))
+                    break;
+                len = half;
+            }
+        }
+        uint64_t kt = UINT64_MAX;  // entries with k >= kt take tiles up to yend
+        if (end < yend && kt_fac > 0) {
+            const double y1 = (double)end + 1.0, k0 = kt_fac * y1 * y1 / kGatherTile;
             const uint64_t k0i = (uint64_t)std::ceil(std::min(k0, 9.2e18));
-            for (size_t i = 0; i < count; ++i) {
+            // the places with k >= k0i (unsorted targets: none)
+            Range r{0, 0, 0.0};
+            for (size_t i = 0; i < count && (count == 1 || sorted); ++i) {
                 if (!qs[i].n && !qs[i].n_hi)
                     continue;
                 const uint64_t xt = (uint64_t)std::min<u128>(qs[i].X, n[i] / k0i);
-                if (xt == 0)
-                    continue;
-                all.push_back({qs[i].off, qs[i].off + xt});
-                kall.push_back(k_between(i, 0.0, (double)xt));
-                sum += kall.back();
+                r.e1 += xt;
+                r.ksum += xt ? k_between(i, 0.0, (double)xt) : 0.0;
             }
-            if (sum * kGatherTile / (y1 * y1) >= kt_min) {
+            if (r.ksum * kGatherTile / (y1 * y1) >= kt_min) {
                 kt = k0i;
-                end = y0 + blen;
+                range = r;
+                for (uint64_t t0 = end; t0 < yend; t0 += len) {
+                    len = std::min(kWheelTileY, yend - t0);
+                    add_tile(t0, len, false);
+                }
             }
         }
         p->ktile.push_back(kt);
-        for (uint64_t t0 = y0; t0 < end; t0 += tile_y) {
-            const uint64_t len = std::min(tile_y, end - t0);
-            if (kt == UINT64_MAX) {
-                // entries whose cut-off lies below the tile's end: all where a
-                // cut-off can be bound by floor(k/jlo), else those of the groups
-                // with dc sqrt(k of the group's last) < t0 + len + 8
-                ranges.clear();
-                ks.clear();
-                for (size_t i = 0; i < count; ++i) {
-                    const WheelQuery &Q = qs[i];
-                    if (!Q.n && !Q.n_hi)
-                        continue;
-                    const double nd = (double)n[i], te = (double)(t0 + len) + 8.0;
-                    uint64_t lo = 0;
-                    if (2.0 * (dc * std::sqrt(nd) + 2.0 * kChunk) < (double)us[i])
-                        lo = (uint64_t)std::max(0.0, std::min((double)Q.X + kWheelGroup,
-                                                              dc * dc * nd / (te * te)) -
-                                                         (double)kWheelGroup) /
-                             kWheelGroup * kWheelGroup;
-                    if (lo >= Q.X)
-                        continue;
-                    const double kv = k_between(i, (double)lo, (double)Q.X);
-                    if (!ranges.empty() && Q.off + lo <= ranges.back().second + 4096) {
-                        ranges.back().second = Q.off + Q.X;
-                        ks.back() += kv;
-                    } else {
-                        ranges.push_back({Q.off + lo, Q.off + Q.X});
-                        ks.push_back(kv);
-                    }
-                }
-            }
-            const auto &rs = kt == UINT64_MAX ? ranges : all;
-            const auto &kv = kt == UINT64_MAX ? ks : kall;
-            const double per_k = (double)len / 3.0 / ((double)(t0 + 1) * (double)(t0 + 1));
-            const uint32_t ti = (uint32_t)(tiles.size() / 2);
-            bool any = false;
-            for (size_t r = 0; r < rs.size(); ++r) {
-                // items of equal numbers of entries, in steps of 1024, with about
-                // item_work terms and checks on the average
-                const double ne = (double)(rs[r].second - rs[r].first);
-                const double work = 2.0 * ne + per_k * kv[r];
-                const uint64_t step = (uint64_t)std::max(
-                    1024.0, std::ceil(ne / std::max(1.0, work / item_work) / 1024.0) * 1024.0);
-                for (uint64_t f = rs[r].first; f < rs[r].second; f += step) {
-                    items.push_back(make_uint4(ti, (uint32_t)f,
-                                               (uint32_t)std::min(f + step, rs[r].second), 0u));
-                    any = true;
-                }
-            }
-            if (any) {
-                tiles.push_back(make_uint2((uint32_t)t0, (uint32_t)(t0 >> 32)));
-                tiles.push_back(make_uint2((uint32_t)len, 0u));
-            }
-        }
     }
     p->gblk.push_back((uint32_t)items.size());
     // chunk records of a block's global gather: an entry with cnt > 16 terms
@@ -848,6 +872,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         take(p->dwide, p->wide.size() * sizeof(WideEntry));
         take(p->dlook, p->lookups.size() * 8);
         up_bytes = off - up0;
+        take(ea.P, sorted ? E * 4 : 0);
         take(p->dK, E * 8);
         take(p->dYCE, E * 8);
         take(p->dJL, E * 4);
@@ -862,7 +887,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             take(p->dsegoff[0], wlen / kSegY * 8);
         }
         take(p->dcarry, (p->nblocks + 1) * 8);
-        take(p->dwgroups, (size_t)G * sizeof(WheelGroup));
+        take(p->dwgroups, (size_t)p->wgroups * sizeof(WheelGroup));
         take(p->dwpre, ((size_t)nblk + 1) * 4);
         take(p->dwtiles, (size_t)ntiles * sizeof(WheelGatherTile));
         if (!table) {
@@ -905,7 +930,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     p->h2d_bytes = up_bytes + np * 4;
     ea.qs = d_qs;
     ea.nq = (uint32_t)count;
+    ea.nent = (uint32_t)E;
+    ea.qgroups = (uint32_t)G;
     ea.ngroups = p->wgroups;
+    if (!sorted)
+        ea.P = nullptr;
+    p->dplace = ea.P;
     ea.dc = dc;
     ea.wide_from = (uint64_t)wide_from;
     ea.K = p->dK;
@@ -1960,7 +1990,8 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
         for (uint64_t X : p->X)
             mx = std::max(mx, X);
         ev_begin(p, kPhResolve, s, &pe);
-        r = wheel_resolve_enqueue(p->dqs, (uint32_t)p->nq, mx, p->dS, p->dA, p->dR6, p->dR, s);
+        r = wheel_resolve_enqueue(p->dqs, (uint32_t)p->nq, mx, p->dplace, p->dS, p->dA, p->dR6,
+                                  p->dR, s);
         if (r >= 0 && !p->lookups.empty()) {
             const int r2 = wheel_lookup_enqueue(p->dlook, (uint32_t)(p->lookups.size() / 2),
                                                 tab->Mloc, tab->segoff, p->dR, s);

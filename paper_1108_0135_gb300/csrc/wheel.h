@@ -106,14 +106,18 @@ __host__ __device__ constexpr uint32_t wheel_block_first(uint32_t b)
 }
 constexpr uint32_t kWheelItem = 256;       // wheel indices of a chunk of the global gather
 
-// A target; n = 0: its value is read from a table (one entry, no terms).
+// A target; n = 0: its value is read from a table (one entry, no terms).  Its
+// entries x = 1 .. X are numbered off + x - 1 in the results; the update works on
+// places: the same numbers for one target, all targets' entries in decreasing
+// order of k for several (so that 64 consecutive places have close k).
 struct WheelQuery {
     uint64_t n, n_hi, X;
-    uint64_t off, goff;     // first entry, first group
+    uint64_t off, goff;     // first entry, first group of 64 entries
+    uint64_t place;         // n = 0: the entry's place
 };
 
 struct WheelGroup {
-    uint32_t first, count;  // entries
+    uint32_t first, count;  // places
     uint64_t yc;            // dense cut-off (a multiple of 6)
     uint64_t kmax;          // largest k of the group
 };
@@ -135,9 +139,12 @@ struct WheelTotals {
 struct WheelEntryArgs {
     const WheelQuery *qs;
     uint32_t nq;
-    uint32_t ngroups;
+    uint32_t nent;
+    uint32_t qgroups;       // groups of 64 entries, target by target
+    uint32_t ngroups;       // groups of 64 places
     double dc;              // dense cut-off factor
     uint64_t wide_from;     // entries with k at or above: two-word ones (k = 0 here)
+    uint32_t *P;            // place of every entry (null: the entry's number)
     uint64_t *K, *YC;
     uint32_t *JL, *JD;
     WheelGroup *groups;
@@ -234,8 +241,9 @@ int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t 
 
 struct QueryDev;
 // R6[x] = M6(floor(n/x)) from the sums S, then M in R (A: the parts of M whose
-// M6 argument lies below the array).
-int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint64_t *S,
-                          const uint64_t *A, uint64_t *R6, uint64_t *R, cudaStream_t s);
+// M6 argument lies below the array; S and A by place).
+int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint32_t *P,
+                          const uint64_t *S, const uint64_t *A, uint64_t *R6, uint64_t *R,
+                          cudaStream_t s);
 
 }  // namespace mert

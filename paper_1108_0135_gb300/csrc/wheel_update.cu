@@ -57,20 +57,16 @@ __device__ __forceinline__ uint64_t warp_max_u64(uint64_t v)
     return v;
 }
 
-// k = floor(n/x), the first j of its gathered terms and the group's dense
-// cut-off: dc sqrt(mean k of the group), at most floor(k/jlo) of every entry
-// (beyond it no term is left), down to a multiple of 6.  Any cut-off gives the
-// same sums; a dense y costs the whole group one term per entry, a gathered j
-// only its own, so the mean of k balances them (with the first entry's k, the
-// first group had four times the dense terms: 14% of all at n = 10^13).  jd stays
-// below 2^32.  The totals' gather_j counts the gathered terms of the full sums'
-// cut-offs (dc sqrt(k of the first one-word entry), up to a multiple of 4096 less
-// one, within [floor(sqrt(k)), floor(k/jlo) - 1]).
+// Every entry's k = floor(n/x) and first gathered j, at its place, and the totals
+// of the full sums (a warp per 64 entries of a target): gather_j counts the
+// gathered terms of the full sums' dense cut-offs, dc sqrt(k of the first
+// one-word entry), up to a multiple of 4096 less one, within [floor(sqrt(k)),
+// floor(k/jlo) - 1].
 __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
 {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    if (g >= a.ngroups)
+    if (g >= a.qgroups)
         return;
     uint32_t lo_q = 0, hi_q = a.nq;  // the last target with goff <= g
     while (hi_q - lo_q > 1) {
@@ -83,15 +79,14 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
     const WheelQuery Q = a.qs[lo_q];
     const uint64_t x0 = (g - Q.goff) * kWheelGroup + 1;
     const uint32_t cnt = (uint32_t)min((uint64_t)kWheelGroup, Q.X - x0 + 1);
-    uint64_t k[2], sq[2], vh[2], jlo[2], cap[2];
+    uint64_t k[2], sq[2], vh[2], jlo[2];
     uint64_t lo = 0, nhi = 0, kf = 0;  // max of s, max of ~vh (= ~min), largest k
-    float ksum = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
         k[h] = 0;
         if (i < cnt) {
-            const uint64_t x = x0 + i;
+            const uint64_t x = x0 + i, e = Q.off + x - 1;
             if (Q.n_hi) {
                 const unsigned __int128 kk = (((unsigned __int128)Q.n_hi << 64) | Q.n) / x;
                 k[h] = kk < a.wide_from ? (uint64_t)kk : 0;
@@ -100,75 +95,116 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
                 if (k[h] >= a.wide_from)
                     k[h] = 0;
             }
+            jlo[h] = k[h] ? Q.X / x + 1 : 1;
+            uint64_t place = e;
+            if (a.P) {
+                // entries before this one in decreasing order of k (ties: by
+                // target): floor(n'/x') >= k for the x' <= floor(n'/k)
+                place = Q.n ? x - 1 : Q.place;
+                for (uint32_t q = 0; q < a.nq && Q.n; ++q)
+                    if (q != lo_q)
+                        place += min(a.qs[q].X, a.qs[q].n / (k[h] + (q < lo_q ? 0u : 1u)));
+                a.P[e] = (uint32_t)place;
+            }
+            a.K[place] = k[h];
+            a.JL[place] = (uint32_t)jlo[h];
             if (k[h]) {
                 kf = max(kf, k[h]);
-                ksum += (float)k[h];
                 sq[h] = isqrt_dev(k[h]);
-                jlo[h] = Q.X / x + 1;
-                cap[h] = k[h] / jlo[h];
-                vh[h] = jlo[h] <= k[h] / (sq[h] + 1) ? cap[h] - 1 : sq[h];
+                vh[h] = jlo[h] <= k[h] / (sq[h] + 1) ? k[h] / jlo[h] - 1 : sq[h];
                 lo = max(lo, sq[h]);
                 nhi = max(nhi, ~vh[h]);
-            } else {
-                const uint64_t e = Q.off + x - 1;
-                a.K[e] = 0;
-                a.YC[e] = 0;
-                a.JL[e] = 1;
-                a.JD[e] = 0;
             }
         }
     }
     kf = warp_max_u64(kf);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1)
-        ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
-    const uint64_t mean = max((uint64_t)(a.dc * sqrt((double)ksum / cnt)), kf / (uint64_t)4000000000u);
     lo = warp_max_u64(lo);
     const uint64_t hi = ~warp_max_u64(nhi);
     uint64_t target = (uint64_t)(a.dc * sqrt((double)kf));
     target = (target + kChunk) / kChunk * kChunk - 1;
-    uint64_t nyc = 0, yce[2];  // max of ~cut-off
+    uint64_t direct = 0, gathered = 0, gather_j = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h)
         if (k[h]) {
-            yce[h] = lo <= hi ? min(max(target, lo), hi) : min(max(target, sq[h]), vh[h]);
-            nyc = max(nyc, ~min(mean, cap[h]));
-        }
-    uint64_t yc = kf ? ~warp_max_u64(nyc) : 0;
-    yc -= yc % 6;
-    uint64_t direct = 0, gathered = 0, gather_j = 0, exec = 0;
-#pragma unroll
-    for (int h = 0; h < 2; ++h)
-        if (k[h]) {
-            const uint64_t e = Q.off + x0 - 1 + lane + 32u * (uint32_t)h;
-            const uint64_t jd = max(k[h] / (yc + 1), jlo[h] - 1);
-            a.K[e] = k[h];
-            a.YC[e] = yc;
-            a.JL[e] = (uint32_t)jlo[h];
-            a.JD[e] = (uint32_t)jd;
+            const uint64_t yce =
+                lo <= hi ? min(max(target, lo), hi) : min(max(target, sq[h]), vh[h]);
             direct += sq[h];
-            const uint64_t jhi = k[h] / (sq[h] + 1), jc = k[h] / (yce[h] + 1);
+            const uint64_t jhi = k[h] / (sq[h] + 1), jc = k[h] / (yce + 1);
             gathered += jhi >= jlo[h] ? jhi - jlo[h] + 1 : 0;
             gather_j += jc >= jlo[h] ? jc - jlo[h] + 1 : 0;
-            exec += phi6(jd) - phi6(jlo[h] - 1);
         }
     direct = warp_sum_u64(direct);
     gathered = warp_sum_u64(gathered);
     gather_j = warp_sum_u64(gather_j);
-    exec = warp_sum_u64(exec);
     if (lane == 0) {
-        WheelGroup G;
-        G.first = (uint32_t)(Q.off + x0 - 1);
-        G.count = cnt;
-        G.yc = yc;
-        G.kmax = kf;
-        a.groups[g] = G;
         WheelTotals *t = a.totals + lo_q;
         atomicAdd(&t->direct, direct);
         atomicAdd(&t->gathered, gathered);
         atomicAdd(&t->gather_j, gather_j);
-        atomicAdd(&t->exec, exec);
-        atomicAdd(&t->dense_y, yc * cnt);
+    }
+}
+
+// A warp per group of 64 places: its dense cut-off dc sqrt(mean k of its one-word
+// entries), at most floor(k/jlo) of every entry (beyond it no term is left), down
+// to a multiple of 6, and every entry's last gathered j.  Any cut-off gives the
+// same sums; a dense y costs the whole group one term per entry, a gathered j only
+// its own, so the mean of k balances them (with the first entry's k, the first
+// group had four times the dense terms: 14% of all at n = 10^13).  jd stays below
+// 2^32.
+__global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
+{
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (g >= a.ngroups)
+        return;
+    const uint32_t e0 = g * kWheelGroup, cnt = min(kWheelGroup, a.nent - e0);
+    uint64_t k[2], jlo[2], kf = 0, ncap = 0;  // largest k, max of ~floor(k/jlo)
+    float ksum = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t i = lane + 32u * (uint32_t)h;
+        k[h] = i < cnt ? a.K[e0 + i] : 0;
+        if (k[h]) {
+            jlo[h] = a.JL[e0 + i];
+            kf = max(kf, k[h]);
+            ksum += (float)k[h];
+            ncap = max(ncap, ~(k[h] / jlo[h]));
+        }
+    }
+    kf = warp_max_u64(kf);
+    ncap = warp_max_u64(ncap);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
+    const uint32_t one = __reduce_add_sync(0xffffffffu, (k[0] ? 1u : 0u) + (k[1] ? 1u : 0u));
+    uint64_t yc = 0;
+    if (kf) {
+        yc = max((uint64_t)(a.dc * sqrt((double)ksum / one)), kf / (uint64_t)4000000000u);
+        yc = min(yc, ~ncap);
+        yc -= yc % 6;
+    }
+    uint64_t exec = 0;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t i = lane + 32u * (uint32_t)h;
+        if (i < cnt) {
+            const uint64_t jd = k[h] ? max(k[h] / (yc + 1), jlo[h] - 1) : 0;
+            a.YC[e0 + i] = k[h] ? yc : 0;
+            a.JD[e0 + i] = (uint32_t)jd;
+            if (k[h])
+                exec += phi6(jd) - phi6(jlo[h] - 1);
+        }
+    }
+    exec = warp_sum_u64(exec);
+    if (lane == 0) {
+        WheelGroup G;
+        G.first = e0;
+        G.count = cnt;
+        G.yc = yc;
+        G.kmax = kf;
+        a.groups[g] = G;
+        atomicAdd(&a.totals->exec, exec);
+        atomicAdd(&a.totals->dense_y, yc * one);
     }
 }
 
@@ -215,7 +251,8 @@ __global__ void wheel_tiles_kernel(WheelEntryArgs a)
 
 int wheel_entries_enqueue(const WheelEntryArgs &a, cudaStream_t s)
 {
-    wheel_entries_kernel<<<(a.ngroups + 3) / 4, 128, 0, s>>>(a);
+    wheel_entries_kernel<<<(a.qgroups + 3) / 4, 128, 0, s>>>(a);
+    wheel_groups_kernel<<<(a.ngroups + 3) / 4, 128, 0, s>>>(a);
     wheel_dense_items_kernel<<<1, 1024, 0, s>>>(a);
     if (a.ntiles)
         wheel_tiles_kernel<<<(a.ntiles + 127) / 128, 128, 0, s>>>(a);
@@ -686,16 +723,73 @@ __device__ __forceinline__ void tile_uniform(const int16_t *Mt, uint2 *jw, const
     }
 }
 
-// A work item is one tile and a range of entries of one target.  Warps take 64
+// The ranges of wheel indices of the j of 64 entries eb .., two per lane, in a tile.
+struct TileRanges {
+    uint64_t k[2];
+    uint32_t wl[2], wh[2];
+    bool big, bound;  // some j beyond 32-bit remainders; some range starts at jlo
+};
+
+__device__ __forceinline__ TileRanges tile_ranges(const WheelGatherArgs &a,
+                                                  const WheelGatherTile &T, uint32_t eb,
+                                                  uint32_t e1, uint32_t lane)
+{
+    TileRanges r;
+    r.big = a.all_long;
+    r.bound = false;
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t e = eb + 32u * (uint32_t)h + lane;
+        r.k[h] = 0;
+        r.wl[h] = r.wh[h] = 0;
+        if (e < e1) {
+            r.k[h] = a.K[e];
+            const uint64_t jd = a.JD[e], jlo = a.JL[e];
+            const uint64_t q1 = div_magic(r.k[h] << 1, T.m1, T.l1);  // floor(k/(t0+1))
+            const uint64_t q2 = div_magic(r.k[h] << 1, T.m2, T.l2);  // floor(k/(t0+len+1))
+            const uint64_t t = jd < q1 ? jd : q1, b = q2 + 1u > jlo ? q2 + 1u : jlo;
+            r.bound |= b != q2 + 1u;
+            if (r.k[h] && t >= b) {
+                r.big |= t >= kGatherJ32;
+                r.wl[h] = phi6_u32((uint32_t)b - 1u);
+                r.wh[h] = phi6_u32((uint32_t)t);
+            }
+        }
+    }
+    return r;
+}
+
+// Sum of one entry's terms [wl, wh) by a warp, added to S[e].
+__device__ __forceinline__ void tile_entry(const WheelGatherArgs &a, const int16_t *Mt,
+                                           const WheelGatherTile &T, uint32_t lim, int64_t base,
+                                           bool big, uint32_t e, uint64_t k, uint32_t wl,
+                                           uint32_t wh, uint32_t lane)
+{
+    const int acc = big ? tile_warp<true>(Mt, k, T.t0, lim, wl, wh, lane)
+                        : tile_warp<false>(Mt, k, T.t0, lim, wl, wh, lane);
+    const int tot = __reduce_add_sync(0xffffffffu, acc);
+    if (lane == 0)
+        atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e),
+                  (unsigned long long)((int64_t)tot + (int64_t)(wh - wl) * base));
+}
+
+// A work item is one tile and a range of places.  Warps take 64
 // entries at a time, two per lane, and find the ranges of wheel indices of
-// their j.  Low tiles where these ranges nearly coincide take tile_uniform;
-// otherwise, 32 entries at a time, when the counts are close (or all small)
+// their j.  Low tiles where these ranges nearly coincide take tile_uniform.
+// The others, 32 entries at a time: when the counts are close (or all small)
 // every lane sums its own entry, else entries with many terms take the whole
-// warp in turn.
+// warp in turn; with many terms in all, at the end of the item, where all warps
+// share them (the first 32 entries of a target hold a third of a tile's terms;
+// on one warp, the other fifteen waited for it).
+constexpr uint32_t kSharedMax = 128;         // sets of 32 left to the end of an item
+constexpr uint32_t kSharedTerms = 16384;     // a set's terms from which it is
+constexpr uint32_t kSharedSlice = 8192;      // an entry's terms from which warps split it
+
 __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
 {
     extern __shared__ __align__(16) int16_t Mt[];  // kGatherTile, a zero, j constants
-    __shared__ uint32_t s_item;
+    __shared__ uint32_t s_item, s_nshared, s_next;
+    __shared__ uint32_t s_shared[kSharedMax];
     __shared__ int64_t s_base;
     __shared__ int32_t s_delta[kGatherTile / kSegY];
     __shared__ uint64_t s_mbar;
@@ -707,8 +801,11 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
         fence_proxy_async_smem();
     }
     for (;;) {
-        if (threadIdx.x == 0)
+        if (threadIdx.x == 0) {
             s_item = atomicAdd(a.counter, 1u);
+            s_nshared = 0;
+            s_next = 0;
+        }
         __syncthreads();
         if (s_item >= a.nitems)
             break;
@@ -751,37 +848,22 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
         const int64_t base = s_base;
         const uint32_t lim = T.len / 3u - 1u;
         const bool low = T.t0 + T.len <= kUniformY;
-        for (uint32_t eb = I.y + warp * 64u; eb < I.z; eb += nwarp * 64u) {
-            uint64_t k[2];
-            uint32_t wl[2], wh[2];
-            bool big = a.all_long, bound = false;  // j beyond 32-bit remainders; jlo binds
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const uint32_t e = eb + 32u * (uint32_t)h + lane;
-                k[h] = 0;
-                wl[h] = wh[h] = 0;
-                if (e < I.z) {
-                    k[h] = a.K[e];
-                    const uint64_t jd = a.JD[e], jlo = a.JL[e];
-                    const uint64_t q1 = div_magic(k[h] << 1, T.m1, T.l1);  // floor(k/(t0+1))
-                    const uint64_t q2 = div_magic(k[h] << 1, T.m2, T.l2);  // floor(k/(t0+len+1))
-                    const uint64_t t = jd < q1 ? jd : q1, b = q2 + 1u > jlo ? q2 + 1u : jlo;
-                    bound |= b != q2 + 1u;
-                    if (k[h] && t >= b) {
-                        big |= t >= kGatherJ32;
-                        wl[h] = phi6_u32((uint32_t)b - 1u);
-                        wh[h] = phi6_u32((uint32_t)t);
-                    }
-                }
-            }
-            const uint32_t c0 = wh[0] - wl[0], c1 = wh[1] - wl[1];
+        for (;;) {
+            uint32_t eb = 0;  // the next 64 entries
+            if (lane == 0)
+                eb = I.y + 64u * atomicAdd(&s_next, 1u);
+            eb = __shfl_sync(0xffffffffu, eb, 0);
+            if (eb >= I.z)
+                break;
+            const TileRanges r = tile_ranges(a, T, eb, I.z, lane);
+            const uint32_t c0 = r.wh[0] - r.wl[0], c1 = r.wh[1] - r.wl[1];
             const uint32_t sum = __reduce_add_sync(0xffffffffu, c0 + c1);
             if (sum == 0)
                 continue;
-            if (low && !__any_sync(0xffffffffu, bound || big)) {
-                const uint32_t w0 = __reduce_min_sync(0xffffffffu, min(c0 ? wl[0] : 0xffffffffu,
-                                                                       c1 ? wl[1] : 0xffffffffu));
-                const uint32_t w1 = __reduce_max_sync(0xffffffffu, max(wh[0], wh[1]));
+            if (low && !__any_sync(0xffffffffu, r.bound || r.big)) {
+                const uint32_t w0 = __reduce_min_sync(0xffffffffu, min(c0 ? r.wl[0] : 0xffffffffu,
+                                                                       c1 ? r.wl[1] : 0xffffffffu));
+                const uint32_t w1 = __reduce_max_sync(0xffffffffu, max(r.wh[0], r.wh[1]));
                 // 64 (w1 - w0) terms at about 11 issue slots each against
                 // `sum` at about 18
                 if (40u * (w1 - w0) <= sum && w1 < kUniformW) {
@@ -790,7 +872,7 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                     for (int h = 0; h < 2; ++h) {
                         const uint32_t e = eb + 32u * (uint32_t)h + lane;
                         lo[h] = lim + 1u;  // no entry: nothing counts
-                        if (k[h]) {
+                        if (r.k[h]) {
                             const uint64_t yc = a.YC[e];
                             lo[h] = yc <= T.t0 ? 0u
                                     : yc >= T.t0 + T.len ? lim + 1u
@@ -799,7 +881,7 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                         b2[h] = 0u - kMagicBits - 1u - (uint32_t)(T.t0 / 3u) - lo[h];
                     }
                     int acc[2];
-                    tile_uniform(Mt, jw, k, b2, lo, lim, w0, w1, lane, acc);
+                    tile_uniform(Mt, jw, r.k, b2, lo, lim, w0, w1, lane, acc);
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         const uint32_t cnt = h ? c1 : c0;
@@ -811,17 +893,29 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                     continue;
                 }
             }
-            big = __any_sync(0xffffffffu, big);
+            const bool big = __any_sync(0xffffffffu, r.big);
 #pragma unroll 1
             for (uint32_t h = 0; h < 2u; ++h) {
-                const uint32_t cnt = h ? c1 : c0, wlh = h ? wl[1] : wl[0], whh = h ? wh[1] : wh[0];
-                const uint64_t kh = h ? k[1] : k[0];
+                const uint32_t cnt = h ? c1 : c0, wlh = h ? r.wl[1] : r.wl[0],
+                               whh = h ? r.wh[1] : r.wh[0];
+                const uint64_t kh = h ? r.k[1] : r.k[0];
                 const uint32_t e0 = eb + 32u * h;
                 const uint32_t mx = __reduce_max_sync(0xffffffffu, cnt);
                 if (mx == 0)
                     continue;
-                const bool lanes = mx <= kWheelLaneTerms ||
-                                   16u * mx <= __reduce_add_sync(0xffffffffu, cnt);
+                const uint32_t hsum = __reduce_add_sync(0xffffffffu, cnt);
+                const bool lanes = mx <= kWheelLaneTerms || 16u * mx <= hsum;
+                if (!lanes && hsum >= kSharedTerms) {
+                    uint32_t slot = 0;
+                    if (lane == 0)
+                        slot = atomicAdd(&s_nshared, 1u);
+                    slot = __shfl_sync(0xffffffffu, slot, 0);
+                    if (slot < kSharedMax) {
+                        if (lane == 0)
+                            s_shared[slot] = e0;
+                        continue;
+                    }
+                }
                 if (cnt && (lanes || cnt <= kWheelLaneTerms)) {
                     const int acc = big ? tile_lane<true>(Mt, kh, T.t0, lim, wlh, whh)
                                         : tile_lane<false>(Mt, kh, T.t0, lim, wlh, whh);
@@ -835,13 +929,37 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                     const uint32_t wls = __shfl_sync(0xffffffffu, wlh, src);
                     const uint32_t whs = __shfl_sync(0xffffffffu, whh, src);
                     const uint64_t ks = __shfl_sync(0xffffffffu, kh, src);
-                    const int acc = big ? tile_warp<true>(Mt, ks, T.t0, lim, wls, whs, lane)
-                                        : tile_warp<false>(Mt, ks, T.t0, lim, wls, whs, lane);
-                    const int tot = __reduce_add_sync(0xffffffffu, acc);
-                    if (lane == 0)
-                        atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e0 + src),
-                                  (unsigned long long)((int64_t)tot + (int64_t)(whs - wls) * base));
+                    tile_entry(a, Mt, T, lim, base, big, e0 + src, ks, wls, whs, lane);
                 }
+            }
+        }
+        __syncthreads();
+        // the groups left: every warp finds the ranges; entries in turn to the
+        // warps, the largest split over all of them
+        const uint32_t nsh = min(s_nshared, kSharedMax);
+        uint32_t turn = 0;
+        for (uint32_t q = 0; q < nsh; ++q) {
+            const uint32_t eb = s_shared[q];
+            const TileRanges r = tile_ranges(a, T, eb, min(I.z, eb + 32u), lane);
+            const bool big = __any_sync(0xffffffffu, r.big);
+#pragma unroll 1
+            for (uint32_t i = 0; i < 32u; ++i) {
+                uint32_t wl = __shfl_sync(0xffffffffu, r.wl[0], i);
+                uint32_t wh = __shfl_sync(0xffffffffu, r.wh[0], i);
+                const uint32_t cnt = wh - wl;
+                if (cnt == 0)
+                    continue;
+                if (cnt >= kSharedSlice) {
+                    const uint32_t part = ((cnt + nwarp - 1) / nwarp + 31u) & ~31u;
+                    wl = min(wl + warp * part, wh);
+                    wh = min(wl + part, wh);
+                    if (wl >= wh)
+                        continue;
+                } else if (turn++ % nwarp != warp) {
+                    continue;
+                }
+                const uint64_t k = __shfl_sync(0xffffffffu, r.k[0], i);
+                tile_entry(a, Mt, T, lim, base, big, eb + i, k, wl, wh, lane);
             }
         }
         __syncthreads();
@@ -1068,42 +1186,69 @@ __global__ void wheel_carry_at_kernel(const int16_t *__restrict__ Mloc,
 // then M[x] = R6[x] - V(2x) - V(3x) + V(6x), V(z) = R6[z] within the array (the
 // values beyond it are in A).  The smallest such j is 5, so the entries of
 // (X/5^(l+1), X/5^l] only read entries above X/5^l: level by level, every entry
-// of a level in parallel, a warp per entry where an entry has many terms.
+// of a level in parallel: a thread per entry, a warp from X/x = 64 on, a CTA from
+// 1024 on (a warp on the 83 000 terms of x = 1 took 243 of 370 us at X = 250 000).
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ void resolve_level(const QueryDev &Q, const uint64_t *S, uint64_t *R6,
+__device__ __forceinline__ uint64_t at_place(const uint64_t *v, const uint32_t *P, uint64_t e)
+{
+    return v[P ? P[e] : e];
+}
+
+__device__ __forceinline__ void resolve_level(const QueryDev &Q, const uint32_t *P,
+                                              const uint64_t *S, uint64_t *R6,
                                               uint64_t xlo, uint64_t xhi, uint64_t tid,
-                                              uint64_t nthreads)
+                                              uint64_t nthreads, uint64_t *sh)
 {
     const uint64_t X = Q.X, base = Q.off;
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     if (X / xhi < 64) {
         for (uint64_t x = xlo + tid; x <= xhi; x += nthreads) {
             const uint32_t nw = (uint32_t)phi6(X / x);
             uint64_t acc = 0;
+#pragma unroll 4
             for (uint32_t w = 1; w < nw; ++w)
                 acc += R6[base + x * wheel_y(w) - 1];
-            R6[base + x - 1] = 1ull - S[base + x - 1] - acc;
+            R6[base + x - 1] = 1ull - at_place(S, P, base + x - 1) - acc;
         }
-    } else {
-        const uint32_t lane = (uint32_t)tid & 31u;
+    } else if (X / xhi < 1024) {
         for (uint64_t x = xlo + (tid >> 5); x <= xhi; x += nthreads >> 5) {
             const uint32_t nw = (uint32_t)phi6(X / x);
             uint64_t acc = 0;
+#pragma unroll 4
             for (uint32_t w = 1 + lane; w < nw; w += 32)
                 acc += R6[base + x * wheel_y(w) - 1];
             acc = warp_sum_u64(acc);
             if (lane == 0)
-                R6[base + x - 1] = 1ull - S[base + x - 1] - acc;
+                R6[base + x - 1] = 1ull - at_place(S, P, base + x - 1) - acc;
+        }
+    } else {
+        for (uint64_t x = xlo + tid / blockDim.x; x <= xhi; x += nthreads / blockDim.x) {
+            const uint32_t nw = (uint32_t)phi6(X / x);
+            uint64_t acc = 0;
+#pragma unroll 4
+            for (uint32_t w = 1 + threadIdx.x; w < nw; w += blockDim.x)
+                acc += R6[base + x * wheel_y(w) - 1];
+            acc = warp_sum_u64(acc);
+            if (lane == 0)
+                sh[warp] = acc;
+            __syncthreads();
+            if (warp == 0) {
+                acc = warp_sum_u64(lane < nwarp ? sh[lane] : 0);
+                if (lane == 0)
+                    R6[base + x - 1] = 1ull - at_place(S, P, base + x - 1) - acc;
+            }
+            __syncthreads();
         }
     }
 }
 
-__device__ __forceinline__ void resolve_final(const QueryDev &Q, const uint64_t *A,
+__device__ __forceinline__ void resolve_final(const QueryDev &Q, const uint32_t *P, const uint64_t *A,
                                               const uint64_t *R6, uint64_t *R, uint64_t tid,
                                               uint64_t nthreads)
 {
     const uint64_t X = Q.X, base = Q.off;
     for (uint64_t x = 1 + tid; x <= X; x += nthreads) {
-        uint64_t v = R6[base + x - 1] + A[base + x - 1];
+        uint64_t v = R6[base + x - 1] + at_place(A, P, base + x - 1);
         if (2 * x <= X)
             v -= R6[base + 2 * x - 1];
         if (3 * x <= X)
@@ -1116,33 +1261,37 @@ __device__ __forceinline__ void resolve_final(const QueryDev &Q, const uint64_t 
 
 // A CTA per target, all levels.
 __global__ void __launch_bounds__(1024) wheel_resolve_kernel(const QueryDev *__restrict__ qs,
+                                                             const uint32_t *__restrict__ P,
                                                              const uint64_t *__restrict__ S,
                                                              const uint64_t *__restrict__ A,
                                                              uint64_t *R6, uint64_t *R)
 {
+    __shared__ uint64_t sh[32];
     const QueryDev Q = qs[blockIdx.x];
     for (uint64_t hi = Q.X; hi >= 1; hi /= 5) {
-        resolve_level(Q, S, R6, hi / 5 + 1, hi, threadIdx.x, blockDim.x);
+        resolve_level(Q, P, S, R6, hi / 5 + 1, hi, threadIdx.x, blockDim.x, sh);
         __syncthreads();
     }
-    resolve_final(Q, A, R6, R, threadIdx.x, blockDim.x);
+    resolve_final(Q, P, A, R6, R, threadIdx.x, blockDim.x);
 }
 
 // One level (the last launch: the values of M) of every target, several CTAs each.
 __global__ void __launch_bounds__(256) wheel_resolve_level_kernel(const QueryDev *__restrict__ qs,
+                                                                  const uint32_t *__restrict__ P,
                                                                   const uint64_t *__restrict__ S,
                                                                   const uint64_t *__restrict__ A,
                                                                   uint64_t *R6, uint64_t *R,
                                                                   uint64_t div, uint32_t last)
 {
+    __shared__ uint64_t sh[32];
     const QueryDev Q = qs[blockIdx.y];
     const uint64_t tid = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint64_t nt = (uint64_t)gridDim.x * blockDim.x;
     const uint64_t hi = Q.X / div;
     if (last)
-        resolve_final(Q, A, R6, R, tid, nt);
+        resolve_final(Q, P, A, R6, R, tid, nt);
     else if (hi)
-        resolve_level(Q, S, R6, hi / 5 + 1, hi, tid, nt);
+        resolve_level(Q, P, S, R6, hi / 5 + 1, hi, tid, nt, sh);
 }
 
 // ---------------------------------------------------------------------------
@@ -1231,18 +1380,19 @@ int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t 
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint64_t *S,
-                          const uint64_t *A, uint64_t *R6, uint64_t *R, cudaStream_t s)
+int wheel_resolve_enqueue(const QueryDev *qs, uint32_t nq, uint64_t max_x, const uint32_t *P,
+                          const uint64_t *S, const uint64_t *A, uint64_t *R6, uint64_t *R,
+                          cudaStream_t s)
 {
     if (max_x <= 16384 || nq >= 32) {
-        wheel_resolve_kernel<<<nq, 1024, 0, s>>>(qs, S, A, R6, R);
+        wheel_resolve_kernel<<<nq, 1024, 0, s>>>(qs, P, S, A, R6, R);
         return cudaGetLastError() == cudaSuccess ? 1 : -1;
     }
     int n = 0;
     const dim3 grid((unsigned)std::min<uint64_t>((max_x + 255) / 256, 608), nq);
     for (uint64_t div = 1; div <= max_x; div *= 5, ++n)
-        wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, S, A, R6, R, div, 0u);
-    wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, S, A, R6, R, 1, 1u);
+        wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, P, S, A, R6, R, div, 0u);
+    wheel_resolve_level_kernel<<<grid, 256, 0, s>>>(qs, P, S, A, R6, R, 1, 1u);
     return cudaGetLastError() == cudaSuccess ? n + 1 : -1;
 }
 
