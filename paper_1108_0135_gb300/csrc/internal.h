@@ -112,6 +112,10 @@ uint32_t prime_count_upto(const PrimeTable *t, uint64_t b);
 // Enqueues the fused steps a1 + a2 for one block.  Returns the number of
 // kernels launched, or -1 on a launch error.
 int sieve_block_enqueue(const PrimeTable *t, const SieveLaunch &L, cudaStream_t s);
+// a2 finish: segoff[s] = *carry_in + sum of segsum[0..s), *carry_out = *carry_in +
+// all of them (segsum 16-byte aligned).
+void seg_carry_enqueue(const int32_t *segsum, uint32_t nseg, const int64_t *carry_in,
+                       int64_t *segoff, int64_t *carry_out, cudaStream_t s);
 // Segments of a block of `len` y values.
 inline uint64_t sieve_segments(uint64_t len) { return (len + kSegY - 1) / kSegY; }
 

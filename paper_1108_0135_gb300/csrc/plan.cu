@@ -2143,6 +2143,7 @@ static int run_enqueue(mertens_plan_s *p, cudaStream_t origin, uint64_t *out)
             sa.EMIT = p->dEMIT;
             sa.JC0 = p->dJC0;
             sa.YCE = p->dYCE;
+            sa.ydense = p->ydense;
             sa.MG = p->dMG;
             sa.S = p->dS;
             sa.queue = p->dqueue;

@@ -1251,39 +1251,34 @@ __global__ void __launch_bounds__(kSieveThreads, 1) mu_sieve_persist_kernel(Byte
                 }
             } else {
                 // bucket entries of this tile: mark, forward to the tile of the
-                // next multiple (warp-aggregated slot allocation)
-                const uint32_t e0 = (job - jm) * kBucketJob;
+                // next multiple.  Four loads per lane are in flight (one at a
+                // time, a warp waited for each), and every lane takes its slot
+                // with its own shared atomic.
+                const uint32_t e0 = (job - jm) * kBucketJob + lane;
                 uint64_t *bk = a.bucket + (size_t)(tb + tt) * a.cap;
 #pragma unroll 1
-                for (uint32_t k = 0; k < kBucketJob / 32u; ++k) {
-                    const uint32_t e = e0 + k * 32u + lane;
-                    uint32_t nt = 0xffffffffu, fwd = 0;
-                    uint64_t ent = 0;
-                    if (e < nb) {
-                        ent = bk[e];
-                        const uint32_t off = (uint32_t)ent & (kByteTile - 1);
-                        const uint32_t wt = (uint32_t)(ent >> 17) & 127u;
-                        const uint32_t p = (uint32_t)(ent >> 24);
+                for (uint32_t k = 0; k < kBucketJob; k += 128u) {
+                    uint64_t ent[4];
+#pragma unroll
+                    for (uint32_t q = 0; q < 4u; ++q)
+                        ent[q] = e0 + k + 32u * q < nb ? bk[e0 + k + 32u * q] : 0ull;
+#pragma unroll
+                    for (uint32_t q = 0; q < 4u; ++q) {
+                        if (ent[q] == 0)
+                            continue;
+                        const uint32_t off = (uint32_t)ent[q] & (kByteTile - 1);
+                        const uint32_t wt = (uint32_t)(ent[q] >> 17) & 127u;
+                        const uint32_t nx = off + (uint32_t)(ent[q] >> 24);
                         atomicAdd(&w[off >> 2], __funnelshift_l(0u, wt, off << 3));
-                        const uint32_t nx = off + p;
-                        if (tt + (nx >> 17) < T) {
-                            nt = tt + (nx >> 17);
-                            fwd = nx & (kByteTile - 1);
+                        const uint32_t nt = tt + (nx >> 17);
+                        if (nt < T) {
+                            const uint32_t slot = atomicAdd(&s_cnt[nt], 1u);
+                            if (slot < a.cap)
+                                a.bucket[(size_t)(tb + nt) * a.cap + slot] =
+                                    (ent[q] & ~(uint64_t)(kByteTile - 1)) | (nx & (kByteTile - 1));
+                            else
+                                atomicOr(a.err, kErrBucket);
                         }
-                    }
-                    const uint32_t peers = __match_any_sync(0xffffffffu, nt);
-                    if (nt != 0xffffffffu) {
-                        const uint32_t leader = __ffs(peers) - 1u;
-                        uint32_t base = 0;
-                        if (lane == leader)
-                            base = atomicAdd(&s_cnt[nt], (uint32_t)__popc(peers));
-                        base = __shfl_sync(peers, base, leader);
-                        const uint32_t slot = base + __popc(peers & ((1u << lane) - 1u));
-                        if (slot < a.cap)
-                            a.bucket[(size_t)(tb + nt) * a.cap + slot] =
-                                (ent & ~(uint64_t)(kByteTile - 1)) | fwd;
-                        else
-                            atomicOr(a.err, kErrBucket);
                     }
                 }
             }
@@ -1292,33 +1287,6 @@ __global__ void __launch_bounds__(kSieveThreads, 1) mu_sieve_persist_kernel(Byte
         byte_tile_decode(a, sb, sq, a0, t1, tl, lane, warp);
         __syncthreads();  // the next tile reuses the shared arrays
     }
-}
-
-// a2 finish: segoff[s] = carry_in + sum of segsum[0..s) (int64), and
-// carry_out = carry_in + all of them.  Each CTA scans 1024 segments and adds
-// the sum of all segments before its range.
-__global__ void __launch_bounds__(1024) seg_carry_kernel(const int32_t *__restrict__ segsum,
-                                                         uint32_t nseg,
-                                                         const int64_t *__restrict__ carry_in,
-                                                         int64_t *__restrict__ segoff,
-                                                         int64_t *__restrict__ carry_out)
-{
-    __shared__ int64_t sh[33];
-    const uint32_t base = blockIdx.x * 1024u;
-    int64_t before = 0;
-    for (uint32_t i = threadIdx.x; i < base; i += 1024u)
-        before += segsum[i];
-    int64_t tb;
-    block_excl_scan<int64_t>(before, sh, &tb);
-    const uint32_t i = base + threadIdx.x;
-    const int64_t v = i < nseg ? segsum[i] : 0;
-    int64_t tot;
-    const int64_t ex = block_excl_scan<int64_t>(v, sh, &tot);
-    const int64_t c0 = *carry_in;
-    if (i < nseg)
-        segoff[i] = c0 + tb + ex;
-    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0)
-        *carry_out = c0 + tb + tot;
 }
 
 __global__ void expand_M_kernel(const int16_t *__restrict__ Mloc, const int64_t *__restrict__ segoff,
@@ -1730,8 +1698,7 @@ int sieve_block_enqueue(const PrimeTable *t, const SieveLaunch &L, cudaStream_t 
             if (L.mid2)
                 cudaEventRecord(L.mid2, s);
             const uint32_t nseg = (uint32_t)sieve_segments(L.len);
-            seg_carry_kernel<<<(nseg + 1023) / 1024, 1024, 0, s>>>(L.segsum, nseg, L.carry_in,
-                                                                  L.segoff, L.carry_out);
+            seg_carry_enqueue(L.segsum, nseg, L.carry_in, L.segoff, L.carry_out, s);
             ++launches;
             return cudaGetLastError() == cudaSuccess ? launches : -1;
         }
@@ -1832,8 +1799,7 @@ int sieve_block_enqueue(const PrimeTable *t, const SieveLaunch &L, cudaStream_t 
     if (L.mid2)
         cudaEventRecord(L.mid2, s);
     const uint32_t nseg = (uint32_t)sieve_segments(L.len);
-    seg_carry_kernel<<<(nseg + 1023) / 1024, 1024, 0, s>>>(L.segsum, nseg, L.carry_in, L.segoff,
-                                                          L.carry_out);
+    seg_carry_enqueue(L.segsum, nseg, L.carry_in, L.segoff, L.carry_out, s);
     ++launches;
     if (cudaGetLastError() != cudaSuccess)
         return -1;

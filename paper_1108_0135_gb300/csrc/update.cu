@@ -303,13 +303,16 @@ __global__ void __launch_bounds__(256) sparse_range_kernel(SparseBlockArgs b, Sp
     const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31u;
     const bool act = e < a.nent;
-    const uint64_t k = act ? a.K[e] : 0ull;
+    // all loads at once: the kernel waits for memory (4.6e6 entries, 53 us with one
+    // load after the other)
+    const uint64_t k = act ? a.K[e] : 0ull, jc = act ? a.JC0[e] : 0ull,
+                   jlo = act ? a.JLO[e] : 0ull;
+    const uint64_t yce = act && b.y1 <= a.ydense ? a.YCE[e] : 0ull;
     const uint64_t k2 = k << 1;
     uint64_t jtop = 0, jbot = 1;
     if (k2 && k < a.kmax) {
         const uint64_t q1 = div_magic(k2, a.m_ylo, a.l_ylo);    // floor(k / y_lo)
         const uint64_t q2 = div_magic(k2, b.m_y2p1, b.l_y2p1);  // floor(k / (y2+1))
-        const uint64_t jc = a.JC0[e], jlo = a.JLO[e];
         jtop = jc < q1 ? jc : q1;
         jbot = (q2 + 1) > jlo ? (q2 + 1) : jlo;
     }
@@ -330,13 +333,8 @@ __global__ void __launch_bounds__(256) sparse_range_kernel(SparseBlockArgs b, Sp
                 emit_levels(a.S, e, em, jbot, jtop, h, 0);
         }
     }
-    if (k2) {
-        const uint64_t yc = a.YCE[e];
-        if (yc >= b.y1 && yc <= b.y2) {
-            const int64_t Myc = block_M(a.segoff, a.Mloc, yc - b.y1);
-            add -= (int64_t)((uint64_t)Myc * a.JC0[e]);
-        }
-    }
+    if (k2 && yce >= b.y1 && yce <= b.y2)
+        add -= (int64_t)((uint64_t)block_M(a.segoff, a.Mloc, yce - b.y1) * jc);
     if (add)
         atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e), (unsigned long long)add);
     // heavy entries: ceil(cnt / kSparseItem) chunk records, slots taken with

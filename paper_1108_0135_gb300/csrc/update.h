@@ -64,6 +64,7 @@ struct SparseArgs {
     uint64_t m_ylo;
     uint32_t l_ylo;
     uint32_t qcap;
+    uint64_t ydense;  // no cut-off in YCE is above
     const uint64_t *K, *JLO, *JC0, *YCE, *MG;
     const uint32_t *EMIT;  // x | L << 29: the entries 2^s x (s <= L) it feeds (update.cu)
     uint64_t *S;

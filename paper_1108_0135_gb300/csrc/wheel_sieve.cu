@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(THREADS, MINB) wheel_sieve_kernel(WSieveArgs a
 // a2 finish: segoff[s] = carry_in + sum of segsum[0..s), carry_out = carry_in
 // + all of them.  Each CTA scans 4096 segments and adds the sum of all
 // segments before its range.
-__global__ void __launch_bounds__(1024) wheel_carry_kernel(const int32_t *__restrict__ segsum,
+__global__ void __launch_bounds__(1024) seg_carry_kernel(const int32_t *__restrict__ segsum,
                                                            uint32_t nseg,
                                                            const int64_t *__restrict__ carry_in,
                                                            int64_t *__restrict__ segoff,
@@ -581,6 +581,13 @@ uint32_t wheel_primes_upto(const WheelSieve *t, uint64_t b)
                       t->host_p.begin());
 }
 
+void seg_carry_enqueue(const int32_t *segsum, uint32_t nseg, const int64_t *carry_in,
+                       int64_t *segoff, int64_t *carry_out, cudaStream_t s)
+{
+    seg_carry_kernel<<<(nseg + 4095) / 4096, 1024, 0, s>>>(segsum, nseg, carry_in, segoff,
+                                                           carry_out);
+}
+
 template <uint32_t TILE, int THREADS, int MINB>
 static int wheel_launch(const WheelSieve *t, const WheelLaunch &L, cudaStream_t s)
 {
@@ -626,8 +633,7 @@ int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t 
     if (L.mid2)
         cudaEventRecord(L.mid2, s);
     const uint32_t nseg = (uint32_t)(L.len >> kSegShift);
-    wheel_carry_kernel<<<(nseg + 4095) / 4096, 1024, 0, s>>>(L.segsum, nseg, L.carry_in, L.segoff,
-                                                             L.carry_out);
+    seg_carry_enqueue(L.segsum, nseg, L.carry_in, L.segoff, L.carry_out, s);
     return cudaGetLastError() == cudaSuccess ? launches + 1 : -1;
 }
 
