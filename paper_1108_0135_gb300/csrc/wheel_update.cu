@@ -36,6 +36,14 @@ __device__ __forceinline__ uint32_t wheel_of_bits(uint32_t bits)
     return (3u * bits + (1u - 3u * kMagicBits)) | 1u;
 }
 
+// v as a float (relative error at most 2^-23) by two 32-bit conversions (a 64-bit
+// one runs on the FP64 pipe here).
+__device__ __forceinline__ float float_u64(uint64_t v)
+{
+    return __fmaf_rn(__uint2float_rn((uint32_t)(v >> 32)), 4294967296.0f,
+                     __uint2float_rn((uint32_t)v));
+}
+
 // ---------------------------------------------------------------------------
 // Plan: the entries of every target, a warp per group of 64 (two per lane).
 // ---------------------------------------------------------------------------
@@ -320,13 +328,13 @@ __device__ __forceinline__ uint32_t count_below(const uint16_t *a, uint32_t n, u
 // in k, in the reciprocal and, from 3y = 2^24 on, in 3y: it errs by less than 1/3
 // for k/(3y) < 2.06e6, or 1.8e6 there (the kernel's rule; n <= 2048 terms, so the
 // sum of the T stays below 2^32).
-__device__ __forceinline__ void dense_float(const uint2 *el, uint32_t n, const float kf[2],
+__device__ __forceinline__ void dense_float(const uint4 *el, uint32_t n, const float kf[2],
                                             const uint32_t kl[2], uint64_t out[2])
 {
     uint32_t st[2] = {0, 0}, ss[2] = {0, 0};
 #pragma unroll 4
     for (uint32_t i = 0; i < n; ++i) {
-        const uint2 v = el[i];
+        const uint4 v = el[i];
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
             const uint32_t T = __float_as_uint(__fmaf_rd(kf[e], __uint_as_float(v.x), kMagicF));
@@ -339,11 +347,40 @@ __device__ __forceinline__ void dense_float(const uint2 *el, uint32_t n, const f
         out[e] = (uint64_t)(uint32_t)(st[e] - n * kMagicBits) + n - ss[e];
 }
 
+// Linear mode: as the float mode with the chunk's middle ym taken out: with
+// q0 = floor(k/(3 ym)) and r0 = k - 3 ym q0, k/(3y) = q0 + (r0 - 3 q0 (y - ym))/(3y),
+// whose second part is below 10^6 in size for k <= 900 y0^2 (y0 the chunk's
+// start, |y - ym| <= 3072): four roundings of 2^-24, so it errs by less than 1/4,
+// and the sum of 2048 of them fits 32 bits.  Staged {1/(3y), -y, y - ym}.
+__device__ __forceinline__ void dense_linear(const uint4 *el, uint32_t n, const uint64_t q0[2],
+                                             const float r0[2], const uint32_t kl[2],
+                                             uint64_t out[2])
+{
+    uint32_t st[2] = {0, 0}, ss[2] = {0, 0};
+    const float a[2] = {-3.0f * float_u64(q0[0]), -3.0f * float_u64(q0[1])};
+    const uint32_t c[2] = {3u * (uint32_t)q0[0] + 1u - 3u * kMagicBits,
+                           3u * (uint32_t)q0[1] + 1u - 3u * kMagicBits};
+#pragma unroll 4
+    for (uint32_t i = 0; i < n; ++i) {
+        const uint4 v = el[i];
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const float R = __fmaf_rn(a[e], __uint_as_float(v.z), r0[e]);
+            const uint32_t T = __float_as_uint(__fmaf_rd(R, __uint_as_float(v.x), kMagicF));
+            ss[e] += (((3u * T + c[e]) | 1u) * v.y + kl[e]) >> 31;
+            st[e] += T;
+        }
+    }
+#pragma unroll
+    for (int e = 0; e < 2; ++e)
+        out[e] = (uint64_t)(int64_t)(int32_t)(st[e] - n * kMagicBits) + n * q0[e] + n - ss[e];
+}
+
 // High-word mode: staged {m, -y}, m = floor(2^(31 + ex)/(3y)) in [2^30, 2^31),
 // ex = floor(log2 3y); kh the top 32 bits of k (b bits), T the floor of
 // (kh m / 2^32) / 2^(ex + 31 - b).  Truncations of 2^-31 and 2^-30 and one of a
 // unit before the shift (at least 4) with k/(3y) < 6e7: less than 0.15.
-__device__ __forceinline__ void dense_high(const uint2 *el, uint32_t n, const uint32_t kh[2],
+__device__ __forceinline__ void dense_high(const uint4 *el, uint32_t n, const uint32_t kh[2],
                                            const uint32_t sb[2], const uint32_t kl[2],
                                            uint64_t out[2])
 {
@@ -351,7 +388,7 @@ __device__ __forceinline__ void dense_high(const uint2 *el, uint32_t n, const ui
     uint32_t ss[2] = {0, 0};
 #pragma unroll 4
     for (uint32_t i = 0; i < n; ++i) {
-        const uint2 v = el[i];
+        const uint4 v = el[i];
         const uint32_t ex = 31u - __clz(0u - 3u * v.y);
 #pragma unroll
         for (int e = 0; e < 2; ++e) {
@@ -369,13 +406,13 @@ __device__ __forceinline__ void dense_high(const uint2 *el, uint32_t n, const ui
 // Two steps, k/(3y) < 3e14, from the same staged values: q1 from the high words as
 // above but in 64 bits (at most 3.3e-9 k/(3y) + 1 below k/(3y)), then the float
 // mode's estimate for the rest k - 3y q1 < 2^35 (its quotient below 1e6).
-__device__ __forceinline__ void dense_two(const uint2 *el, uint32_t n, const uint64_t k[2],
+__device__ __forceinline__ void dense_two(const uint4 *el, uint32_t n, const uint64_t k[2],
                                           const uint32_t kh[2], const uint32_t sb[2],
                                           uint64_t out[2])
 {
     uint64_t st[2] = {0, 0};
     for (uint32_t i = 0; i < n; ++i) {
-        const uint2 v = el[i];
+        const uint4 v = el[i];
         const uint32_t d = 0u - 3u * v.y, ex = 31u - __clz(d);
         const float rf = __uint2float_rn(v.x) * __uint_as_float((96u - ex) << 23);
 #pragma unroll
@@ -414,12 +451,12 @@ __device__ __forceinline__ void dense_wide(const uint16_t *off, uint32_t n, uint
 }
 
 // A work item is part of a chunk's list for kWheelGroupBlock groups.  Items whose
-// k/(3y) all lie below the float mode's bound (and y < 3.5e8) take it; in the
-// others the y up to kmax/9e14 (all y from 3.5e8) take 64-bit division, those up
+// k/(3y) all lie below the float mode's bound (and y < 3.5e8) take it, those with
+// k <= 900 y0^2 the linear mode; in the others the y up to kmax/9e14 (all y from 3.5e8) take 64-bit division, those up
 // to kmax/1.8e8 the two-step mode, the rest the high-word mode.
 __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDenseArgs a)
 {
-    __shared__ uint2 s_el[kSegY];
+    __shared__ uint4 s_el[kSegY];
     __shared__ uint16_t s_off[kSegY];
     __shared__ uint32_t s_item, s_block;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
@@ -458,6 +495,8 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
         const bool small_y = y0 + kWheelSegY < 350000000u;
         const bool fl =
             small_y && kmax < (y0 + kWheelSegY < 5500000u ? 6200000ull : 5400000ull) * (y0 + 1);
+        const bool lin = small_y && !fl && kmax / 900u <= y0 * y0;
+        const uint32_t ym = (uint32_t)y0 + (uint32_t)kWheelSegY / 2u;
         const uint32_t cnt = a.dl_cnt[c];
         const uint32_t cp = cnt & 0xffffu, cm = cnt >> 16;
         const uint32_t p0 = cp * part / a.parts, m0 = cm * part / a.parts;
@@ -470,9 +509,9 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
                 continue;
             const uint32_t y = (uint32_t)y0 + 3u * o + 1u + (o & 1u), d = 3u * y;
             const uint32_t ex = 31u - __clz(d);
-            s_el[i] = make_uint2(fl ? __float_as_uint(__frcp_rn(__uint2float_rn(d)))
-                                    : (uint32_t)((1ull << (31u + ex)) / d),
-                                 0u - y);
+            s_el[i] = make_uint4(fl || lin ? __float_as_uint(__frcp_rn(__uint2float_rn(d)))
+                                           : (uint32_t)((1ull << (31u + ex)) / d),
+                                 0u - y, __float_as_uint((float)(int32_t)(y - ym)), 0u);
         }
         __syncthreads();
         // one group per warp; fewer groups than warps: several warps share a
@@ -504,6 +543,19 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
                 const uint32_t kl[2] = {(uint32_t)k[0], (uint32_t)k[1]};
                 dense_float(s_el + f0, n0, kf, kl, sum);
                 dense_float(s_el + f1, n1, kf, kl, part2);
+                sum[0] -= part2[0];
+                sum[1] -= part2[1];
+            } else if (lin) {
+                uint64_t q0[2];
+                float r0[2];
+                const uint32_t kl[2] = {(uint32_t)k[0], (uint32_t)k[1]};
+#pragma unroll
+                for (int e = 0; e < 2; ++e) {
+                    q0[e] = k[e] / (3u * ym);
+                    r0[e] = __uint2float_rn((uint32_t)(k[e] - q0[e] * (3u * ym)));
+                }
+                dense_linear(s_el + f0, n0, q0, r0, kl, sum);
+                dense_linear(s_el + f1, n1, q0, r0, kl, part2);
                 sum[0] -= part2[0];
                 sum[1] -= part2[1];
             } else {
@@ -570,24 +622,13 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
 constexpr uint32_t kGatherJ32 = 300000000u;  // 32-bit remainders below: 5j < 2^31
 constexpr uint32_t kWheelLaneTerms = 16;     // few terms: always a lane per entry
 
-// v as a float (relative error at most 2^-22) from exact 16-bit pieces.
-__device__ __forceinline__ float float_pieces(uint64_t v)
-{
-    const uint32_t lo = (uint32_t)v, hi = (uint32_t)(v >> 32);
-    const float f3 = __int_as_float(0x4B000000 | (hi >> 16)) - 8388608.0f;
-    const float f2 = __int_as_float(0x4B000000 | (hi & 0xffffu)) - 8388608.0f;
-    const float f1 = __int_as_float(0x4B000000 | (lo >> 16)) - 8388608.0f;
-    const float f0 = __int_as_float(0x4B000000 | (lo & 0xffffu)) - 8388608.0f;
-    return __fmaf_rn(__fmaf_rn(f3, 65536.0f, f2), 4294967296.0f, __fmaf_rn(f1, 65536.0f, f0));
-}
-
 // Constants of a run of terms j = j0 + step i in a tile.
 struct TileStep {
     float dRf, stepf;    // step t0 / 3, step
     uint32_t dR32, step; // step t0 (mod 2^32), step
     uint64_t dR;         // step t0
     __device__ __forceinline__ TileStep(uint64_t t0, uint32_t st)
-        : dRf(float_pieces(t0) * ((float)st / 3.0f)), stepf((float)st), dR32((uint32_t)t0 * st),
+        : dRf(float_u64(t0) * ((float)st / 3.0f)), stepf((float)st), dR32((uint32_t)t0 * st),
           step(st), dR(t0 * st)
     {
     }
@@ -604,8 +645,8 @@ struct TileRun {
     __device__ __forceinline__ TileRun(uint64_t k, uint64_t t0, uint32_t j0)
     {
         R = k - t0 * (uint64_t)j0;
-        Rf0 = float_pieces(R) * (1.0f / 3.0f);
-        jf0 = float_pieces(j0);
+        Rf0 = float_u64(R) * (1.0f / 3.0f);
+        jf0 = __uint2float_rn(j0);
         j = j0;
         nR = ~(uint32_t)R;
     }

@@ -94,3 +94,21 @@ def test_wheel_runs_equal_full_sums(ns, u, bl, quot, monkeypatch):
         monkeypatch.setenv("MERTENS_GATHER_QUOT", quot)  # 64-bit remainders
     for a, b in zip(full, _arrays(ns, u, bl)):
         assert np.array_equal(a, b)
+
+
+def test_linear_estimate_of_the_dense_terms():
+    """The linear mode's estimate of k/(3y) - q0 in single precision (float_u64 of
+    q0, one multiply-add, the reciprocal) errs by less than 1/3 for k <= 900 y0^2."""
+    rng = random.Random(8)
+    f = np.float32
+    for _ in range(20000):
+        y0 = 6144 * rng.randrange(1, 56_000)
+        k = min(rng.randrange(900 * y0 * y0 // 8, 900 * y0 * y0 + 1), 2**63 - 1)
+        ym = y0 + 3072
+        y = y0 + rng.randrange(1, 6144)
+        q0, r0 = divmod(k, 3 * ym)
+        qf = f(float(f(q0 >> 32)) * 2.0**32 + float(f(q0 & 0xffffffff)))
+        R = f(float(f(-3.0) * qf) * float(y - ym) + float(f(r0)))
+        est = float(R) * float(f(1.0) / f(3 * y))
+        exact = (k - 3 * y * q0) / (3 * y)
+        assert abs(est - exact) < 1 / 3 and abs(exact) < 1.0e6
