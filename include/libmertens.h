@@ -105,7 +105,7 @@ int mertens_plan(mertens_plan_t *out, const mertens_u128 *n, size_t count,
 /*
  * Resident M(y) table.  The sieve's output for 1 <= y <= y_max (steps a1 +
  * a2, over the y coprime to 6, from which M(y) follows) is computed once and
- * kept in device memory (about 0.67 bytes per y), together with what the
+ * kept in device memory (about 0.17 bytes per y), together with what the
  * update needs independently of the target for all n <= n_max (the squarefree
  * list of the dense form).  Plans made on it read M(y) from the table for every
  * sieve block that ends at or below y_max and sieve only the blocks above it; their

@@ -151,16 +151,15 @@ inline uint64_t dense_chunks(uint64_t ydense) { return ydense / kChunk + 1; }
 }  // namespace mert
 
 // A resident table (mertens_table_create) in the form of wheel.h: M6(y) for the
-// y <= y_cov (y_max up to whole segments) coprime to 6, in the sieve's layout
-// (int16 relative to the 2048-number segment, int64 segment offsets), and the
-// dense list of the squarefree ones up to ydense.
+// y <= y_cov (y_max up to whole segments) coprime to 6 in the sieve's layout, and
+// the dense list of the squarefree ones up to ydense.
 struct mertens_table_s {
     mert::Allocator al;
     int device = 0;
     uint64_t y_max = 0, y_cov = 0;
     uint64_t n_max_lo = 0, n_max_hi = 0;
     uint64_t ydense = 0;
-    int16_t *Mloc = nullptr;
+    uint2 *Mg = nullptr;
     int64_t *segoff = nullptr;
     uint16_t *dl = nullptr;
     uint32_t *dl_cnt = nullptr;

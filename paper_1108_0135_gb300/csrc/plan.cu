@@ -271,6 +271,7 @@ struct mertens_plan_s {
     bool wheel = false;
     bool wheel_long = false;     // 64-bit remainders for every gathered term
     WheelSieve ws;
+    uint2 *dMg = nullptr;        // a block's M6 (wheel.h)
     uint32_t *dJL = nullptr, *dJD = nullptr;
     uint32_t *dplace = nullptr;  // entries' places (several targets)
     uint64_t *dA = nullptr, *dR6 = nullptr;
@@ -675,9 +676,9 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         delete p;
         return MERTENS_EINVAL;
     }
-    // a block's M6 takes a third of the memory of block_len y in the full form, so
-    // three times as many y make a block (fewer launches: 48.9 -> 45.2 ms at
-    // n = 10^16 with 2^28-y blocks)
+    // three times as many y make a block (in a quarter of the memory that block_len
+    // y take in the full form; fewer launches: 48.9 -> 45.2 ms at n = 10^16 with
+    // 2^28-y blocks)
     block_len = std::min(std::min<uint64_t>(3 * block_len, 3ull << 30), p->y_last);
     // a plan on a table sieves only the blocks that end above it
     p->sieves = !table || p->y_last > table->y_max;
@@ -882,7 +883,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         take(p->dR, E * 8);
         take(p->dqueue, (size_t)p->qcap * sizeof(uint4));
         if (p->sieves) {
-            take(p->dMloc[0], wlen * 2);
+            take(p->dMg, wlen >> kMgShift << 3);
             take(p->dsegsum[0], wlen / kSegY * 4);
             take(p->dsegoff[0], wlen / kSegY * 8);
         }
@@ -1864,12 +1865,12 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
     for (uint64_t b = 0; b < p->nblocks && r >= 0; ++b) {
         const uint64_t y0 = b * p->block_len, len = wheel_block_len(p, b);
         const bool from_table = tab && y0 + len <= tab->y_cov;
-        const int16_t *Mb = from_table ? tab->Mloc + y0 / 3 : p->dMloc[0];
+        const uint2 *Mb = from_table ? tab->Mg + (y0 / 3 >> kMgShift) : p->dMg;
         const int64_t *Sb = from_table ? tab->segoff + y0 / kWheelSegY : p->dsegoff[0];
         PhaseEvents pe, pe2;
         if (!from_table) {
             if (after_table) {
-                r = wheel_carry_at_enqueue(tab->Mloc, tab->segoff, y0, p->dcarry + b, s);
+                r = wheel_carry_at_enqueue(tab->Mg, tab->segoff, y0, p->dcarry + b, s);
                 if (r < 0)
                     break;
                 launches += r;
@@ -1877,7 +1878,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             WheelLaunch L;
             L.w0 = y0 / 3;
             L.len = len / 3;
-            L.Mloc = p->dMloc[0];
+            L.Mg = p->dMg;
             L.segsum = p->dsegsum[0];
             L.segoff = p->dsegoff[0];
             L.carry_in = p->dcarry + b;
@@ -1924,14 +1925,13 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             ga.items = p->dwgitems + p->gblk[b];
             ga.nitems = p->gblk[b + 1] - p->gblk[b];
             ga.counter = p->dcounter_gather;
-            ga.Mloc = Mb;
+            ga.Mg = Mb;
             ga.segoff = Sb;
             ga.K = p->dK;
             ga.YC = p->dYCE;
             ga.JL = p->dJL;
             ga.JD = p->dJD;
             ga.S = p->dS;
-            ga.err = p->derr;
             ga.all_long = p->wheel_long ? 1u : 0u;
             r = wheel_gather_enqueue(ga, s);
             if (r < 0)
@@ -1958,7 +1958,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
         ba.qlen = p->dqlen;
         ba.qcap = p->qcap;
         ba.err = p->derr;
-        ba.Mloc = Mb;
+        ba.Mg = Mb;
         ba.segoff = Sb;
         r = wheel_block_enqueue(ba, s);
         if (r >= 0 && !p->wide.empty()) {
@@ -1967,7 +1967,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             wa.W = p->dwide;
             wa.y0 = y0;
             wa.len = len;
-            wa.Mloc = Mb;
+            wa.Mg = Mb;
             wa.segoff = Sb;
             wa.S = p->dS;
             wa.A = p->dA;
@@ -1994,7 +1994,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
                                   p->dR, s);
         if (r >= 0 && !p->lookups.empty()) {
             const int r2 = wheel_lookup_enqueue(p->dlook, (uint32_t)(p->lookups.size() / 2),
-                                                tab->Mloc, tab->segoff, p->dR, s);
+                                                tab->Mg, tab->segoff, p->dR, s);
             r = r2 < 0 ? r2 : r + r2;
         }
         ev_end(p, s, &pe);

@@ -1,5 +1,5 @@
 // Resident M(y) table: the sieve (steps a1 + a2, in the form of wheel.h) run
-// once up to y_max and kept in device memory (0.67 bytes per y), together with
+// once up to y_max and kept in device memory (0.17 bytes per y), together with
 // the part of the update that does not depend on the target (the dense list of
 // squarefree numbers).  Plans made on a table (mertens_plan_on_table) read M6(y)
 // from it and run only the update and resolve.  The paper sieves per target
@@ -84,7 +84,7 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
     t->y_cov = (y_max + kWheelSegY - 1) / kWheelSegY * kWheelSegY;
     const uint64_t nseg = t->y_cov / kWheelSegY;
     const uint64_t nchunks = (t->ydense + kWheelSegY - 1) / kWheelSegY;
-    t->Mloc = table_alloc<int16_t>(t, nseg * kSegY);
+    t->Mg = table_alloc<uint2>(t, nseg * kSegY >> kMgShift);
     t->segoff = table_alloc<int64_t>(t, nseg);
     t->dl = table_alloc<uint16_t>(t, nchunks * kSegY);
     t->dl_cnt = table_alloc<uint32_t>(t, nchunks);
@@ -97,7 +97,7 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
     const size_t b_ws = up(wheel_sieve_bytes(&ws, L / 3)), b_sum = up(L / kWheelSegY * 4),
                  b_cy = up((nblocks + 1) * 8), bytes = b_ws + b_sum + b_cy + 256;
     char *buf = (char *)dev_alloc(t->al, bytes);
-    int rc = t->Mloc && t->segoff && t->dl && t->dl_cnt && buf ? MERTENS_OK : MERTENS_ENOMEM;
+    int rc = t->Mg && t->segoff && t->dl && t->dl_cnt && buf ? MERTENS_OK : MERTENS_ENOMEM;
     if (rc == MERTENS_OK) {
         int32_t *segsum = (int32_t *)(buf + b_ws);
         int64_t *carry = (int64_t *)(buf + b_ws + b_sum);
@@ -112,7 +112,7 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
             WheelLaunch Lc;
             Lc.w0 = y0 / 3;
             Lc.len = std::min(L, t->y_cov - y0) / 3;
-            Lc.Mloc = t->Mloc + y0 / 3;
+            Lc.Mg = t->Mg + (y0 / 3 >> kMgShift);
             Lc.segsum = segsum;
             Lc.segoff = t->segoff + y0 / kWheelSegY;
             Lc.carry_in = carry + b;
@@ -121,7 +121,7 @@ int mertens_table_create(mertens_table_t *out, uint64_t y_max, mertens_u128 n_ma
                 rc = MERTENS_ECUDA;
         }
         if (rc == MERTENS_OK &&
-            wheel_dense_list_enqueue(t->Mloc, 0, nchunks, t->dl, t->dl_cnt, s) < 0)
+            wheel_dense_list_enqueue(t->Mg, 0, nchunks, t->dl, t->dl_cnt, s) < 0)
             rc = MERTENS_ECUDA;
         uint32_t st = 0;
         if (cudaMemcpyAsync(&st, err, 4, cudaMemcpyDeviceToHost, s) != cudaSuccess ||

@@ -51,6 +51,19 @@ __host__ __device__ __forceinline__ uint32_t wheel_index(uint32_t v)
 
 __host__ __device__ __forceinline__ uint64_t wheel_y(uint64_t w) { return 3 * w + 1 + (w & 1); }
 
+// Wheel numbers per element of Mg.
+constexpr uint32_t kMgShift = 4;
+
+#ifdef __CUDACC__
+// The part of M6 at wheel index i of a block that its Mg holds.
+__device__ __forceinline__ int wheel_value(const uint2 *Mg, uint64_t i)
+{
+    const uint2 v = Mg[i >> kMgShift];
+    const uint32_t upto = (2u << ((uint32_t)i & 15u)) - 1u;  // bits 0 .. i mod 16
+    return (int)v.y + __popc(v.x & upto) - 2 * __popc((v.x >> 16) & upto);
+}
+#endif
+
 // ---- sieve ------------------------------------------------------------------
 // Sieving primes and scratch of a wheel sieve (device arrays, primes >= 5), all
 // in one piece of memory of its owner.
@@ -64,10 +77,14 @@ struct WheelSieve {
 };
 
 // One block: wheel numbers [w0, w0 + len), both multiples of kSegY.
-//   M6(y(w)) = segoff[(w - w0) >> kSegShift] + Mloc[w - w0]
+//   M6(y(w)) = segoff[i >> kSegShift] + wheel_value(Mg, i), i = w - w0
+// Mg holds 8 bytes per 16 numbers (0.5 bytes per number; int16 values took four
+// times as much, and the sieve's decode was bound by writing them): x = the
+// squarefree ones as 16 bits, those with mu = -1 in the high half; y = M6 before
+// the 16 relative to the segment.
 struct WheelLaunch {
     uint64_t w0 = 0, len = 0;
-    int16_t *Mloc = nullptr;
+    uint2 *Mg = nullptr;
     int32_t *segsum = nullptr;
     int64_t *segoff = nullptr;
     const int64_t *carry_in = nullptr;  // device M6(y(w0) - 1)
@@ -174,17 +191,16 @@ struct WheelDenseArgs {
 };
 
 struct WheelGatherArgs {
-    uint64_t y0;            // block start: Mloc index 0 is y0 + 1
+    uint64_t y0;            // block start: wheel index 0 of Mg is y0 + 1
     const WheelGatherTile *tiles;
     const uint4 *items;     // {tile, e0, e1, 0}
     uint32_t nitems;
     uint32_t *counter;
-    const int16_t *Mloc;
+    const uint2 *Mg;
     const int64_t *segoff;
     const uint64_t *K, *YC;
     const uint32_t *JL, *JD;
     uint64_t *S;
-    uint32_t *err;
     uint32_t all_long;      // 64-bit remainders for every term
 };
 
@@ -203,11 +219,11 @@ struct WheelBlockArgs {
     uint32_t *qlen;
     uint32_t qcap;
     uint32_t *err;
-    const int16_t *Mloc;
+    const uint2 *Mg;
     const int64_t *segoff;
 };
 
-int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks, uint16_t *dl,
+int wheel_dense_list_enqueue(const uint2 *Mg, uint64_t c0, uint64_t nchunks, uint16_t *dl,
                              uint32_t *dl_cnt, cudaStream_t s);
 int wheel_dense_enqueue(const WheelDenseArgs &a, uint64_t max_items, cudaStream_t s);
 int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s);
@@ -222,7 +238,7 @@ struct WideEntry;
 struct WheelWideArgs {
     const WideEntry *W;
     uint64_t y0, len;
-    const int16_t *Mloc;
+    const uint2 *Mg;
     const int64_t *segoff;
     uint64_t *S, *A;
 };
@@ -232,11 +248,11 @@ void wheel_wide_units(const WideEntry &W, uint64_t y0, uint64_t len, uint64_t *d
                       uint64_t *wj, uint64_t *gathered);
 int wheel_wide_enqueue(const WheelWideArgs &a, uint32_t nw, uint64_t units, cudaStream_t s);
 
-// Reads of a resident table (Mloc and segoff from y = 0 on): M(y) of (entry, y)
+// Reads of a resident table (Mg and segoff from y = 0 on): M(y) of (entry, y)
 // pairs into R; M6(y0) into *out (y0 a multiple of a segment, > 0).
-int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
+int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const uint2 *Mg,
                          const int64_t *segoff, uint64_t *R, cudaStream_t s);
-int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y0, int64_t *out,
+int wheel_carry_at_enqueue(const uint2 *Mg, const int64_t *segoff, uint64_t y0, int64_t *out,
                            cudaStream_t s);
 
 struct QueryDev;

@@ -118,7 +118,7 @@ struct WSieveArgs {
     const uint4 *pat;
     uint32_t *sqcnt;
     const uint32_t *sqlist;
-    int16_t *Mloc;
+    uint2 *Mg;
     int32_t *segsum;
     uint32_t *err;
 };
@@ -226,26 +226,28 @@ __device__ __forceinline__ void wheel_lane_prime(uint4 q, uint32_t *w, uint32_t 
     }
 }
 
-// Decode + scan of one 2048-number segment (one warp); see t2_segment in
-// sieve.cu for the word arithmetic.  A round covers 1024 numbers, each lane
-// 16 at 16 lane and 16 at 512 + 16 lane; one warp scan carries both halves'
-// lane sums packed in one int32.  kTileThr: one threshold for the tile (bias4);
-// otherwise a threshold per number.
+// Decode + scan of one 2048-number segment (one warp): per byte the square flag
+// and, from the sign of W = (byte & 127) + bias and the weight sum's parity, mu =
+// -1; two words' flags become eight bits by dot products.  A round covers 1024
+// numbers, each lane 16 at 16 lane and 16 at 512 + 16 lane; one warp scan carries
+// both halves' lane sums packed in one int32.  kTileThr: one threshold for the
+// tile (bias4); otherwise a threshold per number.  Returns the segment's sum.
 template <bool kTileThr>
 __device__ __forceinline__ int wheel_segment(const WSieveArgs &a, const uint4 *sb, uint64_t wt0,
                                              uint32_t so, uint32_t lane, uint32_t bias4,
-                                             int16_t *dst0)
+                                             uint2 *dst0)
 {
     int run = 0;
 #pragma unroll 1
     for (uint32_t r = 0; r < (uint32_t)kSegY / 1024u; ++r) {
-        uint32_t D[8];
-        int tot[2] = {0, 0};
+        uint32_t bits[2];
+        int tot[2];
 #pragma unroll
         for (int h = 0; h < 2; ++h) {
             const uint32_t o0 = so + r * 1024u + (uint32_t)h * 512u + lane * 16u;
             const uint4 q4 = sb[o0 >> 4];
             const uint32_t ws[4] = {q4.x, q4.y, q4.z, q4.w};
+            uint32_t free8[2] = {0, 0}, neg8[2] = {0, 0};
 #pragma unroll
             for (int k = 0; k < 4; ++k) {
                 const uint32_t nsq = ~(ws[k] >> 7) & 0x01010101u;
@@ -266,9 +268,13 @@ __device__ __forceinline__ int wheel_segment(const WSieveArgs &a, const uint4 *s
                     }
                     m &= nsq;
                 }
-                D[4 * h + k] = (nsq - 2u * m) * 0x01010101u + 0x04040404u;
-                tot[h] += (int)(D[4 * h + k] >> 24) - 4;
+                const uint32_t weights = (k & 1) ? 0x80402010u : 0x08040201u;
+                free8[k >> 1] = __dp4a(nsq, weights, free8[k >> 1]);
+                neg8[k >> 1] = __dp4a(m, weights, neg8[k >> 1]);
             }
+            const uint32_t sf = free8[0] | (free8[1] << 8), ng = neg8[0] | (neg8[1] << 8);
+            bits[h] = sf | (ng << 16);
+            tot[h] = __popc(sf) - 2 * __popc(ng);
         }
         int inc = tot[0] + tot[1] * 65536;
 #pragma unroll
@@ -280,23 +286,9 @@ __device__ __forceinline__ int wheel_segment(const WSieveArgs &a, const uint4 *s
         const int all = __shfl_sync(0xffffffffu, inc, 31);
         const int incA = (int)(int16_t)(inc & 0xffff), incB = (inc - incA) >> 16;
         const int allA = (int)(int16_t)(all & 0xffff), allB = (all - allA) >> 16;
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t o0 = so + r * 1024u + (uint32_t)h * 512u + lane * 16u;
-            int rb = run + (h == 0 ? incA - tot[0] : allA + incB - tot[1]);
-            uint32_t out[8];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint32_t Dk = D[4 * h + k];
-                const uint32_t bx = (uint32_t)(rb - 4) * 0x00010001u;
-                out[2 * k] = (bx + __byte_perm(Dk, 0x80u, 0x4140)) ^ 0x80008000u;
-                out[2 * k + 1] = (bx + __byte_perm(Dk, 0x80u, 0x4342)) ^ 0x80008000u;
-                rb += (int)(Dk >> 24) - 4;
-            }
-            uint4 *dst = reinterpret_cast<uint4 *>(dst0 + o0);
-            dst[0] = make_uint4(out[0], out[1], out[2], out[3]);
-            dst[1] = make_uint4(out[4], out[5], out[6], out[7]);
-        }
+        uint2 *dst = dst0 + ((so + r * 1024u) >> kMgShift) + lane;
+        dst[0] = make_uint2(bits[0], (uint32_t)(run + incA - tot[0]));
+        dst[32] = make_uint2(bits[1], (uint32_t)(run + allA + incB - tot[1]));
         run += allA + allB;
     }
     return run;
@@ -305,7 +297,7 @@ __device__ __forceinline__ int wheel_segment(const WSieveArgs &a, const uint4 *s
 // The low tiles (a threshold per number), in a function of their own so that
 // they hold no registers of the common path.
 __device__ __noinline__ int wheel_segment_low(const WSieveArgs &a, const uint4 *sb, uint64_t wt0,
-                                              uint32_t so, uint32_t lane, int16_t *dst0)
+                                              uint32_t so, uint32_t lane, uint2 *dst0)
 {
     return wheel_segment<false>(a, sb, wt0, so, lane, 0u, dst0);
 }
@@ -414,7 +406,7 @@ __global__ void __launch_bounds__(THREADS, MINB) wheel_sieve_kernel(WSieveArgs a
         const int thr = (int)floorf(2.0f * log2f(__ull2float_rn(y1)) - a.log2P) & ~1;
         bias4 = (uint32_t)(126 - thr) * 0x01010101u;
     }
-    int16_t *dst0 = a.Mloc + a0;
+    uint2 *dst0 = a.Mg + (a0 >> kMgShift);
     for (uint32_t sgi = 0; sgi < 2; ++sgi) {
         const uint32_t so = warp * (2u * kSegY) + sgi * kSegY;
         if (a0 + so >= a.len)
@@ -613,7 +605,7 @@ static int wheel_launch(const WheelSieve *t, const WheelLaunch &L, cudaStream_t 
     a.pat = t->pat;
     a.sqcnt = t->sqcnt;
     a.sqlist = t->sqlist;
-    a.Mloc = L.Mloc;
+    a.Mg = L.Mg;
     a.segsum = L.segsum;
     a.err = t->err;
     wheel_prep_kernel<<<(a.np + 127) / 128, 128, 0, s>>>(L.w0 / 2, a.np, t->p, t->rec, t->rec2,

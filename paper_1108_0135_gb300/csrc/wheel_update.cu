@@ -270,27 +270,18 @@ int wheel_entries_enqueue(const WheelEntryArgs &a, cudaStream_t s)
 // ---------------------------------------------------------------------------
 // Dense list: chunk c holds the wheel numbers [c kSegY, (c + 1) kSegY), one
 // segment of the sieve; dl gets the offsets of its squarefree numbers, those
-// with mu = +1 first, read off as differences of the segment's M6.
+// with mu = +1 first.  A thread takes half an element of Mg.
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(256) wheel_dense_list_kernel(const int16_t *__restrict__ Mloc,
+__global__ void __launch_bounds__(256) wheel_dense_list_kernel(const uint2 *__restrict__ Mg,
                                                                uint64_t c0,
                                                                uint16_t *__restrict__ dl,
                                                                uint32_t *__restrict__ dl_cnt)
 {
     __shared__ uint32_t sh[33];
-    const int16_t *M = Mloc + (uint64_t)blockIdx.x * kSegY;
-    const uint4 v = reinterpret_cast<const uint4 *>(M)[threadIdx.x];
-    const uint32_t vw[4] = {v.x, v.y, v.z, v.w};
-    int prev = threadIdx.x ? M[threadIdx.x * 8 - 1] : 0;
-    int mu[8];
-    uint32_t cnt = 0;  // +1 in the low half, -1 in the high half
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-        const int m = (int)(int16_t)(vw[k >> 1] >> (16 * (k & 1)));
-        mu[k] = m - prev;
-        prev = m;
-        cnt += mu[k] > 0 ? 1u : (mu[k] < 0 ? 65536u : 0u);
-    }
+    const uint32_t v = Mg[((uint64_t)blockIdx.x * kSegY >> kMgShift) + (threadIdx.x >> 1)].x >>
+                       (8u * (threadIdx.x & 1u));
+    const uint32_t ng = (v >> 16) & 255u, ps = v & 255u & ~ng;
+    const uint32_t cnt = (uint32_t)__popc(ps) + ((uint32_t)__popc(ng) << 16);
     uint32_t tot;
     const uint32_t ex = block_scan_u32(cnt, sh, &tot);
     uint32_t ip = ex & 0xffffu, im = (tot & 0xffffu) + (ex >> 16);
@@ -298,9 +289,9 @@ __global__ void __launch_bounds__(256) wheel_dense_list_kernel(const int16_t *__
 #pragma unroll
     for (int k = 0; k < 8; ++k) {
         const uint16_t o = (uint16_t)(threadIdx.x * 8 + k);
-        if (mu[k] > 0)
+        if ((ps >> k) & 1u)
             d[ip++] = o;
-        else if (mu[k] < 0)
+        else if ((ng >> k) & 1u)
             d[im++] = o;
     }
     if (threadIdx.x == 0)
@@ -715,9 +706,9 @@ __device__ __forceinline__ int tile_warp(const int16_t *Mt, uint64_t k, uint64_t
 }
 
 // M6 at wheel index i of a block.
-__device__ __forceinline__ int64_t wheel_M(const int64_t *segoff, const int16_t *Mloc, uint32_t i)
+__device__ __forceinline__ int64_t wheel_M(const int64_t *segoff, const uint2 *Mg, uint64_t i)
 {
-    return segoff[i >> kSegShift] + (int64_t)Mloc[i];
+    return segoff[i >> kSegShift] + (int64_t)wheel_value(Mg, i);
 }
 
 // Tiles at y <= kUniformY: 64 entries of a warp (two per lane) against the same
@@ -832,15 +823,9 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
     __shared__ uint32_t s_item, s_nshared, s_next;
     __shared__ uint32_t s_shared[kSharedMax];
     __shared__ int64_t s_base;
-    __shared__ int32_t s_delta[kGatherTile / kSegY];
-    __shared__ uint64_t s_mbar;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, nwarp = blockDim.x >> 5;
     uint2 *jw = reinterpret_cast<uint2 *>(Mt + kGatherTile + 8) + warp * 32u;
-    uint32_t staged = 0xffffffffu, phase = 0;
-    if (threadIdx.x == 0) {
-        mbar_init(&s_mbar);
-        fence_proxy_async_smem();
-    }
+    uint32_t staged = 0xffffffffu;
     for (;;) {
         if (threadIdx.x == 0) {
             s_item = atomicAdd(a.counter, 1u);
@@ -853,35 +838,29 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
         const uint4 I = a.items[s_item];
         const WheelGatherTile T = a.tiles[I.x];
         if (I.x != staged) {
-            // one bulk asynchronous copy of the block's int16 values (whole
-            // segments), then each segment's offset added in place
+            // 16 values per element of Mg, relative to M6(t0)
             const uint32_t o1 = (uint32_t)((T.t0 - a.y0) / 3u), n = T.len / 3u;
+            const int64_t b0 = a.segoff[o1 >> kSegShift];
             if (threadIdx.x == 0) {
-                fence_proxy_async_smem();  // earlier readers of Mt passed the barrier
-                mbar_arrive_expect(&s_mbar, n * 2u);
-                bulk_copy_g2s(Mt, a.Mloc + o1, n * 2u, &s_mbar);
-                s_base = a.segoff[o1 >> kSegShift];
-            }
-            __syncthreads();
-            if (threadIdx.x == 0)
+                s_base = b0;
                 Mt[n] = 0;
-            if (threadIdx.x < n / kSegY)
-                s_delta[threadIdx.x] =
-                    (int32_t)(a.segoff[(o1 >> kSegShift) + threadIdx.x] - s_base);
-            if (__syncthreads_or(!mbar_wait(&s_mbar, phase & 1u))) {
-                if (threadIdx.x == 0)
-                    atomicOr(a.err, kErrTimeout);
-                mbar_wait(&s_mbar, phase & 1u);
-                return;
             }
-            ++phase;
-            uint32_t *Mw = reinterpret_cast<uint32_t *>(Mt);
-            for (uint32_t i = threadIdx.x; i < n / 2u; i += blockDim.x) {
-                const uint32_t v = Mw[i];
-                const int32_t dl = s_delta[(2u * i) >> kSegShift];
-                const uint32_t lo = (uint32_t)((int32_t)(int16_t)(v & 0xffffu) + dl) & 0xffffu;
-                const uint32_t hi = (uint32_t)((int32_t)(int16_t)(v >> 16) + dl);
-                Mw[i] = lo | (hi << 16);
+            const uint2 *src = a.Mg + (o1 >> kMgShift);
+            uint4 *Mw = reinterpret_cast<uint4 *>(Mt);
+            for (uint32_t i = threadIdx.x; i < n >> kMgShift; i += blockDim.x) {
+                const uint2 v = src[i];
+                int r = (int)v.y +
+                        (int)(a.segoff[(o1 + (i << kMgShift)) >> kSegShift] - b0);
+                uint32_t o[8];
+#pragma unroll
+                for (int k = 0; k < 8; ++k) {
+                    r += (int)((v.x >> (2 * k)) & 1u) - 2 * (int)((v.x >> (16 + 2 * k)) & 1u);
+                    const uint32_t lo = (uint32_t)r & 0xffffu;
+                    r += (int)((v.x >> (2 * k + 1)) & 1u) - 2 * (int)((v.x >> (17 + 2 * k)) & 1u);
+                    o[k] = lo | ((uint32_t)r << 16);
+                }
+                Mw[2 * i] = make_uint4(o[0], o[1], o[2], o[3]);
+                Mw[2 * i + 1] = make_uint4(o[4], o[5], o[6], o[7]);
             }
             staged = I.x;
         }
@@ -1036,7 +1015,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
         const uint64_t yc = a.YC[e];
         if (yc > a.y0 && yc <= yend)
             atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e),
-                      (unsigned long long)(0ull - (uint64_t)wheel_M(a.segoff, a.Mloc,
+                      (unsigned long long)(0ull - (uint64_t)wheel_M(a.segoff, a.Mg,
                                                                     wheel_index((uint32_t)(yc - a.y0))) *
                                                       phi6(jd)));
         int64_t tail = 0;
@@ -1046,7 +1025,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
                 const uint64_t y = k / m;
                 if (m >= jlo && y > a.y0 && y <= yend) {
                     const int64_t v =
-                        wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+                        wheel_M(a.segoff, a.Mg, wheel_index((uint32_t)(y - a.y0)));
                     tail += m == 6 ? v : -v;
                 }
             }
@@ -1060,7 +1039,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
 #pragma unroll 4
         for (uint32_t w = wl; w < wh; ++w) {
             const uint64_t y = k / (3ull * w + 1u + (w & 1u));
-            acc += wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+            acc += wheel_M(a.segoff, a.Mg, wheel_index((uint32_t)(y - a.y0)));
         }
         atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e), (unsigned long long)acc);
     }
@@ -1104,7 +1083,7 @@ __global__ void __launch_bounds__(256) wheel_chunk_kernel(WheelBlockArgs a)
         for (uint32_t i = lane; i < r.z; i += 32u) {
             const uint32_t w = r.y + i;
             const uint64_t y = k / (3ull * w + 1u + (w & 1u));
-            acc += wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)(y - a.y0)));
+            acc += wheel_M(a.segoff, a.Mg, wheel_index((uint32_t)(y - a.y0)));
         }
         acc = warp_sum_i64(acc);
         if (lane == 0)
@@ -1164,13 +1143,13 @@ __global__ void __launch_bounds__(kWideThreads) wheel_wide_kernel(WheelWideArgs 
         for (const uint64_t ue = u1 < nd ? u1 : nd; u < ue; ++u) {
             const uint64_t yn = wheel_y(w0 + u + 1);
             const uint64_t pn = phi6_quot(k, yn <= W.s ? yn : W.s + 1);
-            acc += (uint64_t)wheel_M(a.segoff, a.Mloc, (uint32_t)u) * (p - pn);
+            acc += (uint64_t)wheel_M(a.segoff, a.Mg, (uint32_t)u) * (p - pn);
             p = pn;
         }
     }
     for (; u < u1; ++u) {
         const uint64_t j = wheel_y(wj + (u - nd));
-        acc += (uint64_t)wheel_M(a.segoff, a.Mloc, wheel_index((uint32_t)((uint64_t)(k / j) - a.y0)));
+        acc += (uint64_t)wheel_M(a.segoff, a.Mg, wheel_index((uint32_t)((uint64_t)(k / j) - a.y0)));
     }
     acc = warp_sum_u64(acc);
     if ((threadIdx.x & 31) == 0)
@@ -1187,7 +1166,7 @@ __global__ void __launch_bounds__(kWideThreads) wheel_wide_kernel(WheelWideArgs 
             for (uint32_t m = 2; m <= 6; m += (m == 2 ? 1u : 3u)) {
                 const u128d y = k / m;
                 if (m >= W.jlo && y > a.y0 && y <= a.y0 + a.len) {
-                    const int64_t v = wheel_M(a.segoff, a.Mloc,
+                    const int64_t v = wheel_M(a.segoff, a.Mg,
                                               wheel_index((uint32_t)((uint64_t)y - a.y0)));
                     tail += m == 6 ? v : -v;
                 }
@@ -1201,7 +1180,7 @@ __global__ void __launch_bounds__(kWideThreads) wheel_wide_kernel(WheelWideArgs 
 // Resident tables.
 // ---------------------------------------------------------------------------
 __global__ void wheel_lookup_kernel(const uint64_t *__restrict__ pairs, uint32_t count,
-                                    const int16_t *__restrict__ Mloc,
+                                    const uint2 *__restrict__ Mg,
                                     const int64_t *__restrict__ segoff, uint64_t *__restrict__ R)
 {
     const uint32_t i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -1210,16 +1189,16 @@ __global__ void wheel_lookup_kernel(const uint64_t *__restrict__ pairs, uint32_t
     const uint64_t y = pairs[2 * i + 1];
     const auto M6 = [&](uint64_t v) -> int64_t {
         const uint64_t w = phi6(v);
-        return w ? segoff[(w - 1) >> kSegShift] + (int64_t)Mloc[w - 1] : 0;
+        return w ? wheel_M(segoff, Mg, w - 1) : 0;
     };
     R[pairs[2 * i]] = (uint64_t)(M6(y) - M6(y / 2) - M6(y / 3) + M6(y / 6));
 }
 
-__global__ void wheel_carry_at_kernel(const int16_t *__restrict__ Mloc,
+__global__ void wheel_carry_at_kernel(const uint2 *__restrict__ Mg,
                                       const int64_t *__restrict__ segoff, uint64_t w,
                                       int64_t *__restrict__ out)
 {
-    *out = segoff[w >> kSegShift] + (int64_t)Mloc[w];
+    *out = wheel_M(segoff, Mg, w);
 }
 
 // ---------------------------------------------------------------------------
@@ -1346,10 +1325,10 @@ static int sm_count()
     return sms;
 }
 
-int wheel_dense_list_enqueue(const int16_t *Mloc, uint64_t c0, uint64_t nchunks, uint16_t *dl,
+int wheel_dense_list_enqueue(const uint2 *Mg, uint64_t c0, uint64_t nchunks, uint16_t *dl,
                              uint32_t *dl_cnt, cudaStream_t s)
 {
-    wheel_dense_list_kernel<<<(unsigned)nchunks, 256, 0, s>>>(Mloc, c0, dl, dl_cnt);
+    wheel_dense_list_kernel<<<(unsigned)nchunks, 256, 0, s>>>(Mg, c0, dl, dl_cnt);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
@@ -1405,19 +1384,19 @@ int wheel_wide_enqueue(const WheelWideArgs &a, uint32_t nw, uint64_t units, cuda
     return cudaGetLastError() == cudaSuccess ? n : -1;
 }
 
-int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const int16_t *Mloc,
+int wheel_lookup_enqueue(const uint64_t *pairs, uint32_t count, const uint2 *Mg,
                          const int64_t *segoff, uint64_t *R, cudaStream_t s)
 {
     if (count == 0)
         return 0;
-    wheel_lookup_kernel<<<(count + 127) / 128, 128, 0, s>>>(pairs, count, Mloc, segoff, R);
+    wheel_lookup_kernel<<<(count + 127) / 128, 128, 0, s>>>(pairs, count, Mg, segoff, R);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
-int wheel_carry_at_enqueue(const int16_t *Mloc, const int64_t *segoff, uint64_t y0, int64_t *out,
+int wheel_carry_at_enqueue(const uint2 *Mg, const int64_t *segoff, uint64_t y0, int64_t *out,
                            cudaStream_t s)
 {
-    wheel_carry_at_kernel<<<1, 1, 0, s>>>(Mloc, segoff, y0 / 3 - 1, out);
+    wheel_carry_at_kernel<<<1, 1, 0, s>>>(Mg, segoff, y0 / 3 - 1, out);
     return cudaGetLastError() == cudaSuccess ? 1 : -1;
 }
 
