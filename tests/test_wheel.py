@@ -112,3 +112,19 @@ def test_linear_estimate_of_the_dense_terms():
         est = float(R) * float(f(1.0) / f(3 * y))
         exact = (k - 3 * y * q0) / (3 * y)
         assert abs(est - exact) < 1 / 3 and abs(exact) < 1.0e6
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("env", [None, "MERTENS_SIEVE_BUCKETS"])
+@pytest.mark.parametrize("y1,ln", [(1, 40_003), (10**9 + 4, 131_073), (10**9 + 5, 98_305),
+                                   (10**12 + 2, 400_001), (10**12 + 3, 262_147)])
+def test_bucketed_sieve_leaves_out_the_multiples_of_4(env, y1, ln, monkeypatch):
+    """mu from every start mod 4 (the bucketed kernel's primes give the multiples of
+    4 no weight), over several tiles and with primes below, in and above a tile."""
+    import torch
+
+    if env:
+        monkeypatch.setenv(env, "1")
+    out = torch.empty(ln, dtype=torch.int8, device="cuda")
+    pm.mertens_sieve_mu(y1, ln, out)
+    assert np.array_equal(out.cpu().numpy(), oracle.mu_window(y1, ln))
