@@ -91,7 +91,9 @@ int mertens_set_allocator(mertens_alloc_fn alloc, mertens_free_fn release, void 
  *              block by block); 0 = chosen by the library.  Any value >= 1
  *              is taken; whole runs, whose M(y) takes a third of the memory
  *              per y of a window plan's, make blocks of three times block_len,
- *              up to a multiple of 6144 (results do not depend on it).
+ *              up to a multiple of 6144, and a window longer than block_len
+ *              blocks of four times block_len (at most 2^30, and where the
+ *              memory for it is there).  Results do not depend on it.
  *
  * Allocates all device memory of the plan on the current device (through the
  * hook above).  Small kernels that make the plan's tables run on a stream of
@@ -285,26 +287,24 @@ typedef struct {
     uint64_t terms;       /* direct + gathered update terms, all targets    */
     uint64_t kernels;     /* kernel launches of the last run                */
     uint64_t dense_y;     /* y values covered by the dense (mu-form) part,
-                             summed over entries                            */
+                             summed over entries (whole runs evaluate the
+                             squarefree ones coprime to 6)                  */
     uint64_t gather_j;    /* gathered terms (one per j), all entries        */
-    double sieve_updates; /* sieve updates: sum over blocks of the block
-                             length times sum_{p <= sqrt(block end)}
-                             (1/p + 1/p^2)                                  */
+    double sieve_updates; /* sieve updates: sum over blocks of the numbers
+                             sieved times the sum over the sieving primes of
+                             1/p + 1/p^2 (whole runs: the y coprime to 6 and
+                             5 <= p <= sqrt(block end); window plans: every y
+                             and p)                                         */
     uint64_t h2d_bytes;   /* host-to-device bytes of the plan's inputs      */
     uint64_t d2h_bytes;   /* device-to-host bytes read by mertens_result
                              since the last mertens_run                     */
-    uint64_t gather_j_exec; /* gathered terms evaluated: entry 2x takes the
-                             terms at j' <= floor(jtop_x/2) from entry x's
-                             even j (floor(floor(n/x)/2j') =
-                             floor(floor(n/2x)/j')), so these are fewer
-                             than gather_j                                  */
-    uint64_t dense_odd_skip; /* odd y left out of the dense sums, summed over
-                             entries: entry 2x takes its odd-y terms up to
-                             half of entry x's cut-off from entry x's
-                             even-y terms (mu(y) floor(floor(n/2x)/y) =
-                             -mu(2y) floor(floor(n/x)/2y)); the squarefree
-                             ones among them, about 8/pi^2 of these, are
-                             not evaluated                                  */
+    uint64_t gather_j_exec; /* gathered terms evaluated: in whole runs those
+                             with j coprime to 6; in window plans all but
+                             those entry 2x takes from entry x's even j
+                             (floor(floor(n/x)/2j) = floor(floor(n/2x)/j))  */
+    uint64_t dense_odd_skip; /* y left out of the dense sums beside those of
+                             dense_y that are not coprime to 6 (whole runs) or
+                             not squarefree: none                           */
 } mertens_run_stats;
 
 /* Enables (1) or disables (0) per-phase events for later runs of `plan`

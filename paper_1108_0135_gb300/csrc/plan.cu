@@ -1010,7 +1010,7 @@ static int wheel_counts(mertens_plan_s *p)
 static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count, mertens_u128 u,
                        uint64_t block_len, const mertens_tuning &tn, bool window = false,
                        uint64_t w_first = 1, uint64_t w_last = UINT64_MAX,
-                       mertens_table_s *table = nullptr)
+                       mertens_table_s *table = nullptr, bool widen = true)
 {
     if (!out)
         return MERTENS_EINVAL;
@@ -1327,6 +1327,12 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         delete p;
         return MERTENS_EINVAL;
     }
+    // a longer window's blocks hold four times as many y, up to 2^30: the sieve sets
+    // up every large prime per block and SM, and each block has seven launches (16
+    // blocks of 2^28 y from 10^13, n = 10^20: 12.55 -> 10.12 ms as four).  Without
+    // the memory for it: block_len y (mertens_plan_window)
+    if (window && widen && span > block_len)
+        block_len = std::max(block_len, std::min({4 * block_len, (uint64_t)1 << 30, span}));
     p->block_len = block_len;
     p->nblocks = (span + block_len - 1) / block_len;
     if (window) {
@@ -2545,7 +2551,11 @@ int mertens_plan_window(mertens_plan_t *out, const mertens_u128 *n, size_t count
         set_last_error("mertens_plan_window: need 1 <= y_first <= y_last");
         return MERTENS_EINVAL;
     }
-    return plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last);
+    const int rc = plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last);
+    if (rc != MERTENS_ENOMEM)
+        return rc;
+    return plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last, nullptr,
+                       false);
 }
 
 int mertens_window_result(mertens_plan_t p, size_t i, uint64_t *S_loc, uint64_t *coef,

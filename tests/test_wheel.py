@@ -128,3 +128,20 @@ def test_bucketed_sieve_leaves_out_the_multiples_of_4(env, y1, ln, monkeypatch):
     out = torch.empty(ln, dtype=torch.int8, device="cuda")
     pm.mertens_sieve_mu(y1, ln, out)
     assert np.array_equal(out.cpu().numpy(), oracle.mu_window(y1, ln))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n,u,y1,ny", [(10**14 + 7, 3 * 10**9, 10**8 + 3, 5 * 10**6 + 11),
+                                       (10**20, 21544346900318, 10**12 + 2, 3 * 10**7 + 1)])
+def test_window_does_not_depend_on_the_block_length(n, u, y1, ny):
+    """A window in one block and in blocks of four times block_len, the last one
+    ragged: the same sums, carry coefficients and mu sum."""
+    got = []
+    for bl in (ny, ny // 5, ny // 13 + 1):
+        plan = pm.mertens_plan_window([n], y1, y1 + ny - 1, u, bl)
+        pm.mertens_run(plan)
+        got.append(pm.mertens_window_result(plan, 0))
+        pm.mertens_destroy(plan)
+    for S, coef, mu in got[1:]:
+        assert mu == got[0][2]
+        assert np.array_equal(S, got[0][0]) and np.array_equal(coef, got[0][1])
