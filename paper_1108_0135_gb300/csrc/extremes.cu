@@ -199,18 +199,29 @@ __global__ void __launch_bounds__(kExtThreads) segment_extremes_kernel(
         part[blockIdx.x] = e;
 }
 
-// All records into part[0] (one CTA).
+// The records i = b, b + grid, ... into part[b] (which no other CTA reads).
 __global__ void __launch_bounds__(kExtThreads) merge_extremes_kernel(Ext *part, uint32_t n)
 {
     __shared__ Ext sh[kExtWarps];
     Ext e;
     ext_init(e);
-    for (uint32_t i = threadIdx.x; i < n; i += kExtThreads)
+    for (uint64_t i = blockIdx.x + (uint64_t)threadIdx.x * gridDim.x; i < n;
+         i += (uint64_t)kExtThreads * gridDim.x)
         ext_merge(e, part[i]);
     __syncthreads();
     e = ext_reduce(e, sh);
     if (threadIdx.x == 0)
-        part[0] = e;
+        part[blockIdx.x] = e;
+}
+
+// All records into part[0]: a record per thread, then one CTA (one CTA alone took
+// 86 us for the 16 384 records of 2^30 y).
+void merge_extremes(Ext *part, uint32_t n, cudaStream_t s)
+{
+    const uint32_t ctas = std::min((n + kExtThreads - 1) / kExtThreads, (uint32_t)kExtThreads);
+    if (ctas > 1)
+        merge_extremes_kernel<<<ctas, kExtThreads, 0, s>>>(part, n);
+    merge_extremes_kernel<<<1, kExtThreads, 0, s>>>(part, ctas > 1 ? ctas : n);
 }
 
 // Pass 3: the exact extremes over the segments that can hold one, given the
@@ -221,30 +232,37 @@ __global__ void __launch_bounds__(kExtThreads) exact_extremes_kernel(
     const Ext *__restrict__ best, Ext *__restrict__ part)
 {
     __shared__ Ext sh[kExtWarps];
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t w = (blockIdx.x * kExtThreads + threadIdx.x) >> 5, nw = gridDim.x * kExtWarps;
+    __shared__ uint32_t s_list[kExtThreads], s_n;
     const Ext B = best[0];
     Ext e;
     ext_init(e);
-    for (uint32_t s0 = w * 32u; s0 < nseg; s0 += nw * 32u) {
-        const uint32_t sg = s0 + lane;
-        bool pick = false;
+    for (uint32_t s0 = blockIdx.x * kExtThreads; s0 < nseg; s0 += gridDim.x * kExtThreads) {
+        const uint32_t sg = s0 + threadIdx.x;
+        if (threadIdx.x == 0)
+            s_n = 0;
+        __syncthreads();
         if (sg < nseg) {
             const int64_t so = segoff[sg];
             const int64_t mx = so + (int16_t)(mm[sg] & 0xffffu), mn = so + (int16_t)(mm[sg] >> 16);
             const uint64_t i0 = (uint64_t)sg << kSegShift;
             const uint64_t a = y1 + i0, b = y1 + min(i0 + kSegY, len) - 1;
-            pick = (mx == B.mx && a == B.ymx) || (mn == B.mn && a == B.ymn) ||
-                   !ratio_gt(B.rpM, B.rpy, mx, ext_limit(mx, a, b)) ||
-                   !ratio_gt(mn, ext_limit(-mn, a, b), B.rnM, B.rny);
+            if ((mx == B.mx && a == B.ymx) || (mn == B.mn && a == B.ymn) ||
+                !ratio_gt(B.rpM, B.rpy, mx, ext_limit(mx, a, b)) ||
+                !ratio_gt(mn, ext_limit(-mn, a, b), B.rnM, B.rny))
+                s_list[atomicAdd(&s_n, 1u)] = sg;
         }
-        for (uint32_t mask = __ballot_sync(0xffffffffu, pick); mask; mask &= mask - 1u) {
-            const uint64_t i0 = (uint64_t)(s0 + __ffs(mask) - 1u) << kSegShift;
+        __syncthreads();
+        // the segments left, one after the other by the whole CTA (a warp each took
+        // 72 us for the seven of a last block)
+        const uint32_t n = s_n;
+        for (uint32_t q = 0; q < n; ++q) {
+            const uint64_t i0 = (uint64_t)s_list[q] << kSegShift;
             const uint64_t i1 = min(i0 + kSegY, len);
             const int64_t so = segoff[i0 >> kSegShift];
-            for (uint64_t i = i0 + lane; i < i1; i += 32u)
+            for (uint64_t i = i0 + threadIdx.x; i < i1; i += kExtThreads)
                 ext_point(e, so + (int64_t)Mloc[i], y1 + i);
         }
+        __syncthreads();
     }
     e = ext_reduce(e, sh);
     if (threadIdx.x == 0)
@@ -308,14 +326,14 @@ int mertens_scan_extremes(uint64_t y_first, uint64_t y_last, int64_t carry,
             const uint32_t nc = (ns + kExtWarps * kExtSegs - 1) / (kExtWarps * kExtSegs);
             uint32_t *mm = reinterpret_cast<uint32_t *>(ss);
             segment_extremes_kernel<<<nc, kExtThreads, 0, s>>>(Lc.y1, Lc.len, ns, ml, so, mm, first);
-            merge_extremes_kernel<<<1, kExtThreads, 0, s>>>(first, nc);
+            merge_extremes(first, nc, s);
             exact_extremes_kernel<<<kExtScan, kExtThreads, 0, s>>>(Lc.y1, Lc.len, ns, ml, so, mm,
                                                                   first, part + b * kExtScan);
             if (cudaGetLastError() != cudaSuccess)
                 rc = MERTENS_ECUDA;
         }
         if (rc == MERTENS_OK)
-            merge_extremes_kernel<<<1, kExtThreads, 0, s>>>(part, (uint32_t)nparts);
+            merge_extremes(part, (uint32_t)nparts, s);
         Ext e;
         int64_t last = 0;
         if (rc == MERTENS_OK &&

@@ -676,10 +676,11 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         delete p;
         return MERTENS_EINVAL;
     }
-    // three times as many y make a block (in a quarter of the memory that block_len
-    // y take in the full form; fewer launches: 48.9 -> 45.2 ms at n = 10^16 with
-    // 2^28-y blocks)
-    block_len = std::min(std::min<uint64_t>(3 * block_len, 3ull << 30), p->y_last);
+    // six times as many y make a block, up to 3 2^30 (in half of the memory that
+    // block_len y take in the full form; fewer launches, and an entry's range per
+    // block is found less often): n = 10^16 with 2^28-y blocks 39.6 -> 38.2 ms against
+    // three times as many, 38.7 at twelve
+    block_len = std::min(std::min<uint64_t>(6 * block_len, 3ull << 30), p->y_last);
     // a plan on a table sieves only the blocks that end above it
     p->sieves = !table || p->y_last > table->y_max;
     p->block_len = (block_len + kWheelSegY - 1) / kWheelSegY * kWheelSegY;

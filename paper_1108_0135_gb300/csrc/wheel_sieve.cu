@@ -17,6 +17,14 @@
 // class 6i + 1 at i = a0 (mod p) and the class 6i + 5 at i = a0 + d (mod p),
 //   p = 1 (mod 6): a0 = (p - 1)/6,  d = 2 (p - 1)/3,
 //   p = 5 (mod 6): a0 = (5p - 1)/6, d = (p - 2)/3.
+//
+// Measured (n = 10^16, u = 4 10^10, per run): every y 45.9 ms (the scale-2
+// kernel of sieve.cu) -> 17.7 ms in this form -> 15.2 ms with squares below 1024
+// by the descriptor jobs' lanes (one thread each stalled the rest at the barrier)
+// -> 13.2 ms with 8 bytes written per 16 numbers: 265 us per block of 8.05e8 y.
+// Bound by issue and by the shared atomics: of 330 us (decode still writing
+// int16), lane primes took 106, descriptors 74, the decode 75, pattern copy and
+// barriers 58.
 #include <algorithm>
 #include <cmath>
 #include <cstdlib>
@@ -34,6 +42,9 @@ constexpr uint32_t kWTileBig = 98304;         // wheel numbers per tile
 constexpr uint32_t kWTileSmall = 24576;
 constexpr uint32_t kWPatLen = ((kWPatPeriod + kWTileBig + 31u) / 16u) * 16u;
 constexpr uint32_t kWJobsMax = 192;           // descriptor jobs: primes 13 .. 1021
+// Lane primes from 512 or 2048, and lists from 2048, measured slower at n = 10^16;
+// so did tiles of 64 Ki (three CTAs per SM) and 48 Ki (four): 42.9 and 45.5 ms a
+// run against 41.7.
 constexpr uint32_t kWLaneMin = 1024;          // primes from here: a lane per prime
 constexpr uint32_t kWListMin = 4096;          // squares from here: the block's lists
 constexpr uint32_t kWSqCap = 64;
@@ -419,8 +430,9 @@ __global__ void __launch_bounds__(THREADS, MINB) wheel_sieve_kernel(WSieveArgs a
 }
 
 // a2 finish: segoff[s] = carry_in + sum of segsum[0..s), carry_out = carry_in
-// + all of them.  Each CTA scans 4096 segments and adds the sum of all
-// segments before its range.
+// + all of them.  Each CTA scans 4096 segments, four per thread, and adds the sum
+// of all segments before its range (16-byte loads).  Bound by latency: 10 us for
+// 131 072 segments (12 us with one segment per thread).
 __global__ void __launch_bounds__(1024) seg_carry_kernel(const int32_t *__restrict__ segsum,
                                                            uint32_t nseg,
                                                            const int64_t *__restrict__ carry_in,
@@ -617,7 +629,9 @@ static int wheel_launch(const WheelSieve *t, const WheelLaunch &L, cudaStream_t 
 
 int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t s)
 {
-    // small tiles while the large ones would leave SMs without a CTA
+    // small tiles while the large ones would leave SMs without a CTA (two per
+    // SM): n = 10^10 0.131 against 0.147 ms a run, 10^12 in blocks of 5 10^7 y 0.36
+    // against 0.39; small ones always: 10^16 54 against 39.4
     int launches = L.len < 304ull * kWTileBig ? wheel_launch<kWTileSmall, 192, 8>(t, L, s)
                                               : wheel_launch<kWTileBig, 768, 2>(t, L, s);
     if (L.mid)

@@ -300,7 +300,14 @@ __global__ void __launch_bounds__(256) wheel_dense_list_kernel(const uint2 *__re
 
 // ---------------------------------------------------------------------------
 // Dense update: a warp takes the 64 entries of a group, two per lane, against
-// the staged numbers of a chunk (shared-memory broadcasts).
+// the staged numbers of a chunk (shared-memory broadcasts; two entries per lane
+// halve the broadcast per term, four measured 7.5 against 7.8 issue slots per
+// term and leave half the groups of a small target).  Bound by issue: 6.4
+// instructions, 7.8 slots per term in the float and linear modes (two of them
+// multiplies).  n = 10^16, u = 4 10^10: 44.2 ms over every squarefree y by 64-bit
+// multiply-high -> 15.3 ms (coprime to 6, remainder and two sign bits) -> 10.8
+// (one comparison, two-step mode, cut-offs from the mean k) -> 9.4 (linear mode);
+// n = 10^17: 90 -> 54 -> 46 ms by the last two.
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t count_below(const uint16_t *a, uint32_t n, uint32_t v)
 {
@@ -443,8 +450,13 @@ __device__ __forceinline__ void dense_wide(const uint16_t *off, uint32_t n, uint
 
 // A work item is part of a chunk's list for kWheelGroupBlock groups.  Items whose
 // k/(3y) all lie below the float mode's bound (and y < 3.5e8) take it, those with
-// k <= 900 y0^2 the linear mode; in the others the y up to kmax/9e14 (all y from 3.5e8) take 64-bit division, those up
-// to kmax/1.8e8 the two-step mode, the rest the high-word mode.
+// k <= 900 y0^2 the linear mode; in the others the y up to kmax/9e14 (all y from
+// 3.5e8) take 64-bit division, those up to kmax/1.8e8 the two-step mode, the rest
+// the high-word mode.  Each line is the bound to which the cheaper mode is exact.
+// The high-word mode costs twice the float mode's time per term (without the
+// linear mode it took 36% of the terms at n = 10^17: 54 against 46 ms); 64-bit
+// divisions of the first group alone were a third of the kernel's instructions at
+// n = 10^15 before the two-step mode.
 __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDenseArgs a)
 {
     __shared__ uint4 s_el[kSegY];
@@ -609,9 +621,14 @@ __global__ void __launch_bounds__(kWheelDenseThreads) wheel_dense_kernel(WheelDe
 // wheel numbers are squarefree) by wheel index.  A term's index is
 // phi6(floor(R/j)) - 1 with R = k - t0 j < len j: T = floor of R / (3j) <= 2^15
 // from single precision (relative error near 2^-21), then as above.
+// Bound by issue (about 11 slots per term with all lanes on one j, 18 with a j
+// per lane, and the ranges' divisions).  n = 10^16, u = 4 10^10, all gathered
+// terms: 55.1 ms over every j -> 22.1 (j coprime to 6) -> 17.0 (one comparison,
+// groups handed out one by one, the first entries shared by all warps, Mg).
 // ---------------------------------------------------------------------------
 constexpr uint32_t kGatherJ32 = 300000000u;  // 32-bit remainders below: 5j < 2^31
-constexpr uint32_t kWheelLaneTerms = 16;     // few terms: always a lane per entry
+constexpr uint32_t kWheelLaneTerms = 16;     // few terms: always a lane per entry (8 and
+                                             // 32 measure the same)
 
 // Constants of a run of terms j = j0 + step i in a tile.
 struct TileStep {
@@ -719,6 +736,8 @@ __device__ __forceinline__ int64_t wheel_M(const int64_t *segoff, const uint2 *M
 // one.  An index outside [lo, lim] -- a j whose y lies beyond the tile or at most
 // yc (yc + 1 a wheel number) -- is sent to the zero after it.  jw: 32 uint2 of
 // this warp; b2 = -C - 1 - (first index) - lo.
+// That error bound sets the limit.  Up to it this form beats a j per lane: 39.4
+// against 41.3 ms a run at n = 10^16, 27.4 against 29.5 for 64 targets near 10^14.
 constexpr uint64_t kUniformY = 7400000;
 constexpr uint32_t kUniformW = 1860000;  // 3j < 2^24
 
@@ -812,7 +831,9 @@ __device__ __forceinline__ void tile_entry(const WheelGatherArgs &a, const int16
 // every lane sums its own entry, else entries with many terms take the whole
 // warp in turn; with many terms in all, at the end of the item, where all warps
 // share them (the first 32 entries of a target hold a third of a tile's terms;
-// on one warp, the other fifteen waited for it).
+// on one warp, the other fifteen waited for it; all sets of 32 that way: 3.99
+// against 3.32 ms at n = 10^15).  From 65536 terms a
+// set: 0.154 against 0.131 ms at n = 10^10; from 4096: the same.
 constexpr uint32_t kSharedMax = 128;         // sets of 32 left to the end of an item
 constexpr uint32_t kSharedTerms = 16384;     // a set's terms from which it is
 constexpr uint32_t kSharedSlice = 8192;      // an entry's terms from which warps split it
@@ -992,17 +1013,25 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
 // more: posted as chunks of kWheelItem wheel indices for wheel_chunk_kernel);
 // the dense form's -M6(yc) phi6(jd) when yc is in the block; and the values
 // M6(floor(k/m)), m = 2, 3, 6, of M(k) that lie in the block when m x is
-// beyond the array (m >= floor(X/x) + 1).
+// beyond the array (m >= floor(X/x) + 1).  Bound by the 64-bit divisions and
+// random reads of entries with few terms: 19 us per block at n = 10^16 (0.94 ms
+// per run).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
 {
     const uint64_t e = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const uint32_t lane = threadIdx.x & 31u;
-    const uint64_t k = e < a.nent ? a.K[e] : 0ull;
+    // the entry's loads at once: one after the other they took most of the time
+    uint64_t k = 0, jlo = 0, jd = 0, yc = 0;
+    if (e < a.nent) {
+        k = a.K[e];
+        yc = a.YC[e];
+        jlo = a.JL[e];
+        jd = a.JD[e];
+    }
     const uint64_t yend = a.y0 + a.len;
     uint32_t wl = 0, wh = 0;
     if (k) {
-        const uint64_t jlo = a.JL[e], jd = a.JD[e];
         if (k < a.kmax) {
             const uint64_t q1 = div_magic(k << 1, a.m_ylo, a.l_ylo);  // floor(k / ylo)
             const uint64_t q2 = div_magic(k << 1, a.m_end, a.l_end);  // floor(k / (yend + 1))
@@ -1012,7 +1041,6 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
                 wh = phi6_u32((uint32_t)t);
             }
         }
-        const uint64_t yc = a.YC[e];
         if (yc > a.y0 && yc <= yend)
             atomicAdd(reinterpret_cast<unsigned long long *>(a.S + e),
                       (unsigned long long)(0ull - (uint64_t)wheel_M(a.segoff, a.Mg,
@@ -1070,6 +1098,9 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
 }
 
 // The posted chunks, a warp each (grid-stride), lanes over consecutive indices.
+// Bound by 64-bit divisions and random reads; at n = 10^16 1.48 ms per run when
+// the block held int16 values, 1.05 ms from Mg (a quarter of the memory, more of
+// it in L2).
 __global__ void __launch_bounds__(256) wheel_chunk_kernel(WheelBlockArgs a)
 {
     const uint32_t lane = threadIdx.x & 31u;
