@@ -89,11 +89,11 @@ int mertens_set_allocator(mertens_alloc_fn alloc, mertens_free_fn release, void 
  *              entries (Sec. 2); X_i >= 2^32 is MERTENS_ENOTSUP.
  *   block_len  length of a sieve block in y (Sec. 3 processes the y-axis
  *              block by block); 0 = chosen by the library.  Any value >= 1
- *              is taken; whole runs, whose M(y) takes a third of the memory
- *              per y of a window plan's, make blocks of three times block_len,
- *              up to a multiple of 6144, and a window longer than block_len
- *              blocks of four times block_len (at most 2^30, and where the
- *              memory for it is there).  Results do not depend on it.
+ *              is taken; whole runs, whose M(y) takes a twelfth of the memory
+ *              per y of a window plan's, make blocks of six times block_len
+ *              (at most 3 2^30), up to a multiple of 6144, and a window longer
+ *              than block_len blocks of four times block_len (at most 2^30, and
+ *              where the memory for it is there).  Results do not depend on it.
  *
  * Allocates all device memory of the plan on the current device (through the
  * hook above).  Small kernels that make the plan's tables run on a stream of
@@ -127,7 +127,7 @@ int mertens_plan(mertens_plan_t *out, const mertens_u128 *n, size_t count,
  *   mertens_plan_on_table: as mertens_plan, on the table's device; u = {0,0}
  *     picks the larger of min(n, y_max + 1) and the automatic limit per
  *     target.  MERTENS_ENOTSUP when a target exceeds n_max or needs dense
- *     cut-offs or divisors beyond the table; block_len must be a multiple of
+ *     cut-offs beyond the table; block_len must be a multiple of
  *     2048 (0: 2^30).  The table must outlive its plans.
  *   mertens_table_destroy: waits for the device, then frees the table.
  */

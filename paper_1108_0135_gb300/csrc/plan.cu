@@ -211,8 +211,8 @@ struct mertens_plan_s {
     bool window = false;
     std::vector<uint64_t> coef;
     uint64_t *dcoef = nullptr;  // the same on the device (window plans)
-    // plans on a resident table: M(y), the divisor magics and the dense list
-    // are the table's; targets n <= table y_max are read from it directly
+    // plans on a resident table: M(y) and the dense list are the table's;
+    // targets n <= table y_max are read from it directly
     // (entry, y) pairs
     mertens_table_s *table = nullptr;
     bool sieves = true;  // some block is sieved (always without a table)
@@ -225,8 +225,8 @@ struct mertens_plan_s {
     PrimeTable pt;
     uint64_t *dK = nullptr, *dJLO = nullptr, *dJC0 = nullptr, *dJCUR = nullptr, *dYCE = nullptr;
     uint32_t *dEMIT = nullptr;
-    uint64_t gather_j_exec = 0;  // gathered terms evaluated (after sharing)
-    uint64_t dense_odd_skip = 0; // odd y left out of dense sums (taken from entries x/2)
+    uint64_t gather_j_exec = 0;  // gathered terms evaluated
+    uint64_t dense_odd_skip = 0; // none (kept for the statistics' layout)
     uint64_t *dS = nullptr, *dR = nullptr;
     // chunks of the global gather's heavy entries, per block (qcap records)
     uint4 *dqueue = nullptr;

@@ -74,10 +74,9 @@ size_t estimate_table_batch_bytes(const std::vector<uint64_t> &ns, uint64_t y_ma
     return above ? estimate_batch_bytes(ns) : (size_t)(110.0 * entries + 64.0e6);
 }
 
-// Device memory a batch's plan will take, estimated from the plan's shapes
-// (entry arrays, one sieve block of int16 M, the divisor-magic table and the
-// squarefree list up to the dense cut-off, dense_c sqrt(n), dense_c at least
-// 1.6), with slack.
+// A bound on the device memory a batch's plan will take, from the plan's shapes:
+// entry arrays, a sieve block (at most 1 byte per y of the block length here) and
+// the squarefree list up to the dense cut-off, dense_c sqrt(n) (2/3 byte per y).
 size_t estimate_batch_bytes(const std::vector<uint64_t> &ns)
 {
     double entries = 0, ymax = 0, nmax = 0;
