@@ -269,6 +269,7 @@ struct mertens_plan_s {
     bool mg_built = false;
     // whole runs over the integers coprime to 6 (wheel.h)
     bool wheel = false;
+    uint32_t long_lane = 0;      // WheelGatherArgs
     bool wheel_long = false;     // 64-bit remainders for every gathered term
     WheelSieve ws;
     uint2 *dMg = nullptr;        // a block's M6 (wheel.h)
@@ -725,6 +726,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     // their few items (0.79 ms at n = 10^13)
     const double item_work = std::min(2.0e6, std::max(4096.0, terms / (456.0 * 24.0)));
     const double item_max = std::max(8192.0, terms / (456.0 * 4.0));
+    // a lane sums an entry's terms of a tile alone up to about the share of two lanes
+    // in all terms (the sets x = 33 .. 256 of a target held one warp while the rest
+    // of the device was done: n = 10^13 0.90 -> 0.77 ms a run, 10^14 2.85 -> 2.72;
+    // for larger n no set is that long, and sharing sets of 2048 terms a lane anyway
+    // took 40.2 against 38.7 ms at 10^16)
+    p->long_lane = (uint32_t)std::min(4.0e9, std::max(2048.0, terms / 1.2e5));
     double yc_min = 1e300;  // about the least dense cut-off
     for (size_t i = 0; i < count; ++i)
         if (qs[i].n || qs[i].n_hi)
@@ -1939,6 +1946,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
             ga.JL = p->dJL;
             ga.JD = p->dJD;
             ga.S = p->dS;
+            ga.long_lane = p->long_lane;
             ga.all_long = p->wheel_long ? 1u : 0u;
             r = wheel_gather_enqueue(ga, s);
             if (r < 0)

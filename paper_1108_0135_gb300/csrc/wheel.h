@@ -201,6 +201,7 @@ struct WheelGatherArgs {
     const uint64_t *K, *YC;
     const uint32_t *JL, *JD;
     uint64_t *S;
+    uint32_t long_lane;     // a lane sums fewer terms of an entry than this
     uint32_t all_long;      // 64-bit remainders for every term
 };
 

@@ -827,8 +827,9 @@ __device__ __forceinline__ void tile_entry(const WheelGatherArgs &a, const int16
 // A work item is one tile and a range of places.  Warps take 64
 // entries at a time, two per lane, and find the ranges of wheel indices of
 // their j.  Low tiles where these ranges nearly coincide take tile_uniform.
-// The others, 32 entries at a time: when the counts are close (or all small)
-// every lane sums its own entry, else entries with many terms take the whole
+// The others, 32 entries at a time: when the counts are close and no lane's sum
+// would take long against the whole kernel (or all are small) every lane sums its
+// own entry, else entries with many terms take the whole
 // warp in turn; with many terms in all, at the end of the item, where all warps
 // share them (the first 32 entries of a target hold a third of a tile's terms;
 // on one warp, the other fifteen waited for it; all sets of 32 that way: 3.99
@@ -945,7 +946,8 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
                 if (mx == 0)
                     continue;
                 const uint32_t hsum = __reduce_add_sync(0xffffffffu, cnt);
-                const bool lanes = mx <= kWheelLaneTerms || 16u * mx <= hsum;
+                const bool lanes =
+                    mx <= kWheelLaneTerms || (16u * mx <= hsum && mx < a.long_lane);
                 if (!lanes && hsum >= kSharedTerms) {
                     uint32_t slot = 0;
                     if (lane == 0)

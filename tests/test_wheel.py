@@ -145,3 +145,19 @@ def test_window_does_not_depend_on_the_block_length(n, u, y1, ny):
     for S, coef, mu in got[1:]:
         assert mu == got[0][2]
         assert np.array_equal(S, got[0][0]) and np.array_equal(coef, got[0][1])
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("n", [3 * 10**12 + 1, 10**13 + 37, 4 * 10**13 + 5])
+def test_long_lanes_equal_the_full_sums(n, monkeypatch):
+    """Targets whose sets of 32 entries have thousands of terms per entry in a tile
+    (all warps share them) give the same array as the full sums."""
+    got = []
+    for share in (None, "0"):
+        if share:
+            monkeypatch.setenv("MERTENS_SHARE", share)
+        plan = pm.mertens_plan([n])
+        pm.mertens_run(plan)
+        got.append(pm.mertens_result(plan, 0, entries=True)[1])
+        pm.mertens_destroy(plan)
+    assert np.array_equal(got[0], got[1])
