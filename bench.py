@@ -385,7 +385,8 @@ def run_sharded(args, world, rank, local):
                   "update_dense": st["dense_ms"], "update_gathered": st["gather_ms"]}
         kernels = int(st["kernels"])
         peaks, _ = load_peaks()
-        roofs = rooflines(phases, st, peaks, int(st["blocks"]), pm.mertens_probe_int_peaks(stream))
+        roofs = rooflines(phases, st, peaks, int(st["blocks"]),
+                          pm.mertens_probe_int_peaks(stream), wheel=False)
     else:
         kernels, roofs = 0, {}
     window = tgt.window
@@ -435,7 +436,7 @@ def run_native(args, world, rank, local):
     plan = pm.mertens_plan(n_list, u, L)
     info = pm.mertens_plan_info(plan, 0)
     terms = info["direct_terms"] + info["gathered_terms"]
-    # warm-up (first run also builds the n-independent divisor table)
+    # warm-up (the second run captures the plan's graph)
     for _ in range(max(args.warmup, 1)):
         pm.mertens_run(plan, stream)
     m_n, _ = pm.mertens_result(plan, 0)
@@ -559,17 +560,16 @@ def run_native(args, world, rank, local):
             "dtype": "int64", "data": "synthetic",
             "config": {"workload": cfg["workload"], "n": n_list[0], "u": u,
                        "block_len": L, "X": info["X"], "terms_per_step": terms,
-                       "M_n": m_n, "l2": "inputs larger than L2 (M block 1 GiB, "
-                                         "divisor table 1.3 GB per step)",
+                       "M_n": m_n, "l2": "inputs larger than L2 (a run writes and reads "
+                                         "6.7 GB of sieve output, block after block)",
                        "parallelism": f"{world} independent replicas"},
             "wall_time_s": ms_max / 1e3,
             # `value` counts the paper's direct + gathered terms (closed form per
-            # entry); the kernels reach the same sums through the mu-form, which
-            # executes one quotient per squarefree y below the dense cut-off and
-            # one per gathered j above it, less the gathered terms entry 2x takes
-            # from entry x's even j (floor(floor(n/x)/2j) = floor(floor(n/2x)/j)):
+            # entry); the kernels reach the same sums over the integers coprime
+            # to 6, in mu-form below the dense cut-off: one term per squarefree y
+            # coprime to 6 there and one per gathered j coprime to 6 above it:
             "terms_executed_per_step": dense_evaluated(stats) + stats["gather_j_exec"],
-            "gathered_terms_shared_per_step": stats["gather_j"] - stats["gather_j_exec"],
+            "gathered_terms_left_out_per_step": stats["gather_j"] - stats["gather_j_exec"],
             "phases_ms": {k: round(v, 3) for k, v in phases.items()},
             "y_sieved_per_s": stats["y_sieved"] * world / (ms_max / 1e3),
             "clocks": clk,
@@ -669,19 +669,18 @@ def window_measure(stream):
 # From ncu captures of the current kernel versions on the n = 10^16 workload
 # (one GB300, --clock-control none), per kernel class:
 #   dram_bytes_per_step: dram__bytes_read.sum + dram__bytes_write.sum summed
-#     over all of the class's launches in one run (a run of the capture, or
-#     one captured launch times the launches per run where every launch does
-#     the same work per y), None when a kernel of the class changed since;
+#     over all of the class's launches in one run, None when a kernel of the
+#     class changed since;
 #   issue_active: smsp__issue_active.avg.pct_of_peak_sustained_active of the
 #     class's main kernel (share of cycles a scheduler issued an instruction);
 #   pipe: the busiest pipe of that kernel and its share of active cycles.
 NCU = {
-    "mu_sieve": {"kernel": "mu_sieve_t2_kernel", "dram_bytes_per_step": 72.3e9,
-                 "issue_active": 0.666, "pipe": ("alu", 0.436)},
-    "update_dense": {"kernel": "dense_update_kernel", "dram_bytes_per_step": 0.87e9,
-                     "issue_active": 0.446, "pipe": ("fmaheavy", 0.799)},
-    "update_gathered": {"kernel": "gather_tile_kernel", "dram_bytes_per_step": 13.9e9,
-                        "issue_active": 0.830, "pipe": ("fmaheavy", 0.668)},
+    "mu_sieve": {"kernel": "wheel_sieve_kernel", "dram_bytes_per_step": 5.19e9,
+                 "issue_active": 0.678, "pipe": ("alu", 0.423)},
+    "update_dense": {"kernel": "wheel_dense_kernel", "dram_bytes_per_step": 0.028e9,
+                     "issue_active": 0.850, "pipe": ("alu", 0.691)},
+    "update_gathered": {"kernel": "wheel_gather_kernel", "dram_bytes_per_step": 4.26e9,
+                        "issue_active": 0.839, "pipe": ("fmaheavy", 0.651)},
 }
 # Issue slots of the chip: 152 SMs x 4 schedulers x one warp instruction per
 # clock at the maximum SM clock.
@@ -690,43 +689,47 @@ ISSUE_PEAK_WARP_INSTR_PER_S = 152 * 4 * 2070e6
 SIX_OVER_PI2 = 6.0 / math.pi ** 2
 
 
-def dense_evaluated(stats):
-    """Squarefree y the dense kernel evaluates: (6/pi^2) of the summed dense
-    y-ranges, less the odd squarefree y (8/pi^2 of the odd y) that entries 2x
-    take from entries x (mu(y) floor(floor(n/2x)/y) = -mu(2y) floor(floor(n/x)/2y))."""
-    return SIX_OVER_PI2 * stats["dense_y"] - (4.0 / 3.0) * SIX_OVER_PI2 * stats["dense_odd_skip"]
+def dense_evaluated(stats, wheel=True):
+    """Squarefree y the dense kernel evaluates: 6/pi^2 of the summed dense
+    y-ranges in a window plan, half of that (3/pi^2: those coprime to 6) in a
+    whole run."""
+    return SIX_OVER_PI2 * stats["dense_y"] * (0.5 if wheel else 1.0)
 
 
-def rooflines(phases, stats, peaks, nblocks, ipk):
+def rooflines(phases, stats, peaks, nblocks, ipk, wheel=True):
     """Roofline records per kernel class of the timed region.
 
     Every class here is bound by integer issue (no tensor cores, no floating
-    point contraction; HBM traffic is about 2 B per sieved y).  MEASURED_PEAKS
-    holds no integer figure, so `peak` is the speed of the class's own inner
-    step, measured on this device by mertens_probe_int_peaks (ipk: independent
-    chains of that step on every SM) -- `frac` is the fraction of that
-    inner-step speed, not of a chip pipe peak.  Beside it, `issue` gives the
-    ncu issue-active share of the class's main kernel and its busiest pipe
-    (NCU above), against the chip's issue slots.
-      update_dense: the update's inner step acc += mulhi64(m, 2k) >> l, in
-        terms/s.  Units: squarefree y the kernel evaluates (dense_evaluated).
-      update_gathered: one term per gathered j evaluated (entry 2x takes
-        part of its terms from entry x's even j, so fewer than the method's
-        gathered terms), against the faster of that step and the
-        shared-memory gather's float-estimate quotient step (the tile kernel
-        takes the latter, the global path the former).
+    point contraction; HBM traffic is about 0.17 B per sieved y).
+    MEASURED_PEAKS holds no integer figure, so `peak` is the speed of an inner
+    step measured on this device by mertens_probe_int_peaks (ipk: independent
+    chains of that step on every SM) -- `frac` is the fraction of that step's
+    speed, not of a chip pipe peak.  Beside it, `issue` gives the ncu
+    issue-active share of the class's main kernel and its busiest pipe (NCU
+    above), against the chip's issue slots.
+      update_dense: squarefree y the kernel evaluates (dense_evaluated) per
+        second.  A whole run's kernel forms no full quotient; its peak is the
+        chip's issue slots over the 6.4 instructions of its inner loop per
+        term.  Window plans: the 64-bit step acc += mulhi64(m, 2k) >> l.
+      update_gathered: one term per gathered j evaluated (whole runs: j coprime
+        to 6), against the faster of that step and the float-estimate quotient
+        step.
       mu_sieve: 32-bit ALU lane operations/s (LOP3 + IADD3 chains).
-        Algorithmic operations: one per sieve update (y, p | y or p^2 | y
-        for every sieving prime p) plus two per y (decision + scan add).
+        Algorithmic operations: one per sieve update (y, p | y or p^2 | y for
+        every sieving prime p) plus two per sieved number (decision + scan add;
+        whole runs sieve the third of the y coprime to 6).
     `achieved` and `traffic` are per step (all launches of the class)."""
     sm_mhz = peaks.get("sm_max_mhz", 2070.0)
     mulhi_peak = ipk["mulhi_terms_per_s"] / 1e12
+    dense_peak = 32.0 * ISSUE_PEAK_WARP_INSTR_PER_S / 6.4 / 1e12 if wheel else mulhi_peak
     alu_peak = 2.0 * ipk["alu_pairs_per_s"] / 1e12
     gather_peak = max(ipk["mulhi_terms_per_s"], ipk.get("fquot_terms_per_s", 0.0)) / 1e12
     work = {
-        "mu_sieve": (stats["sieve_updates"] + 2.0 * stats["y_sieved"], alu_peak, "T int-op/s",
+        "mu_sieve": (stats["sieve_updates"] + 2.0 * stats["y_sieved"] / (3.0 if wheel else 1.0),
+                     alu_peak, "T int-op/s",
                      "inner-step probe: LOP3+IADD3 chains on all SMs, 2 ops per pair"),
-        "update_dense": (dense_evaluated(stats), mulhi_peak, "T mulhi-terms/s",
+        "update_dense": (dense_evaluated(stats, wheel), dense_peak, "T terms/s",
+                         "issue slots x 32 lanes / 6.4 instructions per term" if wheel else
                          "inner-step probe: acc += mulhi64(m,2k) >> l chains on all SMs"),
         "update_gathered": (float(stats["gather_j_exec"]), gather_peak, "T terms/s",
                             "inner-step probe: the faster of the mulhi64 step and the "
@@ -738,10 +741,12 @@ def rooflines(phases, stats, peaks, nblocks, ipk):
         if ms <= 0:
             continue
         achieved = v / (ms / 1e3) / 1e12
-        nc = NCU[k]
+        # the captures are of whole runs: a window plan's kernels are others
+        nc = NCU[k] if wheel else {"kernel": None, "dram_bytes_per_step": None,
+                                   "issue_active": None, "pipe": (None, None)}
         out[k] = {"bound": "alu", "kernel": k, "achieved": achieved, "peak": peak,
                   "unit": unit, "frac": achieved / peak,
-                  "frac_of": "the class's inner-step speed measured by the probe",
+                  "frac_of": "the speed named in peak_source",
                   "traffic": nc["dram_bytes_per_step"], "traffic_per": "step",
                   "issue": {"kernel": nc["kernel"], "ncu_issue_active": nc["issue_active"],
                             "busiest_pipe": nc["pipe"][0], "pipe_active": nc["pipe"][1],

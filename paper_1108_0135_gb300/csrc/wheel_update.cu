@@ -1016,8 +1016,8 @@ __global__ void __launch_bounds__(512, 3) wheel_gather_kernel(WheelGatherArgs a)
 // the dense form's -M6(yc) phi6(jd) when yc is in the block; and the values
 // M6(floor(k/m)), m = 2, 3, 6, of M(k) that lie in the block when m x is
 // beyond the array (m >= floor(X/x) + 1).  Bound by the 64-bit divisions and
-// random reads of entries with few terms: 19 us per block at n = 10^16 (0.94 ms
-// per run).
+// random reads of entries with few terms, and by latency: at n = 10^16 0.64 ms per run
+// of 25 blocks (with the entry's loads one after the other 17 us per block).
 // ---------------------------------------------------------------------------
 __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
 {
@@ -1102,7 +1102,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
 // The posted chunks, a warp each (grid-stride), lanes over consecutive indices.
 // Bound by 64-bit divisions and random reads; at n = 10^16 1.48 ms per run when
 // the block held int16 values, 1.05 ms from Mg (a quarter of the memory, more of
-// it in L2).
+// it in L2), 0.94 ms in blocks of 1.6e9 y.
 __global__ void __launch_bounds__(256) wheel_chunk_kernel(WheelBlockArgs a)
 {
     const uint32_t lane = threadIdx.x & 31u;
