@@ -1106,6 +1106,10 @@ __global__ void __launch_bounds__(THREADS, MINB) mu_sieve_t2_kernel(T2Args a)
 // Multiples of p^2 for p >= 2048 come from a bit array over the block made by
 // square_bits_kernel; primes below 2048 are set up per tile as in the byte
 // kernel.  The tile's bytes, decode and scan are those of the byte kernel.
+// Bound by the latency of bucket loads and shared atomics at half occupancy (one
+// tile and the medium primes fill an SM's shared memory).  2^28 y at 10^13: 912 us
+// -> 769 (four entries in flight per lane) -> 690 (multiples of 4 left out); 2^30 y:
+// 2.39 ms.
 // ---------------------------------------------------------------------------
 constexpr uint32_t kMedMax = 12288;          // primes in [2048, 2^17): 11942
 constexpr uint32_t kPersistTilesMax = 128;   // tiles per CTA (blocks <= 2^30 y, >= 64 CTAs)
@@ -1388,7 +1392,8 @@ __device__ __forceinline__ uint32_t byte_weight(uint32_t p, uint32_t S)
 }
 
 // Everything a prime's records hold, from the prime alone (the host uploads
-// only the primes).
+// only the primes; with records and patterns made on the host and uploaded, a
+// window call of 10^6 y took 0.58 ms against 0.16).
 __global__ void prime_records_kernel(uint32_t np, const uint32_t *__restrict__ primes,
                                      uint32_t *__restrict__ lg, uint64_t *__restrict__ m,
                                      uint8_t *__restrict__ l, uint32_t S, uint4 *__restrict__ pq,
@@ -1777,8 +1782,9 @@ int sieve_block_enqueue(const PrimeTable *t, const SieveLaunch &L, cudaStream_t 
         b.extra_tx = (getenv("MERTENS_TEST_STALL_COPY") && t->perr) ? 16u : 0u;
         const uint32_t btiles = (uint32_t)((L.len + kByteTile - 1) / kByteTile);
         // the bucketed kernel pays once the primes above 2^17 outnumber the
-        // medium ones (2048 <= p < 2^17) more than 3:1 (measured crossover
-        // near y = 4e11); MERTENS_SIEVE_TILES / MERTENS_SIEVE_BUCKETS force
+        // medium ones (2048 <= p < 2^17) more than 3:1 (near y = 4e11; 2^32 y
+        // in blocks of 2^28: scale-2 kernel 7.4 ms at 3e11, 10.0 at 1e12, 14.0
+        // at 3e12, bucketed 9.4 and 10.3 at the last two); MERTENS_SIEVE_TILES / MERTENS_SIEVE_BUCKETS force
         // one kernel (tests)
         const uint32_t nmid = std::min(t->np_mid, np);
         bool persist = np - nmid > 3u * (nmid - std::min(np_small, nmid));

@@ -161,3 +161,38 @@ def test_long_lanes_equal_the_full_sums(n, monkeypatch):
         got.append(pm.mertens_result(plan, 0, entries=True)[1])
         pm.mertens_destroy(plan)
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.gpu
+def test_window_without_the_memory_for_long_blocks():
+    """A window plan whose blocks of four times block_len do not get their memory is
+    made with block_len, with the same results."""
+    import torch
+
+    n, u, y1, bl = 10**14 + 7, 3 * 10**9, 10**9 + 3, 1 << 22
+    sizes, limit, refused = [], [1 << 62], []
+
+    def alloc(nbytes, stream, ctx):
+        if nbytes > limit[0]:
+            refused.append(nbytes)
+            return 0
+        sizes.append(nbytes)
+        return int(torch.cuda.caching_allocator_alloc(int(nbytes), 0, stream or 0))
+
+    def release(ptr, nbytes, stream, ctx):
+        torch.cuda.caching_allocator_delete(ptr)
+
+    got = []
+    pm.mertens_set_allocator(alloc, release)
+    try:
+        for _ in range(2):
+            plan = pm.mertens_plan_window([n], y1, y1 + 9 * bl + 4, u, bl)
+            pm.mertens_run(plan)
+            got.append(pm.mertens_window_result(plan, 0))
+            pm.mertens_destroy(plan)
+            limit[0] = 2 * 4 * bl - 1  # the int16 M of a long block is larger
+    finally:
+        pm.mertens_set_allocator()
+    assert max(sizes) > limit[0] and refused
+    assert got[0][2] == got[1][2]
+    assert np.array_equal(got[0][0], got[1][0]) and np.array_equal(got[0][1], got[1][1])
