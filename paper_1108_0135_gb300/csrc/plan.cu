@@ -202,6 +202,7 @@ struct mertens_plan_s {
     std::vector<uint64_t> n, n_hi, u, X, off;
     std::vector<uint64_t> direct, gathered, ymax_q;
     uint64_t nent = 0;
+    uint64_t nplaces = 0;  // wheel plans: length of the arrays by place
     uint64_t y_max = 0, block_len = 0, nblocks = 0, ydense = 0, jmax = 0, mg_n = 0;
     uint32_t gquot = 1;  // GatherArgs::quot of this plan
     // sieved range: [1, y_max] for a whole run; a window plan runs only the
@@ -579,11 +580,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     const double dc = dense_factor(tn);
     const u128 wide_from = wide_threshold();
     std::vector<WheelQuery> qs(count);
+    std::vector<WheelTarget> wt(count);
     uint64_t E = 0, G = 0, cut = 0;
     double acc = 0, ksum = 0, terms = 0, pairs = 0;
     for (size_t i = 0; i < count; ++i) {
         const uint64_t X = (uint64_t)(n[i] / us[i]);
-        qs[i] = {(uint64_t)n[i], (uint64_t)(n[i] >> 64), X, E, G, 0};
+        qs[i] = {(uint64_t)n[i], (uint64_t)(n[i] >> 64), X, E, G, 0, 0};
         p->n.push_back(qs[i].n);
         p->n_hi.push_back(qs[i].n_hi);
         p->u.push_back(us[i]);
@@ -593,7 +595,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         p->wide_gathered.push_back(0);
         const uint64_t ng = (X + kWheelGroup - 1) / kWheelGroup;
         G += ng;
-        if (table && n[i] <= table->y_max && X == 1) {
+        wt[i] = {n[i], us[i], X, table && n[i] <= table->y_max && X == 1, 0};
+        if (wt[i].lookup) {
             // M(n) is in the table: one entry, no terms, read after resolve
             p->lookups.push_back(E);
             p->lookups.push_back(qs[i].n);
@@ -634,18 +637,39 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         pairs += dc * root / (double)(kWheelSegY * kWheelGroup * kWheelGroupBlock) +
                  (double)ng / kWheelGroupBlock;
     }
-    if (E >= (1ull << 32)) {
+    uint64_t terms_end = 0;  // the places after it are lookups
+    const std::vector<WheelClass> classes = wheel_classes(wt, dc, wide_from, &terms_end);
+    const uint64_t places = terms_end + p->lookups.size() / 2;
+    if (places >= (1ull << 32)) {
         set_last_error("mertens_plan: more than 2^32 array entries");
         delete p;
         return MERTENS_ENOTSUP;
     }
     p->nent = E;
+    p->nplaces = places;
     // several one-word targets: entries in order of k (E count divisions on the
     // device); otherwise target by target
     const bool sorted = count > 1 && p->wide.empty() && (double)E * (double)count < 4.0e9;
-    for (size_t i = 0, l = 0; i < count; ++i)
-        if (!qs[i].n && !qs[i].n_hi)
-            qs[i].place = E - p->lookups.size() / 2 + l++;
+    bool placed = sorted;  // some place is not the entry's number
+    {
+        std::vector<uint64_t> next;  // per class: the next target's place
+        for (const WheelClass &c : classes)
+            next.push_back(c.first);
+        uint64_t l = terms_end;
+        for (size_t i = 0; i < count; ++i) {
+            if (wt[i].lookup) {
+                qs[i].place = l++;
+            } else {
+                qs[i].cls = wt[i].cls;
+                qs[i].place = sorted ? classes[wt[i].cls].first : next[wt[i].cls];
+                next[wt[i].cls] += qs[i].X;
+            }
+            placed = placed || qs[i].place != qs[i].off;
+        }
+        for (size_t i = 0, w = 0; i < count; ++i)
+            for (; w < p->wide.size() && p->wide[w].e < qs[i].off + qs[i].X; ++w)
+                p->wide[w].e += qs[i].place - qs[i].off;
+    }
     p->y_max = std::max<uint64_t>(p->y_max, 1);
     p->y_first = 1;
     p->y_last = p->y_max;
@@ -693,7 +717,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     }
     p->nblocks = (p->y_last + p->block_len - 1) / p->block_len;
     p->wchunks = (p->ydense + kWheelSegY - 1) / kWheelSegY;
-    p->wgroups = (uint32_t)((E + kWheelGroup - 1) / kWheelGroup);
+    p->wgroups = (uint32_t)((places + kWheelGroup - 1) / kWheelGroup);
     // parts of a dense chunk's list while the items would not fill the device
     p->wparts = (uint32_t)std::min(8.0, std::max(1.0, std::ceil(2400.0 / pairs)));
     p->wdense_items = (uint64_t)(pairs * p->wparts * 1.1) + 64;
@@ -732,60 +756,81 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     // for larger n no set is that long, and sharing sets of 2048 terms a lane anyway
     // took 40.2 against 38.7 ms at 10^16)
     p->long_lane = (uint32_t)std::min(4.0e9, std::max(2048.0, terms / 1.2e5));
-    double yc_min = 1e300;  // about the least dense cut-off
+    // per class: about the least dense cut-off, the largest y of a gathered term
+    std::vector<double> yc_min(classes.size(), 1e300);
+    std::vector<uint64_t> y_top(classes.size(), 0);
     for (size_t i = 0; i < count; ++i)
-        if (qs[i].n || qs[i].n_hi)
-            yc_min = std::min(yc_min, dc * std::sqrt((double)n[i] / (double)qs[i].X));
+        if (!wt[i].lookup) {
+            const size_t c = qs[i].cls;
+            yc_min[c] = std::min(yc_min[c], dc * std::sqrt((double)n[i] / (double)qs[i].X));
+            y_top[c] = std::max(y_top[c], (uint64_t)(n[i] / ((u128)qs[i].X + 1)));
+        }
     // sum of k over the x in (a, b] of target i
     const auto k_between = [&](size_t i, double a, double b) {
         return (double)n[i] * std::log((b + 0.5) / (a + 0.5));
     };
     std::vector<uint2> tiles;  // {first y less one, low and high word}, {length, 0}
     std::vector<uint4> items;
+    // the places that an item list takes, per class, and their sum of k
     struct Range {
         uint64_t e0, e1;
         double ksum;
     };
-    Range range{0, 0, 0.0};
-    bool bound = count > 1 && !sorted;  // a cut-off can be bound by floor(k/jlo)
+    std::vector<Range> ranges;
+    // classes where a cut-off can be bound by floor(k/jlo)
+    std::vector<uint8_t> bound(classes.size(), count > 1 && !sorted);
     for (size_t i = 0; i < count; ++i)
-        if (qs[i].n || qs[i].n_hi)
-            bound = bound || 2.0 * (dc * std::sqrt((double)n[i]) + 2.0 * kChunk) >= (double)us[i];
-    // the places with k < kt (before them all others), their sum of k
-    const auto k_below = [&](double kt) {
-        range = {0, sorted ? E - p->lookups.size() / 2 : E, 0.0};
-        for (size_t i = 0; i < count; ++i) {
-            if (!qs[i].n && !qs[i].n_hi)
-                continue;
-            const double lo = std::min((double)qs[i].X, std::floor((double)n[i] / kt));
-            range.e0 += (uint64_t)lo;
-            range.ksum += k_between(i, lo, (double)qs[i].X);
-        }
-    };
-    // places whose cut-off lies below te: all where a cut-off can be bound by
-    // floor(k/jlo), else from the group of the first with dc sqrt(k) < te + 8
+        if (!wt[i].lookup &&
+            2.0 * (dc * std::sqrt((double)n[i]) + 2.0 * kChunk) >= (double)us[i])
+            bound[qs[i].cls] = 1;
+    // places whose cut-off lies below te: all of a bound class, else from the group of
+    // the first with dc sqrt(k) < te + 8
     const auto below = [&](uint64_t te) {
         const double t = ((double)te + 8.0) / dc;
-        k_below(bound ? 1e300 : t * t);
-        range.e0 = std::max<uint64_t>(range.e0, kWheelGroup) - kWheelGroup;
-        range.e0 -= range.e0 % kWheelGroup;
+        ranges.clear();
+        for (const WheelClass &c : classes)
+            ranges.push_back({c.first, c.first + c.entries, 0.0});
+        for (size_t i = 0; i < count; ++i) {
+            if (wt[i].lookup)
+                continue;
+            Range &r = ranges[qs[i].cls];
+            const double lo = bound[qs[i].cls]
+                                  ? 0.0
+                                  : std::min((double)qs[i].X, std::floor((double)n[i] / (t * t)));
+            r.e0 += (uint64_t)lo;
+            r.ksum += k_between(i, lo, (double)qs[i].X);
+        }
+        for (size_t c = 0; c < classes.size(); ++c) {
+            uint64_t &e0 = ranges[c].e0;
+            e0 = std::max(e0, classes[c].first + kWheelGroup) - kWheelGroup;
+            e0 -= e0 % kWheelGroup;
+        }
     };
-    // the tile (t0, t0 + len] with the current range; false: too many terms in
+    // the tile (t0, t0 + len] with the current ranges; false: too many terms in
     // 1024 entries of it
     const auto add_tile = [&](uint64_t t0, uint64_t len, bool may_split) {
-        if (range.e0 >= range.e1)
+        double ne = 0, terms = 0;
+        for (size_t c = 0; c < classes.size(); ++c) {
+            Range &r = ranges[c];
+            if (t0 >= y_top[c])
+                r.e0 = r.e1;
+            if (r.e0 >= r.e1)
+                continue;
+            ne += (double)(r.e1 - r.e0);
+            terms += (1.0 / std::max((double)t0 + 1.0, std::min(yc_min[c], (double)(t0 + len))) -
+                      1.0 / ((double)(t0 + len) + 1.0)) / 3.0 * r.ksum;
+        }
+        if (ne == 0)
             return true;
-        const double terms =
-            (1.0 / std::max((double)t0 + 1.0, std::min(yc_min, (double)(t0 + len))) -
-             1.0 / ((double)(t0 + len) + 1.0)) / 3.0 * range.ksum;
-        const double ne = (double)(range.e1 - range.e0), work = 2.0 * ne + terms;
+        const double work = 2.0 * ne + terms;
         if (may_split && terms > item_max * std::ceil(ne / 1024.0))
             return false;
         const uint64_t step = (uint64_t)std::max(
             1024.0, std::ceil(ne / std::max(1.0, work / item_work) / 1024.0) * 1024.0);
-        for (uint64_t f = range.e0; f < range.e1; f += step)
-            items.push_back(make_uint4((uint32_t)(tiles.size() / 2), (uint32_t)f,
-                                       (uint32_t)std::min(f + step, range.e1), 0u));
+        for (const Range &r : ranges)
+            for (uint64_t f = r.e0; f < r.e1; f += step)
+                items.push_back(make_uint4((uint32_t)(tiles.size() / 2), (uint32_t)f,
+                                           (uint32_t)std::min(f + step, r.e1), 0u));
         tiles.push_back(make_uint2((uint32_t)t0, (uint32_t)(t0 >> 32)));
         tiles.push_back(make_uint2((uint32_t)len, 0u));
         return true;
@@ -813,17 +858,21 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             const double y1 = (double)end + 1.0, k0 = kt_fac * y1 * y1 / kGatherTile;
             const uint64_t k0i = (uint64_t)std::ceil(std::min(k0, 9.2e18));
             // the places with k >= k0i (unsorted targets: none)
-            Range r{0, 0, 0.0};
+            ranges.clear();
+            double ks = 0.0;
+            for (const WheelClass &c : classes)
+                ranges.push_back({c.first, c.first, 0.0});
             for (size_t i = 0; i < count && (count == 1 || sorted); ++i) {
-                if (!qs[i].n && !qs[i].n_hi)
+                if (wt[i].lookup)
                     continue;
                 const uint64_t xt = (uint64_t)std::min<u128>(qs[i].X, n[i] / k0i);
-                r.e1 += xt;
-                r.ksum += xt ? k_between(i, 0.0, (double)xt) : 0.0;
+                const double kx = xt ? k_between(i, 0.0, (double)xt) : 0.0;
+                ranges[qs[i].cls].e1 += xt;
+                ranges[qs[i].cls].ksum += kx;
+                ks += kx;
             }
-            if (r.ksum * kGatherTile / (y1 * y1) >= kt_min) {
+            if (ks * kGatherTile / (y1 * y1) >= kt_min) {
                 kt = k0i;
-                range = r;
                 for (uint64_t t0 = end; t0 < yend; t0 += len) {
                     len = std::min(kWheelTileY, yend - t0);
                     add_tile(t0, len, false);
@@ -881,12 +930,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         take(p->dwide, p->wide.size() * sizeof(WideEntry));
         take(p->dlook, p->lookups.size() * 8);
         up_bytes = off - up0;
-        take(ea.P, sorted ? E * 4 : 0);
-        take(p->dK, E * 8);
-        take(p->dYCE, E * 8);
-        take(p->dJL, E * 4);
-        take(p->dJD, E * 4);
-        take(p->dS, 2 * E * 8);  // S, then A
+        take(ea.P, placed ? E * 4 : 0);
+        take(p->dK, places * 8);
+        take(p->dYCE, places * 8);
+        take(p->dJL, places * 4);
+        take(p->dJD, places * 4);
+        take(p->dS, 2 * places * 8);  // S, then A
         take(p->dR6, E * 8);
         take(p->dR, E * 8);
         take(p->dqueue, (size_t)p->qcap * sizeof(uint4));
@@ -917,7 +966,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         p->dwl = table->dl;
         p->dwl_cnt = table->dl_cnt;
     }
-    p->dA = p->dS + E;
+    p->dA = p->dS + places;
     p->wtotals = d_totals;
     p->derr = (uint32_t *)(d_totals + count);  // status, chunk count, two work counters
     p->dqlen = p->derr + 1;
@@ -939,11 +988,12 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     p->h2d_bytes = up_bytes + np * 4;
     ea.qs = d_qs;
     ea.nq = (uint32_t)count;
-    ea.nent = (uint32_t)E;
+    ea.nplaces = (uint32_t)places;
     ea.qgroups = (uint32_t)G;
     ea.ngroups = p->wgroups;
-    if (!sorted)
+    if (!placed)
         ea.P = nullptr;
+    ea.by_k = sorted ? 1u : 0u;
     p->dplace = ea.P;
     ea.dc = dc;
     ea.wide_from = (uint64_t)wide_from;
@@ -963,6 +1013,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     cudaStream_t s = p->al.alloc ? nullptr : alloc_stream();
     const bool ok =
         (s || p->al.alloc) && cudaMemsetAsync(base, 0, cleared, s) == cudaSuccess &&
+        (places == E || cudaMemsetAsync(p->dK, 0, places * 8, s) == cudaSuccess) &&
         cudaMemcpyAsync(up, img.data(), up_bytes, cudaMemcpyHostToDevice, s) == cudaSuccess &&
         wheel_entries_enqueue(ea, s) >= 0 &&
         (!p->sieves ||
@@ -1850,9 +1901,8 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
 {
     uint64_t launches = 0;
     int r = 0;
-    const size_t E = p->nent;
     const mertens_table_s *tab = p->table;
-    cudaMemsetAsync(p->dS, 0, 2 * E * 8, s);
+    cudaMemsetAsync(p->dS, 0, 2 * p->nplaces * 8, s);
     cudaMemsetAsync(p->dcarry, 0, 8, s);
     cudaMemsetAsync(p->derr, 0, 4, s);
     WheelDenseArgs da;
@@ -1962,7 +2012,7 @@ static int wheel_run(mertens_plan_s *p, cudaStream_t s, uint64_t *out)
         ba.m_end = magic_of(y0 + len + 1);
         ba.l_end = magic_shift(y0 + len + 1);
         ba.kmax = p->ktile[b];
-        ba.nent = E;
+        ba.nplaces = p->nplaces;
         ba.K = p->dK;
         ba.YC = p->dYCE;
         ba.JL = p->dJL;

@@ -20,6 +20,7 @@
 
 #include "common.cuh"
 #include "internal.h"
+#include "wheel_place.h"
 
 namespace mert {
 
@@ -107,7 +108,6 @@ int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t 
 bool wheel_sieve_exact(uint64_t y_max);
 
 // ---- plan -----------------------------------------------------------------------
-constexpr uint32_t kWheelGroup = 64;       // consecutive entries with one dense cut-off
 constexpr uint32_t kWheelGroupBlock = 8;   // groups of a dense work item; the first
                                            // eight groups are items of their own (their
                                            // k is large: more terms take a slow form)
@@ -125,12 +125,14 @@ constexpr uint32_t kWheelItem = 256;       // wheel indices of a chunk of the gl
 
 // A target; n = 0: its value is read from a table (one entry, no terms).  Its
 // entries x = 1 .. X are numbered off + x - 1 in the results; the update works on
-// places: the same numbers for one target, all targets' entries in decreasing
-// order of k for several (so that 64 consecutive places have close k).
+// places: the same numbers for one target; for several, the entries of a class of
+// targets (wheel_place.h) in decreasing order of k (so that 64 consecutive places
+// have close k), class after class.
 struct WheelQuery {
     uint64_t n, n_hi, X;
     uint64_t off, goff;     // first entry, first group of 64 entries
-    uint64_t place;         // n = 0: the entry's place
+    uint64_t place;         // in order of k: the class's first place; else the target's
+    uint64_t cls;           // its class
 };
 
 struct WheelGroup {
@@ -156,12 +158,13 @@ struct WheelTotals {
 struct WheelEntryArgs {
     const WheelQuery *qs;
     uint32_t nq;
-    uint32_t nent;
+    uint32_t nplaces;       // places: the entries, and unused ones (k = 0) after a class
     uint32_t qgroups;       // groups of 64 entries, target by target
     uint32_t ngroups;       // groups of 64 places
     double dc;              // dense cut-off factor
     uint64_t wide_from;     // entries with k at or above: two-word ones (k = 0 here)
     uint32_t *P;            // place of every entry (null: the entry's number)
+    uint32_t by_k;          // places in decreasing order of k
     uint64_t *K, *YC;
     uint32_t *JL, *JD;
     WheelGroup *groups;
@@ -212,7 +215,7 @@ struct WheelBlockArgs {
     uint64_t m_ylo, m_end;  // division magics of ylo and y0 + len + 1
     uint32_t l_ylo, l_end;
     uint64_t kmax;          // entries with k >= kmax take the block's tiles
-    uint64_t nent;
+    uint64_t nplaces;
     const uint64_t *K, *YC;
     const uint32_t *JL, *JD;
     uint64_t *S, *A;

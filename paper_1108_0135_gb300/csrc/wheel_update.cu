@@ -94,7 +94,7 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
         const uint32_t i = lane + 32u * (uint32_t)h;
         k[h] = 0;
         if (i < cnt) {
-            const uint64_t x = x0 + i, e = Q.off + x - 1;
+            const uint64_t x = x0 + i;
             if (Q.n_hi) {
                 const unsigned __int128 kk = (((unsigned __int128)Q.n_hi << 64) | Q.n) / x;
                 k[h] = kk < a.wide_from ? (uint64_t)kk : 0;
@@ -104,16 +104,15 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
                     k[h] = 0;
             }
             jlo[h] = k[h] ? Q.X / x + 1 : 1;
-            uint64_t place = e;
-            if (a.P) {
-                // entries before this one in decreasing order of k (ties: by
-                // target): floor(n'/x') >= k for the x' <= floor(n'/k)
-                place = Q.n ? x - 1 : Q.place;
-                for (uint32_t q = 0; q < a.nq && Q.n; ++q)
-                    if (q != lo_q)
+            uint64_t place = Q.place + x - 1;
+            if (a.by_k && Q.n)
+                // entries of the class before this one in decreasing order of k
+                // (ties: by target): floor(n'/x') >= k for the x' <= floor(n'/k)
+                for (uint32_t q = 0; q < a.nq; ++q)
+                    if (q != lo_q && a.qs[q].n && a.qs[q].cls == Q.cls)
                         place += min(a.qs[q].X, a.qs[q].n / (k[h] + (q < lo_q ? 0u : 1u)));
-                a.P[e] = (uint32_t)place;
-            }
+            if (a.P)
+                a.P[Q.off + x - 1] = (uint32_t)place;
             a.K[place] = k[h];
             a.JL[place] = (uint32_t)jlo[h];
             if (k[h]) {
@@ -158,14 +157,15 @@ __global__ void __launch_bounds__(128) wheel_entries_kernel(WheelEntryArgs a)
 // same sums; a dense y costs the whole group one term per entry, a gathered j only
 // its own, so the mean of k balances them (with the first entry's k, the first
 // group had four times the dense terms: 14% of all at n = 10^13).  jd stays below
-// 2^32.
+// 2^32: the classes of targets (wheel_place.h) keep an entry's floor(k/jlo) from
+// taking the cut-off of a far larger k's group below kf / kWheelMaxJ.
 __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
 {
     const uint32_t lane = threadIdx.x & 31u;
     const uint32_t g = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (g >= a.ngroups)
         return;
-    const uint32_t e0 = g * kWheelGroup, cnt = min(kWheelGroup, a.nent - e0);
+    const uint32_t e0 = g * kWheelGroup, cnt = min(kWheelGroup, a.nplaces - e0);
     uint64_t k[2], jlo[2], kf = 0, ncap = 0;  // largest k, max of ~floor(k/jlo)
     float ksum = 0;
 #pragma unroll
@@ -185,18 +185,13 @@ __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
     for (int o = 16; o > 0; o >>= 1)
         ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
     const uint32_t one = __reduce_add_sync(0xffffffffu, (k[0] ? 1u : 0u) + (k[1] ? 1u : 0u));
-    uint64_t yc = 0;
-    if (kf) {
-        yc = max((uint64_t)(a.dc * sqrt((double)ksum / one)), kf / (uint64_t)4000000000u);
-        yc = min(yc, ~ncap);
-        yc -= yc % 6;
-    }
+    const uint64_t yc = kf ? wheel_cutoff(a.dc, (double)ksum / one, kf, ~ncap) : 0;
     uint64_t exec = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
         if (i < cnt) {
-            const uint64_t jd = k[h] ? max(k[h] / (yc + 1), jlo[h] - 1) : 0;
+            const uint64_t jd = k[h] ? wheel_last_j(k[h], yc, jlo[h]) : 0;
             a.YC[e0 + i] = k[h] ? yc : 0;
             a.JD[e0 + i] = (uint32_t)jd;
             if (k[h])
@@ -1025,7 +1020,7 @@ __global__ void __launch_bounds__(256) wheel_range_kernel(WheelBlockArgs a)
     const uint32_t lane = threadIdx.x & 31u;
     // the entry's loads at once: one after the other they took most of the time
     uint64_t k = 0, jlo = 0, jd = 0, yc = 0;
-    if (e < a.nent) {
+    if (e < a.nplaces) {
         k = a.K[e];
         yc = a.YC[e];
         jlo = a.JL[e];
@@ -1398,7 +1393,7 @@ int wheel_gather_enqueue(const WheelGatherArgs &a, cudaStream_t s)
 int wheel_block_enqueue(const WheelBlockArgs &a, cudaStream_t s)
 {
     cudaMemsetAsync(a.qlen, 0, 4, s);
-    wheel_range_kernel<<<(unsigned)((a.nent + 255) / 256), 256, 0, s>>>(a);
+    wheel_range_kernel<<<(unsigned)((a.nplaces + 255) / 256), 256, 0, s>>>(a);
     const uint32_t grid = std::min<uint32_t>((uint32_t)sm_count() * 8u, (a.qcap + 7u) / 8u);
     wheel_chunk_kernel<<<grid, 256, 0, s>>>(a);
     return cudaGetLastError() == cudaSuccess ? 2 : -1;

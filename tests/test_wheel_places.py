@@ -1,0 +1,199 @@
+"""Places and dense cut-offs of plans over the integers coprime to 6: the rules of
+csrc/wheel_place.h, run by a host program over batches of unlike targets, and on the
+GPU such batches against their targets planned alone."""
+import math
+import os
+import random
+import subprocess
+
+import numpy as np
+import pytest
+
+import paper_1108_0135_gb300 as pm
+
+CSRC = os.path.join(os.path.dirname(os.path.abspath(pm.__file__)), "csrc")
+
+# reads: dc wide_from count by_k, then n u per target (n as high and low word);
+# prints per batch: classes, places, largest j, largest yc, gathered j, bad entries
+PROGRAM = r"""
+#include <cstdio>
+#include "wheel_place.h"
+using namespace mert;
+typedef unsigned __int128 u128;
+int main()
+{
+    double dc;
+    unsigned long long wide, hi, lo, u;
+    int count, by_k;
+    while (scanf("%lf %llu %d %d", &dc, &wide, &count, &by_k) == 4) {
+        std::vector<WheelTarget> t(count);
+        for (auto &v : t) {
+            if (scanf("%llu %llu %llu", &hi, &lo, &u) != 3)
+                return 1;
+            v.n = ((u128)hi << 64) | lo;
+            v.u = u;
+            v.X = (uint64_t)(v.n / u);
+            v.lookup = false;
+        }
+        uint64_t end = 0;
+        const std::vector<WheelClass> cls = wheel_classes(t, dc, wide, &end);
+        struct E { uint64_t k, jlo; };
+        std::vector<E> place(end, E{0, 0});
+        uint64_t bad = 0;
+        for (size_t c = 0; c < cls.size(); ++c) {
+            std::vector<E> e;
+            for (auto &v : t)
+                for (uint64_t x = 1; v.cls == c && x <= v.X; ++x) {
+                    const u128 k = v.n / x;
+                    e.push_back({k < wide ? (uint64_t)k : 0, v.X / x + 1});
+                }
+            if (by_k)
+                std::stable_sort(e.begin(), e.end(),
+                                 [](const E &a, const E &b) { return a.k > b.k; });
+            bad += e.size() != cls[c].entries || cls[c].first % kWheelGroup != 0;
+            for (size_t i = 0; i < e.size(); ++i) {
+                bad += place[cls[c].first + i].jlo != 0;  // places do not overlap
+                place[cls[c].first + i] = e[i];
+            }
+        }
+        uint64_t jmax = 0, ymax = 0;
+        double gathered = 0;
+        for (uint64_t g = 0; g < end; g += kWheelGroup) {
+            uint64_t kf = 0, cap = UINT64_MAX;
+            double sum = 0;
+            int one = 0;
+            const uint64_t to = std::min(end, g + kWheelGroup);
+            for (uint64_t i = g; i < to; ++i)
+                if (place[i].k) {
+                    kf = std::max(kf, place[i].k);
+                    cap = std::min(cap, place[i].k / place[i].jlo);
+                    sum += (double)place[i].k;
+                    ++one;
+                }
+            const uint64_t yc = kf ? wheel_cutoff(dc, sum / one, kf, cap) : 0;
+            ymax = std::max(ymax, yc);
+            for (uint64_t i = g; i < to; ++i)
+                if (place[i].k) {
+                    const uint64_t j = wheel_last_j(place[i].k, yc, place[i].jlo);
+                    jmax = std::max(jmax, j);
+                    gathered += (double)(j - (place[i].jlo - 1));
+                    bad += yc > place[i].k / place[i].jlo;
+                }
+        }
+        printf("%zu %llu %llu %llu %.0f %llu\n", cls.size(), (unsigned long long)end,
+               (unsigned long long)jmax, (unsigned long long)ymax, gathered,
+               (unsigned long long)bad);
+    }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("places")
+    src, exe = d / "places.cpp", d / "places"
+    src.write_text(PROGRAM)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+
+    def run(batches, dc=1.4, wide=1 << 63, by_k=1):
+        text = ""
+        for targets in batches:
+            text += f"{dc} {wide} {len(targets)} {by_k}\n"
+            for n, u in targets:
+                text += f"{n >> 64} {n & (2**64 - 1)} {u}\n"
+        out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True)
+        names = ("classes", "places", "jmax", "ymax", "gathered", "bad")
+        return [dict(zip(names, map(int, line.split()))) for line in out.stdout.splitlines()]
+
+    return run
+
+
+def auto_u(ns):
+    """The documented automatic limits of a batch."""
+    g = min(1.78, max(1.0, (max(ns) / 1e18) ** -0.25))
+    ub = 0.45 * g * float(sum(ns)) ** (2 / 3)
+    return [(n, min(n, max(int(ub), math.isqrt(n) + 1)) if n > 3 else n) for n in ns]
+
+
+BATCHES = [
+    [10**15, 1], [10**17, 5], [10**17, 50], [10**14, 10], [10**14, 100],
+    [10**i for i in range(17)],                       # the paper's table in one call
+    [1000, 10**19], [7, 10**19, 12, 3 * 10**18],      # two-word entries
+    [10**14 + i * 10**9 for i in range(64)],
+    [10**12, 10**12 + 10**6, 5 * 10**9 + 9, 12345, 6, 1],
+    [1], [2, 1], [3, 3, 3, 1, 1],
+]
+
+
+@pytest.mark.parametrize("by_k", [1, 0])
+def test_groups_of_unlike_targets(rules, by_k):
+    """No j reaches 2^32, no cut-off is above an entry's floor(k/jlo), and a batch
+    gathers at most twice what its targets gather one by one at the same limits (a
+    group of a batch takes the mean of its own k)."""
+    rng = random.Random(3)
+    batches = list(BATCHES)
+    for _ in range(40):
+        top = rng.uniform(2, 17)
+        batches.append([int(10 ** rng.uniform(0, top)) for _ in range(rng.randrange(2, 12))])
+    batches = [auto_u(ns) for ns in batches]
+    got = rules(batches, by_k=by_k)
+    for targets, r in zip(batches, got):
+        assert r["bad"] == 0 and r["jmax"] < 2**32 - 6, (targets, r)
+        alone = sum(v["gathered"] for v in rules([[t] for t in targets]))
+        assert r["gathered"] <= 2 * alone + 64 * 6, (targets, r, alone)
+        assert r["places"] < sum(n // u for n, u in targets) + 64 * r["classes"]
+
+
+def test_like_targets_share_a_class(rules):
+    """Close targets, and requests over the serving range, stay one class."""
+    rng = random.Random(4)
+    batches = [[10**14 + i * 10**9 for i in range(64)],
+               [int(10 ** rng.uniform(10, 15)) for _ in range(32)]]
+    for r in rules([auto_u(ns) for ns in batches]):
+        assert r["classes"] == 1
+
+
+@pytest.mark.parametrize("dc", [0.7, 1.4, 7.5, 900.0])
+def test_limits_near_the_square_root(rules, dc):
+    """Explicit limits: every cut-off is bound by floor(k/jlo); the classes stay few."""
+    rng = random.Random(5)
+    batches = []
+    for _ in range(30):
+        u = int(10 ** rng.uniform(1, 5))
+        ns = [int(10 ** rng.uniform(math.log10(u), 2 * math.log10(u))) for _ in range(6)]
+        batches.append([(n, u) for n in ns if math.isqrt(n) < u <= n] or [(u, u)])
+        batches.append([(n, min(n, math.isqrt(n) + 1)) for n in ns])
+    for targets, r in zip(batches, rules(batches, dc=dc)):
+        assert r["bad"] == 0 and r["jmax"] < 2**32 - 6 and r["classes"] <= 8, (targets, r)
+
+
+def _array(n, u):
+    plan = pm.mertens_plan([n], u)
+    try:
+        pm.mertens_run(plan)
+        return pm.mertens_result(plan, 0, entries=True)[1]
+    finally:
+        pm.mertens_destroy(plan)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ns,wide_from", [
+    ([10**15, 1], None),
+    ([10**i for i in range(17)], None),
+    ([50, 10**15, 10**14 + 3, 2, 10**15 + 1, 777], None),
+    ([1000, 10**14, 3], 10**13),          # target by target: two-word entries
+    ([5, 10**15 + 7, 10**6], 10**14),
+])
+def test_unlike_targets_equal_the_same_planned_alone(ns, wide_from, monkeypatch):
+    if wide_from:
+        monkeypatch.setenv("MERTENS_WIDE_FROM", str(wide_from))
+    plan = pm.mertens_plan(ns)
+    try:
+        pm.mertens_run(plan)
+        got = [(pm.mertens_plan_info(plan, i)["u"], pm.mertens_result(plan, i, entries=True)[1])
+               for i in range(len(ns))]
+    finally:
+        pm.mertens_destroy(plan)
+    monkeypatch.delenv("MERTENS_WIDE_FROM", raising=False)
+    for n, (u, arr) in zip(ns, got):
+        assert np.array_equal(arr, _array(n, u)), n
