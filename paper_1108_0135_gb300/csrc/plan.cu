@@ -264,7 +264,6 @@ struct mertens_plan_s {
     // entries with k >= 2^63 (targets n >= 2^63) and the wide kernel's
     // grid width per block (0: no terms in the block)
     std::vector<WideEntry> wide;
-    std::vector<uint64_t> wide_direct, wide_gathered;  // their terms, per target (wheel plans)
     WideEntry *dwide = nullptr;
     std::vector<uint32_t> wide_grid;
     bool mg_built = false;
@@ -279,7 +278,6 @@ struct mertens_plan_s {
     uint64_t *dA = nullptr, *dR6 = nullptr;
     WheelGroup *dwgroups = nullptr;
     uint32_t *dwpre = nullptr;
-    WheelTotals *wtotals = nullptr;
     uint32_t wgroups = 0, wparts = 1;
     uint64_t wdense_items = 0;   // about; the device has their number
     WheelGatherTile *dwtiles = nullptr;
@@ -591,8 +589,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         p->u.push_back(us[i]);
         p->X.push_back(X);
         p->off.push_back(E);
-        p->wide_direct.push_back(0);
-        p->wide_gathered.push_back(0);
+        p->direct.push_back(0);
+        p->gathered.push_back(0);
         const uint64_t ng = (X + kWheelGroup - 1) / kWheelGroup;
         G += ng;
         wt[i] = {n[i], us[i], X, table && n[i] <= table->y_max && X == 1, 0};
@@ -615,8 +613,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             W.jhi = (uint64_t)(k / ((u128)W.s + 1));
             W.e = E + x - 1;
             p->wide.push_back(W);
-            p->wide_direct.back() += W.s;
-            p->wide_gathered.back() += W.jhi >= W.jlo ? W.jhi - W.jlo + 1 : 0;
+            p->direct.back() += W.s;
+            p->gathered.back() += W.jhi >= W.jlo ? W.jhi - W.jlo + 1 : 0;
         }
         if (table)
             cut = std::max(cut, first_cutoff(n[i], X, dc, wide_from));
@@ -967,7 +965,6 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         p->dwl_cnt = table->dl_cnt;
     }
     p->dA = p->dS + places;
-    p->wtotals = d_totals;
     p->derr = (uint32_t *)(d_totals + count);  // status, chunk count, two work counters
     p->dqlen = p->derr + 1;
     p->dcounter_dense = p->derr + 2;
@@ -984,6 +981,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     put(p->dwgitems, items.data(), items.size() * sizeof(uint4));
     put(p->dwide, p->wide.data(), p->wide.size() * sizeof(WideEntry));
     put(p->dlook, p->lookups.data(), p->lookups.size() * 8);
+    std::vector<WheelTotals> totals(count);
     const size_t np = p->ws.host_p.size();
     p->h2d_bytes = up_bytes + np * 4;
     ea.qs = d_qs;
@@ -1021,11 +1019,23 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
           cudaMemcpyAsync(p->ws.p, p->ws.host_p.data(), np * 4, cudaMemcpyHostToDevice, s) ==
               cudaSuccess)) &&
         cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess &&
+        cudaMemcpyAsync(totals.data(), d_totals, count * sizeof(WheelTotals),
+                        cudaMemcpyDeviceToHost, s) == cudaSuccess &&
         cudaStreamSynchronize(s) == cudaSuccess;
     if (!ok) {
         set_last_error("mertens_plan: CUDA error %s", cudaGetErrorString(cudaGetLastError()));
         mertens_destroy(p);
         return MERTENS_ECUDA;
+    }
+    // the term counts are read here, so that mertens_plan_info needs no device (it may
+    // be called by several threads, and while a stream is being captured)
+    for (size_t t = 0; t < count; ++t) {
+        p->direct[t] += totals[t].direct;
+        p->gathered[t] += totals[t].gathered;
+        p->terms += p->direct[t] + p->gathered[t];
+        p->gather_j += totals[t].gather_j;
+        p->gather_j_exec += totals[t].exec;
+        p->dense_y += totals[t].dense_y;
     }
     // sieve updates: sum of 1/p + 1/p^2 over the primes 5 <= p <= sqrt(block
     // end), per wheel number
@@ -1042,27 +1052,6 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         p->sieve_updates += (double)len / 3.0 * pre;
     }
     *out = p;
-    return MERTENS_OK;
-}
-
-// Term counts of a wheel plan's targets, read when they are asked for.
-static int wheel_counts(mertens_plan_s *p)
-{
-    if (!p->wheel || !p->direct.empty())
-        return MERTENS_OK;
-    std::vector<WheelTotals> t(p->nq);
-    if (cudaMemcpy(t.data(), p->wtotals, p->nq * sizeof(WheelTotals), cudaMemcpyDeviceToHost) !=
-        cudaSuccess)
-        return MERTENS_ECUDA;
-    for (size_t i = 0; i < p->nq; ++i) {
-        const WheelTotals &v = t[i];
-        p->direct.push_back(v.direct + p->wide_direct[i]);
-        p->gathered.push_back(v.gathered + p->wide_gathered[i]);
-        p->terms += p->direct[i] + p->gathered[i];
-        p->gather_j += v.gather_j;
-        p->gather_j_exec += v.exec;
-        p->dense_y += v.dense_y;
-    }
     return MERTENS_OK;
 }
 
@@ -2707,8 +2696,6 @@ int mertens_plan_info(mertens_plan_t p, size_t i, mertens_query_info *info)
 {
     if (!p || i >= p->nq || !info)
         return MERTENS_EINVAL;
-    if (wheel_counts(p) != MERTENS_OK)
-        return MERTENS_ECUDA;
     memset(info, 0, sizeof(*info));
     info->n.lo = p->n[i];
     info->n.hi = p->n_hi[i];
@@ -2738,7 +2725,7 @@ int mertens_run_stats_get(mertens_plan_t p, mertens_run_stats *st)
     memset(st, 0, sizeof(*st));
     if (!p->ran)
         return MERTENS_ENOTREADY;
-    if (cudaEventSynchronize(p->done) != cudaSuccess || wheel_counts(p) != MERTENS_OK)
+    if (cudaEventSynchronize(p->done) != cudaSuccess)
         return MERTENS_ECUDA;
     st->blocks = p->nblocks;
     st->y_sieved = p->y_last >= p->y_first ? p->y_last - p->y_first + 1 : 0;

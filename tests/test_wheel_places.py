@@ -197,3 +197,38 @@ def test_unlike_targets_equal_the_same_planned_alone(ns, wide_from, monkeypatch)
     monkeypatch.delenv("MERTENS_WIDE_FROM", raising=False)
     for n, (u, arr) in zip(ns, got):
         assert np.array_equal(arr, _array(n, u)), n
+
+
+@pytest.mark.gpu
+def test_plan_info_needs_no_device():
+    """Term counts of a plan from many threads at once, and inside a stream capture
+    (which a copy on the default stream would break)."""
+    import threading
+
+    import torch
+
+    ns = [10**12 + i for i in range(5)] + [7]
+    plan = pm.mertens_plan(ns)
+    try:
+        g, side = torch.cuda.CUDAGraph(), torch.zeros(1, device="cuda")
+        with torch.cuda.graph(g):
+            side += 1
+            inside = [pm.mertens_plan_info(plan, i) for i in range(len(ns))]
+        got = [None] * 16
+        start = threading.Barrier(16)
+
+        def read(t):
+            start.wait()
+            got[t] = [pm.mertens_plan_info(plan, i) for i in range(len(ns))]
+
+        threads = [threading.Thread(target=read, args=(t,)) for t in range(16)]
+        for t in threads:
+            t.start()
+        for t in threads:
+            t.join()
+        want = [pm.mertens_describe(n, v["u"]) for n, v in zip(ns, inside)]
+        for v in got + [inside]:
+            assert [(x["direct_terms"], x["gathered_terms"]) for x in v] == \
+                [(x["direct_terms"], x["gathered_terms"]) for x in want]
+    finally:
+        pm.mertens_destroy(plan)
