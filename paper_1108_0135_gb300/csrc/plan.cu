@@ -575,10 +575,13 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
                              const mertens_tuning &tn, mertens_table_s *table)
 {
     const size_t count = n.size();
-    const double dc = dense_factor(tn);
+    // at least 1: below, an entry gathers more terms per tile than the tile's 32-bit
+    // sums hold (at 2e-4 and n = 10^12 they wrapped), and none of it pays
+    const double dc = std::max(1.0, dense_factor(tn));
     const u128 wide_from = wide_threshold();
     std::vector<WheelQuery> qs(count);
     std::vector<WheelTarget> wt(count);
+    std::vector<uint8_t> beyond(count, 0);  // the end of a table's list can bind a cut-off
     uint64_t E = 0, G = 0, cut = 0;
     double acc = 0, ksum = 0, terms = 0, pairs = 0;
     for (size_t i = 0; i < count; ++i) {
@@ -623,10 +626,11 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
         const uint64_t yg = (uint64_t)(n[i] / ((u128)X + 1));
         p->ymax_q.push_back(std::max(isqrt128(n[i]), yg));
         p->y_max = std::max(p->y_max, p->ymax_q.back());
-        // no cut-off is above the first group's target value
-        const double nd = (double)n[i], kf = std::min(nd, (double)wide_from);
-        const uint64_t t = ((uint64_t)(dc * std::sqrt(kf)) + kChunk) / kChunk * kChunk;
+        // no cut-off of a group with an entry of this target as its largest k is above
+        const double nd = (double)n[i];
+        const uint64_t t = wheel_cutoff_bound(dc, (uint64_t)std::min(n[i], wide_from));
         p->ydense = std::max(p->ydense, std::min(t, yg));
+        beyond[i] = table && t > table->ydense;
         const double lx = std::log((double)std::max<uint64_t>(X, 2));
         acc += nd * lx;
         ksum += nd * (lx + 1.0);
@@ -778,8 +782,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     // classes where a cut-off can be bound by floor(k/jlo)
     std::vector<uint8_t> bound(classes.size(), count > 1 && !sorted);
     for (size_t i = 0; i < count; ++i)
-        if (!wt[i].lookup &&
-            2.0 * (dc * std::sqrt((double)n[i]) + 2.0 * kChunk) >= (double)us[i])
+        if (!wt[i].lookup && (beyond[i] ||
+            2.0 * (dc * std::sqrt((double)n[i]) + 2.0 * kChunk) >= (double)us[i]))
             bound[qs[i].cls] = 1;
     // places whose cut-off lies below te: all of a bound class, else from the group of
     // the first with dc sqrt(k) < te + 8
@@ -981,7 +985,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     put(p->dwgitems, items.data(), items.size() * sizeof(uint4));
     put(p->dwide, p->wide.data(), p->wide.size() * sizeof(WideEntry));
     put(p->dlook, p->lookups.data(), p->lookups.size() * 8);
-    std::vector<WheelTotals> totals(count);
+    std::vector<WheelTotals> totals(count + 1);  // and the status word behind them
     const size_t np = p->ws.host_p.size();
     p->h2d_bytes = up_bytes + np * 4;
     ea.qs = d_qs;
@@ -994,6 +998,8 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
     ea.by_k = sorted ? 1u : 0u;
     p->dplace = ea.P;
     ea.dc = dc;
+    ea.ydense = table ? table->ydense : p->ydense;
+    ea.err = p->derr;
     ea.wide_from = (uint64_t)wide_from;
     ea.K = p->dK;
     ea.YC = p->dYCE;
@@ -1019,13 +1025,20 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
           cudaMemcpyAsync(p->ws.p, p->ws.host_p.data(), np * 4, cudaMemcpyHostToDevice, s) ==
               cudaSuccess)) &&
         cudaEventCreateWithFlags(&p->done, cudaEventDisableTiming) == cudaSuccess &&
-        cudaMemcpyAsync(totals.data(), d_totals, count * sizeof(WheelTotals),
+        cudaMemcpyAsync(totals.data(), d_totals, count * sizeof(WheelTotals) + 4,
                         cudaMemcpyDeviceToHost, s) == cudaSuccess &&
         cudaStreamSynchronize(s) == cudaSuccess;
     if (!ok) {
         set_last_error("mertens_plan: CUDA error %s", cudaGetErrorString(cudaGetLastError()));
         mertens_destroy(p);
         return MERTENS_ECUDA;
+    }
+    uint32_t status = 0;
+    memcpy(&status, &totals[count], 4);
+    if (status & kErrJ) {
+        set_last_error("mertens_plan: a gathered j does not fit 32 bits");
+        mertens_destroy(p);
+        return MERTENS_ENOTSUP;
     }
     // the term counts are read here, so that mertens_plan_info needs no device (it may
     // be called by several threads, and while a stream is being captured)

@@ -102,6 +102,7 @@ void wheel_sieve_primes(WheelSieve *t, uint64_t y_max);
 // kErrList in *err.
 size_t wheel_sieve_bytes(const WheelSieve *t, uint64_t max_len);
 constexpr uint32_t kErrList = 4u;  // a square list overflowed its capacity
+constexpr uint32_t kErrJ = 32u;    // a plan's gathered j beyond 32 bits
 int wheel_sieve_bind(WheelSieve *t, void *base, uint64_t max_len, uint32_t *err, cudaStream_t s);
 uint32_t wheel_primes_upto(const WheelSieve *t, uint64_t b);
 int wheel_sieve_enqueue(const WheelSieve *t, const WheelLaunch &L, cudaStream_t s);
@@ -162,6 +163,8 @@ struct WheelEntryArgs {
     uint32_t qgroups;       // groups of 64 entries, target by target
     uint32_t ngroups;       // groups of 64 places
     double dc;              // dense cut-off factor
+    uint64_t ydense;        // end of the dense list
+    uint32_t *err;          // kErrJ when a gathered j did not fit 32 bits
     uint64_t wide_from;     // entries with k at or above: two-word ones (k = 0 here)
     uint32_t *P;            // place of every entry (null: the entry's number)
     uint32_t by_k;          // places in decreasing order of k

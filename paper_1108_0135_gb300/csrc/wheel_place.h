@@ -24,17 +24,30 @@ namespace mert {
 
 constexpr uint32_t kWheelGroup = 64;  // consecutive places with one dense cut-off
 
-// Cut-offs from k / kWheelMaxJ on keep every gathered j below 2^32 - 6.
+// Cut-offs from k / kWheelMaxJ + 6 on (down to a multiple of 6) keep every gathered j
+// below 2^32 - 6.
 constexpr uint64_t kWheelMaxJ = 4000000000u;
 
-// Dense cut-off of a group: dc sqrt(mean k of its one-word entries), at least
-// kf / kWheelMaxJ (kf its largest k), at most cap (its least floor(k/jlo): beyond it
-// no term is left), down to a multiple of 6.
-MERT_RULE uint64_t wheel_cutoff(double dc, double mean, uint64_t kf, uint64_t cap)
+// Dense cut-off of a group: dc sqrt(mean k of its one-word entries), at least what
+// keeps j in range for kf, its largest k; at most cap (its least floor(k/jlo): beyond
+// it no term is left) and `listed`, the end of the dense list; down to a multiple of 6.
+MERT_RULE uint64_t wheel_cutoff(double dc, double mean, uint64_t kf, uint64_t cap,
+                                uint64_t listed)
 {
-    const uint64_t want = (uint64_t)(dc * sqrt(mean)), least = kf / kWheelMaxJ;
-    const uint64_t yc = want > least ? want : least;
-    return (yc < cap ? yc : cap) / 6 * 6;
+    const uint64_t want = (uint64_t)(dc * sqrt(mean)), least = kf / kWheelMaxJ + 6;
+    uint64_t yc = want > least ? want : least;
+    yc = yc < cap ? yc : cap;
+    return (yc < listed ? yc : listed) / 6 * 6;
+}
+
+// A bound of all cut-offs of groups whose k are at most k (before cap), a multiple of
+// 4096: the dense list has to reach it.  The mean of a group, summed in double
+// precision, is above k by at most a relative 2^-46, and dc sqrt(k) stays below 2^42,
+// so the cut-off's whole part is at most one above that of dc sqrt(k).
+MERT_RULE uint64_t wheel_cutoff_bound(double dc, uint64_t k)
+{
+    const uint64_t want = (uint64_t)(dc * sqrt((double)k)), least = k / kWheelMaxJ + 6;
+    return ((want > least ? want : least) + 4096) / 4096 * 4096;
 }
 
 // An entry's last gathered j at cut-off yc.

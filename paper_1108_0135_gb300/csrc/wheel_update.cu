@@ -167,7 +167,10 @@ __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
         return;
     const uint32_t e0 = g * kWheelGroup, cnt = min(kWheelGroup, a.nplaces - e0);
     uint64_t k[2], jlo[2], kf = 0, ncap = 0;  // largest k, max of ~floor(k/jlo)
-    float ksum = 0;
+    // in double precision: the dense list and the tiles' ranges of places are laid out
+    // for dc sqrt(k) as a double (in single precision the cut-offs of 64 close targets
+    // near 10^17 could lie 40 above it)
+    double ksum = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
@@ -175,7 +178,7 @@ __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
         if (k[h]) {
             jlo[h] = a.JL[e0 + i];
             kf = max(kf, k[h]);
-            ksum += (float)k[h];
+            ksum += (double)k[h];
             ncap = max(ncap, ~(k[h] / jlo[h]));
         }
     }
@@ -185,8 +188,8 @@ __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
     for (int o = 16; o > 0; o >>= 1)
         ksum += __shfl_xor_sync(0xffffffffu, ksum, o);
     const uint32_t one = __reduce_add_sync(0xffffffffu, (k[0] ? 1u : 0u) + (k[1] ? 1u : 0u));
-    const uint64_t yc = kf ? wheel_cutoff(a.dc, (double)ksum / one, kf, ~ncap) : 0;
-    uint64_t exec = 0;
+    const uint64_t yc = kf ? wheel_cutoff(a.dc, ksum / one, kf, ~ncap, a.ydense) : 0;
+    uint64_t exec = 0, jmax = 0;
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
         const uint32_t i = lane + 32u * (uint32_t)h;
@@ -194,10 +197,13 @@ __global__ void __launch_bounds__(128) wheel_groups_kernel(WheelEntryArgs a)
             const uint64_t jd = k[h] ? wheel_last_j(k[h], yc, jlo[h]) : 0;
             a.YC[e0 + i] = k[h] ? yc : 0;
             a.JD[e0 + i] = (uint32_t)jd;
+            jmax = max(jmax, jd);
             if (k[h])
                 exec += phi6(jd) - phi6(jlo[h] - 1);
         }
     }
+    if (jmax >= (1ull << 32) - 6)
+        atomicOr(a.err, kErrJ);  // the plan is refused
     exec = warp_sum_u64(exec);
     if (lane == 0) {
         WheelGroup G;

@@ -1,10 +1,12 @@
 """Places and dense cut-offs of plans over the integers coprime to 6: the rules of
 csrc/wheel_place.h, run by a host program over batches of unlike targets, and on the
 GPU such batches against their targets planned alone."""
+import ctypes
 import math
 import os
 import random
 import subprocess
+import threading
 
 import numpy as np
 import pytest
@@ -12,6 +14,14 @@ import pytest
 import paper_1108_0135_gb300 as pm
 
 CSRC = os.path.join(os.path.dirname(os.path.abspath(pm.__file__)), "csrc")
+
+
+def compiled(d, name, text):
+    src, exe = d / (name + ".cpp"), d / name
+    src.write_text(text)
+    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    return str(exe)
+
 
 # reads: dc wide_from count by_k, then n u per target (n as high and low word);
 # prints per batch: classes, places, largest j, largest yc, gathered j, bad entries
@@ -70,7 +80,8 @@ int main()
                     sum += (double)place[i].k;
                     ++one;
                 }
-            const uint64_t yc = kf ? wheel_cutoff(dc, sum / one, kf, cap) : 0;
+            const uint64_t yc = kf ? wheel_cutoff(dc, sum / one, kf, cap, UINT64_MAX) : 0;
+            bad += kf && yc > wheel_cutoff_bound(dc, kf);
             ymax = std::max(ymax, yc);
             for (uint64_t i = g; i < to; ++i)
                 if (place[i].k) {
@@ -90,10 +101,7 @@ int main()
 
 @pytest.fixture(scope="module")
 def rules(tmp_path_factory):
-    d = tmp_path_factory.mktemp("places")
-    src, exe = d / "places.cpp", d / "places"
-    src.write_text(PROGRAM)
-    subprocess.run(["g++", "-O2", "-std=c++17", "-I", CSRC, str(src), "-o", str(exe)], check=True)
+    exe = compiled(tmp_path_factory.mktemp("places"), "places", PROGRAM)
 
     def run(batches, dc=1.4, wide=1 << 63, by_k=1):
         text = ""
@@ -101,7 +109,7 @@ def rules(tmp_path_factory):
             text += f"{dc} {wide} {len(targets)} {by_k}\n"
             for n, u in targets:
                 text += f"{n >> 64} {n & (2**64 - 1)} {u}\n"
-        out = subprocess.run([str(exe)], input=text, capture_output=True, text=True, check=True)
+        out = subprocess.run([exe], input=text, capture_output=True, text=True, check=True)
         names = ("classes", "places", "jmax", "ymax", "gathered", "bad")
         return [dict(zip(names, map(int, line.split()))) for line in out.stdout.splitlines()]
 
@@ -167,6 +175,74 @@ def test_limits_near_the_square_root(rules, dc):
         assert r["bad"] == 0 and r["jmax"] < 2**32 - 6 and r["classes"] <= 8, (targets, r)
 
 
+# reads: dc, largest k, then 64 k of a group; prints the cut-off, its bound, the
+# largest j (all without floor(k/jlo) and the list's end)
+CUTOFF = r"""
+#include <cstdio>
+#include "wheel_place.h"
+using namespace mert;
+int main()
+{
+    double dc;
+    unsigned long long kf, k[64];
+    while (scanf("%lf %llu", &dc, &kf) == 2) {
+        double sum = 0;
+        for (auto &v : k) {
+            if (scanf("%llu", &v) != 1)
+                return 1;
+            sum += (double)v;
+        }
+        const uint64_t yc = wheel_cutoff(dc, sum / 64, kf, UINT64_MAX, UINT64_MAX);
+        uint64_t j = 0;
+        for (auto v : k)
+            j = std::max(j, wheel_last_j(v, yc, 1));
+        printf("%llu %llu %llu\n", (unsigned long long)yc,
+               (unsigned long long)wheel_cutoff_bound(dc, kf), (unsigned long long)j);
+    }
+}
+"""
+
+
+def test_dense_list_reaches_every_cutoff(tmp_path):
+    """The bound that sizes the dense list is at least the cut-off of every group, for
+    factors over the accepted range, k up to 2^63 and groups of close or equal k (where
+    the rounding of the mean counts), and j stays in range."""
+    rng = random.Random(9)
+    text, n = "", 0
+    for _ in range(4000):
+        dc = 10 ** rng.uniform(-7, 2.999)
+        kf = min(2**63 - 1, int(10 ** rng.uniform(0, 18.97)))
+        if rng.random() < 0.3:  # dc sqrt(k) just below a multiple of 4096
+            v = 4096 * rng.randrange(1, 10**6)
+            kf = max(1, min(2**63 - 1, int((v / dc) ** 2) - rng.randrange(3)))
+        spread = rng.choice([0, 0, 1e-15, 1e-9, 1e-3, 1])
+        ks = [kf - int(kf * spread * rng.random()) for _ in range(63)] + [kf]
+        text += f"{dc!r} {kf} " + " ".join(str(max(1, k)) for k in ks) + "\n"
+        n += 1
+    out = subprocess.run([compiled(tmp_path, "cutoff", CUTOFF)], input=text,
+                         capture_output=True, text=True, check=True).stdout.split("\n")
+    assert len(out) == n + 1
+    for line, given in zip(out, text.split("\n")):
+        if line:
+            yc, bound, j = map(int, line.split())
+            assert yc <= bound and j < 2**32 - 6, (given[:60], yc, bound, j)
+
+
+@pytest.mark.gpu
+def test_small_dense_factor_does_not_change_results(monkeypatch):
+    """A factor far below 1 (the accepted range starts above 0): the same array as the
+    full sums."""
+    n, u = 10**12 + 39, 10**11
+    tuning = pm.mertens_get_tuning()
+    try:
+        pm.mertens_set_tuning(dense_c=2e-4)
+        got = _array(n, u)
+    finally:
+        pm.mertens_set_tuning(**tuning)
+    monkeypatch.setenv("MERTENS_SHARE", "0")
+    assert np.array_equal(got, _array(n, u))
+
+
 def _array(n, u):
     plan = pm.mertens_plan([n], u)
     try:
@@ -203,17 +279,23 @@ def test_unlike_targets_equal_the_same_planned_alone(ns, wide_from, monkeypatch)
 def test_plan_info_needs_no_device():
     """Term counts of a plan from many threads at once, and inside a stream capture
     (which a copy on the default stream would break)."""
-    import threading
-
-    import torch
-
     ns = [10**12 + i for i in range(5)] + [7]
     plan = pm.mertens_plan(ns)
     try:
-        g, side = torch.cuda.CUDAGraph(), torch.zeros(1, device="cuda")
-        with torch.cuda.graph(g):
-            side += 1
+        # a capture of a stream that waits for the default stream: a copy on that would
+        # break it
+        with open("/proc/self/maps") as f:
+            rt = ctypes.CDLL(next(line.split()[-1] for line in f if "libcudart" in line))
+        side, graph = ctypes.c_void_p(), ctypes.c_void_p()
+        assert rt.cudaStreamCreate(ctypes.byref(side)) == 0
+        assert rt.cudaStreamBeginCapture(side, 0) == 0
+        try:
             inside = [pm.mertens_plan_info(plan, i) for i in range(len(ns))]
+        finally:
+            ended = rt.cudaStreamEndCapture(side, ctypes.byref(graph))
+            rt.cudaStreamDestroy(side)
+        assert ended == 0
+        rt.cudaGraphDestroy(graph)
         got = [None] * 16
         start = threading.Barrier(16)
 
