@@ -1071,7 +1071,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
 static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count, mertens_u128 u,
                        uint64_t block_len, const mertens_tuning &tn, bool window = false,
                        uint64_t w_first = 1, uint64_t w_last = UINT64_MAX,
-                       mertens_table_s *table = nullptr, bool widen = true)
+                       mertens_table_s *table = nullptr, bool *longer = nullptr)
 {
     if (!out)
         return MERTENS_EINVAL;
@@ -1392,8 +1392,11 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     // up every large prime per block and SM, and each block has seven launches (16
     // blocks of 2^28 y from 10^13, n = 10^20: 12.55 -> 10.12 ms as four).  Without
     // the memory for it: block_len y (mertens_plan_window)
-    if (window && widen && span > block_len)
-        block_len = std::max(block_len, std::min({4 * block_len, (uint64_t)1 << 30, span}));
+    if (longer && span > block_len) {
+        const uint64_t l = std::min({4 * block_len, (uint64_t)1 << 30, span});
+        *longer = l > block_len;
+        block_len = std::max(block_len, l);
+    }
     p->block_len = block_len;
     p->nblocks = (span + block_len - 1) / block_len;
     if (window) {
@@ -2612,11 +2615,12 @@ int mertens_plan_window(mertens_plan_t *out, const mertens_u128 *n, size_t count
         set_last_error("mertens_plan_window: need 1 <= y_first <= y_last");
         return MERTENS_EINVAL;
     }
-    const int rc = plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last);
-    if (rc != MERTENS_ENOMEM)
+    bool longer = false;  // the blocks are longer than block_len
+    const int rc = plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last,
+                               nullptr, &longer);
+    if (rc != MERTENS_ENOMEM || !longer)
         return rc;
-    return plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last, nullptr,
-                       false);
+    return plan_create(out, n, count, u, block_len, tuning_now(), true, y_first, y_last);
 }
 
 int mertens_window_result(mertens_plan_t p, size_t i, uint64_t *S_loc, uint64_t *coef,

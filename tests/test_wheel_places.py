@@ -314,3 +314,24 @@ def test_plan_info_needs_no_device():
                 [(x["direct_terms"], x["gathered_terms"]) for x in want]
     finally:
         pm.mertens_destroy(plan)
+
+
+def test_windows_are_planned_again_only_for_shorter_blocks():
+    """A window plan that gets no memory is tried again with block_len only when its
+    blocks were longer than that (each attempt asks for the same number of buffers)."""
+    asked = []
+
+    def alloc(nbytes, stream, ctx):
+        asked[-1] += 1
+        return 0
+
+    pm.mertens_set_allocator(alloc, lambda *a: None)
+    try:
+        for span in (10**6, 10**6 + 1):
+            asked.append(0)
+            with pytest.raises(pm.MertensError) as e:
+                pm.mertens_plan_window([10**14 + 7], 10**9, 10**9 + span - 1, 3 * 10**9, 10**6)
+            assert e.value.code == pm.MERTENS_ENOMEM
+    finally:
+        pm.mertens_set_allocator()
+    assert asked[0] > 0 and asked[1] == 2 * asked[0]
