@@ -1375,6 +1375,26 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     p->y_first = window ? w_first : 1;
     p->y_last = window ? std::min(w_last, p->y_max) : p->y_max;
     const uint64_t span = p->y_last >= p->y_first ? p->y_last - p->y_first + 1 : 0;
+    // end of the shared-memory gather tiles of all entries
+    {
+        // Gathered terms per y near y are about (n / y^2) ln X summed over
+        // the targets; shared-memory tiles pay while that is at least ~2,
+        // i.e. up to y ~ sqrt(sum n ln X / 2) (2.5e8 for n = 1e16, X = 2.5e5).
+        // A tile pays while its terms (32768 (sum n ln X) / y^2) are at least
+        // a quarter of the entries it must check (all of them, E).
+        double acc = 0;
+        for (size_t i = 0; i < count; ++i)
+            acc += ((double)p->n[i] + 18446744073709551616.0 * (double)p->n_hi[i]) *
+                   std::log((double)std::max<uint64_t>(p->X[i], 2));
+        const double E = (double)std::max<uint64_t>(p->nent, 1);
+        const double gs = tn.gather_scale > 0 ? tn.gather_scale : 1.0;
+        uint64_t ys = (uint64_t)(gs * std::min(std::sqrt(acc / 2.0),
+                                               std::sqrt(4.0 * kGatherTile * acc / E)));
+        const char *e = getenv("MERTENS_GATHER_END");
+        if (e)
+            ys = strtoull(e, nullptr, 10);
+        p->gather_smem_end = std::min(ys, p->y_max);
+    }
     if (block_len == 0) {
         // one block when it fits 2^28 y, else 2^28 (up to 2^36 y) or 2^30 y blocks
         uint64_t cap = p->y_last > (1ull << 36) ? (1ull << 30) : (1ull << 28);
@@ -1390,9 +1410,13 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
     }
     // a longer window's blocks hold four times as many y, up to 2^30: the sieve sets
     // up every large prime per block and SM, and each block has seven launches (16
-    // blocks of 2^28 y from 10^13, n = 10^20: 12.55 -> 10.12 ms as four).  Without
+    // blocks of 2^28 y from 10^13, n = 10^20: 12.55 -> 10.12 ms as four).  Not where
+    // the tiles of all entries end inside a short window: the rest of that block takes
+    // the global path, a block after it tiles for its large k (n = 10^16, [1, 4e9] in
+    // 2^28 y: gather 48.1 ms, as four blocks 50.5; [1, 4e10]: 55.1 and 52.4).  Without
     // the memory for it: block_len y (mertens_plan_window)
-    if (longer && span > block_len) {
+    if (longer && span > block_len &&
+        (p->y_first > p->gather_smem_end || span >= 32 * block_len)) {
         const uint64_t l = std::min({4 * block_len, (uint64_t)1 << 30, span});
         *longer = l > block_len;
         block_len = std::max(block_len, l);
@@ -1467,25 +1491,6 @@ static int plan_create(mertens_plan_t *out, const mertens_u128 *n, size_t count,
         }
     }
     const double kItemWork = 2.0e5;
-    {
-        // Gathered terms per y near y are about (n / y^2) ln X summed over
-        // the targets; shared-memory tiles pay while that is at least ~2,
-        // i.e. up to y ~ sqrt(sum n ln X / 2) (2.5e8 for n = 1e16, X = 2.5e5).
-        // A tile pays while its terms (32768 (sum n ln X) / y^2) are at least
-        // a quarter of the entries it must check (all of them, E).
-        double acc = 0;
-        for (size_t i = 0; i < count; ++i)
-            acc += ((double)p->n[i] + 18446744073709551616.0 * (double)p->n_hi[i]) *
-                   std::log((double)std::max<uint64_t>(p->X[i], 2));
-        const double E = (double)std::max<uint64_t>(p->nent, 1);
-        const double gs = tn.gather_scale > 0 ? tn.gather_scale : 1.0;
-        uint64_t ys = (uint64_t)(gs * std::min(std::sqrt(acc / 2.0),
-                                               std::sqrt(4.0 * kGatherTile * acc / E)));
-        const char *e = getenv("MERTENS_GATHER_END");
-        if (e)
-            ys = strtoull(e, nullptr, 10);
-        p->gather_smem_end = std::min(ys, p->y_max);
-    }
     std::vector<GatherTile> gtiles;
     std::vector<GatherItem> gitems;
     // Blocks above the tile range: tiles over the whole block for the

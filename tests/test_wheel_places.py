@@ -335,3 +335,16 @@ def test_windows_are_planned_again_only_for_shorter_blocks():
     finally:
         pm.mertens_set_allocator()
     assert asked[0] > 0 and asked[1] == 2 * asked[0]
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("y1,blocks", [(1, 10), (10**9 + 1, 3)])
+def test_short_windows_over_the_tile_range_keep_their_blocks(y1, blocks):
+    """Ten blocks from y = 1, where the tiles of all entries end inside, and above."""
+    bl = 1 << 22
+    plan = pm.mertens_plan_window([10**14 + 7], y1, y1 + 10 * bl - 1, 3 * 10**9, bl)
+    try:
+        pm.mertens_run(plan)
+        assert pm.mertens_run_stats_get(plan)["blocks"] == blocks
+    finally:
+        pm.mertens_destroy(plan)
