@@ -73,12 +73,14 @@ struct WheelClass {
 // Splits the targets into classes.  For every entry of target i floor(k/jlo) is at
 // least n/(2X) (k/jlo = floor(floor(n/x) / (floor(X/x) + 1)), and x (floor(X/x) + 1)
 // <= X + x <= 2X).  A class's head is the largest target left; a target joins it when
-// its n/(2X) reaches the head's largest cut-off, dc sqrt(n), or -- sieve limits near
-// sqrt(n) bound every cut-off -- an eighth of the head's u, and in any case what keeps
-// the head's j below 2^32.  With automatic limits that leaves targets below about
-// 3 sqrt(n) out: 64 targets near 10^14 and requests from 10^10 to 10^15 are one class.
-// Targets with k up to `wide_from` have one-word entries.  Returns the classes with
-// their places; *end is the first place after them all (lookups come there).
+// its n/(2X) reaches the head's largest cut-off, dc sqrt(n), or -- limits near sqrt(n)
+// and small targets bound every cut-off -- an eighth of the head's u, and in any case
+// what keeps the head's j below 2^32.  So targets alike are one class, and a class's u
+// (or, with one entry, n) are below a quarter of the last one's: 32 classes at most.
+// With automatic limits targets below about 3 sqrt(n) are left out: 64 targets near
+// 10^14 and requests from 10^10 to 10^15 are one class.  Targets with k up to
+// `wide_from` have one-word entries.  Returns the classes with their places; *end is
+// the first place after them all (lookups come there).
 inline std::vector<WheelClass> wheel_classes(std::vector<WheelTarget> &t, double dc,
                                              unsigned __int128 wide_from, uint64_t *end)
 {
@@ -94,9 +96,9 @@ inline std::vector<WheelClass> wheel_classes(std::vector<WheelTarget> &t, double
             if (t[i].n > t[head].n)
                 head = i;
         const uint64_t k = (uint64_t)std::min(t[head].n, wide_from);
-        const uint64_t least = k / kWheelMaxJ + 12;
+        const uint64_t least = k < kWheelMaxJ ? 0 : k / kWheelMaxJ + 12;
         const uint64_t want = std::max((uint64_t)(dc * std::sqrt((double)k)) + 12, least);
-        const uint64_t thr = std::min(want, std::max(t[head].u / 8, least));
+        const uint64_t thr = std::max(least, std::min(want, t[head].u / 8));
         place = (place + kWheelGroup - 1) / kWheelGroup * kWheelGroup;
         WheelClass c{place, 0};
         rest.clear();

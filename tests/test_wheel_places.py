@@ -161,6 +161,15 @@ def test_like_targets_share_a_class(rules):
         assert r["classes"] == 1
 
 
+def test_many_small_targets(rules):
+    """A hundred thousand tiny targets make a few classes, not one each."""
+    rng = random.Random(6)
+    for ns in ([3] * 100_000 + [1], [rng.randrange(1, 30) for _ in range(100_000)],
+               [int(10 ** rng.uniform(0, 9)) for _ in range(100_000)]):
+        r, = rules([auto_u(ns)])
+        assert r["bad"] == 0 and r["classes"] <= 6
+
+
 @pytest.mark.parametrize("dc", [0.7, 1.4, 7.5, 900.0])
 def test_limits_near_the_square_root(rules, dc):
     """Explicit limits: every cut-off is bound by floor(k/jlo); the classes stay few."""
@@ -271,6 +280,23 @@ def test_unlike_targets_equal_the_same_planned_alone(ns, wide_from, monkeypatch)
     finally:
         pm.mertens_destroy(plan)
     monkeypatch.delenv("MERTENS_WIDE_FROM", raising=False)
+    for n, (u, arr) in zip(ns, got):
+        assert np.array_equal(arr, _array(n, u)), n
+
+
+@pytest.mark.gpu
+def test_unlike_targets_on_a_table():
+    """Lookups, tiny targets with terms and large ones in one plan on a table."""
+    table = pm.mertens_table_create(1 << 26, 10**15)
+    ns = [10**i for i in range(15)] + [(1 << 26) + 1, 3]
+    try:
+        plan = pm.mertens_plan_on_table(table, ns)
+        pm.mertens_run(plan)
+        got = [(pm.mertens_plan_info(plan, i)["u"], pm.mertens_result(plan, i, entries=True)[1])
+               for i in range(len(ns))]
+        pm.mertens_destroy(plan)
+    finally:
+        pm.mertens_table_destroy(table)
     for n, (u, arr) in zip(ns, got):
         assert np.array_equal(arr, _array(n, u)), n
 
