@@ -347,10 +347,12 @@ __device__ __forceinline__ void dense_float(const uint4 *el, uint32_t n, const f
 }
 
 // Linear mode: as the float mode with the chunk's middle ym taken out: with
-// q0 = floor(k/(3 ym)) and r0 = k - 3 ym q0, k/(3y) = q0 + (r0 - 3 q0 (y - ym))/(3y),
-// whose second part is below 10^6 in size for k <= 900 y0^2 (y0 the chunk's
-// start, |y - ym| <= 3072): four roundings of 2^-24, so it errs by less than 1/4,
-// and the sum of 2048 of them fits 32 bits.  Staged {1/(3y), -y, y - ym}.
+// q0 = floor(k/(3 ym)) and r0 = k - 3 ym q0, k/(3y) = q0 + (r0 - 3 q0 (y - ym))/(3y).
+// For k <= 900 y0^2 (y0 the chunk's start, |y - ym| <= 3071) q0 is below 300 y0 and the
+// second part below 300 3071 + 1 = 921 301 in size.  Six roundings of a relative 2^-24
+// at most -- two in q0, then the product by 3, the multiply-add, 3y and its reciprocal
+// -- make 0.3295 of it: less than the 1/3 needed, so that 900 is the most the rule may
+// be.  The sum of 2048 of them fits 32 bits.  Staged {1/(3y), -y, y - ym}.
 __device__ __forceinline__ void dense_linear(const uint4 *el, uint32_t n, const uint64_t q0[2],
                                              const float r0[2], const uint32_t kl[2],
                                              uint64_t out[2])
