@@ -19,13 +19,15 @@ import numpy as np
 
 from . import _lib as L
 
-# Measured per-unit costs on GB300 (n = 10^16 workload: 68 ms of sieve for
-# 4e10 y, 58 ms for 1.0e11 dense terms, 65 ms for 6.2e10 gathered terms), in
-# seconds: sieve per y, dense (squarefree) term, gathered term.  Integrated
-# over [1, y_max] they give 0.19 s, the measured step.
-SIEVE_S_PER_Y = 1.7e-12
-DENSE_S_PER_TERM = 0.58e-12
-GATHER_S_PER_TERM = 1.05e-12
+# Measured per-unit costs of window plans on GB300 (n = 10^16, u = 4 10^10, the window
+# [1, y_max]: 43.3 ms of sieve for 4e10 y, 52.3 ms for 1.0e11 dense terms, 52.4 ms for
+# 6.2e10 gathered terms), in seconds: sieve per y, dense (squarefree) term, gathered
+# term.  Integrated over [1, y_max] they give about the measured 0.149 s.  (A whole run
+# over the integers coprime to 6 takes 0.039 s on one GPU: windows return sums over
+# every y, so sharding such a target pays from about four ranks on.)
+SIEVE_S_PER_Y = 1.08e-12
+DENSE_S_PER_TERM = 0.52e-12
+GATHER_S_PER_TERM = 0.85e-12
 
 
 def work_density(y: np.ndarray, n: int, X: int, c: float = 1.4) -> np.ndarray:
