@@ -302,6 +302,22 @@ def test_unlike_targets_on_a_table():
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("ns", [[7 * 10**11 + 3], [7 * 10**11 + 3, 7 * 10**11 + 10**6, 10**6]])
+def test_table_whose_list_ends_below_the_factor_times_sqrt_n(ns):
+    """1.4 sqrt(n) lies above the table, floor(k/jlo) of every entry below its end."""
+    table = pm.mertens_table_create(1 << 20, 10**12)
+    try:
+        plan = pm.mertens_plan_on_table(table, ns, 10**6)
+        pm.mertens_run(plan)
+        got = [pm.mertens_result(plan, i, entries=True)[1] for i in range(len(ns))]
+        pm.mertens_destroy(plan)
+    finally:
+        pm.mertens_table_destroy(table)
+    for n, arr in zip(ns, got):
+        assert np.array_equal(arr, _array(n, 10**6)), n
+
+
+@pytest.mark.gpu
 def test_plan_info_needs_no_device():
     """Term counts of a plan from many threads at once, and inside a stream capture
     (which a copy on the default stream would break)."""
