@@ -620,7 +620,7 @@ static int plan_create_wheel(mertens_plan_t *out, mertens_plan_s *p, const std::
             p->gathered.back() += W.jhi >= W.jlo ? W.jhi - W.jlo + 1 : 0;
         }
         if (table)
-            cut = std::max(cut, first_cutoff(n[i], X, dc, wide_from));
+            cut = std::max(cut, first_cutoff(n[i], X, dense_factor(tn), wide_from));
         E += X;
         // the largest y read: a direct term's, or the gathered range's of x = 1
         const uint64_t yg = (uint64_t)(n[i] / ((u128)X + 1));
